@@ -1241,13 +1241,48 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 const TcKnobs kDefaultKnobs = {0, 0, 0, 0, -1, 0, 0, 0, 0, 0};
 
-int choose_bn(int N, bool pair, const TcKnobs& kn) {
+// Tile width. Wide tiles move the fewest operand bytes per product, but a product of few tiles leaves most of the chip
+// idle, and the read-out of its last (often only) tile, whose time grows with the width, is not hidden by anything. The
+// CTA-pair form therefore takes the width with the smallest modelled time (in cycles):
+//   K block (128 bytes of K): the tensor pipe's 2 cycles per column, at least 480 (step latency), at least the operand
+//     bytes of all resident CTAs at the 5500 bytes per cycle that L2 delivers to the whole chip;
+//   read-out: 1500 + 16 (16-bit) or 24 (fp32) per column, half as much again with mirror stores;
+//   waves of tiles, the read-out hidden behind the next tile's products except in the last wave.
+// Measured against width 256: symmetric 1024^3 tf32 22.2 -> 16.1 us (width 64), 1000^3 half 18.3 -> 12.8 (64), 2048^3 tf32
+// 32.5 -> 27.2 (128); 12 x 768^3 19.9 -> 17.8 (192); 4 x 517 x 517 x 1003 53 -> 22 (64); 24 x 1024^3 and everything
+// larger stays at 256 (42.8 us, 128: 48.5). The single-CTA form keeps the widest tile. (Edge tiles only compute the
+// columns that exist, rounded up to 16, or 32 for a CTA pair.)
+int choose_bn(const GemmDesc& g, bool pair, const TcKnobs& kn, int num_sms) {
   const int q = pair ? 32 : 16;
   if (kn.bn >= q && kn.bn <= 256 && kn.bn % q == 0) return kn.bn;
-  // widest tile; edge tiles only compute the columns that exist (rounded up to 16, or 32 for a CTA pair), so
-  // a wide tile wastes at most q - 1 columns per tile row
-  const int r = (N + q - 1) & ~(q - 1);
-  return r < 256 ? r : 256;
+  const int r = (g.N + q - 1) & ~(q - 1);
+  const int top = r < 256 ? r : 256;
+  // (the residual norm's partial sums are laid out per tile by the caller, the split-B panels are one tile wide)
+  if (!pair || top <= 64 || g.epilogue == EPI_RESID_NORM || g.b_split == 2) return top;
+  const int esize = (int)dtype_size(g.in_dtype), span = KBYTES / esize;
+  const double pairs = num_sms / 2;
+  const double out_col = (g.out_dtype == F32 ? 24.0 : 16.0) * (g.symmetric || g.transpose_out ? 1.5 : 1.0);
+  const bool b_mn = g.sb_k[0] != 1;
+  int best = top;
+  double best_t = 0.0;
+  for (int bn = top; bn >= 64; bn = (bn - 1) & ~31) {
+    const int tm = (g.M + 255) / 256, tn = (g.N + bn - 1) / bn;
+    double tiles = 0.0;
+    for (int i = 0; i < tm; ++i) { const int first = g.symmetric ? i * 256 / bn : 0; if (first < tn) tiles += tn - first; }
+    tiles *= g.batch;
+    double kb = (g.K[0] + span - 1) / span;
+    if (g.nseg == 2) kb += ((g.seg1_identity ? bn : g.K[1]) + span - 1) / span;
+    const int bcols = b_mn ? (bn / 2 + span - 1) / span * span : bn / 2;      // an MN-major operand moves whole boxes
+    const double bytes = (128.0 + bcols) * KBYTES, resident = 2.0 * (tiles < pairs ? tiles : pairs);
+    double block = 2.0 * bn;
+    if (block < 480.0) block = 480.0;
+    if (block < bytes * resident / 5500.0) block = bytes * resident / 5500.0;
+    const double read_out = 1500.0 + bn * out_col, products = kb * block;
+    const double waves = (double)(long long)((tiles + pairs - 1.0) / pairs);
+    const double t = (waves - 1.0) * (products > read_out ? products : read_out) + products + read_out;
+    if (bn == top || t < best_t) { best = bn; best_t = t; }
+  }
+  return best;
 }
 
 int choose_tile_m_impl(int M, const TcKnobs& kn) {
@@ -1342,7 +1377,7 @@ TcKnobs tc_knobs_from_env() {
 
 int gemm_tc_partials_per_batch(const GemmDesc& g, const TcKnobs* knobs) {
   const TcKnobs& kn = knobs ? *knobs : kDefaultKnobs;
-  const int bn = choose_bn(g.N, choose_pair(g.M, g.N, kn), kn), tmh = choose_tile_m_impl(g.M, kn);
+  const int bn = choose_bn(g, choose_pair(g.M, g.N, kn), kn, 148), tmh = choose_tile_m_impl(g.M, kn);
   return ((g.M + tmh - 1) / tmh) * ((g.N + bn - 1) / bn) * (tmh == 256 ? 2 : 1) * EPI_WARPS;
 }
 
@@ -1360,7 +1395,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word,
   p.M = g.M; p.N = g.N; p.batch = g.batch;
   p.tile_m = choose_tile_m_impl(g.M, kn);
   p.pair = choose_pair(g.M, g.N, kn) ? 1 : 0;
-  p.BN = choose_bn(g.N, p.pair != 0, kn);
+  p.BN = choose_bn(g, p.pair != 0, kn, num_sms);
   p.tiles_m = (g.M + p.tile_m - 1) / p.tile_m;
   p.tiles_n = (g.N + p.BN - 1) / p.BN;
   p.tiles_per_matrix = p.tiles_m * p.tiles_n;
