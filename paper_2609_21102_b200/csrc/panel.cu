@@ -273,13 +273,19 @@ cudaError_t panel_apply_launch(const float* In, long long in_bs, int ld_in, cons
 // ---------------------------------------------------------------------------------------------
 // One-sided Jacobi eigensolver of the symmetric positive semidefinite core C = sum of partials
 // (l x l). Columns of A = C V are rotated pairwise until mutually orthogonal; then ||a_j|| are the
-// eigenvalues and V the eigenvectors. One warp per column pair (round-robin pairing), lanes over
-// rows, dot products by warp shuffles; fp64 throughout. Outputs (sorted by decreasing eigenvalue):
+// eigenvalues and the normalised columns the eigenvectors (A = C V = V diag(lambda), so V itself is not carried).
+// Eight lanes per column pair (round-robin pairing), dot products by warp shuffles; fp64 throughout.
+// Outputs (sorted by decreasing eigenvalue):
 //   s[b, l]     = sqrt(eigenvalue)             (singular values of the panel whose Gram this is)
 //   E[b, l, l]  = eigenvectors in columns      (fp32)
 //   Es[b, l, l] = E diag(1/s)                  (fp32; zero column where s is numerically zero)
-// With `signed_input` the matrix is a general symmetric one (Rayleigh quotient of Algorithm 2):
-// eigenvalues keep their sign (lambda_j = v_j^T a_j), sorted by decreasing magnitude, s = lambda.
+// With `signed_input` the matrix is a general symmetric one (Rayleigh quotient of Algorithm 2), sorted by decreasing
+// magnitude, s = lambda. It is shifted by 2 ||C||_F first and the shift taken off the eigenvalues again: the columns of
+// C V itself are orthogonal as soon as V spans {v(+mu), v(-mu)}, so a pair of eigenvalues of equal magnitude and opposite
+// sign stays mixed in them by an angle up to 1e-11 over the relative gap of the magnitudes; the shifted pair is far apart.
+// What bounds it is the chain of dependent operations of a round (l - 1 rounds a sweep, one barrier each, half a dozen
+// sweeps), not its arithmetic: the block has only the warps that own pairs, and the rotation angle, which merely steers
+// the iteration, comes from approximate fp32 functions.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -295,7 +301,12 @@ __device__ __forceinline__ double group8_sum(double v) {
   return v;
 }
 
-constexpr int JAC_THREADS = 256;        // 32 column pairs x 8 lanes
+// fp32 reciprocal and square root of the hardware's approximation unit (about 1e-7, no special-case handling)
+__device__ __forceinline__ float rcp_approx(float x) { float r; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
+__device__ __forceinline__ float sqrt_approx(float x) { float r; asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
+__device__ __forceinline__ float rsqrt_approx(float x) { float r; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
+
+constexpr int JAC_THREADS = 256;        // at most 32 column pairs x 8 lanes
 constexpr int JAC_NR = MAX_L / 8;       // rows per lane
 
 __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* __restrict__ partial, int nchunk, int l,
@@ -305,43 +316,36 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
   extern __shared__ double sm[];
   const int ls = l | 1;       // column stride (odd: the four pairs of a warp start in different banks)
   double* A = sm;             // column-major: A[c * ls + r]
-  double* V = sm + MAX_L * (MAX_L + 1);     // column-major
-  __shared__ double lam[MAX_L];
+  __shared__ double lam[MAX_L];       // column norms (eigenvalues of the scaled, shifted matrix), then the eigenvalues
+  __shared__ double len[MAX_L];
   __shared__ double nrm2[MAX_L];      // squared column norms of A, carried along by the rotations
   __shared__ int order[MAX_L];
   __shared__ int rotated;
-  const int bz = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int bz = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nt = blockDim.x;
   const double* pb = partial + (long long)bz * nchunk * l * l;
-  for (int e = tid; e < l * l; e += blockDim.x) {
-    const int r = e / l, c = e % l;
-    double t = 0.0, u = 0.0;
-    for (int ch = 0; ch < nchunk; ++ch) {
-      t += pb[(long long)ch * l * l + r * l + c];
-      u += pb[(long long)ch * l * l + c * l + r];
-    }
-    A[c * ls + r] = 0.5 * (t + u);
-    V[c * ls + r] = (r == c) ? 1.0 : 0.0;
+  for (int e = tid; e < l * l; e += nt) {
+    double t = 0.0;
+#pragma unroll 8
+    for (int ch = 0; ch < nchunk; ++ch) t += pb[(long long)ch * l * l + e];
+    A[(e % l) * ls + e / l] = t;
+  }
+  __syncthreads();
+  // symmetrise (one thread per pair of entries)
+  for (int e = tid; e < l * l; e += nt) {
+    const int i = e / l, j = e % l;
+    if (i < j) { const double a = 0.5 * (A[i * ls + j] + A[j * ls + i]); A[i * ls + j] = a; A[j * ls + i] = a; }
   }
   __syncthreads();
   const int np = (l + 1) & ~1;        // players, padded to even
   const int npairs = np / 2;
-  // Eight lanes per column pair, four pairs per warp: the three dot products of a pair take three shuffle steps
-  // each instead of five, and a round issues a sixth of the shuffles of the one-warp-per-pair form (whose
-  // shuffle traffic, not its arithmetic, filled the round).
+  // Eight lanes per column pair, four pairs per warp: the dot product of a pair takes three shuffle steps.
   const int grp = tid >> 3, sub = tid & 7;
   const int nr = (l + 7) >> 3;        // rows per lane actually present
-  // The eigenvector accumulation V is needed only for a signed spectrum (to tell the sign of an eigenvalue). For
-  // a Gram matrix the columns of A converge to lambda_j v_j with lambda_j >= 0, so the eigenvectors are the
-  // normalised columns: the rotations skip V, a third of the fp64 work (fp64 issue is what bounds this kernel).
-  const bool track_v = signed_input != 0;
-  int sweep = 0;
-  for (; sweep < max_sweeps; ++sweep) {
-    if (tid == 0) rotated = 0;
-    // Squared column norms, exact at the start of every sweep. Within the sweep a rotation by tan t moves
-    // t gamma from one column's squared norm to the other's (alpha' = alpha - t gamma, beta' = beta + t gamma), so
-    // a round computes one dot product per pair instead of three; the sweep that finds nothing to rotate, which
-    // ends the iteration, has tested every pair against exact norms.
-    for (int j0 = 0; j0 < l; j0 += JAC_THREADS / 8) {      // (the same trip count for every lane: shuffles inside)
+  // Squared norms of the columns (Frobenius norm for the shift, and for the scale: the matrix is multiplied by the power
+  // of two that brings its norm near one, exactly, so that squared norms and dot products of columns down to 1e-18 of it
+  // are ordinary fp32 numbers for the angle).
+  auto column_norms = [&]() {
+    for (int j0 = 0; j0 < l; j0 += nt >> 3) {      // (the same trip count for every lane: shuffles inside)
       const int j = j0 + grp;
       double acc = 0.0;
 #pragma unroll
@@ -353,6 +357,32 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
       if (sub == 0 && j < l) nrm2[j] = acc;
     }
     __syncthreads();
+  };
+  column_norms();
+  double fro2 = 0.0;
+  for (int j = 0; j < l; ++j) fro2 += nrm2[j];
+  const double fro = sqrt(fro2);
+  double scale = 1.0, unscale = 1.0;
+  if (fro > 1e-290 && fro < 1e290) {
+    const int ex = (int)((__double_as_longlong(fro) >> 52) & 0x7ff);             // fro in [2^(ex-1023), 2^(ex-1022))
+    scale = __longlong_as_double((long long)(2046 - ex) << 52);                  // 2^(1023 - ex)
+    unscale = __longlong_as_double((long long)ex << 52);
+  }
+  const double shift = signed_input ? 2.0 * fro * scale : 0.0;
+  __syncthreads();
+  for (int e = tid; e < l * l; e += nt) {
+    const int c = e / l, r = e % l;
+    A[c * ls + r] = A[c * ls + r] * scale + ((r == c) ? shift : 0.0);
+  }
+  __syncthreads();
+  int sweep = 0;
+  for (; sweep < max_sweeps; ++sweep) {
+    if (tid == 0) rotated = 0;
+    // Squared column norms, exact at the start of every sweep. Within the sweep a rotation by tan t moves
+    // t gamma from one column's squared norm to the other's (alpha' = alpha - t gamma, beta' = beta + t gamma), so
+    // a round computes one dot product per pair instead of three; the sweep that finds nothing to rotate, which
+    // ends the iteration, has tested every pair against exact norms.
+    column_norms();
     for (int round = 0; round < np - 1; ++round) {
       int p = 0, q = l;
       if (grp < npairs) {
@@ -366,8 +396,9 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
       }
       const bool live = q < l;            // (a pair with the padding player, or a group beyond the pairs, idles)
       double* ap = A + p * ls; double* aq = A + (live ? q : p) * ls;
+      const double alpha = live ? nrm2[p] : 0.0, beta = live ? nrm2[q] : 0.0;
       double x[JAC_NR], y[JAC_NR];
-      double pg = 0.0;
+      double pg0 = 0.0, pg1 = 0.0;
 #pragma unroll
       for (int i = 0; i < JAC_NR; ++i) {
         if (i < nr) {
@@ -375,58 +406,40 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
           const bool in = live && r < l;
           x[i] = in ? ap[r] : 0.0;
           y[i] = in ? aq[r] : 0.0;
-          pg = fma(x[i], y[i], pg);
+          if (i & 1) pg1 = fma(x[i], y[i], pg1); else pg0 = fma(x[i], y[i], pg0);
         }
       }
-      const double gamma = group8_sum(pg);
-      const double alpha = live ? nrm2[p] : 0.0, beta = live ? nrm2[q] : 0.0;
+      const double gamma = group8_sum(pg0 + pg1);
       // rotate when |gamma| > 1e-11 sqrt(alpha beta) (compared in squares): the eigenvalues are then good to about
       // 1e-22 and the vectors to 1e-11 over the relative gap, far beyond the fp32 outputs
       if (live && gamma != 0.0 && gamma * gamma > 1e-22 * (alpha * beta)) {
         if (sub == 0) rotated = 1;
-        // The rotation angle only steers the iteration (any exact rotation keeps V orthogonal and the invariants
-        // intact), so tan is computed in fp32 from the exponent-scaled pair (beta - alpha, 2 gamma); cos comes
-        // from an fp32 reciprocal square root refined by two Newton steps in fp64, which makes c^2 + s^2 = 1 hold
-        // to fp64 rounding. A rotation then leaves 1e-7 of the inner product instead of none, and the pair's
-        // next visit removes that. The chain of dependent fp64 operations, which is the latency of a round,
-        // shrinks to a third. Out-of-range exponents take the fp64 formula.
+        // The rotation angle only steers the iteration (any exact rotation keeps the invariants intact), so tan is
+        // computed in fp32 with approximate functions; cos comes from an fp32 reciprocal square root refined by two
+        // Newton steps in fp64, which makes c^2 + s^2 = 1 hold to fp64 rounding. A rotation then leaves 1e-7 of the
+        // inner product instead of none, and the pair's next visit removes that. The chain of dependent fp64
+        // operations, which is the latency of a round, shrinks to a third. What fp32 cannot hold takes the fp64 formula.
         const double d = beta - alpha, g2 = 2.0 * gamma;
-        const double big = fmax(fabs(d), fabs(g2));
-        const int ex = (int)((__double_as_longlong(big) >> 52) & 0x7ff);
-        const double sc = __longlong_as_double((long long)(2046 - ex) << 52);       // 2^(1023 - ex)
-        const float df = (float)(d * sc), gf = (float)(g2 * sc);
-        double c, sn, tg;
-        if (ex >= 1 && ex <= 2045 && fabsf(gf) > 1e-30f) {
-          const float zf = df / gf, az = fabsf(zf);
+        const float df = (float)d, gf = (float)g2;
+        double t;
+        if (fabsf(gf) > 1e-30f && fabsf(df) < 1e30f) {
+          const float zf = df * rcp_approx(gf), az = fabsf(zf);
           // t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)): the root of t^2 + 2 zeta t - 1 = 0 of smaller magnitude
-          const float tf = (az > 1e15f) ? 0.5f / zf : copysignf(1.0f / (az + sqrtf(fmaf(zf, zf, 1.0f))), zf);
-          const double t = (double)tf;
-          const double w = fma(t, t, 1.0), h = 0.5 * w;            // w in [1, 2]
-          double yv = (double)rsqrtf((float)w);
-          yv = yv * fma(-h * yv, yv, 1.5);
-          yv = yv * fma(-h * yv, yv, 1.5);
-          c = yv; sn = yv * t;
-          tg = t * gamma;
+          t = (double)copysignf((az > 1e15f) ? 0.5f * rcp_approx(az) : rcp_approx(az + sqrt_approx(fmaf(zf, zf, 1.0f))), zf);
         } else {
           const double zeta = d / g2;
-          const double w = 1.0 + zeta * zeta;
-          const double root = w * rsqrt(w);                          // sqrt(1 + zeta^2)
-          const double t = ((zeta >= 0.0) ? 1.0 : -1.0) / (fabs(zeta) + root);
-          c = rsqrt(1.0 + t * t); sn = c * t;
-          tg = t * gamma;
+          t = ((zeta >= 0.0) ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
         }
+        const double w = fma(t, t, 1.0), h = 0.5 * w;                // w in [1, 2]
+        double c = (double)rsqrt_approx((float)w);
+        c = c * fma(-h * c, c, 1.5);
+        c = c * fma(-h * c, c, 1.5);
+        const double sn = c * t, tg = t * gamma;
         if (sub == 0) { nrm2[p] = alpha - tg; nrm2[q] = beta + tg; }
-        double* vp = V + p * ls; double* vq = V + q * ls;
 #pragma unroll
         for (int i = 0; i < JAC_NR; ++i) {
           const int r = sub + 8 * i;
-          if (i < nr && r < l) {
-            ap[r] = c * x[i] - sn * y[i]; aq[r] = sn * x[i] + c * y[i];
-            if (track_v) {
-              const double a = vp[r], b = vq[r];
-              vp[r] = c * a - sn * b; vq[r] = sn * a + c * b;
-            }
-          }
+          if (i < nr && r < l) { ap[r] = c * x[i] - sn * y[i]; aq[r] = sn * x[i] + c * y[i]; }
         }
       }
       __syncthreads();
@@ -436,24 +449,11 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
   }
   if (tid == 0 && sweep >= max_sweeps && status) atomicOr(&status[bz], 2);
   // eigenvalues
-  if (warp < 32) {
-    for (int j = warp; j < l; j += (blockDim.x >> 5)) {
-      const double* aj = A + j * ls; const double* vj = V + j * ls;
-      const double a0 = (lane < l) ? aj[lane] : 0.0, a1 = (lane + 32 < l) ? aj[lane + 32] : 0.0;
-      const double v0 = (lane < l) ? vj[lane] : 0.0, v1 = (lane + 32 < l) ? vj[lane + 32] : 0.0;
-      const double nrm = sqrt(warp_sum(a0 * a0 + a1 * a1));
-      const double rq = warp_sum(a0 * v0 + a1 * v1);
-      if (lane == 0) lam[j] = signed_input ? ((rq >= 0.0) ? nrm : -nrm) : nrm;
-      if (!track_v) {
-        // v_j = a_j / lambda_j; a column that vanished (rank-deficient input) keeps its unit vector, which only
-        // ever meets a zero singular value
-        const double inv = (nrm > 1e-150) ? 1.0 / nrm : 0.0;
-        if (nrm > 1e-150) {
-          if (lane < l) V[j * ls + lane] = a0 * inv;
-          if (lane + 32 < l) V[j * ls + lane + 32] = a1 * inv;
-        }
-      }
-    }
+  for (int j = warp; j < l; j += nt >> 5) {
+    const double* aj = A + j * ls;
+    const double a0 = (lane < l) ? aj[lane] : 0.0, a1 = (lane + 32 < l) ? aj[lane + 32] : 0.0;
+    const double nrm = sqrt(warp_sum(a0 * a0 + a1 * a1));
+    if (lane == 0) { len[j] = nrm; lam[j] = (nrm - shift) * unscale; }
   }
   __syncthreads();
   if (tid < l) {
@@ -470,10 +470,12 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
     order[rank] = tid;
   }
   __syncthreads();
-  for (int e = tid; e < l * l; e += blockDim.x) {
+  for (int e = tid; e < l * l; e += nt) {
     const int r = e / l, cc = e % l;
     const int src = order[cc];
-    const double v = V[src * ls + r];
+    // v_j = a_j / ||a_j||; a column that vanished (rank-deficient input) takes its unit vector, which only ever meets a
+    // zero singular value
+    const double v = (len[src] > 1e-150) ? A[src * ls + r] / len[src] : ((r == src) ? 1.0 : 0.0);
     const double lm = lam[src];
     const double sv = signed_input ? lm : sqrt(lm > 0.0 ? lm : 0.0);
     if (E) E[(long long)bz * l * l + e] = (float)v;
@@ -484,10 +486,10 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
 
 cudaError_t jacobi_eig_launch(const double* partial, int nchunk, int batch, int l, int signed_input, float* s_out,
                               float* E, float* Es, int* status, cudaStream_t st, long long* launches, int max_sweeps) {
-  const size_t smem = 2 * (size_t)MAX_L * (MAX_L + 1) * sizeof(double);
-  cudaFuncSetAttribute(jacobi_eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  jacobi_eig_kernel<<<batch, JAC_THREADS, smem, st>>>(partial, nchunk, l, signed_input, s_out, E, Es, status,
-                                                      max_sweeps > 0 ? max_sweeps : 40);
+  const size_t smem = (size_t)MAX_L * (MAX_L + 1) * sizeof(double);
+  const int threads = (((l + 1) / 2) * 8 + 31) & ~31;        // eight lanes per pair, whole warps
+  jacobi_eig_kernel<<<batch, threads, smem, st>>>(partial, nchunk, l, signed_input, s_out, E, Es, status,
+                                                  max_sweeps > 0 ? max_sweeps : 40);
   if (launches) ++*launches;
   return cudaGetLastError();
 }

@@ -85,6 +85,28 @@ def test_psd_matches_oracle_with_tracked_basis(ctx, n, K, k, engine_name):
     assert bulk_err <= 2e-2, bulk_err
 
 
+@pytest.mark.parametrize("gap", [0.0, 1e-6])
+def test_eigenvalues_of_equal_magnitude_and_opposite_sign_are_told_apart(ctx, gap):
+    """A head of +-1000 whose magnitudes agree to `gap`, seen through a basis that mixes its directions: the Ritz step must
+    separate +mu from -mu (their images are orthogonal to each other however v(+mu) and v(-mu) are mixed). The error is
+    judged on the bulk alone: a mixing angle t leaves 1000 t in the projection."""
+    n, K, k = 256, 12, 8
+    lam = torch.cat([1000.0 * (1.0 + gap * torch.arange(k).double()) * torch.tensor([1.0, -1.0] * (k // 2)).double(),
+                     2.0 * inputs.rand((n - k,), 4215) - 1.0])
+    q = inputs.haar(n, n, 4210)
+    x = (q * lam.unsqueeze(0)) @ q.T
+    X = (0.5 * (x + x.T)).float().cuda()
+    V0 = _orth(torch.cat([q[:, :k] @ inputs.haar(k, k, 4211), inputs.randn((n, K - k), 4212)], dim=1).numpy())
+    V = torch.from_numpy(V0).float().cuda()
+    v0 = inputs.gaussian_vector(n, 5, inputs.PURPOSE_LANCZOS).cuda()
+    Vin = _orth(V.double().cpu().numpy())
+    P = ctx.defl_psd_project(X, k, V, SCHED7, gamma=1.1, lanczos_start=v0)
+    Po = oracle.psd_project(X.double().cpu().numpy(), Vin, k, oracle.schedule(SCHED7), gamma=1.1,
+                            lanczos_v0=v0.double().cpu().numpy())[0]
+    bulk = float(torch.clamp(lam[k:], min=0).norm())
+    assert float(np.linalg.norm(P.double().cpu().numpy() - Po)) <= 2e-3 * bulk
+
+
 def test_psd_undeflated_baseline_and_frobenius_scale(ctx):
     from paper_2609_21102_b200 import binding
     n = 192
