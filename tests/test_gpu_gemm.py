@@ -62,6 +62,26 @@ def test_tensor_engine(ctx, b, M, N, K, ta, tb, dtype):
         assert err < 2e-3, float(err)
 
 
+@pytest.mark.parametrize("n", [8, 16, 17, 32, 33, 65])
+@pytest.mark.parametrize("k", [1, 15, 64, 65, 130])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16, torch.float16])
+def test_simt_engine_tile_forms_and_operand_walks(ctx, n, k, dtype):
+    """Every tile form (16, 32 and 64 columns wide) at its edges, with operands contiguous along K and along the rows,
+    aligned for whole-quad loads and not. fp32 sums of k products: the bound is k rounding errors of 2^-24 each on the sum
+    of the magnitudes (plus one for the store)."""
+    from paper_2609_21102_b200 import binding
+    for m in (31, 64, 132):
+        for ta, tb in ((False, False), (True, True)):
+            g = torch.Generator().manual_seed(1000 * n + 10 * k + m + ta)
+            A = torch.randn((2, k, m) if ta else (2, m, k), generator=g).to(dtype).cuda()
+            B = torch.randn((2, n, k) if tb else (2, k, n), generator=g).to(dtype).cuda()
+            C = ctx.defl_debug_gemm(A, B, ta, tb, engine=binding.ENGINE_SIMT, out_dtype=torch.float32)
+            Ad = A.double().transpose(1, 2) if ta else A.double()
+            Bd = B.double().transpose(1, 2) if tb else B.double()
+            bound = (k + 1) * 2.0 ** -24 * (Ad.abs() @ Bd.abs()) + 1e-30
+            assert bool(((C.double() - Ad @ Bd).abs() <= bound).all()), (m, ta, tb)
+
+
 def test_tensor_engine_bf16_output_and_large_tiles(ctx):
     from paper_2609_21102_b200 import binding
     A = _mk(2, 520, 1600, torch.bfloat16, 5)     # X X^T with a ragged 1600 = 12.5 tiles of 128
