@@ -59,8 +59,21 @@ bool use_tensor_engine(const GemmDesc& g, int engine) {
   return gemm_tc_supported(g);
 }
 
+// A product of a matrix with its own transpose (X X^T, A A for the symmetric A, the polynomial a I + b A + c A A with A
+// itself as `aux`) computes (i, j) and (j, i) from the same terms in the same order on either engine: the upper tiles and
+// their mirror image are the same result, bit for bit, for half the work, whatever exploit_symmetry says.
+static bool self_product(const GemmDesc& g) {
+  if (g.nseg != 1 || g.M != g.N || g.b_split == 2 || g.transpose_out || g.in_dtype != g.b_dtype) return false;
+  if (g.A[0] != g.B[0] || g.sa_i[0] != g.sb_j[0] || g.sa_k[0] != g.sb_k[0] || (g.batch > 1 && g.batch_a[0] != g.batch_b[0])) return false;
+  if (g.epilogue == EPI_STORE) return true;
+  return g.epilogue == EPI_POLY && g.aux == g.A[0] && g.aux_dtype == g.in_dtype && g.ld_aux == g.sa_i[0] && g.sa_k[0] == 1 &&
+         (g.batch <= 1 || g.batch_aux == g.batch_a[0]);
+}
+
 // Run one product on the engine the options ask for. Returns a DEFL_* code.
-int run_gemm(defl_ctx* c, const GemmDesc& g, int engine, const char* what) {
+int run_gemm(defl_ctx* c, const GemmDesc& desc, int engine, const char* what) {
+  GemmDesc g = desc;
+  if (self_product(g)) g.symmetric = 1;
   const bool tc = use_tensor_engine(g, engine);
   if ((engine == DEFL_ENGINE_TENSOR || g.transpose_out) && !tc) {
     snprintf(c->err, sizeof(c->err), "%s: shape/type not supported by the tensor engine", what);
