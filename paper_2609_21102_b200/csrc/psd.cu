@@ -647,23 +647,34 @@ __global__ void __launch_bounds__(256) admm_x_kernel(const float* __restrict__ C
 }
 
 // the three eigenvalue-free KKT terms of the iteration (Appendix E.4, "Experimental Details"), from the partial sums and b^T y, ||b||, ||C||_F
-__global__ void admm_residual_kernel(const double* __restrict__ partial, int nblk, const float* __restrict__ b,
-                                     const float* __restrict__ y, int n, double norm_b, double norm_c,
-                                     float* __restrict__ out3) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__global__ void __launch_bounds__(256) admm_residual_kernel(const double* __restrict__ partial, int nblk, const float* __restrict__ b,
+                                                            const float* __restrict__ y, int n, double norm_b, double norm_c,
+                                                            float* __restrict__ out3) {
+  __shared__ double red[32];
   double dres = 0.0, obj = 0.0, pres = 0.0, by = 0.0;
-  for (int i = 0; i < nblk; ++i) { dres += partial[3 * i]; obj += partial[3 * i + 1]; pres += partial[3 * i + 2]; }
-  for (int i = 0; i < n; ++i) by += (double)b[i] * (double)y[i];
+  for (int i = threadIdx.x; i < nblk; i += blockDim.x) { dres += partial[3 * i]; obj += partial[3 * i + 1]; pres += partial[3 * i + 2]; }
+  for (int i = threadIdx.x; i < n; i += blockDim.x) by += (double)b[i] * (double)y[i];
+  dres = block_sum(dres, red); obj = block_sum(obj, red); pres = block_sum(pres, red); by = block_sum(by, red);
+  if (threadIdx.x != 0) return;
   out3[0] = (float)(sqrt(pres) / (1.0 + norm_b));
   out3[1] = (float)(sqrt(dres) / (1.0 + norm_c));
   out3[2] = (float)(fabs(obj - by) / (1.0 + fabs(obj) + fabs(by)));
 }
 
-// sum of squares of a float array in one CTA (norms of b and C, once per call)
+// Sum of squares of a float array in fp64 (norms of b and C, once per call): CTA i leaves the sum of its share in out[i],
+// and sum_kernel adds those up.
 __global__ void __launch_bounds__(1024) sumsq_kernel(const float* __restrict__ x, long long count, double* out) {
   __shared__ double red[32];
   double a = 0.0;
-  for (long long i = threadIdx.x; i < count; i += blockDim.x) a += (double)x[i] * (double)x[i];
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x)
+    a += (double)x[i] * (double)x[i];
+  a = block_sum(a, red);
+  if (threadIdx.x == 0) out[blockIdx.x] = a;
+}
+__global__ void __launch_bounds__(256) sum_kernel(const double* __restrict__ sums, int count, double* out) {
+  __shared__ double red[32];
+  double a = 0.0;
+  for (int i = threadIdx.x; i < count; i += blockDim.x) a += sums[i];
   a = block_sum(a, red);
   if (threadIdx.x == 0) *out = a;
 }
@@ -1033,8 +1044,9 @@ int defl_admm_diag_sdp(defl_ctx* c, const void* Cv, const float* b, int n, float
   double* norms = reinterpret_cast<double*>(aux + align_up((size_t)nblk * 3 * sizeof(double), 256) +
                                             align_up((size_t)(iters > 0 ? iters : 1) * 3 * sizeof(float), 256));
   sumsq_kernel<<<1, 1024, 0, c->stream>>>(b, n, norms);
-  sumsq_kernel<<<1, 1024, 0, c->stream>>>(C, (long long)n * n, norms + 1);
-  c->launches += 2;
+  sumsq_kernel<<<c->num_sms, 1024, 0, c->stream>>>(C, (long long)n * n, partial);
+  sum_kernel<<<1, 256, 0, c->stream>>>(partial, c->num_sms, norms + 1);
+  c->launches += 3;
   double hn[2] = {0.0, 0.0};
   if (ctx_fail(c, cudaMemcpyAsync(hn, norms, sizeof(hn), cudaMemcpyDeviceToHost, c->stream), "norms") ||
       ctx_fail(c, cudaStreamSynchronize(c->stream), "synchronize"))
@@ -1052,7 +1064,7 @@ int defl_admm_diag_sdp(defl_ctx* c, const void* Cv, const float* b, int n, float
     const int rc = defl_psd_project(c, Z, S, n, k, warm_basis, K, coeff_schedule, T, &o, nullptr);
     if (rc) return rc;
     admm_x_kernel<<<nblk, 256, 0, c->stream>>>(C, S, y, b, X, n, sigma, partial);
-    admm_residual_kernel<<<1, 32, 0, c->stream>>>(partial, nblk, b, y, n, norm_b, norm_c, hist + 3 * it);
+    admm_residual_kernel<<<1, 256, 0, c->stream>>>(partial, nblk, b, y, n, norm_b, norm_c, hist + 3 * it);
     c->launches += 2;
     if (ctx_fail(c, cudaGetLastError(), "ADMM X")) return DEFL_ERR_CUDA;
   }
