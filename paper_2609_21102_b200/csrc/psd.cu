@@ -116,6 +116,12 @@ struct LanczosState {
   double* beta_prev;
 };
 
+__device__ __forceinline__ double lz_warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 __device__ double block_sum(double v, double* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
@@ -243,23 +249,17 @@ __global__ void __launch_bounds__(1024) lanczos_step_reg_kernel(int j, int n, in
 }
 
 // ---------------------------------------------------------------------------------------------
-// Largest eigenpair of the Lanczos matrix (symmetric tridiagonal, dense fp64 storage [steps, steps], rows after a
-// breakdown all zero), by one warp: the eigenvalue by multi-section on the Sturm count (32 shifts per round, one
-// per lane), the eigenvector by inverse iteration (elimination with row exchanges, pivots floored at eps ||T||).
-// Only the leading unreduced block takes part: the Krylov space ends where an off-diagonal entry is zero, and the
-// entries of the vector beyond it are exact zeros. Outputs rho[0] and column 0 of E (fp32, [steps, steps] row-major).
-// A general symmetric eigensolver on this 20 x 20 matrix cost a fifth of the whole scale estimate.
+// Largest eigenpair of the Lanczos matrix (symmetric tridiagonal: diagonal al, off-diagonal be, zero after a breakdown),
+// by one warp: the eigenvalue by multi-section on the Sturm count (32 shifts per round, one per lane, to 1e-13 of its
+// size: the result is an fp32 number), the eigenvector by two inverse iterations (elimination with row exchanges, pivots
+// floored at eps ||T||). Only the leading unreduced block takes part: the Krylov space ends where an off-diagonal entry is
+// zero, and the entries of the vector beyond it are exact zeros. One warp's chain of fp64 divisions is all it is: 46 us
+// with multi-section to the last bit and three inverse iterations. Returns the eigenvalue; y[0 .. steps) the vector.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(32) tridiag_top_kernel(const double* __restrict__ T, int steps, float* __restrict__ rho,
-                                                         float* __restrict__ E) {
+__device__ double tridiag_top(const double* al, const double* be, int steps, double* y) {
   constexpr int MS = DEFL_LANCZOS_STEPS;
-  __shared__ double al[MS], be[MS], y[MS];
-  const int lane = threadIdx.x;
-  if (lane < steps) {
-    al[lane] = T[lane * steps + lane];
-    be[lane] = (lane + 1 < steps) ? T[lane * steps + lane + 1] : 0.0;
-    E[lane * steps] = 0.f;
-  }
+  const int lane = threadIdx.x & 31;
+  if (lane < steps) y[lane] = 0.0;
   __syncwarp();
   int m = 1;
   while (m < steps && be[m - 1] != 0.0) ++m;                 // size of the leading unreduced block
@@ -288,11 +288,10 @@ __global__ void __launch_bounds__(32) tridiag_top_kernel(const double* __restric
     const double nb = (first < 32) ? __shfl_sync(0xffffffffu, x, first) : b;
     const double na = (first > 0) ? __shfl_sync(0xffffffffu, x, first - 1) : a;
     a = na; b = nb;
-    if (b - a <= 2.0 * eps * fmax(fabs(a), fabs(b)) + 2.0 * pivmin) break;
+    if (b - a <= 1e-13 * fmax(fabs(a), fabs(b)) + 2.0 * pivmin) break;
   }
   const double lam = 0.5 * (a + b);
   if (lane == 0) {
-    rho[0] = (float)lam;
     if (m == 1) y[0] = 1.0;
     else {
       // inverse iteration from the vector of ones (the off-diagonal entries of a Lanczos matrix are positive, so the
@@ -300,7 +299,7 @@ __global__ void __launch_bounds__(32) tridiag_top_kernel(const double* __restric
       double d[MS], du[MS], du2[MS], dl[MS], z[MS];
       const double floor_p = eps * tn;
       for (int i = 0; i < m; ++i) z[i] = 1.0;
-      for (int iter = 0; iter < 3; ++iter) {
+      for (int iter = 0; iter < 2; ++iter) {
         for (int i = 0; i < m; ++i) { d[i] = al[i] - lam; du[i] = (i + 1 < m) ? be[i] : 0.0; dl[i] = du[i]; du2[i] = 0.0; }
         for (int i = 0; i + 1 < m; ++i) {
           if (fabs(d[i]) >= fabs(dl[i])) {
@@ -336,7 +335,22 @@ __global__ void __launch_bounds__(32) tridiag_top_kernel(const double* __restric
     }
   }
   __syncwarp();
-  if (lane < m) E[lane * steps] = (float)y[lane];
+  return lam;
+}
+
+// the same from the dense matrix [steps, steps] in device memory: rho[0] and column 0 of E (fp32, [steps, steps] row-major)
+__global__ void __launch_bounds__(32) tridiag_top_kernel(const double* __restrict__ T, int steps, float* __restrict__ rho,
+                                                         float* __restrict__ E) {
+  __shared__ double al[DEFL_LANCZOS_STEPS], be[DEFL_LANCZOS_STEPS], y[DEFL_LANCZOS_STEPS];
+  const int lane = threadIdx.x;
+  if (lane < steps) {
+    al[lane] = T[lane * steps + lane];
+    be[lane] = (lane + 1 < steps) ? T[lane * steps + lane + 1] : 0.0;
+  }
+  __syncwarp();
+  const double lam = tridiag_top(al, be, steps, y);
+  if (lane == 0) rho[0] = (float)lam;
+  if (lane < steps) E[lane * steps] = (float)y[lane];
 }
 
 // v = sum_p E[p][0] q_p (the Ritz vector of the largest Ritz value); E is [steps, steps] row-major fp32; rows of Q that
@@ -372,6 +386,398 @@ __global__ void __launch_bounds__(1024) lanczos_theta_kernel(int n, const float*
     inv_theta[0] = ok ? (float)(1.0 / th) : 0.f;
     if (!ok && status) atomicOr(status, 4);
   }
+}
+
+// ---------------------------------------------------------------------------------------------
+// The whole scale estimate in one launch. As 63 dependent launches (two matrix-vector products and one single-CTA
+// reorthogonalisation per step) it was bound by launches and by one SM's memory path: 440 us at n = 1000, 640 at n = 4096.
+// Here every CTA owns `rows` consecutive rows of A and of all vectors: as many of its rows of A as fit stay in shared
+// memory for the whole run, its slices of the Lanczos basis too, and what has to meet across CTAs are two vectors and a few
+// dozen partial sums per step.
+//   step j:  t = A q_j  |  w = A t, partial sums of Q_j^T w and of the new Gram row Q_j^T q_j  |
+//            w -= Q_j (2 c - G c), c = Q_j^T w, G = Q_j^T Q_j;  ||w||^2 partial, w  |  q_{j+1} = w / ||w||
+// alpha_j is c_j. The second projection of the two-pass scheme, Q^T (w - Q c) = c - G c, needs no pass of its own: G comes
+// from the stored (rounded) basis, and the correction is applied in fp64 before w is rounded again. Sums over CTAs are
+// fp64 in a fixed order, so every CTA computes the same coefficients, takes the same decisions and finds the same Ritz pair.
+//
+// CLUSTER: one cluster of 16 CTAs, vectors and partial sums written straight into the other CTAs' shared memory, the
+// hardware's cluster barrier between phases. The barrier and the exchange then take a fraction of a microsecond instead of
+// about four through L2 and a counter, which is what bounds small n; 16 SMs can only read 16 times 64 bytes per cycle
+// of what does not fit in their shared memory, which bounds large n. Up to n = LZ_CLUSTER_N the cluster, above it the
+// cooperative grid (n = 1000: 361 us with the grid; n = 4096: 655).
+// ---------------------------------------------------------------------------------------------
+constexpr int LZ_THREADS = 512;
+constexpr int LZ_WARPS = LZ_THREADS / 32;
+constexpr int LZ_MAX_GRID = 160;      // CTAs the partial sums are laid out for
+constexpr int LZ_CLUSTER = 16;
+constexpr int LZ_CLUSTER_N = 1536;
+constexpr int LZ_PW = 2 * DEFL_LANCZOS_STEPS + 1;      // partial sums per CTA: projections, Gram row, ||w||^2
+
+struct LanczosRun {
+  const float* A; const float* v0;
+  int n, steps, rows, resident;      // rows per CTA, how many of them stay in shared memory
+  int aligned;                       // rows of A may be read 16 bytes at a time
+  float* t; float* w;                // [n]                       (grid form)
+  double* part;                      // [2][grid][LZ_PW]          (grid form)
+  unsigned int* bar;                 // barrier counter, zero at launch (grid form)
+  int* wait_status;                  // bit 8 when a barrier runs out of time
+  unsigned long long wait_ns;
+  float* theta; float* inv_theta; int* status;
+};
+
+// y_i = A[row_i] . x for up to NR rows at once by the calling warp (x in shared memory, read once for all); every lane
+// gets the sums
+template <int NR>
+__device__ __forceinline__ void row_dots(const float* const* row, const float* x, int n, bool vec, int lane, float* out) {
+  float acc[NR];
+  if (vec) {
+    const float4* x4 = reinterpret_cast<const float4*>(x);
+    float a[NR][4];
+#pragma unroll
+    for (int q = 0; q < NR; ++q)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) a[q][j] = 0.f;
+    const int n4 = n / 4;
+    constexpr int U = NR >= 4 ? 2 : 4;          // 16-byte loads of every row in flight per lane
+    int i = lane;
+    for (; i + 32 * (U - 1) < n4; i += 32 * U) {
+      float4 r[NR][U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int q = 0; q < NR; ++q) r[q][u] = reinterpret_cast<const float4*>(row[q])[i + 32 * u];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float4 v = x4[i + 32 * u];
+#pragma unroll
+        for (int q = 0; q < NR; ++q) {
+          a[q][0] = fmaf(r[q][u].x, v.x, a[q][0]); a[q][1] = fmaf(r[q][u].y, v.y, a[q][1]);
+          a[q][2] = fmaf(r[q][u].z, v.z, a[q][2]); a[q][3] = fmaf(r[q][u].w, v.w, a[q][3]);
+        }
+      }
+    }
+    for (; i < n4; i += 32) {
+      const float4 v = x4[i];
+#pragma unroll
+      for (int q = 0; q < NR; ++q) {
+        const float4 r = reinterpret_cast<const float4*>(row[q])[i];
+        a[q][0] = fmaf(r.x, v.x, a[q][0]); a[q][1] = fmaf(r.y, v.y, a[q][1]);
+        a[q][2] = fmaf(r.z, v.z, a[q][2]); a[q][3] = fmaf(r.w, v.w, a[q][3]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NR; ++q) acc[q] = (a[q][0] + a[q][1]) + (a[q][2] + a[q][3]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < NR; ++q) acc[q] = 0.f;
+#pragma unroll 4
+    for (int i = lane; i < n; i += 32) {
+      const float v = x[i];
+#pragma unroll
+      for (int q = 0; q < NR; ++q) acc[q] = fmaf(row[q][i], v, acc[q]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < NR; ++q) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+    out[q] = acc[q];
+  }
+}
+
+// shared memory of CTA `rank` of the cluster at the place of `p` in this one's
+template <typename T>
+__device__ __forceinline__ uint32_t peer_smem(const T* p, int rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void peer_store(uint32_t a, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+__device__ __forceinline__ void peer_store(uint32_t a, double v) { asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory"); }
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <bool CLUSTER>
+__global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const LanczosRun p) {
+  extern __shared__ __align__(16) float lz[];
+  constexpr int MS = DEFL_LANCZOS_STEPS;
+  const int n = p.n, steps = p.steps, R = p.rows, G = gridDim.x, blk = blockIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int first = blk * R, mine = max(0, min(R, n - first));      // this CTA's rows
+  const int np = (n + 3) & ~3;
+  float* xq = lz;                             // [n] the vector being multiplied: q_j (or v), then t
+  float* xt = CLUSTER ? xq + np : xq;         // (the cluster form's CTAs write into each other's: two buffers)
+  float* wl = xt + np;                        // [R] own slice of w (or t)
+  float* Qs = wl + ((R + 3) & ~3);            // [steps][R] own slices of the basis
+  float* As = Qs + (((long long)MS * R + 3) & ~3);  // [resident][n] own rows of A
+  __shared__ double red[LZ_WARPS], tot[LZ_PW], coef[MS], gram[MS][MS], al[MS], be[MS], y[MS];
+  __shared__ double cpart[2][CLUSTER ? LZ_CLUSTER : 1][CLUSTER ? LZ_PW : 1];     // cluster form: everybody's partial sums
+  __shared__ double rho_s;
+  __shared__ int alive;
+  unsigned int epoch = 0;
+  const bool vec = (n & 3) == 0 && p.aligned;
+
+  {
+    const float* src = p.A + (long long)first * n;
+    const int count = min(p.resident, mine) * n;
+    if (vec) {
+#pragma unroll 8
+      for (int e = tid; e < count / 4; e += LZ_THREADS) reinterpret_cast<float4*>(As)[e] = __ldg(reinterpret_cast<const float4*>(src) + e);
+    } else {
+#pragma unroll 8
+      for (int e = tid; e < count; e += LZ_THREADS) As[e] = __ldg(src + e);
+    }
+  }
+  if (tid < MS) { al[tid] = 0.0; be[tid] = 0.0; }
+  if (tid == 0) alive = 1;
+  __syncthreads();
+
+  // All CTAs meet. Grid form: a counter with a time limit, false (everywhere in the CTA) when it ran out.
+  auto meet = [&]() -> bool {
+    if (CLUSTER) { cluster_barrier(); return true; }
+    __syncthreads();
+    ++epoch;
+    if (tid == 0) {
+      __threadfence();
+      atomicAdd(p.bar, 1u);
+      const unsigned int want = epoch * (unsigned int)G;
+      unsigned long long t0 = 0;
+      for (unsigned int polls = 0;; ++polls) {
+        unsigned int v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p.bar) : "memory");
+        if (v >= want) break;
+        if ((polls & 1023u) == 1023u) {
+          unsigned long long now;
+          asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
+          if (t0 == 0) t0 = now;
+          else if (now - t0 > p.wait_ns) { alive = 0; atomicOr(p.wait_status, DEFL_ST_DEVICE_WAIT); break; }
+        }
+      }
+      __threadfence();
+    }
+    __syncthreads();
+    return alive != 0;
+  };
+  // own slice of a vector to everybody: into their x buffer, or to global memory
+  auto publish = [&](float* x, float* v) {
+    if (CLUSTER) {
+      for (int e = tid; e < mine * G; e += LZ_THREADS) {
+        const int g = e / mine, r = e - g * mine;
+        peer_store(peer_smem(x + first + r, g), wl[r]);
+      }
+    } else {
+      for (int r = tid; r < mine; r += LZ_THREADS) v[first + r] = wl[r];
+    }
+  };
+  // x <- the vector that all CTAs have published (grid form: through L2, the L1 may hold the previous one), times `scale`
+  auto stage = [&](float* x, const float* v, float scale) {
+    if (!CLUSTER || scale != 1.f) {
+      for (int i = tid; i < n; i += LZ_THREADS) x[i] = (CLUSTER ? x[i] : __ldcg(v + i)) * scale;
+      __syncthreads();
+    }
+  };
+  // (A x)[r] for the own rows, in wl
+  auto multiply = [&](const float* x) {
+    for (int r = warp; r < mine; r += 4 * LZ_WARPS) {
+      const float* row[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int rr = r + q * LZ_WARPS;
+        row[q] = (rr < p.resident) ? As + (long long)rr * n : p.A + (long long)(first + (rr < mine ? rr : r)) * n;
+      }
+      float o[4];
+      if (r + LZ_WARPS >= mine) row_dots<1>(row, x, n, vec, lane, o);
+      else if (r + 2 * LZ_WARPS >= mine) row_dots<2>(row, x, n, vec, lane, o);
+      else row_dots<4>(row, x, n, vec, lane, o);
+      if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) if (r + q * LZ_WARPS < mine) wl[r + q * LZ_WARPS] = o[q];
+      }
+    }
+    __syncthreads();
+  };
+  // one partial sum of this CTA (the same in every lane of the warp) to where everybody adds them up
+  auto give = [&](int set, int q, double d) {
+    if (CLUSTER) { if (lane < G) peer_store(peer_smem(&cpart[set][blk][q], lane), d); }
+    else if (lane == 0) p.part[((long long)set * G + blk) * LZ_PW + q] = d;
+  };
+  auto total = [&](int set, int q) -> double {     // sum over the CTAs by one warp, fixed order
+    double d = 0.0;
+    if (CLUSTER) { if (lane < G) d = cpart[set][lane][q]; }
+    else for (int g = lane; g < G; g += 32) d += __ldcg(p.part + ((long long)set * G + g) * LZ_PW + q);
+    return lz_warp_sum(d);
+  };
+  auto square = [&](int set) {          // this CTA's share of ||w||^2
+    if (warp == 0) {
+      double d = 0.0;
+      for (int r = lane; r < mine; r += 32) d += (double)wl[r] * (double)wl[r];
+      give(set, LZ_PW - 1, lz_warp_sum(d));
+    }
+  };
+
+  // q_0
+  double a = 0.0;
+  for (int i = tid; i < n; i += LZ_THREADS) { const float v = __ldg(p.v0 + i); xq[i] = v; a += (double)v * (double)v; }
+  a = lz_warp_sum(a);
+  if (lane == 0) red[warp] = a;
+  __syncthreads();
+  double nv = 0.0;
+  for (int i = 0; i < LZ_WARPS; ++i) nv += red[i];
+  nv = sqrt(nv);
+  const bool started = nv > 0.0;
+  for (int i = tid; i < n; i += LZ_THREADS) xq[i] = started ? (float)((double)xq[i] / nv) : 0.f;
+  __syncthreads();
+  for (int r = tid; r < mine; r += LZ_THREADS) Qs[r] = xq[first + r];
+  __syncthreads();
+  if (CLUSTER) cluster_barrier();             // nobody writes into a CTA that has not started
+
+  for (int j = 0; started && j < steps; ++j) {
+    multiply(xq);                             // t = A q_j
+    publish(xt, p.t);
+    if (!meet()) return;
+    stage(xt, p.t, 1.f);
+    multiply(xt);                             // w = A t
+    // this CTA's shares of c_q = q_q . w and of G_jq = q_q . q_j, q = 0 .. j
+    for (int q = warp; q < 2 * (j + 1); q += LZ_WARPS) {
+      const int b = q > j ? q - j - 1 : q;
+      const float* other = q > j ? Qs + (long long)j * R : wl;
+      double d = 0.0;
+      for (int r = lane; r < mine; r += 32) d += (double)Qs[b * R + r] * (double)other[r];
+      give(0, q > j ? MS + b : b, lz_warp_sum(d));
+    }
+    if (!meet()) return;
+    for (int q = warp; q < 2 * (j + 1); q += LZ_WARPS) {
+      const int slot = q > j ? MS + q - j - 1 : q;
+      const double d = total(0, slot);
+      if (lane == 0) tot[slot] = d;
+    }
+    __syncthreads();
+    if (tid <= j) { gram[j][tid] = tot[MS + tid]; gram[tid][j] = tot[MS + tid]; }
+    if (tid == 0) al[j] = tot[j];
+    __syncthreads();
+    if (tid <= j) {
+      double gc = 0.0;
+      for (int q = 0; q <= j; ++q) gc = fma(gram[tid][q], tot[q], gc);
+      coef[tid] = 2.0 * tot[tid] - gc;
+    }
+    __syncthreads();
+    if (j + 1 == steps) break;
+    for (int r = tid; r < mine; r += LZ_THREADS) {
+      double v = (double)wl[r];
+      for (int q = 0; q <= j; ++q) v = fma(-coef[q], (double)Qs[q * R + r], v);
+      wl[r] = (float)v;
+    }
+    __syncthreads();
+    square(1);
+    publish(xq, p.w);
+    if (!meet()) return;
+    if (warp == 0) { const double d = total(1, LZ_PW - 1); if (lane == 0) tot[LZ_PW - 1] = sqrt(d); }
+    __syncthreads();
+    const double b = tot[LZ_PW - 1];
+    if (!(b > 1e-12 * fabs(al[0]))) break;    // the Krylov space ends here (the same decision in every CTA)
+    if (tid == 0) be[j] = b;
+    stage(xq, p.w, (float)(1.0 / b));
+    for (int r = tid; r < mine; r += LZ_THREADS) Qs[(j + 1) * R + r] = xq[first + r];
+    __syncthreads();
+  }
+  __syncthreads();
+
+  // largest Ritz pair (rho, v), theta = sqrt(max(rho, 0) + ||A A v - rho v||)
+  if (warp == 0) {
+    const double lam = tridiag_top(al, be, steps, y);
+    if (lane == 0) rho_s = (double)(float)lam;
+  }
+  __syncthreads();
+  for (int r = tid; r < mine; r += LZ_THREADS) {
+    double v = 0.0;
+    for (int q = 0; q < steps; ++q) if (y[q] != 0.0) v += (double)(float)y[q] * (double)Qs[q * R + r];
+    wl[r] = (float)v;
+    Qs[r] = (float)v;                         // (row 0 is this thread's own to overwrite now)
+  }
+  if (CLUSTER) cluster_barrier(); else __syncthreads();     // (the last x_q may still be read by a slower CTA)
+  publish(xq, p.w);
+  if (!meet()) return;
+  stage(xq, p.w, 1.f);
+  multiply(xq);
+  publish(xt, p.t);
+  if (!meet()) return;
+  stage(xt, p.t, 1.f);
+  multiply(xt);
+  const double rho = rho_s;
+  for (int r = tid; r < mine; r += LZ_THREADS) wl[r] = (float)((double)wl[r] - rho * (double)Qs[r]);
+  __syncthreads();
+  square(0);
+  if (!meet()) return;                        // (the last access to another CTA's shared memory lies before this)
+  if (blk == 0 && warp == 0) {
+    const double d = sqrt(total(0, LZ_PW - 1));
+    if (lane == 0) {
+      const double th = sqrt((rho > 0.0 ? rho : 0.0) + d);
+      const bool ok = th > 0.0 && isfinite(th);
+      p.theta[0] = (float)th;
+      p.inv_theta[0] = ok ? (float)(1.0 / th) : 0.f;
+      if (!ok && p.status) atomicOr(p.status, 4);
+    }
+  }
+}
+
+// Launches it, or returns false (nothing launched) where a CTA cannot hold its vectors or the device cannot hold the grid.
+static bool lanczos_launch(defl_ctx* c, const float* A, const float* start, int n, int steps, float* t, float* w, double* part,
+                           unsigned int* bar, float* theta, float* inv_theta, int* status, cudaError_t* err) {
+  *err = cudaSuccess;
+  LanczosRun p;
+  memset(&p, 0, sizeof(p));
+  p.A = A; p.v0 = start; p.n = n; p.steps = steps; p.t = t; p.w = w; p.part = part; p.bar = bar;
+  p.aligned = (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+  p.wait_status = c->wait_status;
+  p.wait_ns = (unsigned long long)(c->tc_knobs.wait_ms > 0 ? c->tc_knobs.wait_ms : 2000) * 1000000ull;
+  p.theta = theta; p.inv_theta = inv_theta; p.status = status;
+  const size_t budget = 210 * 1024;           // (static shared memory comes on top)
+  // rows per CTA, resident rows and shared memory of a form; 0 = does not fit
+  auto layout = [&](int grid, int vectors) -> size_t {
+    p.rows = (n + grid - 1) / grid;
+    const size_t fixed = sizeof(float) * ((size_t)vectors * ((n + 3) & ~3) + (size_t)((p.rows + 3) & ~3) +
+                                          (size_t)((DEFL_LANCZOS_STEPS * p.rows + 3) & ~3));
+    if (fixed > budget) return 0;
+    const size_t fit = (budget - fixed) / ((size_t)n * sizeof(float));
+    p.resident = fit < (size_t)p.rows ? (int)fit : p.rows;
+    return fixed + (size_t)p.resident * n * sizeof(float);
+  };
+  if (n <= LZ_CLUSTER_N) {
+    const size_t smem = layout(LZ_CLUSTER, 2);
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = LZ_CLUSTER; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(LZ_CLUSTER, 1, 1); cfg.blockDim = dim3(LZ_THREADS, 1, 1); cfg.dynamicSmemBytes = smem; cfg.stream = c->stream;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    int clusters = 0;
+    if (smem > 0 && cudaFuncSetAttribute(lanczos_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+        cudaFuncSetAttribute(lanczos_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&clusters, lanczos_kernel<true>, &cfg) == cudaSuccess && clusters > 0) {
+      *err = cudaLaunchKernelEx(&cfg, lanczos_kernel<true>, p);
+      ++c->launches;
+      return true;
+    }
+    cudaGetLastError();
+  }
+  // one CTA per SM at most, at least a row per warp
+  int grid = (n + LZ_WARPS - 1) / LZ_WARPS;
+  if (grid > c->num_sms) grid = c->num_sms;
+  if (grid > LZ_MAX_GRID) grid = LZ_MAX_GRID;
+  const size_t smem = layout(grid, 1);
+  if (smem == 0) return false;
+  grid = (n + p.rows - 1) / p.rows;
+  if (cudaFuncSetAttribute(lanczos_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) { cudaGetLastError(); return false; }
+  if ((*err = cudaMemsetAsync(bar, 0, sizeof(unsigned int), c->stream)) != cudaSuccess) return true;
+  void* args[] = {&p};
+  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)lanczos_kernel<false>, dim3(grid), dim3(LZ_THREADS), args, smem, c->stream);
+  if (e == cudaErrorCooperativeLaunchTooLarge) { cudaGetLastError(); return false; }
+  ++c->launches;
+  *err = e;
+  return true;
 }
 
 // P <- (P + P^T)/2 in place, 32 x 32 tiles through shared memory; tile pair (bi <= bj) per CTA
@@ -469,6 +875,7 @@ struct PsdWs {
   float* Rinv; float* E; float* Es; float* lam; float* coef;   // [K,K] x3, [K], [K]
   float* Q; double* T; float* lw; float* lt; float* lv; float* lE; float* lrho;   // Lanczos state
   int* done; double* beta_prev;
+  double* lpart; unsigned int* lbar;   // partial sums and barrier counter of the one-launch estimate
   double* npart; float* theta; float* inv_theta; float* dummy; float* rscale;
   int* status;
   int* keff;        // [1] size of the deflated set (gate)
@@ -503,6 +910,7 @@ static PsdWs carve_psd(void* base, int n, int K) {
   w.lw = cv.take<float>(n); w.lt = cv.take<float>(n); w.lv = cv.take<float>(n);
   w.lE = cv.take<float>(S * S); w.lrho = cv.take<float>(S);
   w.done = cv.take<int>(1); w.beta_prev = cv.take<double>(1);
+  w.lpart = cv.take<double>((size_t)2 * LZ_MAX_GRID * LZ_PW); w.lbar = cv.take<unsigned int>(1);
   w.npart = cv.take<double>(1184);
   w.theta = cv.take<float>(1); w.inv_theta = cv.take<float>(1); w.dummy = cv.take<float>(S * S); w.rscale = cv.take<float>(1);
   w.status = cv.take<int>(1);
@@ -524,6 +932,13 @@ static int estimate_scale(defl_ctx* c, const float* A, int n, int norm_mode, con
   }
   int steps = DEFL_LANCZOS_STEPS;
   if (steps > n) steps = n;
+  {
+    cudaError_t e;
+    if (lanczos_launch(c, A, start, n, steps, w.lt, w.lw, w.lpart, w.lbar, w.theta, w.inv_theta, w.status, &e)) {
+      if (ctx_fail(c, e, "scale estimate")) return DEFL_ERR_CUDA;
+      return DEFL_OK;
+    }
+  }
   LanczosState s;
   s.Q = w.Q; s.T = w.T; s.w = w.lw; s.t = w.lt; s.done = w.done; s.beta_prev = w.beta_prev;
   lanczos_init_kernel<<<1, 1024, 0, c->stream>>>(start, n, steps, s);
