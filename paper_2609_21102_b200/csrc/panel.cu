@@ -85,148 +85,99 @@ cudaError_t gram_partial_launch(const float* Y, long long batch_stride, int batc
 }
 
 // ---------------------------------------------------------------------------------------------
-// Cholesky of W = sum of partials (l x l, fp64, shared memory), W = R^T R, output Rinv = R^-1
-// (upper triangular, fp32, row-major [l,l]). A non-positive pivot restarts with W + shift I and
-// sets DEFL_ST_CHOL_SHIFT (bit 1) in status[b].
+// Cholesky of W = sum of partials (l x l, fp64), W = R^T R, output Rinv = R^-1 (upper triangular, fp32, row-major [l,l]).
+// A non-positive pivot restarts with W + shift I and sets DEFL_ST_CHOL_SHIFT (bit 1) in status[b].
+//
+// Symmetric elimination of [W | I] in one l x l array: step j subtracts f_i = W_ij / d_j times row j from every row i > j,
+// the columns right of j holding what is left of W, those up to j the unit lower factor's inverse Z as it grows (column j
+// becomes -f_i). Then L^-1 = diag(d)^(-1/2) Z and R^-1 is its transpose, so factor and inverse take one sweep of l steps
+// with one barrier each, and the only chain per step is barrier, pivot, reciprocal, one multiply-add. Every thread keeps its
+// elements in registers; shared memory carries only the pivot row and column (double buffered). Measured for l = 16, one
+// matrix: 16 -> 8.6 us, l = 48, 48 matrices: 46 -> 41 us (right-looking Cholesky and a substitution after it, both in shared
+// memory); a step still takes 800 cycles at l = 8 and 1450 at l = 48, three times its chain.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(512) chol_inv_kernel(const double* __restrict__ partial, int nchunk, int l,
+constexpr int CHOL_ROWS = MAX_L / 8;     // rows per thread: r = first + 8 u
+
+__global__ void __launch_bounds__(512) chol_inv_kernel(const double* __restrict__ partial, int nchunk, int l, int cw_log2,
                                                        float* __restrict__ Rinv, int* __restrict__ status) {
-  extern __shared__ double sm[];
-  // rows are padded to an odd number of doubles: a column walk (row stride apart) then touches every bank once
-  // instead of one bank 32 times (l = 48 doubles = 96 words = 0 mod 32)
-  const int ls = l | 1;
-  double* W = sm;                              // [l][ls] original Gram
-  double* Lm = sm + MAX_L * (MAX_L + 1);       // [l][ls] lower factor, then its inverse
-  __shared__ int bad;
-  __shared__ double rdiag[MAX_L];
+  __shared__ double prow[2][MAX_L], pcol[2][MAX_L], diag[MAX_L], wdiag[MAX_L];
   const int bz = blockIdx.x, tid = threadIdx.x;
+  const int c = tid & ((1 << cw_log2) - 1), r0 = tid >> cw_log2;       // column, first row (0 .. 7)
   const double* pb = partial + (long long)bz * nchunk * l * l;
-  for (int e = tid; e < l * l; e += blockDim.x) {
-    double t = 0.0;
-#pragma unroll 8
-    for (int c = 0; c < nchunk; ++c) t += pb[(long long)c * l * l + e];
-    W[(e / l) * ls + e % l] = t;
-  }
-  __syncthreads();
-  // symmetrise exactly
-  for (int e = tid; e < l * l; e += blockDim.x) {
-    const int i = e / l, j = e % l;
-    if (i < j) { const double a = 0.5 * (W[i * ls + j] + W[j * ls + i]); Lm[i * ls + j] = a; Lm[j * ls + i] = a; }
-    else if (i == j) Lm[i * ls + j] = W[i * ls + j];
-  }
-  __syncthreads();
-  for (int e = tid; e < l * l; e += blockDim.x) { const int o = (e / l) * ls + e % l; W[o] = Lm[o]; }
-  __syncthreads();
-  double trace = 0.0;
-  for (int i = 0; i < l; ++i) trace += W[i * ls + i];
-  double shift = 0.0;
-  for (int attempt = 0; attempt < 6; ++attempt) {
-    for (int e = tid; e < l * l; e += blockDim.x) {
-      const int i = e / l, j = e % l;
-      Lm[i * ls + j] = W[i * ls + j] + ((i == j) ? shift : 0.0);
+  double w[CHOL_ROWS], m[CHOL_ROWS];
+#pragma unroll
+  for (int u = 0; u < CHOL_ROWS; ++u) w[u] = 0.0;
+  if (c < l) {
+#pragma unroll 2
+    for (int ch = 0; ch < nchunk; ++ch) {
+      const double* pe = pb + (long long)ch * l * l + c;
+#pragma unroll
+      for (int u = 0; u < CHOL_ROWS; ++u) w[u] += (r0 + 8 * u < l) ? pe[(r0 + 8 * u) * l] : 0.0;
     }
+#pragma unroll
+    for (int u = 0; u < CHOL_ROWS; ++u) if (r0 + 8 * u == c) wdiag[c] = w[u];
+  }
+  double shift = 0.0;
+  bool failed = false;
+  for (int attempt = 0; attempt < 6; ++attempt) {
     __syncthreads();
-    // Right-looking Cholesky on the lower triangle, one barrier per column: in phase j every thread reads the
-    // pivot d_j itself (so a bad pivot is seen by all alike), the trailing block is updated from the UNSCALED
-    // column j times 1/d_j, and column j-1 (which nobody reads any more) is scaled in passing.
-    // (one reciprocal square root per column and thread: 1/d = rsqrt(d)^2, sqrt(d) = d rsqrt(d); a division and a
-    // square root in fp64 cost several hundred cycles of latency each, more than the rest of the column)
-    bool failed = false;
-    double sd_prev = 1.0, isd_prev = 1.0;
-    const int ti = tid >> 6, tc = tid & 63;        // 8 rows x 64 columns of the trailing block per pass
+    // row j and column j of the array as it stands; below the pivot the column's place is cleared for Z
+    auto publish = [&](int j) {
+      const int buf = j & 1;
+      if (r0 == (j & 7)) {
+#pragma unroll
+        for (int u = 0; u < CHOL_ROWS; ++u) if (u == (j >> 3)) prow[buf][c] = m[u];
+      }
+      if (c == j) {
+#pragma unroll
+        for (int u = 0; u < CHOL_ROWS; ++u) {
+          pcol[buf][r0 + 8 * u] = m[u];
+          if (r0 + 8 * u > j) m[u] = 0.0;
+        }
+      }
+    };
+#pragma unroll
+    for (int u = 0; u < CHOL_ROWS; ++u) m[u] = w[u] + ((r0 + 8 * u == c) ? shift : 0.0);
+    publish(0);
+    __syncthreads();
+    failed = false;
     for (int j = 0; j < l; ++j) {
-      const double d = Lm[j * ls + j];
+      const int buf = j & 1;
+      const double d = prow[buf][j], pr = prow[buf][c];       // every thread reads the pivot itself: a bad one is seen by all alike
+      double f[CHOL_ROWS];
+#pragma unroll
+      for (int u = 0; u < CHOL_ROWS; ++u) f[u] = (r0 + 8 * u > j) ? pcol[buf][r0 + 8 * u] : 0.0;     // (rows past l: zeros)
       if (!(d > 0.0) || !isfinite(d)) { failed = true; break; }
-      const double isd = rsqrt(d), inv_d = isd * isd;
-      if (j > 0) {
-        for (int i = j - 1 + tid; i < l; i += blockDim.x) Lm[i * ls + j - 1] = (i == j - 1) ? sd_prev : Lm[i * ls + j - 1] * isd_prev;
-      }
-      const int c = j + 1 + tc;
-      if (c < l) {
-        const double lc = Lm[c * ls + j] * inv_d;
-        // all loads of the thread's (up to MAX_L / 8) rows first, then the updates: written as one loop, every
-        // iteration's loads wait for the previous iteration's store (the compiler cannot tell they do not alias)
-        double a[MAX_L / 8], bj[MAX_L / 8];
+      const double inv = 1.0 / d;
+      if (tid == 0) diag[j] = d;
+      const double s = (c == j) ? inv : inv * pr;
 #pragma unroll
-        for (int u = 0; u < MAX_L / 8; ++u) {
-          const int i = j + 1 + ti + 8 * u;
-          const bool on = i < l && c <= i;
-          a[u] = on ? Lm[i * ls + c] : 0.0;
-          bj[u] = on ? Lm[i * ls + j] : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < MAX_L / 8; ++u) {
-          const int i = j + 1 + ti + 8 * u;
-          if (i < l && c <= i) Lm[i * ls + c] = a[u] - bj[u] * lc;
-        }
-      }
-      sd_prev = d * isd; isd_prev = isd;
+      for (int u = 0; u < CHOL_ROWS; ++u) if (r0 + 8 * u > j) m[u] = fma(-f[u], s, m[u]);
+      if (j + 1 < l) publish(j + 1);       // (into the other buffer: nobody reads that one before the barrier)
       __syncthreads();
     }
-    if (!failed && tid == 0) Lm[(l - 1) * ls + l - 1] = sd_prev;
-    if (tid == 0) bad = failed ? 1 : 0;
-    __syncthreads();
-    if (!bad) break;
+    if (!failed) break;
     // shift as in shifted CholeskyQR: proportional to the trace, growing per attempt
+    double trace = 0.0;
+    for (int i = 0; i < l; ++i) trace += wdiag[i];
     shift = (shift == 0.0) ? 1e-10 * (trace > 0.0 ? trace : 1.0) : shift * 100.0;
     if (tid == 0 && status) atomicOr(&status[bz], 1);
-    __syncthreads();
   }
-  // Linv by forward substitution, one column per thread: L X = I
-  // X[:,c] for c: x_c = 1/L_cc; x_i = -(sum_{t=c}^{i-1} L_it x_t)/L_ii
+  // Rinv(c, r) = Z(r, c) / sqrt(d_r): upper triangular; all zeros if every attempt failed
+  if (tid < l) wdiag[tid] = failed ? 0.0 : 1.0 / sqrt(diag[tid]);
   __syncthreads();
-  double* X = W;   // reuse
-  for (int e = tid; e < l * ls; e += blockDim.x) X[e] = 0.0;
-  if (tid < l) rdiag[tid] = bad ? 0.0 : 1.0 / Lm[tid * ls + tid];
-  __syncthreads();
-  if (!bad) {
-    // Eight lanes per column c of X = L^-1 (blockDim / 8 = 64 columns at once), column-oriented: lane `sub` keeps,
-    // in registers, the running sums s_r = sum_{k<i} L_rk x_k of the rows r = sub (mod 8). Step i: the owner of row i
-    // hands s_i to the group (one shuffle), everybody forms x_i = (delta_ic - s_i) / L_ii, and adds L_ri x_i to its
-    // sums of the rows below. Per step that is one shuffle and one multiply on the critical path and at most
-    // MAX_L / 8 independent multiply-adds per lane; the row-oriented form (a dot product split over the lanes,
-    // three shuffle levels and a warp barrier per row) spent 2.5x the fp64 instructions, which is what bounds it.
-    const int c = tid >> 3, sub = tid & 7;
-    const int c_warp0 = (tid >> 5) * 4;          // first column of this warp
-    double srow[MAX_L / 8];
-#pragma unroll
-    for (int u = 0; u < MAX_L / 8; ++u) srow[u] = 0.0;
-    if (c_warp0 < l) {                           // (a warp whose four columns all lie beyond l has nothing to do)
-#pragma unroll
-      for (int u = 0; u < MAX_L / 8; ++u) {
-#pragma unroll
-        for (int w = 0; w < 8; ++w) {
-          const int i = 8 * u + w;
-          if (i < l && i >= c_warp0) {           // uniform in the warp: rows above its first column give x_i = 0
-            const double si = __shfl_sync(0xffffffffu, srow[u], w, 8);
-            double xi = 0.0;
-            if (c < l && i >= c) xi = ((i == c) ? 1.0 - si : -si) * rdiag[i];
-            if (sub == w && c < l) X[i * ls + c] = xi;
-#pragma unroll
-            for (int u2 = u; u2 < MAX_L / 8; ++u2) {
-              const int r = 8 * u2 + sub;
-              if (r > i && r < l) srow[u2] = fma(Lm[r * ls + i], xi, srow[u2]);
-            }
-          }
-        }
-      }
-    }
-  }
-  __syncthreads();
-  // Rinv = Linv^T (upper triangular)
   float* out = Rinv + (long long)bz * l * l;
-  for (int e = tid; e < l * l; e += blockDim.x) {
-    const int i = e / l, j = e % l;
-    out[e] = (float)X[j * ls + i];
+#pragma unroll
+  for (int u = 0; u < CHOL_ROWS; ++u) {
+    const int r = r0 + 8 * u;
+    if (r < l && c < l) out[c * l + r] = failed ? 0.f : (float)(((c < r) ? m[u] : (c == r ? 1.0 : 0.0)) * wdiag[r]);
   }
 }
 
 cudaError_t chol_inv_launch(const double* partial, int nchunk, int batch, int l, float* Rinv, int* status,
                             cudaStream_t st, long long* launches) {
-  const size_t smem = 2 * (size_t)MAX_L * (MAX_L + 1) * sizeof(double);
-  // (the attribute belongs to the current device's copy of the kernel: set at every launch, a host-side call)
-  cudaFuncSetAttribute(chol_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  chol_inv_kernel<<<batch, 512, smem, st>>>(partial, nchunk, l, Rinv, status);
+  const int cw_log2 = l <= 16 ? 4 : (l <= 32 ? 5 : 6);       // eight rows of 16, 32 or 64 columns per pass
+  chol_inv_kernel<<<batch, 8 << cw_log2, 0, st>>>(partial, nchunk, l, cw_log2, Rinv, status);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -349,10 +300,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
       const int j = j0 + grp;
       double acc = 0.0;
 #pragma unroll
-      for (int i = 0; i < JAC_NR; ++i) {
-        const int r = sub + 8 * i;
-        if (i < nr && r < l && j < l) { const double v = A[j * ls + r]; acc = fma(v, v, acc); }
-      }
+      for (int i = 0; i < NR; ++i) { const double v = A[min(j, l) * ls + sub + 8 * i]; acc = fma(v, v, acc); }
       acc = group8_sum(acc);
       if (sub == 0 && j < l) nrm2[j] = acc;
     }
@@ -361,6 +309,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
   column_norms();
   double fro2 = 0.0;
   for (int j = 0; j < l; ++j) fro2 += nrm2[j];
+  if (tid == 0) nrm2[l] = 0.0;
   const double fro = sqrt(fro2);
   double scale = 1.0, unscale = 1.0;
   if (fro > 1e-290 && fro < 1e290) {
@@ -394,25 +343,21 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
         }
         if (p > q) { const int t = p; p = q; q = t; }
       }
-      const bool live = q < l;            // (a pair with the padding player, or a group beyond the pairs, idles)
-      double* ap = A + p * ls; double* aq = A + (live ? q : p) * ls;
-      const double alpha = live ? nrm2[p] : 0.0, beta = live ? nrm2[q] : 0.0;
-      double x[JAC_NR], y[JAC_NR];
+      // (a pair with the padding player, or a group beyond the pairs, meets the zero column: nothing to rotate)
+      double* ap = A + p * ls + sub; double* aq = A + q * ls + sub;
+      const double alpha = nrm2[p], beta = nrm2[q];
+      double x[NR], y[NR];
       double pg0 = 0.0, pg1 = 0.0;
 #pragma unroll
-      for (int i = 0; i < JAC_NR; ++i) {
-        if (i < nr) {
-          const int r = sub + 8 * i;
-          const bool in = live && r < l;
-          x[i] = in ? ap[r] : 0.0;
-          y[i] = in ? aq[r] : 0.0;
-          if (i & 1) pg1 = fma(x[i], y[i], pg1); else pg0 = fma(x[i], y[i], pg0);
-        }
+      for (int i = 0; i < NR; ++i) { x[i] = ap[8 * i]; y[i] = aq[8 * i]; }
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        if (i & 1) pg1 = fma(x[i], y[i], pg1); else pg0 = fma(x[i], y[i], pg0);
       }
       const double gamma = group8_sum(pg0 + pg1);
       // rotate when |gamma| > 1e-11 sqrt(alpha beta) (compared in squares): the eigenvalues are then good to about
       // 1e-22 and the vectors to 1e-11 over the relative gap, far beyond the fp32 outputs
-      if (live && gamma != 0.0 && gamma * gamma > 1e-22 * (alpha * beta)) {
+      if (gamma != 0.0 && gamma * gamma > 1e-22 * (alpha * beta)) {
         if (sub == 0) rotated = 1;
         // The rotation angle only steers the iteration (any exact rotation keeps the invariants intact), so tan is
         // computed in fp32 with approximate functions; cos comes from an fp32 reciprocal square root refined by two
@@ -437,10 +382,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
         const double sn = c * t, tg = t * gamma;
         if (sub == 0) { nrm2[p] = alpha - tg; nrm2[q] = beta + tg; }
 #pragma unroll
-        for (int i = 0; i < JAC_NR; ++i) {
-          const int r = sub + 8 * i;
-          if (i < nr && r < l) { ap[r] = c * x[i] - sn * y[i]; aq[r] = sn * x[i] + c * y[i]; }
-        }
+        for (int i = 0; i < NR; ++i) { ap[8 * i] = c * x[i] - sn * y[i]; aq[8 * i] = sn * x[i] + c * y[i]; }
       }
       __syncthreads();
     }
@@ -486,10 +428,13 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
 
 cudaError_t jacobi_eig_launch(const double* partial, int nchunk, int batch, int l, int signed_input, float* s_out,
                               float* E, float* Es, int* status, cudaStream_t st, long long* launches, int max_sweeps) {
-  const size_t smem = (size_t)MAX_L * (MAX_L + 1) * sizeof(double);
   const int threads = (((l + 1) / 2) * 8 + 31) & ~31;        // eight lanes per pair, whole warps
-  jacobi_eig_kernel<<<batch, threads, smem, st>>>(partial, nchunk, l, signed_input, s_out, E, Es, status,
-                                                  max_sweeps > 0 ? max_sweeps : 40);
+  const int nr = (l + 7) / 8;
+  const size_t smem = (size_t)(l + 1) * (8 * nr + 1) * sizeof(double);
+  auto kern = nr <= 1 ? jacobi_eig_kernel<1> : nr == 2 ? jacobi_eig_kernel<2> : nr == 3 ? jacobi_eig_kernel<3>
+            : nr == 4 ? jacobi_eig_kernel<4> : nr == 5 ? jacobi_eig_kernel<5> : nr == 6 ? jacobi_eig_kernel<6>
+            : nr == 7 ? jacobi_eig_kernel<7> : jacobi_eig_kernel<8>;
+  kern<<<batch, threads, smem, st>>>(partial, nchunk, l, signed_input, s_out, E, Es, status, max_sweeps > 0 ? max_sweeps : 40);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
