@@ -258,22 +258,26 @@ __device__ __forceinline__ float sqrt_approx(float x) { float r; asm("sqrt.appro
 __device__ __forceinline__ float rsqrt_approx(float x) { float r; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
 
 constexpr int JAC_THREADS = 256;        // at most 32 column pairs x 8 lanes
-constexpr int JAC_NR = MAX_L / 8;       // rows per lane
 
+template <int NR>      // rows per lane, ceil(l / 8)
 __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* __restrict__ partial, int nchunk, int l,
                                                                  int signed_input, float* __restrict__ s_out,
                                                                  float* __restrict__ E, float* __restrict__ Es,
                                                                  int* __restrict__ status, int max_sweeps) {
   extern __shared__ double sm[];
-  const int ls = l | 1;       // column stride (odd: the four pairs of a warp start in different banks)
-  double* A = sm;             // column-major: A[c * ls + r]
+  // column-major: A[c * ls + r], rows l .. 8 NR - 1 and column l (the padding player's) all zero, so that no access of a
+  // round needs a test; the stride is odd (the four pairs of a warp start in different banks)
+  constexpr int ls = 8 * NR + 1;
+  double* A = sm;
   __shared__ double lam[MAX_L];       // column norms (eigenvalues of the scaled, shifted matrix), then the eigenvalues
   __shared__ double len[MAX_L];
-  __shared__ double nrm2[MAX_L];      // squared column norms of A, carried along by the rotations
+  __shared__ double nrm2[MAX_L + 1];  // squared column norms of A, carried along by the rotations
   __shared__ int order[MAX_L];
   __shared__ int rotated;
   const int bz = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nt = blockDim.x;
   const double* pb = partial + (long long)bz * nchunk * l * l;
+  for (int e = tid; e < (l + 1) * ls; e += nt) A[e] = 0.0;
+  __syncthreads();
   for (int e = tid; e < l * l; e += nt) {
     double t = 0.0;
 #pragma unroll 8
@@ -291,7 +295,6 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
   const int npairs = np / 2;
   // Eight lanes per column pair, four pairs per warp: the dot product of a pair takes three shuffle steps.
   const int grp = tid >> 3, sub = tid & 7;
-  const int nr = (l + 7) >> 3;        // rows per lane actually present
   // Squared norms of the columns (Frobenius norm for the shift, and for the scale: the matrix is multiplied by the power
   // of two that brings its norm near one, exactly, so that squared norms and dot products of columns down to 1e-18 of it
   // are ordinary fp32 numbers for the angle).
@@ -306,10 +309,10 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
     }
     __syncthreads();
   };
+  if (tid == 0) nrm2[l] = 0.0;
   column_norms();
   double fro2 = 0.0;
   for (int j = 0; j < l; ++j) fro2 += nrm2[j];
-  if (tid == 0) nrm2[l] = 0.0;
   const double fro = sqrt(fro2);
   double scale = 1.0, unscale = 1.0;
   if (fro > 1e-290 && fro < 1e290) {
