@@ -603,22 +603,29 @@ cudaError_t rho_identity_launch(const double* partial, int nper, int batch, cons
 // 4096 more spread evenly over the matrix, and raises bit 16 of status[b] when one of them is Inf or NaN. A sample is
 // enough: a non-finite entry of an iterate (non-finite input, or a value that left the range of the iterate's
 // storage format) reaches the Gram matrix of the next step and from there every entry of the following iterate.
-__global__ void __launch_bounds__(256) finite_probe_kernel(const void* __restrict__ X, int dtype, long long count,
+__global__ void __launch_bounds__(1024) finite_probe_kernel(const void* __restrict__ X, int dtype, long long count,
                                                            int* __restrict__ status) {
   const int bz = blockIdx.x, tid = threadIdx.x;
   const long long base = (long long)bz * count;
-  const long long head = min(count, (long long)4096);
   const long long stride = max((long long)1, count / 4096);
+  // all eight loads of a thread are on their way before the first is looked at
+  float v[8];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const long long j = tid + 1024 * i;
+    v[i] = (j < count) ? ld_as_float(X, base + j, dtype) : 0.f;
+    v[4 + i] = (j * stride < count) ? ld_as_float(X, base + j * stride, dtype) : 0.f;
+  }
   bool bad = false;
-  for (long long i = tid; i < head; i += 256) bad |= !isfinite(ld_as_float(X, base + i, dtype));
-  for (long long j = tid; j < 4096 && j * stride < count; j += 256) bad |= !isfinite(ld_as_float(X, base + j * stride, dtype));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) bad |= !isfinite(v[i]);
   if (__syncthreads_or(bad ? 1 : 0) && tid == 0) atomicOr(&status[bz], 16);
 }
 
 cudaError_t finite_probe_launch(const void* X, int dtype, int batch, long long count, int* status, cudaStream_t st,
                                 long long* launches) {
   if (batch <= 0 || count <= 0) return cudaSuccess;
-  finite_probe_kernel<<<batch, 256, 0, st>>>(X, dtype, count, status);
+  finite_probe_kernel<<<batch, 1024, 0, st>>>(X, dtype, count, status);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
