@@ -148,7 +148,7 @@ PolarWs carve_polar(void* base, int b, int m, int n, int dtype, int k, int l, in
   const int le = l > 0 ? l : 1, ke = k > 0 ? k : 1;
   w.Lp = cv.take<float>((size_t)b * ml * le);
   w.Sp = cv.take<float>((size_t)b * ms * le);
-  w.gram = cv.take<double>((size_t)b * gram_num_chunks(ml) * le * le);
+  w.gram = cv.take<double>((size_t)b * fused_max_chunks(ml) * le * le);
   w.Rinv = cv.take<float>((size_t)b * le * le);
   w.E = cv.take<float>((size_t)b * le * le);
   w.Es = cv.take<float>((size_t)b * le * le);

@@ -16,7 +16,7 @@ namespace defl {
 // partial[b, chunk, l, l] = sum over its rows of y_r y_r^T  (fp32 products over 32-row groups,
 // groups added in fp64).
 // ---------------------------------------------------------------------------------------------
-constexpr int GRAM_ROWS = 256;   // rows per CTA
+constexpr int GRAM_ROWS = 64;    // rows per CTA (256 rows: 35 us for the one panel of n = 1024 it serves)
 constexpr int GRAM_SUB = 32;     // rows per fp32 sub-accumulation
 
 __global__ void __launch_bounds__(256) gram_partial_kernel(const float* __restrict__ Y, const float* __restrict__ Y2,
@@ -937,7 +937,8 @@ constexpr int FUSED_TS = MAX_L + 4;
 // Rows are split over CTAs in whole 128-row tiles. The split is chosen so that all CTAs of the launch are resident
 // at once (two per SM with this kernel's registers): a fixed 512-row split gave 624 CTAs for 592 places on
 // the 48 x 6400-row panels, i.e. a second wave for 32 CTAs, and left two thirds of the GPU idle on 1600-row panels.
-// At least two tiles per CTA, so the count never exceeds gram_num_chunks(rows), which sizes the partials buffer.
+// A panel of few matrices spreads over one CTA per tile, the most that fused_max_chunks (which sizes the partials) allows.
+int fused_max_chunks(int rows) { return (rows + FUSED_TILE - 1) / FUSED_TILE; }
 int fused_num_chunks(int rows, int batch) {
   static int sms = 0;
   if (sms <= 0) {
@@ -947,7 +948,7 @@ int fused_num_chunks(int rows, int batch) {
   }
   const int places = sms * 2;
   const int tiles = (rows + FUSED_TILE - 1) / FUSED_TILE;
-  int t = 2;
+  int t = 1;
   while (t < tiles && (long long)((tiles + t - 1) / t) * batch > places) ++t;
   return (tiles + t - 1) / t;
 }
@@ -1134,31 +1135,29 @@ __global__ void __launch_bounds__(256, 2) panel_fused_kernel(const float* In, lo
     }
   }
   if (partial) {
-    // sum over the groups in fp64 (group order fixed: the result does not depend on timing), in the tile's memory
-    // (rows padded to an odd stride: the blocks of a group lie 4 rows apart and the mirror reads walk a column, both
-    // of which land on one shared-memory bank when a row is 48 doubles = 96 words)
-    const int wr = wout | 1;
-    double* red = reinterpret_cast<double*>(fsm);        // [wout][wr], upper blocks only
+    // Sum over the groups in fp64 (group order fixed: the result does not depend on timing). Every thread leaves its block
+    // in the tile's memory, then one thread per element of W adds up the groups. (Groups taking turns on one shared
+    // array, a barrier and 32 dependent updates each, took 10 of the 14 us of a gram pass over a short panel.)
+    float4* part = reinterpret_cast<float4*>(fsm);       // [ngrp][nblk][8] quads: at most 256 x 128 bytes
     __syncthreads();
-    for (int e = tid; e < wout * wr; e += 256) red[e] = 0.0;
-    __syncthreads();
-    for (int g = 0; g < ngrp; ++g) {
-      if (gram_on && grp == g) {
+    if (gram_on) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int gi = bi * 4 + i, gj = bj * 8 + j;
-            if (gi < wout && gj < wout) red[gi * wr + gj] += (double)g8[i][j];
-          }
-      }
-      __syncthreads();
+        for (int h = 0; h < 2; ++h)
+          part[(i * 2 + h) * 256 + tid] = make_float4(g8[i][4 * h], g8[i][4 * h + 1], g8[i][4 * h + 2], g8[i][4 * h + 3]);
     }
     double* out = partial + ((long long)bz * nchunk + chunk) * wout * wout;
     for (int e = tid; e < wout * wout; e += 256) {
-      const int gi = e / wout, gj = e - gi * wout;
+      int gi = e / wout, gj = e - gi * wout;
       // blocks below the block diagonal were not computed: take the mirror image
-      out[e] = ((gi >> 3) <= (gj >> 3)) ? red[gi * wr + gj] : red[gj * wr + gi];
+      if ((gi >> 3) > (gj >> 3)) { const int t = gi; gi = gj; gj = t; }
+      // block columns before this one hold 2, 4, 6, .. blocks
+      const int blk = (gj >> 3) * ((gj >> 3) + 1) + (gi >> 2);
+      const float* q = pf + ((gi & 3) * 2 + ((gj >> 2) & 1)) * 1024 + (gj & 3);
+      double t = 0.0;
+      for (int g = 0; g < ngrp; ++g) t += (double)q[(g * nblk + blk) * 4];
+      out[e] = t;
     }
   }
 }
@@ -1179,6 +1178,8 @@ cudaError_t panel_fused_launch(const float* In, long long in_bs, int ld_in, int 
 // Momentum of a Muon step, element-wise in fp32: Mom <- mu Mom + Grad, stored in the momentum's type; when `look`
 // is given it receives Grad + mu Mom' with Mom' the STORED (rounded) new momentum, i.e. the Nesterov look-ahead
 // is a function of the optimizer state as it is kept in memory.
+    __syncthreads();
+    const float* pf = fsm;
 // ---------------------------------------------------------------------------------------------
 template <typename T, int V>
 __global__ void __launch_bounds__(256) momentum_vec_kernel(T* Mom, const T* __restrict__ Grad, T* look, long long nvec, float mu) {
