@@ -75,6 +75,7 @@ struct TcParams {
   int dup_ok;                  // symmetric pair-form product of a matrix with itself, BN = 256: diagonal tiles share one operand fetch
   int diag_exact;              // symmetric output of two different operands: diagonal blocks mirrored element by element
   int aux_f16, out_f16;        // a 16-bit aux / output is IEEE half (else bf16); the operands' kind is in idesc
+  int vec_ok;                  // rows of C (and of `aux`) start on 16-byte boundaries, their base pointers too
   void* C; long long ldc, batch_c;
   const void* aux; long long ld_aux, batch_aux;
   float alpha, aux_scale, pa, pb, pc;
@@ -745,8 +746,7 @@ __device__ __forceinline__ void epilogue_half(const TcParams& p, uint32_t taddr,
   const size_t cbatch = (size_t)bz * p.batch_c;
   const size_t crow = cbatch + (size_t)gi * p.ldc;
   const size_t xrow = (size_t)bz * p.batch_aux + (size_t)gi * p.ld_aux;
-  const bool vec_ok = ((p.ldc & 7) == 0) && ((p.batch_c & 7) == 0) && ((p.ld_aux & 7) == 0 || EPI == EPI_STORE) &&
-                      ((p.batch_aux & 7) == 0 || EPI == EPI_STORE);
+  const bool vec_ok = p.vec_ok != 0;
   const bool a2 = (p.aux_dtype != F32), o2 = (p.out_dtype != F32);
   // the coalesced path wants `aux` and the output in the same type (true of every product the library makes)
   // (symmetric output: the mirror stores of the coalesced path assume 32 complete rows)
@@ -1475,6 +1475,8 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word,
   p.out_f16 = (g.out_dtype == F16) ? 1 : 0;
   p.C = g.C; p.ldc = g.ldc; p.batch_c = g.batch_c;
   p.aux = g.aux; p.ld_aux = g.ld_aux; p.batch_aux = g.batch_aux;
+  p.vec_ok = ((g.ldc | g.batch_c) & 7) == 0 && aligned16(g.C) &&
+             (g.epilogue == EPI_STORE || (((g.ld_aux | g.batch_aux) & 7) == 0 && aligned16(g.aux)));
   p.alpha = g.alpha; p.aux_scale = g.aux_scale; p.pa = g.pa; p.pb = g.pb; p.pc = g.pc;
   p.alpha_dev = g.alpha_dev; p.aux_scale_dev = g.aux_scale_dev;
   p.partials = g.partials; p.partials_per_batch = g.partials_per_batch;

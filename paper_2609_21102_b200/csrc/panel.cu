@@ -868,11 +868,36 @@ cudaError_t split_concat3_launch(const float* In, long long in_bs, int ld_in, in
   return cudaGetLastError();
 }
 
+// Row-padded copy of 16-bit matrices: Out [b, rows, ld] from In [b, rows, n], columns n .. ld - 1 zero (ld a multiple of 8).
+// Rows of n elements that are not whole 16-byte packets are out of the copy engine's reach; one pass over them puts the
+// whole call on the tensor cores. Bound by memory: 16 bytes per store, the eight loads of a thread side by side.
+__global__ void __launch_bounds__(256) pad_rows_kernel(const uint16_t* __restrict__ In, uint16_t* __restrict__ Out, long long rows,
+                                                       int n, int ld) {
+  const int per = ld / 8;
+  const long long total = rows * per, stride = (long long)gridDim.x * blockDim.x;
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += stride) {
+    const long long r = e / per;
+    const int c = (int)(e - r * per) * 8;
+    uint32_t v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = (c + j < n) ? In[r * n + c + j] : 0;
+    reinterpret_cast<uint4*>(Out)[e] = make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+  }
+}
+
+cudaError_t pad_rows_launch(const void* In, void* Out, int batch, int rows, int n, int ld, cudaStream_t st, long long* launches) {
+  const long long total = (long long)batch * rows * (ld / 8);
+  const int nblk = (int)min((long long)148 * 16, (total + 255) / 256);
+  pad_rows_kernel<<<nblk, 256, 0, st>>>((const uint16_t*)In, (uint16_t*)Out, (long long)batch * rows, n, ld);
+  if (launches) ++*launches;
+  return cudaGetLastError();
+}
+
 // Matrices whose residual counts as zero (status bit 4: 1/rho = 0) get the padded head alone as filter input,
 // X0 = scale * P[:, :keff] W[:, :keff]^T; every other matrix is left untouched (its CTAs return at once).
 __global__ void __launch_bounds__(256) zero_residual_entry_kernel(const int* __restrict__ status, const float* __restrict__ P,
                                                                   const float* __restrict__ W, const int* __restrict__ keff,
-                                                                  int m, int n, int k, float scale, void* __restrict__ X0,
+                                                                  int m, int n, int ld, int k, float scale, void* __restrict__ X0,
                                                                   int dtype) {
   const int bz = blockIdx.y;
   if (!(status[bz] & 4)) return;
@@ -884,13 +909,13 @@ __global__ void __launch_bounds__(256) zero_residual_entry_kernel(const int* __r
     const int i = (int)(e / n), j = (int)(e % n);
     float t = 0.f;
     for (int q = 0; q < ke; ++q) t = fmaf(Pb[(long long)i * k + q], Wb[(long long)j * k + q], t);
-    st_from_float(X0, (long long)bz * tot + e, dtype, scale * t);
+    st_from_float(X0, ((long long)bz * m + i) * ld + j, dtype, scale * t);
   }
 }
 
 cudaError_t zero_residual_entry_launch(const int* status, const float* P, const float* W, const int* keff, int batch, int m,
-                                       int n, int k, float scale, void* X0, int dtype, cudaStream_t st, long long* launches) {
-  zero_residual_entry_kernel<<<dim3(64, batch), 256, 0, st>>>(status, P, W, keff, m, n, k, scale, X0, dtype);
+                                       int n, int ld, int k, float scale, void* X0, int dtype, cudaStream_t st, long long* launches) {
+  zero_residual_entry_kernel<<<dim3(64, batch), 256, 0, st>>>(status, P, W, keff, m, n, ld, k, scale, X0, dtype);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -1147,6 +1172,8 @@ __global__ void __launch_bounds__(256, 2) panel_fused_kernel(const float* In, lo
         for (int h = 0; h < 2; ++h)
           part[(i * 2 + h) * 256 + tid] = make_float4(g8[i][4 * h], g8[i][4 * h + 1], g8[i][4 * h + 2], g8[i][4 * h + 3]);
     }
+    __syncthreads();
+    const float* pf = fsm;
     double* out = partial + ((long long)bz * nchunk + chunk) * wout * wout;
     for (int e = tid; e < wout * wout; e += 256) {
       int gi = e / wout, gj = e - gi * wout;
@@ -1178,8 +1205,6 @@ cudaError_t panel_fused_launch(const float* In, long long in_bs, int ld_in, int 
 // Momentum of a Muon step, element-wise in fp32: Mom <- mu Mom + Grad, stored in the momentum's type; when `look`
 // is given it receives Grad + mu Mom' with Mom' the STORED (rounded) new momentum, i.e. the Nesterov look-ahead
 // is a function of the optimizer state as it is kept in memory.
-    __syncthreads();
-    const float* pf = fsm;
 // ---------------------------------------------------------------------------------------------
 template <typename T, int V>
 __global__ void __launch_bounds__(256) momentum_vec_kernel(T* Mom, const T* __restrict__ Grad, T* look, long long nvec, float mu) {

@@ -49,16 +49,18 @@ cudaError_t split_concat3_launch(const float* In, long long in_bs, int ld_in, in
                                  __nv_bfloat16* Out, cudaStream_t st, long long* launches, const int* keff = nullptr,
                                  int f16 = 0, int transposed = 0, float mult = 1.f, const float* rho = nullptr);
 cudaError_t zero_residual_entry_launch(const int* status, const float* P, const float* W, const int* keff, int batch, int m,
-                                       int n, int k, float scale, void* X0, int dtype, cudaStream_t st, long long* launches);
+                                       int n, int ld, int k, float scale, void* X0, int dtype, cudaStream_t st, long long* launches);
+// row-padded copy of 16-bit matrices, [b, rows, n] -> [b, rows, ld]
+cudaError_t pad_rows_launch(const void* In, void* Out, int batch, int rows, int n, int ld, cudaStream_t st, long long* launches);
 cudaError_t gate_launch(const float* s, int ld_s, int batch, int window, int kmax, float tau, int* keff, cudaStream_t st,
                         long long* launches);
 }  // namespace defl
 
 namespace defl {
 int fused_num_chunks(int rows, int batch);
+int fused_max_chunks(int rows);
 // Out = In * Mtx[:, :kout] (Mtx null: identity), optional fp32 / bf16 hi+lo outputs, optional Gram partials of Out
 // ([b, fused_num_chunks(rows, b), w, w] fp64 with w = width of Out)
-int fused_max_chunks(int rows);
 cudaError_t panel_fused_launch(const float* In, long long in_bs, int ld_in, int batch, int rows, int l, const float* Mtx,
                                int ldm, int kout, float* Out, long long out_bs, int ld_out, __nv_bfloat16* hi,
                                __nv_bfloat16* lo, int lp, double* partial, cudaStream_t st, long long* launches);

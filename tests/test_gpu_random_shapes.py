@@ -105,3 +105,38 @@ def test_random_configurations_add_restore(ctx, seed):
                 worst[name] = max(worst[name], err / tol)
                 assert err <= tol, (case, i, err, tol)
     print("ADD restore, seed %d: worst error / tolerance" % seed, worst)
+
+
+@pytest.mark.parametrize("m,n", [(65, 97), (97, 65), (66, 136), (136, 66), (131, 520), (520, 131), (257, 257)])
+@pytest.mark.parametrize("form", ["plain", "padded", "gated", "add", "odd_base", "muon"])
+def test_rows_of_no_whole_packets_agree_with_the_fp32_engine(ctx, m, n, form):
+    """bf16 shapes whose rows are not whole 16-byte packets run on padded copies and the tensor engine; the fp32 engine takes
+    the same call as it is. Both store the same 16-bit iterates from products that differ in the last bits, so single
+    roundings differ: each result is within the library's 3e-2 of the exact one (half of that here: spectrum with a gap),
+    their distance within twice that."""
+    from paper_2609_21102_b200 import binding
+    rng = np.random.default_rng(m * 1000 + n)
+    b, ms = 2, min(m, n)
+    k = 0 if form == "plain" else 6
+    sigma = np.concatenate([np.linspace(60, 20, 6), rng.uniform(0.05, 1.0, ms - 6)])
+    G = torch.stack([inputs.from_spectrum(m, n, sigma, 9100 + i) for i in range(b)]).to(torch.bfloat16).cuda()
+    Om = torch.tensor(rng.standard_normal((b, ms, 10)), dtype=torch.float32).cuda()
+    if form == "odd_base":                    # buffers that start one element past a 16-byte boundary
+        flat = torch.empty(b * m * n + 1, dtype=torch.bfloat16, device="cuda")
+        flat[1:] = G.reshape(-1)
+        G = flat[1:].view(b, m, n)
+    outs = []
+    for engine in (binding.ENGINE_AUTO, binding.ENGINE_SIMT):
+        kw = dict(sketch=Om if k else None, gamma=1.05, engine=engine, tau=0.1 if form == "gated" else 0.0,
+                  restore_mode=binding.RESTORE_ADD if form == "add" else binding.RESTORE_PADDED)
+        if form == "muon":
+            W, M = torch.zeros((b, m, n), device="cuda"), G.clone()
+            ctx.defl_muon_step_batched(W, M, None, 1.0, 0.0, k, 4, 1, list(binding.MUON_QUINTIC), steps=5, **kw)
+            outs.append(-W)
+        else:
+            out = torch.empty(b * m * n + 1, dtype=torch.bfloat16, device="cuda")[1:].view(b, m, n) if form == "odd_base" else None
+            outs.append(ctx.defl_polar_batched(G, k, 4 if k else 0, 1 if k else 0, [list(binding.MUON_QUINTIC)] * 5, out=out, **kw).float())
+    torch.cuda.synchronize()
+    assert bool(torch.isfinite(outs[0]).all())
+    for i in range(b):
+        assert float((outs[0][i] - outs[1][i]).norm() / outs[1][i].norm()) <= 3e-2
