@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
+#include <utility>
 
 namespace defl {
 
@@ -91,6 +92,28 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word,
                            const TcKnobs* knobs = nullptr, TmCache* cache = nullptr);
 bool gemm_tc_supported(const GemmDesc& g);
 int gemm_tc_partials_per_batch(const GemmDesc& g, const TcKnobs* knobs = nullptr);
+
+// Programmatic dependent launch. Every kernel of the library is launched so that its CTAs may start while the kernel before
+// it on the stream is still draining, and begins with pdl_wait(), which returns when that kernel has finished and its
+// writes are visible; nothing in global memory is touched before it. (A kernel is finished only after its own pdl_wait, so
+// the order along the stream is the usual one.) What a chain of short kernels loses at every boundary, launch latency and
+// the start of the CTAs, is then mostly overlapped: tiny fp32 batch 272 -> 196 us, 12 x 768 x 768 669 -> 597, ADMM at
+// n = 1000 4.68 -> 4.12 ms. pdl_launch() lets the next kernel's CTAs start before this one's are through. Only the tensor
+// engine does (its successor's set-up is worth it): after the other kernels the early CTAs are packed two or three to an SM
+// that has room while others go idle, which cost the fp32 products of one or two CTAs per SM 15 %.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 __device__ __forceinline__ float ld_as_float(const void* p, long long idx, int dt) {
   return dt == BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p)[idx])

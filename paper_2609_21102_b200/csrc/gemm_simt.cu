@@ -195,6 +195,7 @@ __device__ __forceinline__ void emit4(const GemmDesc& g, int gi, int gj, const f
 
 template <typename TIn, typename TB, int BM, int BN, int BK, int TM, int TN>
 __global__ void __launch_bounds__(NT, 2) gemm_simt_kernel(const GemmDesc g) {
+  pdl_wait();
   constexpr int TX = BN / TN, TY = BM / TM;          // threads of one K group
   constexpr int GT = TX * TY, KS = NT / GT;
   constexpr int PARTS = KS / 2;                      // the upper half of the groups hands its sums to the lower half, and again
@@ -332,6 +333,7 @@ __global__ void __launch_bounds__(NT, 2) gemm_simt_kernel(const GemmDesc g) {
 constexpr int RU_ROWS = 4;      // rows per thread; 32 per CTA
 template <int KMAX>
 __global__ void __launch_bounds__(NT) rank_update_kernel(const GemmDesc g) {
+  pdl_wait();
   __shared__ __align__(16) float ua[32][KMAX];
   __shared__ __align__(16) float ub[KMAX][128 + 4];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, bz = blockIdx.z;
@@ -413,9 +415,9 @@ template <typename TIn, typename TB>
 void launch_form(const GemmDesc& g, SimtForm f, cudaStream_t st) {
   const int bm = f == FORM_32x32 ? 32 : 64, bn = f == FORM_64x64 ? 64 : (f == FORM_32x32 ? 32 : 16);
   const dim3 grid((g.N + bn - 1) / bn, (g.M + bm - 1) / bm, g.batch);
-  if (f == FORM_64x64) gemm_simt_kernel<TIn, TB, 64, 64, 32, 8, 8><<<grid, NT, 0, st>>>(g);
-  else if (f == FORM_32x32) gemm_simt_kernel<TIn, TB, 32, 32, 64, 4, 8><<<grid, NT, 0, st>>>(g);
-  else gemm_simt_kernel<TIn, TB, 64, 16, 64, 8, 4><<<grid, NT, 0, st>>>(g);
+  if (f == FORM_64x64) launch_kernel(gemm_simt_kernel<TIn, TB, 64, 64, 32, 8, 8>, grid, NT, 0, st, g);
+  else if (f == FORM_32x32) launch_kernel(gemm_simt_kernel<TIn, TB, 32, 32, 64, 4, 8>, grid, NT, 0, st, g);
+  else launch_kernel(gemm_simt_kernel<TIn, TB, 64, 16, 64, 8, 4>, grid, NT, 0, st, g);
 }
 
 }  // namespace
@@ -431,8 +433,8 @@ cudaError_t gemm_simt_launch(const GemmDesc& g, cudaStream_t st, long long* laun
   if (g.b_split == 2) return cudaErrorNotSupported;      // (split panels go to the tensor engine only)
   if (rank_update_form(g)) {
     const dim3 grid((g.N + 127) / 128, (g.M + 31) / 32, g.batch);
-    if (g.K[0] <= 8) rank_update_kernel<8><<<grid, NT, 0, st>>>(g);
-    else rank_update_kernel<16><<<grid, NT, 0, st>>>(g);
+    if (g.K[0] <= 8) launch_kernel(rank_update_kernel<8>, grid, NT, 0, st, g);
+    else launch_kernel(rank_update_kernel<16>, grid, NT, 0, st, g);
     if (launches) ++*launches;
     return cudaGetLastError();
   }

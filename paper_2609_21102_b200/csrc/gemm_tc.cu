@@ -825,6 +825,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_tc_kernel(const __grid_co
     return (long long)tnum;
   };
 
+  if (warp == 2 && lane == 0) {
+    // the descriptors are on their way while the CTA sets itself up
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&p.tmA[0]) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&p.tmB[0]) : "memory");
+    if (p.nseg > 1) asm volatile("prefetch.tensormap [%0];" ::"l"(&p.tmA[1]) : "memory");
+    if (p.nseg > 1 || BSPLIT == 2) asm volatile("prefetch.tensormap [%0];" ::"l"(&p.tmB[1]) : "memory");
+  }
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 1); }
@@ -848,6 +855,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_tc_kernel(const __grid_co
   if (PAIR) cluster_sync_all();      // the peer's barriers are initialised before anything signals them
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
+  // (barriers, tensor memory and the descriptor fetch above overlap the end of the previous kernel)
+  pdl_wait();
+  pdl_launch();
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -1516,9 +1526,11 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word,
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.blockDim = dim3(NUM_THREADS, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -1543,6 +1555,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word,
     long long npairs = p.total_tiles < pairs ? p.total_tiles : pairs;
     if (npairs < 1) npairs = 1;
     cfg.gridDim = dim3((unsigned)(2 * npairs), 1, 1);
+    cfg.numAttrs = 2;
     e = cudaLaunchKernelEx(&cfg, kern, p);
     if (launches) ++*launches;
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -1553,7 +1566,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word,
   if (e != cudaSuccess) return e;
   long long grid = p.total_tiles < num_sms ? p.total_tiles : num_sms;
   if (grid < 1) grid = 1;
-  kern<<<(unsigned)grid, NUM_THREADS, smem, st>>>(p);
+  launch_kernel(kern, dim3((unsigned)grid), dim3(NUM_THREADS), smem, st, p);
   if (launches) ++*launches;
   return cudaGetLastError();
 }

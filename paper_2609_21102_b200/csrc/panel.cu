@@ -22,6 +22,7 @@ constexpr int GRAM_SUB = 32;     // rows per fp32 sub-accumulation
 __global__ void __launch_bounds__(256) gram_partial_kernel(const float* __restrict__ Y, const float* __restrict__ Y2,
                                                            long long batch_stride, int rows, int l, int ld, int nchunk,
                                                            double* __restrict__ partial) {
+  pdl_wait();
   __shared__ float tile[GRAM_SUB][MAX_L + 1];
   __shared__ float tile2[GRAM_SUB][MAX_L + 1];
   const int chunk = blockIdx.x, bz = blockIdx.y, tid = threadIdx.x;
@@ -79,7 +80,7 @@ int gram_num_chunks(int rows) { return (rows + GRAM_ROWS - 1) / GRAM_ROWS; }
 cudaError_t gram_partial_launch(const float* Y, long long batch_stride, int batch, int rows, int l, int ld,
                                 double* partial, cudaStream_t st, long long* launches, const float* Y2) {
   const int nchunk = gram_num_chunks(rows);
-  gram_partial_kernel<<<dim3(nchunk, batch), 256, 0, st>>>(Y, Y2, batch_stride, rows, l, ld, nchunk, partial);
+  launch_kernel(gram_partial_kernel, dim3(nchunk, batch), 256, 0, st, Y, Y2, batch_stride, rows, l, ld, nchunk, partial);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -100,6 +101,7 @@ constexpr int CHOL_ROWS = MAX_L / 8;     // rows per thread: r = first + 8 u
 
 __global__ void __launch_bounds__(512) chol_inv_kernel(const double* __restrict__ partial, int nchunk, int l, int cw_log2,
                                                        float* __restrict__ Rinv, int* __restrict__ status) {
+  pdl_wait();
   __shared__ double prow[2][MAX_L], pcol[2][MAX_L], diag[MAX_L], wdiag[MAX_L];
   const int bz = blockIdx.x, tid = threadIdx.x;
   const int c = tid & ((1 << cw_log2) - 1), r0 = tid >> cw_log2;       // column, first row (0 .. 7)
@@ -177,7 +179,7 @@ __global__ void __launch_bounds__(512) chol_inv_kernel(const double* __restrict_
 cudaError_t chol_inv_launch(const double* partial, int nchunk, int batch, int l, float* Rinv, int* status,
                             cudaStream_t st, long long* launches) {
   const int cw_log2 = l <= 16 ? 4 : (l <= 32 ? 5 : 6);       // eight rows of 16, 32 or 64 columns per pass
-  chol_inv_kernel<<<batch, 8 << cw_log2, 0, st>>>(partial, nchunk, l, cw_log2, Rinv, status);
+  launch_kernel(chol_inv_kernel, batch, 8 << cw_log2, 0, st, partial, nchunk, l, cw_log2, Rinv, status);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -189,6 +191,7 @@ constexpr int PA_ROWS = 64;
 __global__ void __launch_bounds__(256) panel_apply_kernel(const float* In, long long in_bs, int ld_in,
                                                           const float* __restrict__ Mtx, int ldm, int rows, int l,
                                                           int kout, float* Out, long long out_bs, int ld_out) {
+  pdl_wait();
   __shared__ float tile[PA_ROWS][MAX_L + 1];
   __shared__ float mt[MAX_L][MAX_L + 1];
   const int bz = blockIdx.y, tid = threadIdx.x;
@@ -215,7 +218,7 @@ cudaError_t panel_apply_launch(const float* In, long long in_bs, int ld_in, cons
                                int rows, int l, int kout, float* Out, long long out_bs, int ld_out, cudaStream_t st,
                                long long* launches) {
   if (kout <= 0) return cudaSuccess;
-  panel_apply_kernel<<<dim3((rows + PA_ROWS - 1) / PA_ROWS, batch), 256, 0, st>>>(In, in_bs, ld_in, Mtx, ldm, rows, l,
+  launch_kernel(panel_apply_kernel, dim3((rows + PA_ROWS - 1) / PA_ROWS, batch), 256, 0, st, In, in_bs, ld_in, Mtx, ldm, rows, l,
                                                                                  kout, Out, out_bs, ld_out);
   if (launches) ++*launches;
   return cudaGetLastError();
@@ -264,6 +267,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
                                                                  int signed_input, float* __restrict__ s_out,
                                                                  float* __restrict__ E, float* __restrict__ Es,
                                                                  int* __restrict__ status, int max_sweeps) {
+  pdl_wait();
   extern __shared__ double sm[];
   // column-major: A[c * ls + r], rows l .. 8 NR - 1 and column l (the padding player's) all zero, so that no access of a
   // round needs a test; the stride is odd (the four pairs of a warp start in different banks)
@@ -437,7 +441,7 @@ cudaError_t jacobi_eig_launch(const double* partial, int nchunk, int batch, int 
   auto kern = nr <= 1 ? jacobi_eig_kernel<1> : nr == 2 ? jacobi_eig_kernel<2> : nr == 3 ? jacobi_eig_kernel<3>
             : nr == 4 ? jacobi_eig_kernel<4> : nr == 5 ? jacobi_eig_kernel<5> : nr == 6 ? jacobi_eig_kernel<6>
             : nr == 7 ? jacobi_eig_kernel<7> : jacobi_eig_kernel<8>;
-  kern<<<batch, threads, smem, st>>>(partial, nchunk, l, signed_input, s_out, E, Es, status, max_sweeps > 0 ? max_sweeps : 40);
+  launch_kernel(kern, batch, threads, smem, st, partial, nchunk, l, signed_input, s_out, E, Es, status, max_sweeps > 0 ? max_sweeps : 40);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -447,6 +451,7 @@ cudaError_t jacobi_eig_launch(const double* partial, int nchunk, int batch, int 
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) frob_partial_kernel(const void* __restrict__ X, int dtype, long long count,
                                                            int nblk, double* __restrict__ partial) {
+  pdl_wait();
   __shared__ double red[8];
   const int bz = blockIdx.y, tid = threadIdx.x;
   const long long per = (count + nblk - 1) / nblk;
@@ -474,7 +479,7 @@ __global__ void __launch_bounds__(256) frob_partial_kernel(const void* __restric
 
 cudaError_t frob_partial_launch(const void* X, int dtype, int batch, long long count, int nblk, double* partial,
                                 cudaStream_t st, long long* launches) {
-  frob_partial_kernel<<<dim3(nblk, batch), 256, 0, st>>>(X, dtype, count, nblk, partial);
+  launch_kernel(frob_partial_kernel, dim3(nblk, batch), 256, 0, st, X, dtype, count, nblk, partial);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -484,6 +489,7 @@ cudaError_t frob_partial_launch(const void* X, int dtype, int batch, long long c
 __global__ void rho_finalize_kernel(const double* __restrict__ partial, int nper, int batch, float* __restrict__ rho,
                                     float* __restrict__ inv_rho, float* __restrict__ inv_rho2,
                                     int* __restrict__ status) {
+  pdl_wait();
   const int bz = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (bz >= batch) return;
   double t = 0.0;
@@ -501,7 +507,7 @@ __global__ void rho_finalize_kernel(const double* __restrict__ partial, int nper
 
 cudaError_t rho_finalize_launch(const double* partial, int nper, int batch, float* rho, float* inv_rho,
                                 float* inv_rho2, int* status, cudaStream_t st, long long* launches) {
-  rho_finalize_kernel<<<(batch + 3) / 4, 128, 0, st>>>(partial, nper, batch, rho, inv_rho, inv_rho2, status);
+  launch_kernel(rho_finalize_kernel, (batch + 3) / 4, 128, 0, st, partial, nper, batch, rho, inv_rho, inv_rho2, status);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -512,6 +518,7 @@ cudaError_t rho_finalize_launch(const double* partial, int nper, int batch, floa
 template <typename T, int V>
 __global__ void __launch_bounds__(256) frob_partial_vec_kernel(const T* __restrict__ X, long long count, int nblk,
                                                                double* __restrict__ partial) {
+  pdl_wait();
   struct alignas(16) Pack { T v[V]; };
   __shared__ double red[8];
   const int bz = blockIdx.y, tid = threadIdx.x;
@@ -560,8 +567,8 @@ cudaError_t frob_partial_vec_launch(const void* X, int dtype, int batch, long lo
   const int es = (int)dtype_size(dtype);
   const bool aligned = (reinterpret_cast<uintptr_t>(X) & 15) == 0 && ((count * es) & 15) == 0;
   if (!aligned || dtype == F16) return frob_partial_launch(X, dtype, batch, count, nblk, partial, st, launches);
-  if (dtype == BF16) frob_partial_vec_kernel<__nv_bfloat16, 8><<<dim3(nblk, batch), 256, 0, st>>>((const __nv_bfloat16*)X, count, nblk, partial);
-  else frob_partial_vec_kernel<float, 4><<<dim3(nblk, batch), 256, 0, st>>>((const float*)X, count, nblk, partial);
+  if (dtype == BF16) launch_kernel(frob_partial_vec_kernel<__nv_bfloat16, 8>, dim3(nblk, batch), 256, 0, st, (const __nv_bfloat16*)X, count, nblk, partial);
+  else launch_kernel(frob_partial_vec_kernel<float, 4>, dim3(nblk, batch), 256, 0, st, (const float*)X, count, nblk, partial);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -573,6 +580,7 @@ cudaError_t frob_partial_vec_launch(const void* X, int dtype, int batch, long lo
 __global__ void rho_identity_kernel(const double* __restrict__ partial, int nper, int batch, const float* __restrict__ s,
                                     int ld_s, const int* __restrict__ keff, float* __restrict__ rho,
                                     float* __restrict__ inv_rho, float* __restrict__ inv_rho2, int* __restrict__ status) {
+  pdl_wait();
   const int bz = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (bz >= batch) return;
   double t = 0.0;
@@ -594,7 +602,7 @@ __global__ void rho_identity_kernel(const double* __restrict__ partial, int nper
 cudaError_t rho_identity_launch(const double* partial, int nper, int batch, const float* s, int ld_s, const int* keff,
                                 float* rho, float* inv_rho, float* inv_rho2, int* status, cudaStream_t st,
                                 long long* launches) {
-  rho_identity_kernel<<<(batch + 3) / 4, 128, 0, st>>>(partial, nper, batch, s, ld_s, keff, rho, inv_rho, inv_rho2, status);
+  launch_kernel(rho_identity_kernel, (batch + 3) / 4, 128, 0, st, partial, nper, batch, s, ld_s, keff, rho, inv_rho, inv_rho2, status);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -605,6 +613,7 @@ cudaError_t rho_identity_launch(const double* partial, int nper, int batch, cons
 // storage format) reaches the Gram matrix of the next step and from there every entry of the following iterate.
 __global__ void __launch_bounds__(1024) finite_probe_kernel(const void* __restrict__ X, int dtype, long long count,
                                                            int* __restrict__ status) {
+  pdl_wait();
   const int bz = blockIdx.x, tid = threadIdx.x;
   const long long base = (long long)bz * count;
   const long long stride = max((long long)1, count / 4096);
@@ -625,7 +634,7 @@ __global__ void __launch_bounds__(1024) finite_probe_kernel(const void* __restri
 cudaError_t finite_probe_launch(const void* X, int dtype, int batch, long long count, int* status, cudaStream_t st,
                                 long long* launches) {
   if (batch <= 0 || count <= 0) return cudaSuccess;
-  finite_probe_kernel<<<batch, 1024, 0, st>>>(X, dtype, count, status);
+  launch_kernel(finite_probe_kernel, batch, 1024, 0, st, X, dtype, count, status);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -635,6 +644,7 @@ __global__ void scale_cols_kernel(const float* __restrict__ In, long long in_bs,
                                   const float* __restrict__ s, int ld_s, const float* __restrict__ inv_rho, float c0,
                                   float c1, float* __restrict__ Out, long long out_bs, int ld_out,
                                   const int* __restrict__ keff) {
+  pdl_wait();
   const int bz = blockIdx.y;
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)rows * k) return;
@@ -649,7 +659,7 @@ cudaError_t scale_cols_launch(const float* In, long long in_bs, int ld_in, int b
                               int ld_out, cudaStream_t st, long long* launches, const int* keff) {
   if (k <= 0) return cudaSuccess;
   const long long tot = (long long)rows * k;
-  scale_cols_kernel<<<dim3((unsigned)((tot + 255) / 256), batch), 256, 0, st>>>(In, in_bs, ld_in, rows, k, s, ld_s,
+  launch_kernel(scale_cols_kernel, dim3((unsigned)((tot + 255) / 256), batch), 256, 0, st, In, in_bs, ld_in, rows, k, s, ld_s,
                                                                                inv_rho, c0, c1, Out, out_bs, ld_out, keff);
   if (launches) ++*launches;
   return cudaGetLastError();
@@ -658,6 +668,7 @@ cudaError_t scale_cols_launch(const float* In, long long in_bs, int ld_in, int b
 // Out[b, i] = scale[b] * In[b, i]  (type conversion allowed)
 __global__ void scale_kernel(const void* __restrict__ In, int in_dt, void* __restrict__ Out, int out_dt,
                              long long count, const float* __restrict__ scale, int round_tf32, float mult) {
+  pdl_wait();
   const int bz = blockIdx.y;
   const float sc = (scale ? scale[bz] : 1.f) * mult;
   const long long base = (long long)bz * count;
@@ -672,7 +683,7 @@ __global__ void scale_kernel(const void* __restrict__ In, int in_dt, void* __res
 cudaError_t scale_launch(const void* In, int in_dt, void* Out, int out_dt, int batch, long long count,
                          const float* scale, cudaStream_t st, long long* launches, int round_tf32, float mult) {
   const int nblk = (int)min((long long)1184, (count + 255) / 256);
-  scale_kernel<<<dim3(nblk, batch), 256, 0, st>>>(In, in_dt, Out, out_dt, count, scale, round_tf32, mult);
+  launch_kernel(scale_kernel, dim3(nblk, batch), 256, 0, st, In, in_dt, Out, out_dt, count, scale, round_tf32, mult);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -689,6 +700,7 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
 
 __global__ void fill_gaussian_kernel(void* __restrict__ dst, long long count, int dtype, unsigned long long seed,
                                      long long per_stream, unsigned long long seed_stride) {
+  pdl_wait();
   // element e belongs to stream e / per_stream (seed + stream * seed_stride), index e % per_stream
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < count;
        e += (long long)gridDim.x * blockDim.x) {
@@ -710,18 +722,19 @@ cudaError_t fill_gaussian_launch(void* dst, long long count, int dtype, unsigned
                                  unsigned long long seed_stride, cudaStream_t st, long long* launches) {
   if (count <= 0) return cudaSuccess;
   const int nblk = (int)min((long long)2368, (count + 255) / 256);
-  fill_gaussian_kernel<<<nblk, 256, 0, st>>>(dst, count, dtype, seed, per_stream, seed_stride);
+  launch_kernel(fill_gaussian_kernel, nblk, 256, 0, st, dst, count, dtype, seed, per_stream, seed_stride);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
 
 __global__ void fill_int_kernel(int* p, int n, int v) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) p[i] = v;
 }
 cudaError_t fill_int_launch(int* p, int n, int v, cudaStream_t st, long long* launches) {
   if (n <= 0) return cudaSuccess;
-  fill_int_kernel<<<(n + 255) / 256, 256, 0, st>>>(p, n, v);
+  launch_kernel(fill_int_kernel, (n + 255) / 256, 256, 0, st, p, n, v);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -730,12 +743,13 @@ cudaError_t fill_int_launch(int* p, int n, int v, cudaStream_t st, long long* la
 
 namespace defl {
 __global__ void or_status_kernel(int* status, int n, const int* word) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) status[i] |= *word;
 }
 cudaError_t or_status_launch(int* status, int n, const int* word, cudaStream_t st, long long* launches) {
   if (n <= 0) return cudaSuccess;
-  or_status_kernel<<<(n + 255) / 256, 256, 0, st>>>(status, n, word);
+  launch_kernel(or_status_kernel, (n + 255) / 256, 256, 0, st, status, n, word);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -779,9 +793,9 @@ extern "C" int defl_frobenius_norms_noalloc(const void* X, int dtype, int b, lon
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   // every slot read by the second kernel is written by the first, so nothing needs clearing
-  frob_partial_kernel<<<dim3(NOALLOC_NBLK, b), 256, 0, st>>>(X, dtype, count, NOALLOC_NBLK, scratch);
+  launch_kernel(frob_partial_kernel, dim3(NOALLOC_NBLK, b), 256, 0, st, X, dtype, count, NOALLOC_NBLK, scratch);
   if (cudaGetLastError() != cudaSuccess) return DEFL_ERR_CUDA;
-  rho_finalize_kernel<<<(b + 3) / 4, 128, 0, st>>>(scratch, NOALLOC_NBLK, b, norms, nullptr, nullptr, nullptr);
+  launch_kernel(rho_finalize_kernel, (b + 3) / 4, 128, 0, st, scratch, NOALLOC_NBLK, b, norms, nullptr, nullptr, nullptr);
   if (cudaGetLastError() != cudaSuccess) return DEFL_ERR_CUDA;
   return DEFL_OK;
 }
@@ -795,6 +809,7 @@ namespace defl {
 // hi, lo [b, rows, lp] from In [b, rows, l] (leading dimension ld_in); columns l..lp-1 are zero.
 __global__ void split_panel_kernel(const float* __restrict__ In, long long in_bs, int ld_in, int rows, int l, int lp,
                                    __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
+  pdl_wait();
   const int bz = blockIdx.y;
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)rows * lp) return;
@@ -809,7 +824,7 @@ __global__ void split_panel_kernel(const float* __restrict__ In, long long in_bs
 cudaError_t split_panel_launch(const float* In, long long in_bs, int ld_in, int batch, int rows, int l, int lp,
                                __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t st, long long* launches) {
   const long long tot = (long long)rows * lp;
-  split_panel_kernel<<<dim3((unsigned)((tot + 255) / 256), batch), 256, 0, st>>>(In, in_bs, ld_in, rows, l, lp, hi, lo);
+  launch_kernel(split_panel_kernel, dim3((unsigned)((tot + 255) / 256), batch), 256, 0, st, In, in_bs, ld_in, rows, l, lp, hi, lo);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -825,6 +840,7 @@ __global__ void split_concat3_kernel(const float* __restrict__ In, long long in_
                                      const float* __restrict__ s, int ld_s, const float* __restrict__ inv_rho, float c0,
                                      float c1, float mult, int pattern, uint16_t* __restrict__ Out,
                                      const int* __restrict__ keff, const float* __restrict__ rho) {
+  pdl_wait();
   const int bz = blockIdx.y;
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)rows * kp) return;
@@ -860,10 +876,10 @@ cudaError_t split_concat3_launch(const float* In, long long in_bs, int ld_in, in
   const long long tot = (long long)rows * kp;
   const dim3 grid((unsigned)((tot + 255) / 256), batch);
   uint16_t* o = reinterpret_cast<uint16_t*>(Out);
-  if (f16 && transposed) split_concat3_kernel<true, true><<<grid, 256, 0, st>>>(In, in_bs, ld_in, rows, k, kp, s, ld_s, inv_rho, c0, c1, mult, pattern, o, keff, rho);
-  else if (f16) split_concat3_kernel<true, false><<<grid, 256, 0, st>>>(In, in_bs, ld_in, rows, k, kp, s, ld_s, inv_rho, c0, c1, mult, pattern, o, keff, rho);
-  else if (transposed) split_concat3_kernel<false, true><<<grid, 256, 0, st>>>(In, in_bs, ld_in, rows, k, kp, s, ld_s, inv_rho, c0, c1, mult, pattern, o, keff, rho);
-  else split_concat3_kernel<false, false><<<grid, 256, 0, st>>>(In, in_bs, ld_in, rows, k, kp, s, ld_s, inv_rho, c0, c1, mult, pattern, o, keff, rho);
+  if (f16 && transposed) launch_kernel(split_concat3_kernel<true, true>, grid, 256, 0, st, In, in_bs, ld_in, rows, k, kp, s, ld_s, inv_rho, c0, c1, mult, pattern, o, keff, rho);
+  else if (f16) launch_kernel(split_concat3_kernel<true, false>, grid, 256, 0, st, In, in_bs, ld_in, rows, k, kp, s, ld_s, inv_rho, c0, c1, mult, pattern, o, keff, rho);
+  else if (transposed) launch_kernel(split_concat3_kernel<false, true>, grid, 256, 0, st, In, in_bs, ld_in, rows, k, kp, s, ld_s, inv_rho, c0, c1, mult, pattern, o, keff, rho);
+  else launch_kernel(split_concat3_kernel<false, false>, grid, 256, 0, st, In, in_bs, ld_in, rows, k, kp, s, ld_s, inv_rho, c0, c1, mult, pattern, o, keff, rho);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -873,6 +889,7 @@ cudaError_t split_concat3_launch(const float* In, long long in_bs, int ld_in, in
 // whole call on the tensor cores. Bound by memory: 16 bytes per store, the eight loads of a thread side by side.
 __global__ void __launch_bounds__(256) pad_rows_kernel(const uint16_t* __restrict__ In, uint16_t* __restrict__ Out, long long rows,
                                                        int n, int ld) {
+  pdl_wait();
   const int per = ld / 8;
   const long long total = rows * per, stride = (long long)gridDim.x * blockDim.x;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += stride) {
@@ -888,7 +905,7 @@ __global__ void __launch_bounds__(256) pad_rows_kernel(const uint16_t* __restric
 cudaError_t pad_rows_launch(const void* In, void* Out, int batch, int rows, int n, int ld, cudaStream_t st, long long* launches) {
   const long long total = (long long)batch * rows * (ld / 8);
   const int nblk = (int)min((long long)148 * 16, (total + 255) / 256);
-  pad_rows_kernel<<<nblk, 256, 0, st>>>((const uint16_t*)In, (uint16_t*)Out, (long long)batch * rows, n, ld);
+  launch_kernel(pad_rows_kernel, nblk, 256, 0, st, (const uint16_t*)In, (uint16_t*)Out, (long long)batch * rows, n, ld);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -899,6 +916,7 @@ __global__ void __launch_bounds__(256) zero_residual_entry_kernel(const int* __r
                                                                   const float* __restrict__ W, const int* __restrict__ keff,
                                                                   int m, int n, int ld, int k, float scale, void* __restrict__ X0,
                                                                   int dtype) {
+  pdl_wait();
   const int bz = blockIdx.y;
   if (!(status[bz] & 4)) return;
   const float* Pb = P + (long long)bz * m * k;
@@ -915,7 +933,7 @@ __global__ void __launch_bounds__(256) zero_residual_entry_kernel(const int* __r
 
 cudaError_t zero_residual_entry_launch(const int* status, const float* P, const float* W, const int* keff, int batch, int m,
                                        int n, int ld, int k, float scale, void* X0, int dtype, cudaStream_t st, long long* launches) {
-  zero_residual_entry_kernel<<<dim3(64, batch), 256, 0, st>>>(status, P, W, keff, m, n, ld, k, scale, X0, dtype);
+  launch_kernel(zero_residual_entry_kernel, dim3(64, batch), 256, 0, st, status, P, W, keff, m, n, ld, k, scale, X0, dtype);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -925,6 +943,7 @@ cudaError_t zero_residual_entry_launch(const int* status, const float* P, const 
 //   tau > 0 : if |s_window| < tau |s_1| then keff = #{i < kmax : |s_i| > tau |s_1|}, else keff = 0.
 __global__ void gate_kernel(const float* __restrict__ s, int ld_s, int batch, int window, int kmax, float tau,
                             int* __restrict__ keff) {
+  pdl_wait();
   const int bz = blockIdx.x * blockDim.x + threadIdx.x;
   if (bz >= batch) return;
   const float* sb = s + (long long)bz * ld_s;
@@ -940,7 +959,7 @@ __global__ void gate_kernel(const float* __restrict__ s, int ld_s, int batch, in
 
 cudaError_t gate_launch(const float* s, int ld_s, int batch, int window, int kmax, float tau, int* keff, cudaStream_t st,
                         long long* launches) {
-  gate_kernel<<<(batch + 127) / 128, 128, 0, st>>>(s, ld_s, batch, window, kmax, tau, keff);
+  launch_kernel(gate_kernel, (batch + 127) / 128, 128, 0, st, s, ld_s, batch, window, kmax, tau, keff);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -983,6 +1002,7 @@ __global__ void __launch_bounds__(256, 2) panel_fused_kernel(const float* In, lo
                                                           float* Out, long long out_bs, int ld_out,
                                                           __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
                                                           int lp, double* __restrict__ partial, int nchunk) {
+  pdl_wait();
   extern __shared__ __align__(16) float fsm[];
   // row stride 68 floats: rows stay 16-byte aligned, so register blocks are fetched with 128-bit loads
   float (*tile)[FUSED_TS] = reinterpret_cast<float (*)[FUSED_TS]>(fsm);                          // [128][68]
@@ -1195,7 +1215,7 @@ cudaError_t panel_fused_launch(const float* In, long long in_bs, int ld_in, int 
   const size_t smem = (size_t)(FUSED_TILE + MAX_L) * FUSED_TS * sizeof(float);
   cudaFuncSetAttribute(panel_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int nchunk = fused_num_chunks(rows, batch);
-  panel_fused_kernel<<<dim3(nchunk, batch), 256, smem, st>>>(In, in_bs, ld_in, rows, l, Mtx, ldm, kout, Out, out_bs, ld_out,
+  launch_kernel(panel_fused_kernel, dim3(nchunk, batch), 256, smem, st, In, in_bs, ld_in, rows, l, Mtx, ldm, kout, Out, out_bs, ld_out,
                                                             hi, lo, lp, partial, nchunk);
   if (launches) ++*launches;
   return cudaGetLastError();
@@ -1208,6 +1228,7 @@ cudaError_t panel_fused_launch(const float* In, long long in_bs, int ld_in, int 
 // ---------------------------------------------------------------------------------------------
 template <typename T, int V>
 __global__ void __launch_bounds__(256) momentum_vec_kernel(T* Mom, const T* __restrict__ Grad, T* look, long long nvec, float mu) {
+  pdl_wait();
   // V elements (16 bytes) per thread and trip
   struct alignas(16) Pack { T v[V]; };
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -1228,6 +1249,7 @@ __global__ void __launch_bounds__(256) momentum_vec_kernel(T* Mom, const T* __re
 
 __global__ void __launch_bounds__(256) momentum_kernel(void* Mom, const void* __restrict__ Grad, void* look, int dtype,
                                                        long long first, long long count, float mu) {
+  pdl_wait();
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long i = first + (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += stride) {
     const float g = ld_as_float(Grad, i, dtype);
@@ -1244,13 +1266,13 @@ cudaError_t momentum_launch(void* Mom, const void* Grad, void* look, int dtype, 
   if (nvec > 0) {
     const int nblk = (int)min((long long)148 * 16, (nvec + 255) / 256);
     if (dtype == BF16)
-      momentum_vec_kernel<__nv_bfloat16, 8><<<nblk, 256, 0, st>>>((__nv_bfloat16*)Mom, (const __nv_bfloat16*)Grad, (__nv_bfloat16*)look, nvec, mu);
+      launch_kernel(momentum_vec_kernel<__nv_bfloat16, 8>, nblk, 256, 0, st, (__nv_bfloat16*)Mom, (const __nv_bfloat16*)Grad, (__nv_bfloat16*)look, nvec, mu);
     else
-      momentum_vec_kernel<float, 4><<<nblk, 256, 0, st>>>((float*)Mom, (const float*)Grad, (float*)look, nvec, mu);
+      launch_kernel(momentum_vec_kernel<float, 4>, nblk, 256, 0, st, (float*)Mom, (const float*)Grad, (float*)look, nvec, mu);
     if (launches) ++*launches;
   }
   if (nvec * per < count) {      // the unaligned or leftover part
-    momentum_kernel<<<1, 256, 0, st>>>(Mom, Grad, look, dtype, nvec * per, count, mu);
+    launch_kernel(momentum_kernel, 1, 256, 0, st, Mom, Grad, look, dtype, nvec * per, count, mu);
     if (launches) ++*launches;
   }
   return cudaGetLastError();

@@ -23,6 +23,7 @@ namespace defl {
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) symv_kernel(const float* __restrict__ A, const float* __restrict__ x,
                                                    float* __restrict__ y, int n, const int* __restrict__ skip) {
+  pdl_wait();
   if (skip && *skip) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool vec = (n & 3) == 0;
@@ -80,6 +81,7 @@ __global__ void __launch_bounds__(256) symv_kernel(const float* __restrict__ A, 
 // out[i] = sum over s of part[s * count + i], s in ascending order (fixed order: reproducible)
 __global__ void __launch_bounds__(256) sum_slices_kernel(const float* __restrict__ part, int slices, long long count,
                                                          float* __restrict__ out) {
+  pdl_wait();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   float t = 0.f;
@@ -88,7 +90,7 @@ __global__ void __launch_bounds__(256) sum_slices_kernel(const float* __restrict
 }
 static cudaError_t sum_slices_launch(const float* part, int slices, long long count, float* out, cudaStream_t st,
                                      long long* launches) {
-  sum_slices_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(part, slices, count, out);
+  launch_kernel(sum_slices_kernel, (unsigned)((count + 255) / 256), 256, 0, st, part, slices, count, out);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -97,7 +99,7 @@ static cudaError_t symv_launch(const float* A, const float* x, float* y, int n, 
                                long long* launches) {
   int grid = (n + 7) / 8;
   if (grid > 148 * 8) grid = 148 * 8;
-  symv_kernel<<<grid, 256, 0, st>>>(A, x, y, n, skip);
+  launch_kernel(symv_kernel, grid, 256, 0, st, A, x, y, n, skip);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -135,6 +137,7 @@ __device__ double block_sum(double v, double* red) {
 }
 
 __global__ void __launch_bounds__(1024) lanczos_init_kernel(const float* __restrict__ v0, int n, int steps, LanczosState s) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) a += (double)v0[i] * (double)v0[i];
@@ -145,6 +148,7 @@ __global__ void __launch_bounds__(1024) lanczos_init_kernel(const float* __restr
 }
 
 __global__ void __launch_bounds__(1024) lanczos_step_kernel(int j, int n, int steps, LanczosState s) {
+  pdl_wait();
   __shared__ double red[32];
   __shared__ double coef[DEFL_LANCZOS_STEPS];
   if (*s.done) return;
@@ -195,6 +199,7 @@ __global__ void __launch_bounds__(1024) lanczos_step_kernel(int j, int n, int st
 // spent 22 us per step on fp64 instruction issue alone.
 template <int EPT>
 __global__ void __launch_bounds__(1024) lanczos_step_reg_kernel(int j, int n, int steps, LanczosState s) {
+  pdl_wait();
   __shared__ double part[32][DEFL_LANCZOS_STEPS];
   __shared__ double coef[DEFL_LANCZOS_STEPS];
   __shared__ double red[32];
@@ -341,6 +346,7 @@ __device__ double tridiag_top(const double* al, const double* be, int steps, dou
 // the same from the dense matrix [steps, steps] in device memory: rho[0] and column 0 of E (fp32, [steps, steps] row-major)
 __global__ void __launch_bounds__(32) tridiag_top_kernel(const double* __restrict__ T, int steps, float* __restrict__ rho,
                                                          float* __restrict__ E) {
+  pdl_wait();
   __shared__ double al[DEFL_LANCZOS_STEPS], be[DEFL_LANCZOS_STEPS], y[DEFL_LANCZOS_STEPS];
   const int lane = threadIdx.x;
   if (lane < steps) {
@@ -357,6 +363,7 @@ __global__ void __launch_bounds__(32) tridiag_top_kernel(const double* __restric
 // carry a zero coefficient (those after a breakdown, never written) are not read
 __global__ void lanczos_ritz_kernel(int n, int steps, const float* __restrict__ Q, const float* __restrict__ E,
                                     float* __restrict__ v) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double a = 0.0;
@@ -371,6 +378,7 @@ __global__ void lanczos_ritz_kernel(int n, int steps, const float* __restrict__ 
 __global__ void __launch_bounds__(1024) lanczos_theta_kernel(int n, const float* __restrict__ rho_p,
                                                              const float* __restrict__ v, const float* __restrict__ w,
                                                              float* theta, float* inv_theta, int* status) {
+  pdl_wait();
   __shared__ double red[32];
   const double rho = (double)rho_p[0];
   double a = 0.0;
@@ -501,6 +509,7 @@ __device__ __forceinline__ void cluster_barrier() {
 
 template <bool CLUSTER>
 __global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const LanczosRun p) {
+  pdl_wait();
   extern __shared__ __align__(16) float lz[];
   constexpr int MS = DEFL_LANCZOS_STEPS;
   const int n = p.n, steps = p.steps, R = p.rows, G = gridDim.x, blk = blockIdx.x;
@@ -748,7 +757,9 @@ static bool lanczos_launch(defl_ctx* c, const float* A, const float* start, int 
     const size_t smem = layout(LZ_CLUSTER, 2);
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = LZ_CLUSTER; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(LZ_CLUSTER, 1, 1); cfg.blockDim = dim3(LZ_THREADS, 1, 1); cfg.dynamicSmemBytes = smem; cfg.stream = c->stream;
@@ -757,6 +768,7 @@ static bool lanczos_launch(defl_ctx* c, const float* A, const float* start, int 
     if (smem > 0 && cudaFuncSetAttribute(lanczos_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
         cudaFuncSetAttribute(lanczos_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
         cudaOccupancyMaxActiveClusters(&clusters, lanczos_kernel<true>, &cfg) == cudaSuccess && clusters > 0) {
+      cfg.numAttrs = 2;
       *err = cudaLaunchKernelEx(&cfg, lanczos_kernel<true>, p);
       ++c->launches;
       return true;
@@ -782,6 +794,7 @@ static bool lanczos_launch(defl_ctx* c, const float* A, const float* start, int 
 
 // P <- (P + P^T)/2 in place, 32 x 32 tiles through shared memory; tile pair (bi <= bj) per CTA
 __global__ void __launch_bounds__(256) symmetrise_kernel(float* __restrict__ P, int n) {
+  pdl_wait();
   __shared__ float ta[32][33], tb[32][33];
   const int bi = blockIdx.y, bj = blockIdx.x;
   if (bj < bi) return;
@@ -803,6 +816,7 @@ __global__ void __launch_bounds__(256) symmetrise_kernel(float* __restrict__ P, 
 
 // hi = tf32(x) (round to nearest), lo = tf32(x - hi)
 __global__ void split_tf32_kernel(const float* __restrict__ X, float* __restrict__ hi, float* __restrict__ lo, long long count) {
+  pdl_wait();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x) {
     const float x = X[i];
     const float h = round_to_tf32(x);
@@ -817,6 +831,7 @@ __global__ void split_tf32_kernel(const float* __restrict__ X, float* __restrict
 __global__ void ritz_scale_kernel(const float* __restrict__ lam, int k, int mode, float gamma, int neg, float* __restrict__ out,
                                   const int* __restrict__ keff, const float* __restrict__ root_scale, float z_pad, int p,
                                   int* __restrict__ status) {
+  pdl_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= k) return;
   if (t >= keff[0]) { out[t] = 0.f; return; }     // not in the deflated set (gate)
@@ -834,6 +849,7 @@ __global__ void ritz_scale_kernel(const float* __restrict__ lam, int k, int mode
 
 // root_scale = theta^(-1/p) (0 when theta is not a positive number: the status bit is already set by the estimate)
 __global__ void root_scale_kernel(const float* __restrict__ theta, int p, float* __restrict__ out) {
+  pdl_wait();
   const double th = (double)theta[0];
   out[0] = (th > 0.0 && isfinite(th)) ? (float)pow(th, -1.0 / (double)p) : 0.f;
 }
@@ -841,6 +857,7 @@ __global__ void root_scale_kernel(const float* __restrict__ theta, int p, float*
 // T = a I + b M for n x n fp32 matrices (the step matrix of the coupled Newton iteration), optionally rounded to tf32
 __global__ void __launch_bounds__(256) affine_identity_kernel(const float* __restrict__ M, float a, float b,
                                                               float* __restrict__ T, int n, int round_tf32) {
+  pdl_wait();
   const long long total = (long long)n * n;
   const long long stride = (long long)gridDim.x * blockDim.x;
   if ((n & 3) == 0) {
@@ -941,28 +958,28 @@ static int estimate_scale(defl_ctx* c, const float* A, int n, int norm_mode, con
   }
   LanczosState s;
   s.Q = w.Q; s.T = w.T; s.w = w.lw; s.t = w.lt; s.done = w.done; s.beta_prev = w.beta_prev;
-  lanczos_init_kernel<<<1, 1024, 0, c->stream>>>(start, n, steps, s);
+  launch_kernel(lanczos_init_kernel, 1, 1024, 0, c->stream, start, n, steps, s);
   ++c->launches;
   if (ctx_fail(c, cudaGetLastError(), "lanczos init")) return DEFL_ERR_CUDA;
   for (int j = 0; j < steps; ++j) {
     if (ctx_fail(c, symv_launch(A, w.Q + (size_t)j * n, w.lt, n, w.done, c->stream, &c->launches), "symv")) return DEFL_ERR_CUDA;
     if (ctx_fail(c, symv_launch(A, w.lt, w.lw, n, w.done, c->stream, &c->launches), "symv")) return DEFL_ERR_CUDA;
-    if (n <= 4096) lanczos_step_reg_kernel<4><<<1, 1024, 0, c->stream>>>(j, n, steps, s);
-    else if (n <= 8192) lanczos_step_reg_kernel<8><<<1, 1024, 0, c->stream>>>(j, n, steps, s);
-    else lanczos_step_kernel<<<1, 1024, 0, c->stream>>>(j, n, steps, s);
+    if (n <= 4096) launch_kernel(lanczos_step_reg_kernel<4>, 1, 1024, 0, c->stream, j, n, steps, s);
+    else if (n <= 8192) launch_kernel(lanczos_step_reg_kernel<8>, 1, 1024, 0, c->stream, j, n, steps, s);
+    else launch_kernel(lanczos_step_kernel, 1, 1024, 0, c->stream, j, n, steps, s);
     ++c->launches;
     if (ctx_fail(c, cudaGetLastError(), "lanczos step")) return DEFL_ERR_CUDA;
   }
   // largest Ritz pair of the (zero-padded) tridiagonal matrix
-  tridiag_top_kernel<<<1, 32, 0, c->stream>>>(w.T, steps, w.lrho, w.lE);
+  launch_kernel(tridiag_top_kernel, 1, 32, 0, c->stream, w.T, steps, w.lrho, w.lE);
   ++c->launches;
   if (ctx_fail(c, cudaGetLastError(), "ritz")) return DEFL_ERR_CUDA;
-  lanczos_ritz_kernel<<<(n + 255) / 256, 256, 0, c->stream>>>(n, steps, w.Q, w.lE, w.lv);
+  launch_kernel(lanczos_ritz_kernel, (n + 255) / 256, 256, 0, c->stream, n, steps, w.Q, w.lE, w.lv);
   ++c->launches;
   if (ctx_fail(c, cudaGetLastError(), "ritz vector")) return DEFL_ERR_CUDA;
   if (ctx_fail(c, symv_launch(A, w.lv, w.lt, n, nullptr, c->stream, &c->launches), "symv")) return DEFL_ERR_CUDA;
   if (ctx_fail(c, symv_launch(A, w.lt, w.lw, n, nullptr, c->stream, &c->launches), "symv")) return DEFL_ERR_CUDA;
-  lanczos_theta_kernel<<<1, 1024, 0, c->stream>>>(n, w.lrho, w.lv, w.lw, w.theta, w.inv_theta, w.status);
+  launch_kernel(lanczos_theta_kernel, 1, 1024, 0, c->stream, n, w.lrho, w.lv, w.lw, w.theta, w.inv_theta, w.status);
   ++c->launches;
   if (ctx_fail(c, cudaGetLastError(), "theta")) return DEFL_ERR_CUDA;
   return DEFL_OK;
@@ -972,7 +989,7 @@ static int estimate_scale(defl_ctx* c, const float* A, int n, int norm_mode, con
 static int rank_update(defl_ctx* c, const PsdWs& w, int n, int K, int k, int coef_mode, float gamma, int neg,
                        const float* aux, float aux_scale, const float* aux_scale_dev, float* C, int round_tf32 = 0,
                        float z_pad = 0.f, int root_p = 1) {
-  ritz_scale_kernel<<<1, 64, 0, c->stream>>>(w.lam, k, coef_mode, gamma, neg, w.coef, w.keff, w.rscale, z_pad, root_p, w.status);
+  launch_kernel(ritz_scale_kernel, 1, 64, 0, c->stream, w.lam, k, coef_mode, gamma, neg, w.coef, w.keff, w.rscale, z_pad, root_p, w.status);
   ++c->launches;
   if (ctx_fail(c, cudaGetLastError(), "ritz scale")) return DEFL_ERR_CUDA;
   if (ctx_fail(c, scale_cols_launch(w.U, 0, K, 1, n, k, w.coef, K, nullptr, 1.f, 0.f, w.Us, 0, K, c->stream, &c->launches), "U diag"))
@@ -995,6 +1012,7 @@ static int rank_update(defl_ctx* c, const PsdWs& w, int n, int K, int k, int coe
 // y_i = b_i / sigma - (X_ii / sigma + S_ii - C_ii)
 __global__ void admm_y_kernel(const float* __restrict__ C, const float* __restrict__ X, const float* __restrict__ S,
                               const float* __restrict__ b, float* __restrict__ y, int n, float inv_sigma) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const long long d = (long long)i * n + i;
@@ -1005,6 +1023,7 @@ __global__ void admm_y_kernel(const float* __restrict__ C, const float* __restri
 __global__ void __launch_bounds__(256) admm_z_kernel(const float* __restrict__ C, const float* __restrict__ X,
                                                      const float* __restrict__ y, float* __restrict__ Z, int n,
                                                      float inv_sigma) {
+  pdl_wait();
   const long long total4 = (long long)n * n / 4;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total4; q += stride) {
@@ -1023,6 +1042,7 @@ __global__ void __launch_bounds__(256) admm_x_kernel(const float* __restrict__ C
                                                      const float* __restrict__ y, const float* __restrict__ b,
                                                      float* __restrict__ X, int n, float sigma,
                                                      double* __restrict__ partial) {
+  pdl_wait();
   __shared__ double red[3][8];
   const long long total4 = (long long)n * n / 4;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -1065,6 +1085,7 @@ __global__ void __launch_bounds__(256) admm_x_kernel(const float* __restrict__ C
 __global__ void __launch_bounds__(256) admm_residual_kernel(const double* __restrict__ partial, int nblk, const float* __restrict__ b,
                                                             const float* __restrict__ y, int n, double norm_b, double norm_c,
                                                             float* __restrict__ out3) {
+  pdl_wait();
   __shared__ double red[32];
   double dres = 0.0, obj = 0.0, pres = 0.0, by = 0.0;
   for (int i = threadIdx.x; i < nblk; i += blockDim.x) { dres += partial[3 * i]; obj += partial[3 * i + 1]; pres += partial[3 * i + 2]; }
@@ -1079,6 +1100,7 @@ __global__ void __launch_bounds__(256) admm_residual_kernel(const double* __rest
 // Sum of squares of a float array in fp64 (norms of b and C, once per call): CTA i leaves the sum of its share in out[i],
 // and sum_kernel adds those up.
 __global__ void __launch_bounds__(1024) sumsq_kernel(const float* __restrict__ x, long long count, double* out) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 0.0;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x)
@@ -1087,6 +1109,7 @@ __global__ void __launch_bounds__(1024) sumsq_kernel(const float* __restrict__ x
   if (threadIdx.x == 0) out[blockIdx.x] = a;
 }
 __global__ void __launch_bounds__(256) sum_kernel(const double* __restrict__ sums, int count, double* out) {
+  pdl_wait();
   __shared__ double red[32];
   double a = 0.0;
   for (int i = threadIdx.x; i < count; i += blockDim.x) a += sums[i];
@@ -1238,12 +1261,12 @@ static int psd_core(defl_ctx* c, const void* Xv, void* Pv, int n, int k, float* 
       return run_gemm(c, g, gemm_tc_supported(g) ? engine : DEFL_ENGINE_SIMT, what);
     };
     if (T == 0) {
-      affine_identity_kernel<<<ablk, 256, 0, c->stream>>>(M, 1.f, 0.f, zc, n, 0);
+      launch_kernel(affine_identity_kernel, ablk, 256, 0, c->stream, M, 1.f, 0.f, zc, n, 0);
       ++c->launches;
       if (ctx_fail(c, cudaGetLastError(), "identity")) return DEFL_ERR_CUDA;
     }
     for (int t = 0; t < T; ++t) {
-      affine_identity_kernel<<<ablk, 256, 0, c->stream>>>(M, (float)(root_p + 1) / (float)root_p, -1.f / (float)root_p, Tm, n, tf32_round);
+      launch_kernel(affine_identity_kernel, ablk, 256, 0, c->stream, M, (float)(root_p + 1) / (float)root_p, -1.f / (float)root_p, Tm, n, tf32_round);
       ++c->launches;
       if (ctx_fail(c, cudaGetLastError(), "step matrix")) return DEFL_ERR_CUDA;
       if (t == 0) {
@@ -1330,7 +1353,7 @@ static int psd_core(defl_ctx* c, const void* Xv, void* Pv, int n, int k, float* 
 
   // ---- stage 5 (inverse root): out = theta^(-1/p) (Z - z_pad U U^T) + U diag(lambda^(-1/p)) U^T, symmetrised ----
   if (root_p) {
-    root_scale_kernel<<<1, 1, 0, c->stream>>>(w.theta, root_p, w.rscale);
+    launch_kernel(root_scale_kernel, 1, 1, 0, c->stream, w.theta, root_p, w.rscale);
     ++c->launches;
     if (ctx_fail(c, cudaGetLastError(), "root scale")) return DEFL_ERR_CUDA;
     if (deflate) {
@@ -1346,7 +1369,7 @@ static int psd_core(defl_ctx* c, const void* Xv, void* Pv, int n, int k, float* 
       if (ctx_fail(c, scale_launch(root_z, F32, P, F32, 1, (long long)n * n, w.rscale, c->stream, &c->launches, 0), "scale"))
         return DEFL_ERR_CUDA;
     }
-    symmetrise_kernel<<<dim3((n + 31) / 32, (n + 31) / 32), 256, 0, c->stream>>>(P, n);
+    launch_kernel(symmetrise_kernel, dim3((n + 31) / 32, (n + 31) / 32), 256, 0, c->stream, P, n);
     ++c->launches;
     if (ctx_fail(c, cudaGetLastError(), "symmetrise")) return DEFL_ERR_CUDA;
     // the iteration diverges on an eigenvalue of X0 that is not positive (an indefinite input, or a basis that has not
@@ -1364,7 +1387,7 @@ static int psd_core(defl_ctx* c, const void* Xv, void* Pv, int n, int k, float* 
     if (tf32_round && gemm_tc_supported(g)) {
       // R carries the large entries of this product: feed it as two tf32 terms R = R_hi + R_lo (two K
       // segments against the same g) so that the tensor core does not truncate it
-      split_tf32_kernel<<<1184, 256, 0, c->stream>>>(Rm, w.W, w.Tt, (long long)n * n);
+      launch_kernel(split_tf32_kernel, 1184, 256, 0, c->stream, Rm, w.W, w.Tt, (long long)n * n);
       ++c->launches;
       if (ctx_fail(c, cudaGetLastError(), "split R")) return DEFL_ERR_CUDA;
       g.nseg = 2; g.K[1] = n;
@@ -1378,7 +1401,7 @@ static int psd_core(defl_ctx* c, const void* Xv, void* Pv, int n, int k, float* 
     if (deflate) {
       if ((rc = rank_update(c, w, n, K, kcols, 2, gamma, 0, P, 1.f, nullptr, P))) return rc;
     }
-    symmetrise_kernel<<<dim3((n + 31) / 32, (n + 31) / 32), 256, 0, c->stream>>>(P, n);
+    launch_kernel(symmetrise_kernel, dim3((n + 31) / 32, (n + 31) / 32), 256, 0, c->stream, P, n);
     ++c->launches;
     if (ctx_fail(c, cudaGetLastError(), "symmetrise")) return DEFL_ERR_CUDA;
   }
@@ -1458,9 +1481,9 @@ int defl_admm_diag_sdp(defl_ctx* c, const void* Cv, const float* b, int n, float
   float* hist = reinterpret_cast<float*>(aux + align_up((size_t)nblk * 3 * sizeof(double), 256));
   double* norms = reinterpret_cast<double*>(aux + align_up((size_t)nblk * 3 * sizeof(double), 256) +
                                             align_up((size_t)(iters > 0 ? iters : 1) * 3 * sizeof(float), 256));
-  sumsq_kernel<<<1, 1024, 0, c->stream>>>(b, n, norms);
-  sumsq_kernel<<<c->num_sms, 1024, 0, c->stream>>>(C, (long long)n * n, partial);
-  sum_kernel<<<1, 256, 0, c->stream>>>(partial, c->num_sms, norms + 1);
+  launch_kernel(sumsq_kernel, 1, 1024, 0, c->stream, b, n, norms);
+  launch_kernel(sumsq_kernel, c->num_sms, 1024, 0, c->stream, C, (long long)n * n, partial);
+  launch_kernel(sum_kernel, 1, 256, 0, c->stream, partial, c->num_sms, norms + 1);
   c->launches += 3;
   double hn[2] = {0.0, 0.0};
   if (ctx_fail(c, cudaMemcpyAsync(hn, norms, sizeof(hn), cudaMemcpyDeviceToHost, c->stream), "norms") ||
@@ -1471,15 +1494,15 @@ int defl_admm_diag_sdp(defl_ctx* c, const void* Cv, const float* b, int n, float
   defl_opts o;
   if (opts) o = *opts; else memset(&o, 0, sizeof(o));
   for (int it = 0; it < iters; ++it) {
-    admm_y_kernel<<<(n + 255) / 256, 256, 0, c->stream>>>(C, X, S, b, y, n, inv_sigma);
-    admm_z_kernel<<<nblk, 256, 0, c->stream>>>(C, X, y, Z, n, inv_sigma);
+    launch_kernel(admm_y_kernel, (n + 255) / 256, 256, 0, c->stream, C, X, S, b, y, n, inv_sigma);
+    launch_kernel(admm_z_kernel, nblk, 256, 0, c->stream, C, X, y, Z, n, inv_sigma);
     c->launches += 2;
     if (ctx_fail(c, cudaGetLastError(), "ADMM y, Z")) return DEFL_ERR_CUDA;
     o.warmup = (it < warmup_iters) ? 1 : (opts ? opts->warmup : 0);
     const int rc = defl_psd_project(c, Z, S, n, k, warm_basis, K, coeff_schedule, T, &o, nullptr);
     if (rc) return rc;
-    admm_x_kernel<<<nblk, 256, 0, c->stream>>>(C, S, y, b, X, n, sigma, partial);
-    admm_residual_kernel<<<1, 256, 0, c->stream>>>(partial, nblk, b, y, n, norm_b, norm_c, hist + 3 * it);
+    launch_kernel(admm_x_kernel, nblk, 256, 0, c->stream, C, S, y, b, X, n, sigma, partial);
+    launch_kernel(admm_residual_kernel, 1, 256, 0, c->stream, partial, nblk, b, y, n, norm_b, norm_c, hist + 3 * it);
     c->launches += 2;
     if (ctx_fail(c, cudaGetLastError(), "ADMM X")) return DEFL_ERR_CUDA;
   }
