@@ -423,7 +423,7 @@ def extra_sdp(ctx, peaks, device, n=4096, calls=20, warm=2, tf32_peak=True):
                                 "achieved": flops / (prod_ms * 1e-3) / 1e12, "peak": tf32_peak, "unit": "TFLOP/s",
                                 "frac": flops / (prod_ms * 1e-3) / 1e12 / tf32_peak,
                                 "peak_kind": "torch.matmul 8192^3 with tf32 allowed, best of 10, this run"},
-            "roofline_lanczos": {"bound": "hbm", "kernel": "symv_kernel (42 passes over R) + lanczos_step_kernel",
+            "roofline_lanczos": {"bound": "hbm", "kernel": "lanczos_kernel (42 passes over R)",
                                  "achieved": symv_bytes / (st[2] * 1e-3) / 1e9, "peak": float(peaks.get("hbm_gbs", 6650.0)),
                                  "unit": "GB/s", "frac": symv_bytes / (st[2] * 1e-3) / 1e9 / float(peaks.get("hbm_gbs", 6650.0)),
                                  "note": "R (67 MB) fits the 126 MB L2: passes after the first are served from it"}}
