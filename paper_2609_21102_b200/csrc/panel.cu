@@ -92,71 +92,89 @@ cudaError_t gram_partial_launch(const float* Y, long long batch_stride, int batc
 // Symmetric elimination of [W | I] in one l x l array: step j subtracts f_i = W_ij / d_j times row j from every row i > j,
 // the columns right of j holding what is left of W, those up to j the unit lower factor's inverse Z as it grows (column j
 // becomes -f_i). Then L^-1 = diag(d)^(-1/2) Z and R^-1 is its transpose, so factor and inverse take one sweep of l steps
-// with one barrier each, and the only chain per step is barrier, pivot, reciprocal, one multiply-add. Every thread keeps its
-// elements in registers; shared memory carries only the pivot row and column (double buffered). Measured for l = 16, one
-// matrix: 16 -> 8.6 us, l = 48, 48 matrices: 46 -> 41 us (right-looking Cholesky and a substitution after it, both in shared
-// memory); a step still takes 800 cycles at l = 8 and 1450 at l = 48, three times its chain.
+// with one barrier each, and the only chain per step is barrier, pivot, reciprocal, one multiply-add. Every thread keeps NR
+// consecutive rows of one column in registers; shared memory carries only the pivot row and column (double buffered). The
+// steps run in blocks of NR, so that the pivot's place among a thread's rows is known to the compiler and who takes part
+// is a comparison of warp-uniform numbers: with rows eight apart the selection took more instructions than the update.
 // ---------------------------------------------------------------------------------------------
-constexpr int CHOL_ROWS = MAX_L / 8;     // rows per thread: r = first + 8 u
+// 1 / d for a positive finite d: the hardware's approximation and two Newton steps (a division costs twice the latency)
+__device__ __forceinline__ double reciprocal(double d) {
+  if (!(d > 1e-290 && d < 1e290)) return 1.0 / d;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  y = fma(y, fma(-d, y, 1.0), y);
+  y = fma(y, fma(-d, y, 1.0), y);
+  return fma(y, fma(-d, y, 1.0), y);
+}
 
+template <int NR>      // rows per thread, ceil(l / 8)
 __global__ void __launch_bounds__(512) chol_inv_kernel(const double* __restrict__ partial, int nchunk, int l, int cw_log2,
                                                        float* __restrict__ Rinv, int* __restrict__ status) {
   pdl_wait();
   __shared__ double prow[2][MAX_L], pcol[2][MAX_L], diag[MAX_L], wdiag[MAX_L];
   const int bz = blockIdx.x, tid = threadIdx.x;
-  const int c = tid & ((1 << cw_log2) - 1), r0 = tid >> cw_log2;       // column, first row (0 .. 7)
+  const int c = tid & ((1 << cw_log2) - 1), g = tid >> cw_log2;       // column, group of rows g NR .. g NR + NR - 1
   const double* pb = partial + (long long)bz * nchunk * l * l;
-  double w[CHOL_ROWS], m[CHOL_ROWS];
+  double w[NR], m[NR];
 #pragma unroll
-  for (int u = 0; u < CHOL_ROWS; ++u) w[u] = 0.0;
+  for (int u = 0; u < NR; ++u) w[u] = 0.0;
   if (c < l) {
-#pragma unroll 2
+#pragma unroll 4
     for (int ch = 0; ch < nchunk; ++ch) {
       const double* pe = pb + (long long)ch * l * l + c;
 #pragma unroll
-      for (int u = 0; u < CHOL_ROWS; ++u) w[u] += (r0 + 8 * u < l) ? pe[(r0 + 8 * u) * l] : 0.0;
+      for (int u = 0; u < NR; ++u) w[u] += (g * NR + u < l) ? pe[(g * NR + u) * l] : 0.0;
     }
 #pragma unroll
-    for (int u = 0; u < CHOL_ROWS; ++u) if (r0 + 8 * u == c) wdiag[c] = w[u];
+    for (int u = 0; u < NR; ++u) if (g * NR + u == c) wdiag[c] = w[u];
   }
   double shift = 0.0;
   bool failed = false;
   for (int attempt = 0; attempt < 6; ++attempt) {
     __syncthreads();
-    // row j and column j of the array as it stands; below the pivot the column's place is cleared for Z
-    auto publish = [&](int j) {
-      const int buf = j & 1;
-      if (r0 == (j & 7)) {
-#pragma unroll
-        for (int u = 0; u < CHOL_ROWS; ++u) if (u == (j >> 3)) prow[buf][c] = m[u];
-      }
+    // row j = a NR + u and column j of the array as it stands; below the pivot the column's place is cleared for Z
+    auto publish = [&](int a, int u, int j) {
+      if (g == a) prow[j & 1][c] = m[u];
       if (c == j) {
 #pragma unroll
-        for (int u = 0; u < CHOL_ROWS; ++u) {
-          pcol[buf][r0 + 8 * u] = m[u];
-          if (r0 + 8 * u > j) m[u] = 0.0;
+        for (int v = 0; v < NR; ++v) {
+          pcol[j & 1][g * NR + v] = m[v];
+          if (g > a || (g == a && v > u)) m[v] = 0.0;
         }
       }
     };
 #pragma unroll
-    for (int u = 0; u < CHOL_ROWS; ++u) m[u] = w[u] + ((r0 + 8 * u == c) ? shift : 0.0);
-    publish(0);
+    for (int u = 0; u < NR; ++u) m[u] = w[u] + ((g * NR + u == c) ? shift : 0.0);
+    publish(0, 0, 0);
     __syncthreads();
     failed = false;
-    for (int j = 0; j < l; ++j) {
-      const int buf = j & 1;
-      const double d = prow[buf][j], pr = prow[buf][c];       // every thread reads the pivot itself: a bad one is seen by all alike
-      double f[CHOL_ROWS];
+    for (int a = 0; a < 8 && !failed; ++a) {
 #pragma unroll
-      for (int u = 0; u < CHOL_ROWS; ++u) f[u] = (r0 + 8 * u > j) ? pcol[buf][r0 + 8 * u] : 0.0;     // (rows past l: zeros)
-      if (!(d > 0.0) || !isfinite(d)) { failed = true; break; }
-      const double inv = 1.0 / d;
-      if (tid == 0) diag[j] = d;
-      const double s = (c == j) ? inv : inv * pr;
+      for (int u = 0; u < NR; ++u) {
+        const int j = a * NR + u;
+        if (j < l && !failed) {            // (uniform in the block)
+          const int buf = j & 1;
+          const double d = prow[buf][j], pr = prow[buf][c];       // every thread reads the pivot itself: a bad one is seen by all alike
+          double f[NR];
 #pragma unroll
-      for (int u = 0; u < CHOL_ROWS; ++u) if (r0 + 8 * u > j) m[u] = fma(-f[u], s, m[u]);
-      if (j + 1 < l) publish(j + 1);       // (into the other buffer: nobody reads that one before the barrier)
-      __syncthreads();
+          for (int v = 0; v < NR; ++v) f[v] = pcol[buf][g * NR + v];      // (rows past l: zeros)
+          if (!(d > 0.0) || !isfinite(d)) failed = true;
+          else {
+            const double inv = reciprocal(d);
+            if (tid == 0) diag[j] = d;
+            const double s = (c == j) ? inv : inv * pr;
+            if (g > a) {
+#pragma unroll
+              for (int v = 0; v < NR; ++v) m[v] = fma(-f[v], s, m[v]);
+            } else if (g == a) {
+#pragma unroll
+              for (int v = u + 1; v < NR; ++v) m[v] = fma(-f[v], s, m[v]);
+            }
+            if (j + 1 < l) publish(u + 1 < NR ? a : a + 1, u + 1 < NR ? u + 1 : 0, j + 1);   // (into the other buffer)
+          }
+          __syncthreads();
+        }
+      }
     }
     if (!failed) break;
     // shift as in shifted CholeskyQR: proportional to the trace, growing per attempt
@@ -170,16 +188,20 @@ __global__ void __launch_bounds__(512) chol_inv_kernel(const double* __restrict_
   __syncthreads();
   float* out = Rinv + (long long)bz * l * l;
 #pragma unroll
-  for (int u = 0; u < CHOL_ROWS; ++u) {
-    const int r = r0 + 8 * u;
+  for (int u = 0; u < NR; ++u) {
+    const int r = g * NR + u;
     if (r < l && c < l) out[c * l + r] = failed ? 0.f : (float)(((c < r) ? m[u] : (c == r ? 1.0 : 0.0)) * wdiag[r]);
   }
 }
 
 cudaError_t chol_inv_launch(const double* partial, int nchunk, int batch, int l, float* Rinv, int* status,
                             cudaStream_t st, long long* launches) {
-  const int cw_log2 = l <= 16 ? 4 : (l <= 32 ? 5 : 6);       // eight rows of 16, 32 or 64 columns per pass
-  launch_kernel(chol_inv_kernel, batch, 8 << cw_log2, 0, st, partial, nchunk, l, cw_log2, Rinv, status);
+  const int cw_log2 = l <= 16 ? 4 : (l <= 32 ? 5 : 6);       // eight groups of rows x 16, 32 or 64 columns
+  const int nr = (l + 7) / 8;
+  auto kern = nr <= 1 ? chol_inv_kernel<1> : nr == 2 ? chol_inv_kernel<2> : nr == 3 ? chol_inv_kernel<3>
+            : nr == 4 ? chol_inv_kernel<4> : nr == 5 ? chol_inv_kernel<5> : nr == 6 ? chol_inv_kernel<6>
+            : nr == 7 ? chol_inv_kernel<7> : chol_inv_kernel<8>;
+  launch_kernel(kern, batch, 8 << cw_log2, 0, st, partial, nchunk, l, cw_log2, Rinv, status);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
