@@ -531,12 +531,13 @@ __device__ __forceinline__ void store_block_transposed16(const TcParams& p, cons
   }
   __syncwarp();
   uint8_t* mbase = reinterpret_cast<uint8_t*>(p.C) + ((size_t)bz * p.batch_c + (size_t)gj0 * p.ldc + gi_warp0) * 2;
+  uint4 q[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int c = (lane >> 2) + 8 * i;
-    const uint4 q = *reinterpret_cast<const uint4*>(stg + c * 64 + (lane & 3) * 16);
-    *reinterpret_cast<uint4*>(mbase + (size_t)c * p.ldc * 2 + (lane & 3) * 16) = q;
-  }
+  for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const uint4*>(stg + ((lane >> 2) + 8 * i) * 64 + (lane & 3) * 16);
+  uint8_t* mp = mbase + (size_t)(lane >> 2) * p.ldc * 2 + (lane & 3) * 16;
+  const size_t mstep = (size_t)8 * p.ldc * 2;
+#pragma unroll
+  for (int i = 0; i < 4; ++i, mp += mstep) *reinterpret_cast<uint4*>(mp) = q[i];
   __syncwarp();
 }
 
@@ -640,12 +641,17 @@ __device__ __forceinline__ void epilogue_block_fast(const TcParams& p, uint32_t 
   __syncwarp();
   if (!p.transposed) {
     uint8_t* cbase = reinterpret_cast<uint8_t*>(p.C) + ((size_t)bz * p.batch_c + (size_t)gi_warp0 * p.ldc + gj0) * ES;
+    // (all reads of the staged block before the first store: the compiler cannot tell that they do not alias, and one by
+    // one every store waits for its own read)
+    uint4 q[pp];
 #pragma unroll
-    for (int i = 0; i < pp; ++i) {
-      const int row = prow + rpi * i;
-      const uint4 q = *reinterpret_cast<const uint4*>(stg + stage_off(row, piece, rowb, pp));
-      if (gi_warp0 + row < p.M) *reinterpret_cast<uint4*>(cbase + (size_t)row * p.ldc * ES + piece * 16) = q;
-    }
+    for (int i = 0; i < pp; ++i) q[i] = *reinterpret_cast<const uint4*>(stg + stage_off(prow + rpi * i, piece, rowb, pp));
+    uint8_t* cp = cbase + (size_t)prow * p.ldc * ES + piece * 16;
+    const size_t cstep = (size_t)rpi * p.ldc * ES;
+    const int rows_left = p.M - gi_warp0 - prow;
+#pragma unroll
+    for (int i = 0; i < pp; ++i, cp += cstep)
+      if (rpi * i < rows_left) *reinterpret_cast<uint4*>(cp) = q[i];
   }
   // (a transposed output is written the way a symmetric one is mirrored)
   if (p.transposed || (p.symmetric && gj0 > gi_warp0)) {
@@ -653,11 +659,12 @@ __device__ __forceinline__ void epilogue_block_fast(const TcParams& p, uint32_t 
     // block is 32 values = pp pieces of 16 bytes; pp consecutive lanes write one such row, each lane gathering its
     // epp values from one column of the staged block
     uint8_t* mbase = reinterpret_cast<uint8_t*>(p.C) + ((size_t)bz * p.batch_c + (size_t)gj0 * p.ldc + gi_warp0) * ES;
+    uint4 qm[pp];
 #pragma unroll
     for (int i = 0; i < pp; ++i) {
       const int c = rpi * i + prow;                 // column of the block = row of the mirror image
       const int cp = c / epp, ce = (c % epp) * ES;  // its piece and byte offset within a staged row
-      uint4 q;
+      uint4& q = qm[i];
       if (ES == 2) {
         uint16_t h[8];
 #pragma unroll
@@ -672,8 +679,11 @@ __device__ __forceinline__ void epilogue_block_fast(const TcParams& p, uint32_t 
           w[e] = *reinterpret_cast<const uint32_t*>(stg + stage_off(piece * epp + e, cp, rowb, pp) + ce);
         q = make_uint4(w[0], w[1], w[2], w[3]);
       }
-      *reinterpret_cast<uint4*>(mbase + (size_t)c * p.ldc * ES + piece * 16) = q;
     }
+    uint8_t* mp = mbase + (size_t)prow * p.ldc * ES + piece * 16;
+    const size_t mstep = (size_t)rpi * p.ldc * ES;
+#pragma unroll
+    for (int i = 0; i < pp; ++i, mp += mstep) *reinterpret_cast<uint4*>(mp) = qm[i];
   }
   __syncwarp();
 }
