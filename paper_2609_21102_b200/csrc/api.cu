@@ -665,7 +665,10 @@ static int polar_core(defl_ctx* c, const void* G, void* out, int b, int m, int n
   if (k > 0) {
     const float* sk = resolve_sketch(c, opts, b, ms, l, w, &rc);
     if (rc) return rc;
-    if ((rc = run_brsvd(c, G, ldg, b, m, n, dtype, l, power_iters, k, sk, w, engine))) return rc;
+    // (A padded call keeps its panels in fp32 on the FMA engine, as without the padding. The tensor form of these products
+    // splits a panel into bf16 hi + lo, 2^-17 of it, and what that leaves of the head in the residual grows with
+    // ||head|| / ||R||: 4e-2 .. 2e-1 of the result at 300 and 600, against 8e-3 with fp32 panels.)
+    if ((rc = run_brsvd(c, G, ldg, b, m, n, dtype, l, power_iters, k, sk, w, padded ? (int)DEFL_ENGINE_SIMT : engine))) return rc;
   }
   ctx_stage_mark(c);
 

@@ -140,3 +140,28 @@ def test_rows_of_no_whole_packets_agree_with_the_fp32_engine(ctx, m, n, form):
     assert bool(torch.isfinite(outs[0]).all())
     for i in range(b):
         assert float((outs[0][i] - outs[1][i]).norm() / outs[1][i].norm()) <= 3e-2
+
+
+@pytest.mark.parametrize("m,n", [(65, 97), (97, 65), (131, 264), (264, 131), (203, 203)])
+@pytest.mark.parametrize("ratio", [30.0, 300.0, 600.0])
+def test_rows_of_no_whole_packets_with_a_dominant_head(ctx, m, n, ratio):
+    """A head of `ratio` times the residual's norm: what the rounding of the panels leaves of the head in the residual is
+    amplified by that ratio, so they have to stay fp32 (2^-17 of a panel is 4e-2 and more of the result at 300). Against the
+    fp64 algorithm, within the library's 3e-2 for bf16 storage."""
+    from paper_2609_21102_b200 import binding
+    b, k, p, J = 2, 6, 6, 2
+    g = torch.Generator().manual_seed(int(ratio) + m)
+    bulk = torch.randn((b, m, n), generator=g, dtype=torch.float64)
+    bulk /= bulk[0].norm()
+    u = torch.linalg.qr(torch.randn((b, m, k), generator=g, dtype=torch.float64))[0]
+    v = torch.linalg.qr(torch.randn((b, n, k), generator=g, dtype=torch.float64))[0]
+    s = torch.linspace(1.0, 0.4, k, dtype=torch.float64)
+    G = (bulk + (u * (s * (ratio / s.norm()))) @ v.transpose(1, 2)).to(torch.bfloat16).cuda()
+    Om = torch.randn((b, min(m, n), k + p), generator=g).cuda()
+    out, info = ctx.defl_polar_batched(G, k, p, J, [list(binding.MUON_QUINTIC)] * 5, sketch=Om, gamma=1.01, want_info=True)
+    torch.cuda.synchronize()
+    assert info["status"].cpu().tolist() == [0] * b
+    for i in range(b):
+        ref, *_ = oracle.deflated_polar(G[i].double().cpu().numpy(), k, k + p, Om[i].double().cpu().numpy(), J,
+                                        oracle.schedule([list(binding.MUON_QUINTIC)] * 5), gamma=1.01)
+        assert float(np.linalg.norm(out[i].double().cpu().numpy() - ref) / np.linalg.norm(ref)) <= 3e-2
