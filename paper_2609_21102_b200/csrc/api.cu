@@ -330,8 +330,8 @@ int defl_create(defl_ctx** out, int device) {
   c->knobs.jacobi_sweeps = getenv("DEFL_JACOBI_SWEEPS") ? atoi(getenv("DEFL_JACOBI_SWEEPS")) : 0;
   c->knobs.paired_steps = getenv("DEFL_NO_PAIRED_STEPS") ? 0 : 1;
   cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
-  int ok = 1;
-  if (cudaMalloc(&c->wait_status, 2 * sizeof(int)) != cudaSuccess) ok = 0;      // status word, tile counter
+  int ok = gemm_tc_prepare() == cudaSuccess && panel_prepare() == cudaSuccess && psd_prepare() == cudaSuccess ? 1 : 0;
+  if (ok && cudaMalloc(&c->wait_status, 2 * sizeof(int)) != cudaSuccess) ok = 0;      // status word, tile counter
   if (ok) cudaMemset(c->wait_status, 0, 2 * sizeof(int));
   if (ok) {
     // identity tile of the tensor engine's identity segment (X0 = (G - head) / rho adds G in the accumulator)

@@ -91,6 +91,12 @@ int gemm_simt_partials_per_batch(const GemmDesc& g);
 cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word, int num_sms, long long* launches,
                            const TcKnobs* knobs = nullptr, TmCache* cache = nullptr);
 bool gemm_tc_supported(const GemmDesc& g);
+// Shared-memory limits of the kernels that take more than the default, set when a context is created and never on the call
+// path. The limit belongs to the kernel, which all contexts of the process share, so it is the largest size that any call
+// takes: with each launch's own size set just before it, a context on another thread could lower it in between.
+cudaError_t gemm_tc_prepare();
+cudaError_t panel_prepare();
+cudaError_t psd_prepare();
 int gemm_tc_partials_per_batch(const GemmDesc& g, const TcKnobs* knobs = nullptr);
 
 // Programmatic dependent launch. Every kernel of the library is launched so that its CTAs may start while the kernel before

@@ -24,6 +24,7 @@
 // operands. Every wait is bounded: when one runs out the kernel raises DEFL_ST_DEVICE_WAIT in the status word,
 // stops waiting and drains.
 #include "common.cuh"
+#include <atomic>
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <mutex>
@@ -1257,6 +1258,11 @@ bool encode_map(CUtensorMap* tm, const void* base, int esize, bool tf32, bool mn
   return r == CUDA_SUCCESS;
 }
 
+// Shared memory of a launch: pipeline stages and the epilogue warps' staging buffers, and 1 KB to align the stages
+constexpr uint32_t STAGE_BUDGET = 224 * 1024 - EPI_WARPS * STAGING_BYTES;
+constexpr size_t SMEM_EXTRA = 1024 + EPI_WARPS * STAGING_BYTES;
+constexpr size_t SMEM_LIMIT = STAGE_BUDGET + SMEM_EXTRA;
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 const TcKnobs kDefaultKnobs = {0, 0, 0, 0, -1, 0, 0, 0, 0, 0};
@@ -1401,6 +1407,17 @@ int gemm_tc_partials_per_batch(const GemmDesc& g, const TcKnobs* knobs) {
   return ((g.M + tmh - 1) / tmh) * ((g.N + bn - 1) / bn) * (tmh == 256 ? 2 : 1) * EPI_WARPS;
 }
 
+cudaError_t gemm_tc_prepare() {
+  const void* forms[] = {(const void*)gemm_tc_kernel<0, 1, 0>, (const void*)gemm_tc_kernel<0, 2, 0>, (const void*)gemm_tc_kernel<1, 1, 0>,
+                         (const void*)gemm_tc_kernel<1, 2, 0>, (const void*)gemm_tc_kernel<0, 1, 1>, (const void*)gemm_tc_kernel<0, 2, 1>,
+                         (const void*)gemm_tc_kernel<1, 1, 1>, (const void*)gemm_tc_kernel<1, 2, 1>};
+  for (const void* f : forms) {
+    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word, int num_sms, long long* launches,
                            const TcKnobs* knobs, TmCache* cache) {
   if (!gemm_tc_supported(g)) return cudaErrorNotSupported;
@@ -1447,7 +1464,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word,
   }
   // a pair's K block is half the work per CTA of the single-CTA form, too short to hide the per-step cost of the
   // two issuing threads (barrier wait, commit): its pipeline steps cover two K blocks when three such stages fit
-  const uint32_t smem_budget = 224 * 1024 - EPI_WARPS * STAGING_BYTES;
+  const uint32_t smem_budget = STAGE_BUDGET;
   const uint32_t sub_bytes = p.a_stage_bytes + p.b_stage_bytes;
   p.ksub = (p.pair && 3u * 2u * sub_bytes <= smem_budget) ? 2 : 1;
   if ((kn.ksub == 1 || kn.ksub == 2) && (uint32_t)kn.ksub * sub_bytes * 2u <= smem_budget) p.ksub = kn.ksub;
@@ -1527,13 +1544,11 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word,
   // are short (one more hand-off per tile), and the whole step comes out the same.
   p.tile_counter = (p.pair && status_word && kn.dynamic) ? reinterpret_cast<unsigned int*>(status_word + 1) : nullptr;
 
-  const size_t smem = (size_t)stages * stage_bytes + 1024 + EPI_WARPS * STAGING_BYTES;
+  const size_t smem = (size_t)stages * stage_bytes + SMEM_EXTRA;
   cudaError_t e;
   if (p.pair) {
     auto kern = tf32 ? (p.b_split == 2 ? gemm_tc_kernel<1, 2, 1> : gemm_tc_kernel<1, 1, 1>)
                      : (p.b_split == 2 ? gemm_tc_kernel<0, 2, 1> : gemm_tc_kernel<0, 1, 1>);
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cudaLaunchAttribute attr[2];
@@ -1542,16 +1557,16 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word,
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.blockDim = dim3(NUM_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = SMEM_LIMIT;      // (for the question below, which is asked once for all products)
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     // how many CTA pairs the device can hold at once (a GPC with an odd number of free SMs leaves one out)
-    static int max_pairs[4][64];   // per kernel variant and device; 0 = not asked yet
+    static std::atomic<int> max_pairs[4][64];   // per kernel variant and device; 0 = not asked yet
     int dev = 0;
     cudaGetDevice(&dev);
     const int variant = (tf32 ? 2 : 0) + (p.b_split == 2 ? 1 : 0);
-    int pairs = (dev >= 0 && dev < 64) ? max_pairs[variant][dev] : 0;
+    int pairs = (dev >= 0 && dev < 64) ? max_pairs[variant][dev].load() : 0;
     if (pairs <= 0) {
       cfg.gridDim = dim3((unsigned)(num_sms & ~1), 1, 1);
       int n = 0;
@@ -1565,6 +1580,7 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word,
     long long npairs = p.total_tiles < pairs ? p.total_tiles : pairs;
     if (npairs < 1) npairs = 1;
     cfg.gridDim = dim3((unsigned)(2 * npairs), 1, 1);
+    cfg.dynamicSmemBytes = smem;
     cfg.numAttrs = 2;
     e = cudaLaunchKernelEx(&cfg, kern, p);
     if (launches) ++*launches;
@@ -1572,8 +1588,6 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word,
   }
   auto kern = tf32 ? (p.b_split == 2 ? gemm_tc_kernel<1, 2, 0> : gemm_tc_kernel<1, 1, 0>)
                    : (p.b_split == 2 ? gemm_tc_kernel<0, 2, 0> : gemm_tc_kernel<0, 1, 0>);
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   long long grid = p.total_tiles < num_sms ? p.total_tiles : num_sms;
   if (grid < 1) grid = 1;
   launch_kernel(kern, dim3((unsigned)grid), dim3(NUM_THREADS), smem, st, p);

@@ -999,6 +999,7 @@ namespace defl {
 
 constexpr int FUSED_TILE = 128;
 constexpr int FUSED_TS = MAX_L + 4;
+constexpr size_t FUSED_SMEM = (size_t)(FUSED_TILE + MAX_L) * FUSED_TS * sizeof(float);
 
 // Rows are split over CTAs in whole 128-row tiles. The split is chosen so that all CTAs of the launch are resident
 // at once (two per SM with this kernel's registers): a fixed 512-row split gave 624 CTAs for 592 places on
@@ -1231,13 +1232,15 @@ __global__ void __launch_bounds__(256, 2) panel_fused_kernel(const float* In, lo
   }
 }
 
+cudaError_t panel_prepare() {
+  return cudaFuncSetAttribute(panel_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM);
+}
+
 cudaError_t panel_fused_launch(const float* In, long long in_bs, int ld_in, int batch, int rows, int l, const float* Mtx,
                                int ldm, int kout, float* Out, long long out_bs, int ld_out, __nv_bfloat16* hi,
                                __nv_bfloat16* lo, int lp, double* partial, cudaStream_t st, long long* launches) {
-  const size_t smem = (size_t)(FUSED_TILE + MAX_L) * FUSED_TS * sizeof(float);
-  cudaFuncSetAttribute(panel_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int nchunk = fused_num_chunks(rows, batch);
-  launch_kernel(panel_fused_kernel, dim3(nchunk, batch), 256, smem, st, In, in_bs, ld_in, rows, l, Mtx, ldm, kout, Out, out_bs, ld_out,
+  launch_kernel(panel_fused_kernel, dim3(nchunk, batch), 256, FUSED_SMEM, st, In, in_bs, ld_in, rows, l, Mtx, ldm, kout, Out, out_bs, ld_out,
                                                             hi, lo, lp, partial, nchunk);
   if (launches) ++*launches;
   return cudaGetLastError();

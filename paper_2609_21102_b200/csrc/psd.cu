@@ -731,6 +731,15 @@ __global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const LanczosRun
   }
 }
 
+constexpr size_t LZ_SMEM = 210 * 1024;        // dynamic shared memory at most (static shared memory comes on top)
+
+cudaError_t psd_prepare() {
+  cudaError_t e = cudaFuncSetAttribute(lanczos_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LZ_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(lanczos_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(lanczos_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LZ_SMEM);
+  return e;
+}
+
 // Launches it, or returns false (nothing launched) where a CTA cannot hold its vectors or the device cannot hold the grid.
 static bool lanczos_launch(defl_ctx* c, const float* A, const float* start, int n, int steps, float* t, float* w, double* part,
                            unsigned int* bar, float* theta, float* inv_theta, int* status, cudaError_t* err) {
@@ -742,14 +751,13 @@ static bool lanczos_launch(defl_ctx* c, const float* A, const float* start, int 
   p.wait_status = c->wait_status;
   p.wait_ns = (unsigned long long)(c->tc_knobs.wait_ms > 0 ? c->tc_knobs.wait_ms : 2000) * 1000000ull;
   p.theta = theta; p.inv_theta = inv_theta; p.status = status;
-  const size_t budget = 210 * 1024;           // (static shared memory comes on top)
   // rows per CTA, resident rows and shared memory of a form; 0 = does not fit
   auto layout = [&](int grid, int vectors) -> size_t {
     p.rows = (n + grid - 1) / grid;
     const size_t fixed = sizeof(float) * ((size_t)vectors * ((n + 3) & ~3) + (size_t)((p.rows + 3) & ~3) +
                                           (size_t)((DEFL_LANCZOS_STEPS * p.rows + 3) & ~3));
-    if (fixed > budget) return 0;
-    const size_t fit = (budget - fixed) / ((size_t)n * sizeof(float));
+    if (fixed > LZ_SMEM) return 0;
+    const size_t fit = (LZ_SMEM - fixed) / ((size_t)n * sizeof(float));
     p.resident = fit < (size_t)p.rows ? (int)fit : p.rows;
     return fixed + (size_t)p.resident * n * sizeof(float);
   };
@@ -765,9 +773,7 @@ static bool lanczos_launch(defl_ctx* c, const float* A, const float* start, int 
     cfg.gridDim = dim3(LZ_CLUSTER, 1, 1); cfg.blockDim = dim3(LZ_THREADS, 1, 1); cfg.dynamicSmemBytes = smem; cfg.stream = c->stream;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int clusters = 0;
-    if (smem > 0 && cudaFuncSetAttribute(lanczos_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
-        cudaFuncSetAttribute(lanczos_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        cudaOccupancyMaxActiveClusters(&clusters, lanczos_kernel<true>, &cfg) == cudaSuccess && clusters > 0) {
+    if (smem > 0 && cudaOccupancyMaxActiveClusters(&clusters, lanczos_kernel<true>, &cfg) == cudaSuccess && clusters > 0) {
       cfg.numAttrs = 2;
       *err = cudaLaunchKernelEx(&cfg, lanczos_kernel<true>, p);
       ++c->launches;
@@ -782,7 +788,6 @@ static bool lanczos_launch(defl_ctx* c, const float* A, const float* start, int 
   const size_t smem = layout(grid, 1);
   if (smem == 0) return false;
   grid = (n + p.rows - 1) / p.rows;
-  if (cudaFuncSetAttribute(lanczos_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) { cudaGetLastError(); return false; }
   if ((*err = cudaMemsetAsync(bar, 0, sizeof(unsigned int), c->stream)) != cudaSuccess) return true;
   void* args[] = {&p};
   const cudaError_t e = cudaLaunchCooperativeKernel((const void*)lanczos_kernel<false>, dim3(grid), dim3(LZ_THREADS), args, smem, c->stream);
