@@ -19,6 +19,7 @@ reports the whole-job aggregate; without an outer torchrun the script starts its
 `--impl reference` times the fp64 CPU oracle on a bounded sample of the same workload.
 """
 import argparse
+import functools
 import json
 import os
 import socket
@@ -256,6 +257,26 @@ def time_steps(fn, steps, sync):
     e1.record()
     sync()
     return e0.elapsed_time(e1) / steps
+
+
+def run_in_threads(calls):
+    """Runs every call on a host thread of its own and waits for all of them; the first exception (in the order of the calls)
+    is raised here. A plain thread prints and drops it, and the step would be timed without that call's work."""
+    failed = [None] * len(calls)
+
+    def run(i):
+        try:
+            calls[i]()
+        except BaseException as e:
+            failed[i] = e
+    threads = [threading.Thread(target=run, args=(i,)) for i in range(len(calls))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for e in failed:
+        if e is not None:
+            raise e
 
 
 def workload_flops(wl, sym, add=False, iterates=0, per_step=False):
@@ -675,11 +696,7 @@ def main():
         def e2e_step():
             # the call blocks until its output sits in host memory; the shape groups run from host threads of their
             # own (one context each), so that one group's copies overlap the other's computation
-            ts = [threading.Thread(target=e2e_group, args=(c, s, h, o, g)) for c, s, h, o, g in zip(e2e_ctx, e2e_streams, hG, hO, groups)]
-            for t in ts:
-                t.start()
-            for t in ts:
-                t.join()
+            run_in_threads([functools.partial(e2e_group, *x) for x in zip(e2e_ctx, e2e_streams, hG, hO, groups)])
         e2e_step()
         barrier()
         t0 = time.perf_counter()

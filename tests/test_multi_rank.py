@@ -89,3 +89,18 @@ def test_gpus_flag_starts_its_own_ranks_when_no_launcher_did(monkeypatch):
     assert cmd[1:4] == ["-m", "torch.distributed.run", "--nnodes=1"]
     assert cmd[cmd.index("--nproc-per-node") + 1] == "4" and cmd[cmd.index("--master-addr") + 1] == "127.0.0.1"
     assert cmd[-4:] == ["--gpus", "4", "--steps", "2"] and cmd[-5].endswith("bench.py")
+
+
+def test_an_exception_on_a_work_thread_ends_the_step():
+    """The end-to-end leg runs the shape groups on host threads: all of them finish, and a failed one fails the step."""
+    import threading
+    import bench
+    done, here = [], threading.get_ident()
+
+    def bad():
+        raise RuntimeError("group 1")
+    bench.run_in_threads([lambda: done.append(threading.get_ident()), lambda: done.append(threading.get_ident())])
+    assert len(done) == 2 and here not in done
+    with pytest.raises(RuntimeError, match="group 1"):
+        bench.run_in_threads([lambda: done.append(0), bad, lambda: done.append(0)])
+    assert len(done) == 4
