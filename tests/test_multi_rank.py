@@ -4,6 +4,8 @@ import json
 import os
 import subprocess
 import sys
+
+import pytest
 import textwrap
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
