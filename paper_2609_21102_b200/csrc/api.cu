@@ -329,6 +329,8 @@ int defl_create(defl_ctx** out, int device) {
   c->knobs.host_chunks = getenv("DEFL_HOST_CHUNKS") ? atoi(getenv("DEFL_HOST_CHUNKS")) : 0;
   c->knobs.jacobi_sweeps = getenv("DEFL_JACOBI_SWEEPS") ? atoi(getenv("DEFL_JACOBI_SWEEPS")) : 0;
   c->knobs.paired_steps = getenv("DEFL_NO_PAIRED_STEPS") ? 0 : 1;
+  c->knobs.lanczos_form = getenv("DEFL_LANCZOS_FORM") ? atoi(getenv("DEFL_LANCZOS_FORM")) : 0;
+  c->knobs.lanczos_hold = getenv("DEFL_LANCZOS_HOLD") ? 1 : 0;
   cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
   int ok = gemm_tc_prepare() == cudaSuccess && panel_prepare() == cudaSuccess && psd_prepare() == cudaSuccess ? 1 : 0;
   if (ok && cudaMalloc(&c->wait_status, 2 * sizeof(int)) != cudaSuccess) ok = 0;      // status word, tile counter

@@ -430,6 +430,7 @@ struct LanczosRun {
   unsigned int* bar;                 // barrier counter, zero at launch (grid form)
   int* wait_status;                  // bit 8 when a barrier runs out of time
   unsigned long long wait_ns;
+  unsigned int hold;                 // test hook (grid form): arrivals that a meeting waits for and that never come
   float* theta; float* inv_theta; int* status;
 };
 
@@ -541,6 +542,8 @@ __global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const LanczosRun
   }
   if (tid < MS) { al[tid] = 0.0; be[tid] = 0.0; }
   if (tid == 0) alive = 1;
+  // (a wait that runs out returns from the middle: the scale is then zero, not what an earlier call left there)
+  if (blk == 0 && tid == 0) { p.theta[0] = 0.f; p.inv_theta[0] = 0.f; }
   __syncthreads();
 
   // All CTAs meet. Grid form: a counter with a time limit, false (everywhere in the CTA) when it ran out.
@@ -551,7 +554,7 @@ __global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const LanczosRun
     if (tid == 0) {
       __threadfence();
       atomicAdd(p.bar, 1u);
-      const unsigned int want = epoch * (unsigned int)G;
+      const unsigned int want = epoch * (unsigned int)G + p.hold;
       unsigned long long t0 = 0;
       for (unsigned int polls = 0;; ++polls) {
         unsigned int v;
@@ -750,6 +753,7 @@ static bool lanczos_launch(defl_ctx* c, const float* A, const float* start, int 
   p.aligned = (reinterpret_cast<uintptr_t>(A) & 15) == 0;
   p.wait_status = c->wait_status;
   p.wait_ns = (unsigned long long)(c->tc_knobs.wait_ms > 0 ? c->tc_knobs.wait_ms : 2000) * 1000000ull;
+  p.hold = (unsigned int)c->knobs.lanczos_hold;
   p.theta = theta; p.inv_theta = inv_theta; p.status = status;
   // rows per CTA, resident rows and shared memory of a form; 0 = does not fit
   auto layout = [&](int grid, int vectors) -> size_t {
@@ -761,7 +765,7 @@ static bool lanczos_launch(defl_ctx* c, const float* A, const float* start, int 
     p.resident = fit < (size_t)p.rows ? (int)fit : p.rows;
     return fixed + (size_t)p.resident * n * sizeof(float);
   };
-  if (n <= LZ_CLUSTER_N) {
+  if (n <= LZ_CLUSTER_N && c->knobs.lanczos_form == 0) {
     const size_t smem = layout(LZ_CLUSTER, 2);
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));

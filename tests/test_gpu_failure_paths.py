@@ -118,3 +118,36 @@ def test_half_iterate_overflow_is_reported(ctx):
     assert all(s & binding.ST_NONFINITE for s in info["status"].cpu().tolist())
     fine, info2 = ctx.defl_polar_batched(G, 0, 0, 0, [MUON] * 5, want_info=True, bf16_iterates=2)
     assert info2["status"].cpu().tolist() == [0, 0] and bool(torch.isfinite(fine.float()).all())
+
+
+@pytest.mark.parametrize("root", [0, 2])
+def test_scale_estimate_whose_wait_runs_out_is_reported_and_takes_nothing_from_an_earlier_call(monkeypatch, root):
+    """The grid form of the scale estimate with a meeting that waits for one arrival too many and a limit of 2 ms: the call
+    returns, says so, and its scale is zero whatever estimate the context made before. The context stays usable."""
+    from paper_2609_21102_b200 import binding
+    for k, v in (("DEFL_LANCZOS_FORM", "1"), ("DEFL_LANCZOS_HOLD", "1"), ("DEFL_TC_WAIT_MS", "2")):
+        monkeypatch.setenv(k, v)
+    c = binding.Context(0)
+    n, K = 136, 6
+    x = inputs.randn((n, n), 8601)
+    X = (x @ x.T / n + torch.eye(n, dtype=x.dtype)).float().cuda()
+    V = torch.linalg.qr(inputs.randn((n, K), 8602).float())[0].contiguous().cuda()
+
+    def call(A, norm_mode):
+        if root:
+            return c.defl_inv_root(A, root, 3, V.clone(), 6, gamma=1.1, seed=3, norm_mode=norm_mode, want_info=True)
+        return c.defl_psd_project(A, 3, V.clone(), [[1.875, -1.25, 0.375]] * 4, gamma=1.1, seed=3, norm_mode=norm_mode, want_info=True)
+
+    held = []
+    for scale in (1.0, 7.0):                       # an estimate of another size before each
+        _, fine = call(scale * X, binding.NORM_FROBENIUS)
+        assert int(fine["status"]) == 0 and float(fine["theta"]) > 0
+        out, info = call(X, binding.NORM_LANCZOS)
+        torch.cuda.synchronize()
+        assert int(info["status"]) & binding.ST_DEVICE_WAIT
+        assert float(info["theta"]) == 0.0
+        held.append(out.clone())
+    assert torch.equal(held[0], held[1])
+    _, fine = call(X, binding.NORM_FROBENIUS)
+    assert int(fine["status"]) == 0
+    c.close()
