@@ -85,7 +85,9 @@ typedef struct defl_opts {
   int warmup;            /* PSD: non-zero = gate off, return the undeflated projection of Eq. 7 but still
                             advance the basis (the paper keeps the gate off while the basis stabilises) */
   int engine;            /* DEFL_ENGINE_* */
-  int exploit_symmetry;  /* non-zero: compute only the upper tiles of X X^T and of A^2 and mirror them */
+  int exploit_symmetry;  /* non-zero: compute only the upper tiles of every product that is symmetric up to rounding and
+                            mirror them. (A product of a stored matrix with its own transpose, X X^T or A^2, whose
+                            mirror image is the result itself, is computed so in either case.) */
   float tau;             /* deflation gate of Algorithms 1 and 2. <= 0 (default): deflate exactly k components.
                             > 0: with s the k estimated magnitudes, deflate only if s_k < tau * s_1, and then the
                             components with s_i > tau * s_1 (PSD: among all K Ritz values); otherwise the call
@@ -309,7 +311,8 @@ int defl_frobenius_norms_noalloc(const void* X, int dtype, int b, long long coun
  * symmetric (upper tiles computed and mirrored); bit 1 = the product is written transposed, C row-major [N,M]
  * (tensor engine only; DEFL_ERR_UNSUPPORTED otherwise); bit 2 = test of the bounded waits (tensor engine, outputs
  * of at most 128 rows): the first pipeline step of every CTA's first tile is never copied, so the wait for it runs
- * out after the context's wait limit, C is not written and defl_device_wait_status reports DEFL_ST_DEVICE_WAIT. */
+ * out after the context's wait limit, C is not written and defl_device_wait_status reports DEFL_ST_DEVICE_WAIT; bit 3 = the
+ * polynomial epilogue, C = I + A + alpha A opB(B) (M = N = K, sa_k = 1, else DEFL_ERR_ARG). */
 int defl_debug_gemm(defl_ctx* ctx, int engine, int batch, int M, int N, int K,
                     const void* A, long long sa_i, long long sa_k, long long batch_a,
                     const void* B, long long sb_k, long long sb_j, long long batch_b,

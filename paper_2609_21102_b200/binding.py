@@ -400,9 +400,10 @@ class Context:
         return dst
 
     def defl_debug_gemm(self, A, B, trans_a=False, trans_b=False, engine=ENGINE_AUTO, out_dtype=None, alpha=1.0,
-                        exploit_symmetry=False, transpose_out=False, withhold_first_step=False):
+                        exploit_symmetry=False, transpose_out=False, withhold_first_step=False, polynomial=False):
         """C[b] = alpha * op(A[b]) op(B[b]); op = transpose of the stored matrix when the flag is set. With
-        transpose_out the engine writes the product transposed: the result has shape [b, N, M]."""
+        transpose_out the engine writes the product transposed: the result has shape [b, N, M]. With polynomial (square
+        operands, A not transposed) C[b] = I + A[b] + alpha * A[b] op(B[b]), the epilogue of the filter's polynomials."""
         _dev(A, "A"), _dev(B, "B")
         b = A.shape[0]
         if trans_a:
@@ -423,7 +424,8 @@ class Context:
         rc = lib().defl_debug_gemm(self._h, engine, b, M, N, K, _ptr(A), sa_i, sa_k, A.shape[1] * A.shape[2],
                                    _ptr(B), sb_k, sb_j, B.shape[1] * B.shape[2], _ptr(C), _dtype_code(A),
                                    {torch.bfloat16: BF16, torch.float16: F16}.get(out_dtype, F32), alpha,
-                                   int(bool(exploit_symmetry)) | (2 if transpose_out else 0) | (4 if withhold_first_step else 0))
+                                   int(bool(exploit_symmetry)) | (2 if transpose_out else 0) | (4 if withhold_first_step else 0) |
+                                   (8 if polynomial else 0))
         self._check(rc)
         return C
 

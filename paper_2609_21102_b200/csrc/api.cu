@@ -59,14 +59,17 @@ bool use_tensor_engine(const GemmDesc& g, int engine) {
   return gemm_tc_supported(g);
 }
 
-// A product of a matrix with its own transpose (X X^T, A A for the symmetric A, the polynomial a I + b A + c A A with A
-// itself as `aux`) computes (i, j) and (j, i) from the same terms in the same order on either engine: the upper tiles and
-// their mirror image are the same result, bit for bit, for half the work, whatever exploit_symmetry says.
+// A product of a matrix with its own transpose (X X^T, A A for the symmetric A, the polynomial a I + b A + c A A with the
+// exactly symmetric A itself as `aux`) computes (i, j) and (j, i) from the same terms in the same order on either engine:
+// the upper tiles and their mirror image are the full product for half the work, whatever exploit_symmetry says. On the
+// tensor engine to the bit; the FMA engine counts the tiles when it picks a tile form, and another form adds its K groups
+// in another order. (A_{t+1} = B_t^2 A_t of a paired step is a product of two matrices: without exploit_symmetry it is
+// symmetric up to rounding only, and its polynomial is computed in full.)
 static bool self_product(const GemmDesc& g) {
   if (g.nseg != 1 || g.M != g.N || g.b_split == 2 || g.transpose_out || g.in_dtype != g.b_dtype) return false;
   if (g.A[0] != g.B[0] || g.sa_i[0] != g.sb_j[0] || g.sa_k[0] != g.sb_k[0] || (g.batch > 1 && g.batch_a[0] != g.batch_b[0])) return false;
   if (g.epilogue == EPI_STORE) return true;
-  return g.epilogue == EPI_POLY && g.aux == g.A[0] && g.aux_dtype == g.in_dtype && g.ld_aux == g.sa_i[0] && g.sa_k[0] == 1 &&
+  return g.epilogue == EPI_POLY && g.aux_symmetric && g.aux == g.A[0] && g.aux_dtype == g.in_dtype && g.ld_aux == g.sa_i[0] && g.sa_k[0] == 1 &&
          (g.batch <= 1 || g.batch_aux == g.batch_a[0]);
 }
 
@@ -516,6 +519,11 @@ int defl_debug_gemm(defl_ctx* c, int engine, int batch, int M, int N, int K, con
   g.epilogue = EPI_STORE; g.alpha = alpha; g.symmetric = (exploit_symmetry & 1) ? 1 : 0;
   if (exploit_symmetry & 2) { g.transpose_out = 1; g.ldc = M; }
   if (exploit_symmetry & 4) g.debug_hold_stage = 1;
+  if (exploit_symmetry & 8) {
+    if (M != N || K != N || sa_k != 1) return DEFL_ERR_ARG;
+    g.epilogue = EPI_POLY; g.pa = 1.f; g.pb = 1.f; g.pc = alpha;
+    g.aux = A; g.ld_aux = sa_i; g.batch_aux = batch_a; g.aux_dtype = in_dtype;
+  }
   return run_gemm(c, g, engine, "debug gemm");
 }
 
@@ -874,6 +882,7 @@ static int polar_core(defl_ctx* c, const void* G, void* out, int b, int m, int n
       g.B[0] = (q == 0) ? w.Am : prev; g.sb_k[0] = 1; g.sb_j[0] = lds; g.batch_b[0] = (long long)ms * lds;   // symmetric: rows as columns
       g.C = dst; g.ldc = lds; g.batch_c = (long long)ms * lds;
       g.aux = w.Am; g.ld_aux = lds; g.batch_aux = (long long)ms * lds; g.aux_dtype = it_dtype;
+      g.aux_symmetric = 1;
       g.epilogue = EPI_POLY; g.symmetric = sym;
       if (q == 0) { g.pa = cf[terms - 3]; g.pb = cf[terms - 2] * iy2; g.pc = cf[terms - 1] * iy2 * iy2; }
       else { g.pa = cf[terms - 3 - q]; g.pb = 0.f; g.pc = iy2; }

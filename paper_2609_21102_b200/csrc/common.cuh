@@ -35,6 +35,7 @@ struct GemmDesc {
   int b_dtype;                  // type of B (both segments); the tensor engine needs b_dtype == in_dtype
   void* C; long long ldc, batch_c; int out_dtype;
   const void* aux; long long ld_aux, batch_aux; int aux_dtype;
+  int aux_symmetric;            // the caller knows `aux` to be symmetric to the bit (a stored product of a matrix with its own transpose)
   int epilogue;
   float alpha, aux_scale, pa, pb, pc;
   const float* alpha_dev;       // optional per-batch multiplier of alpha (device, [batch])

@@ -1345,7 +1345,7 @@ static int psd_core(defl_ctx* c, const void* Xv, void* Pv, int n, int k, float* 
     g.C = w.W; g.ldc = n; g.epilogue = EPI_STORE; g.symmetric = sym; g.round_tf32 = tf32_round;
     if ((rc = run_gemm(c, g, gemm_tc_supported(g) ? engine : DEFL_ENGINE_SIMT, "X^2"))) return rc;
     g.A[0] = w.W; g.B[0] = w.W; g.C = w.Tt;
-    g.aux = w.W; g.ld_aux = n; g.aux_dtype = F32;
+    g.aux = w.W; g.ld_aux = n; g.aux_dtype = F32; g.aux_symmetric = 1;
     g.epilogue = EPI_POLY; g.pa = ca; g.pb = cb; g.pc = cc;
     if ((rc = run_gemm(c, g, gemm_tc_supported(g) ? engine : DEFL_ENGINE_SIMT, "polynomial"))) return rc;
     g.A[0] = X; g.B[0] = w.Tt; g.C = Xn; g.aux = nullptr;

@@ -213,3 +213,37 @@ def test_bounded_wait_runs_out_and_is_reported(monkeypatch):
     assert torch.allclose(C, _ref(A, B, False, True), rtol=1e-4, atol=2e-3)
     assert ctx.defl_device_wait_status() == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("engine_name", ["simt", "tensor"])
+@pytest.mark.parametrize("n,K", [(24, 24), (72, 200), (256, 64), (264, 264), (328, 1000), (640, 640)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float16])
+def test_product_with_itself_is_the_full_product(ctx, engine_name, n, K, dtype):
+    """A A^T given one buffer twice is computed by upper tiles and mirrored; given a copy as the second operand, in full. The
+    tensor engine must give the same bits. The FMA engine may take another tile form, i.e. another order of the K terms:
+    each of the two sums is within K rounding errors of 2^-24 on the sum of the magnitudes."""
+    from paper_2609_21102_b200 import binding
+    engine = binding.ENGINE_SIMT if engine_name == "simt" else binding.ENGINE_TENSOR
+    A = _mk(2, n, K, dtype, 51)
+    one = ctx.defl_debug_gemm(A, A, False, True, engine=engine, out_dtype=torch.float32)
+    full = ctx.defl_debug_gemm(A, A.clone(), False, True, engine=engine, out_dtype=torch.float32)
+    assert torch.equal(one, one.transpose(1, 2)) and torch.equal(full, full.transpose(1, 2))
+    if engine_name == "tensor":
+        assert torch.equal(one, full)
+    else:
+        bound = 2.0 * (K + 1) * 2.0 ** -24 * (A.double().abs() @ A.double().abs().transpose(1, 2))
+        assert bool(((one.double() - full.double()).abs() <= bound).all())
+
+
+@pytest.mark.parametrize("engine_name", ["simt", "tensor"])
+@pytest.mark.parametrize("n", [40, 264, 520])
+def test_polynomial_of_an_unsymmetric_matrix_is_computed_in_full(ctx, engine_name, n):
+    """I + A + alpha A A^T for an A that is not symmetric, without exploit_symmetry: the product with itself alone does not
+    make the result symmetric. (The second polynomial of a paired step meets this: its A is symmetric up to rounding.)"""
+    from paper_2609_21102_b200 import binding
+    engine = binding.ENGINE_SIMT if engine_name == "simt" else binding.ENGINE_TENSOR
+    A = _mk(2, n, n, torch.float16, 52)
+    C = ctx.defl_debug_gemm(A, A, False, True, engine=engine, out_dtype=torch.float32, alpha=0.125, polynomial=True)
+    ref = torch.eye(n, device="cuda", dtype=torch.float64) + A.double() + 0.125 * (A.double() @ A.double().transpose(1, 2))
+    bound = (n + 3) * 2.0 ** -23 * (1.0 + A.double().abs() + 0.125 * (A.double().abs() @ A.double().abs().transpose(1, 2)))
+    assert bool(((C.double() - ref).abs() <= bound).all())
