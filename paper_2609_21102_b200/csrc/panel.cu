@@ -256,9 +256,11 @@ cudaError_t panel_apply_launch(const float* In, long long in_bs, int ld_in, cons
 //   E[b, l, l]  = eigenvectors in columns      (fp32)
 //   Es[b, l, l] = E diag(1/s)                  (fp32; zero column where s is numerically zero)
 // With `signed_input` the matrix is a general symmetric one (Rayleigh quotient of Algorithm 2), sorted by decreasing
-// magnitude, s = lambda. It is shifted by 2 ||C||_F first and the shift taken off the eigenvalues again: the columns of
-// C V itself are orthogonal as soon as V spans {v(+mu), v(-mu)}, so a pair of eigenvalues of equal magnitude and opposite
-// sign stays mixed in them by an angle up to 1e-11 over the relative gap of the magnitudes; the shifted pair is far apart.
+// magnitude, s = lambda. It is shifted by 2 ||C||_F first: the columns of C V itself are orthogonal as soon as V spans
+// {v(+mu), v(-mu)}, so a pair of eigenvalues of equal magnitude and opposite sign stays mixed in them by an angle up to
+// 1e-11 over the relative gap of the magnitudes; the shifted pair is far apart. The eigenvalues are the Rayleigh quotients
+// v^T C v with the unshifted matrix (a copy in shared memory): as shifted norms less the shift, 1e-16 ||C||_F is all that
+// would be left of a small one beside a large one. One product of C with V for it: 1 us of 50 at l = 16.
 // What bounds it is the chain of dependent operations of a round (l - 1 rounds a sweep, one barrier each, half a dozen
 // sweeps), not its arithmetic: the block has only the warps that own pairs, and the rotation angle, which merely steers
 // the iteration, comes from approximate fp32 functions.
@@ -295,6 +297,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
   // round needs a test; the stride is odd (the four pairs of a warp start in different banks)
   constexpr int ls = 8 * NR + 1;
   double* A = sm;
+  double* C = sm + (l + 1) * ls;      // signed input: the matrix before the shift, stored like A
   __shared__ double lam[MAX_L];       // column norms (eigenvalues of the scaled, shifted matrix), then the eigenvalues
   __shared__ double len[MAX_L];
   __shared__ double nrm2[MAX_L + 1];  // squared column norms of A, carried along by the rotations
@@ -350,8 +353,12 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
   __syncthreads();
   for (int e = tid; e < l * l; e += nt) {
     const int c = e / l, r = e % l;
-    A[c * ls + r] = A[c * ls + r] * scale + ((r == c) ? shift : 0.0);
+    const double v = A[c * ls + r] * scale;
+    A[c * ls + r] = v + ((r == c) ? shift : 0.0);
+    if (signed_input) C[c * ls + r] = v;
   }
+  if (signed_input)
+    for (int e = tid; e < l * (ls - l); e += nt) C[(e / (ls - l)) * ls + l + e % (ls - l)] = 0.0;
   __syncthreads();
   int sweep = 0;
   for (; sweep < max_sweeps; ++sweep) {
@@ -424,9 +431,31 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
     const double* aj = A + j * ls;
     const double a0 = (lane < l) ? aj[lane] : 0.0, a1 = (lane + 32 < l) ? aj[lane + 32] : 0.0;
     const double nrm = sqrt(warp_sum(a0 * a0 + a1 * a1));
-    if (lane == 0) { len[j] = nrm; lam[j] = (nrm - shift) * unscale; }
+    if (lane == 0) { len[j] = nrm; lam[j] = nrm * unscale; }
   }
   __syncthreads();
+  if (signed_input) {
+    // lambda_j = a_j^T C a_j / ||a_j||^2, eight lanes per column
+    for (int j0 = 0; j0 < l; j0 += nt >> 3) {      // (the same trip count for every lane: shuffles inside)
+      const int j = min(j0 + grp, l);
+      const double* aj = A + j * ls;
+      double t[NR];
+#pragma unroll
+      for (int i = 0; i < NR; ++i) t[i] = 0.0;
+      for (int c = 0; c < l; ++c) {
+        const double a = aj[c];
+#pragma unroll
+        for (int i = 0; i < NR; ++i) t[i] = fma(C[c * ls + sub + 8 * i], a, t[i]);
+      }
+      double acc = 0.0;
+#pragma unroll
+      for (int i = 0; i < NR; ++i) acc = fma(t[i], aj[sub + 8 * i], acc);
+      acc = group8_sum(acc);
+      // (a zero matrix has zero columns and no shift)
+      if (sub == 0 && j < l) lam[j] = (len[j] <= 1e-150) ? 0.0 : acc / (len[j] * len[j]) * unscale;
+    }
+    __syncthreads();
+  }
   if (tid < l) {
     // (a NaN compares false with everything: it ranks as magnitude -1, after every number, so that `order` is a
     // permutation whatever the input holds)
@@ -459,7 +488,7 @@ cudaError_t jacobi_eig_launch(const double* partial, int nchunk, int batch, int 
                               float* E, float* Es, int* status, cudaStream_t st, long long* launches, int max_sweeps) {
   const int threads = (((l + 1) / 2) * 8 + 31) & ~31;        // eight lanes per pair, whole warps
   const int nr = (l + 7) / 8;
-  const size_t smem = (size_t)(l + 1) * (8 * nr + 1) * sizeof(double);
+  const size_t smem = (size_t)(l + 1 + (signed_input ? l : 0)) * (8 * nr + 1) * sizeof(double);
   auto kern = nr <= 1 ? jacobi_eig_kernel<1> : nr == 2 ? jacobi_eig_kernel<2> : nr == 3 ? jacobi_eig_kernel<3>
             : nr == 4 ? jacobi_eig_kernel<4> : nr == 5 ? jacobi_eig_kernel<5> : nr == 6 ? jacobi_eig_kernel<6>
             : nr == 7 ? jacobi_eig_kernel<7> : jacobi_eig_kernel<8>;
@@ -1233,7 +1262,12 @@ __global__ void __launch_bounds__(256, 2) panel_fused_kernel(const float* In, lo
 }
 
 cudaError_t panel_prepare() {
-  return cudaFuncSetAttribute(panel_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM);
+  // (the Jacobi core with a signed input of more than 48 columns; up to there it stays within the default limit)
+  constexpr int jac = (int)((2 * MAX_L + 1) * (MAX_L + 1) * sizeof(double));
+  cudaError_t e = cudaFuncSetAttribute(jacobi_eig_kernel<7>, cudaFuncAttributeMaxDynamicSharedMemorySize, jac);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(jacobi_eig_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, jac);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(panel_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM);
+  return e;
 }
 
 cudaError_t panel_fused_launch(const float* In, long long in_bs, int ld_in, int batch, int rows, int l, const float* Mtx,

@@ -243,3 +243,17 @@ def test_half_filter_needs_the_tensor_engine_and_aligned_rows(ctx):
     with pytest.raises(binding.DeflError) as e:
         ctx.defl_psd_project(torch.eye(204, device="cuda"), 0, None, SCHED7, half_filter=True)     # 204 = 8 * 25.5
     assert e.value.code == -4
+
+
+@pytest.mark.parametrize("K", [3, 8, 16, 33, 56, 64])
+def test_small_ritz_values_beside_large_ones(ctx, K):
+    """A diagonal matrix from 1e10 down to 1e-6, of either sign, and the basis of the first unit vectors: the Rayleigh quotient
+    is that diagonal, exactly, and so are its eigenvalues (2^-23: one rounding to fp32, and one of fp64)."""
+    n = K + 1 + (-(K + 1)) % 4
+    d = torch.logspace(10.0, -6.0, n, dtype=torch.float64) * torch.tensor([1.0, -1.0]).double().repeat(n)[:n]
+    X = torch.diag(d).float().cuda()
+    V = torch.eye(n, K).cuda()
+    _, info = ctx.defl_psd_project(X, K - 1, V, SCHED7, gamma=1.1, seed=1, want_info=True)
+    want = torch.diagonal(X)[:K].double().cpu()
+    assert bool(((info["lam"].double().cpu() - want).abs() <= 2.0 ** -23 * want.abs()).all())
+    assert int(info["status"]) == 0
