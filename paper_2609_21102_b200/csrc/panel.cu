@@ -97,16 +97,6 @@ cudaError_t gram_partial_launch(const float* Y, long long batch_stride, int batc
 // steps run in blocks of NR, so that the pivot's place among a thread's rows is known to the compiler and who takes part
 // is a comparison of warp-uniform numbers: with rows eight apart the selection took more instructions than the update.
 // ---------------------------------------------------------------------------------------------
-// 1 / d for a positive finite d: the hardware's approximation and two Newton steps (a division costs twice the latency)
-__device__ __forceinline__ double reciprocal(double d) {
-  if (!(d > 1e-290 && d < 1e290)) return 1.0 / d;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  y = fma(y, fma(-d, y, 1.0), y);
-  y = fma(y, fma(-d, y, 1.0), y);
-  return fma(y, fma(-d, y, 1.0), y);
-}
-
 template <int NR>      // rows per thread, ceil(l / 8)
 __global__ void __launch_bounds__(512) chol_inv_kernel(const double* __restrict__ partial, int nchunk, int l, int cw_log2,
                                                        float* __restrict__ Rinv, int* __restrict__ status) {
@@ -160,7 +150,7 @@ __global__ void __launch_bounds__(512) chol_inv_kernel(const double* __restrict_
           for (int v = 0; v < NR; ++v) f[v] = pcol[buf][g * NR + v];      // (rows past l: zeros)
           if (!(d > 0.0) || !isfinite(d)) failed = true;
           else {
-            const double inv = reciprocal(d);
+            const double inv = 1.0 / d;
             if (tid == 0) diag[j] = d;
             const double s = (c == j) ? inv : inv * pr;
             if (g > a) {
