@@ -1267,17 +1267,27 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 const TcKnobs kDefaultKnobs = {0, 0, 0, 0, -1, 0, 0, 0, 0, 0};
 
+// a matrix times its own transpose
+bool same_operand(const GemmDesc& g) {
+  return g.nseg == 1 && g.b_split != 2 && g.A[0] == g.B[0] && g.sa_i[0] == g.sb_j[0] && g.sa_k[0] == g.sb_k[0] && g.batch_a[0] == g.batch_b[0];
+}
+
 // Tile width. Wide tiles move the fewest operand bytes per product, but a product of few tiles leaves most of the chip
 // idle, and the read-out of its last (often only) tile, whose time grows with the width, is not hidden by anything. The
 // CTA-pair form therefore takes the width with the smallest modelled time (in cycles):
-//   K block (128 bytes of K): the tensor pipe's 2 cycles per column, at least 480 (step latency), at least the operand
-//     bytes of all resident CTAs at the 5500 bytes per cycle that L2 delivers to the whole chip;
+//   K block (128 bytes of K): the tensor pipe's 2 cycles per column that exists, at least 480 (step latency), at least the
+//     operand bytes of all resident CTAs at the 5500 bytes per cycle that L2 delivers to the whole chip (a full tile on the
+//     diagonal of a product of a matrix with itself fetches one operand, at width 256 only);
 //   read-out: 1500 + 16 (16-bit) or 24 (fp32) per column, half as much again with mirror stores;
 //   waves of tiles, the read-out hidden behind the next tile's products except in the last wave.
-// Measured against width 256: symmetric 1024^3 tf32 22.2 -> 16.1 us (width 64), 1000^3 half 18.3 -> 12.8 (64), 2048^3 tf32
-// 32.5 -> 27.2 (128); 12 x 768^3 19.9 -> 17.8 (192); 4 x 517 x 517 x 1003 53 -> 22 (64); 24 x 1024^3 and everything
-// larger stays at 256 (42.8 us, 128: 48.5). The single-CTA form keeps the widest tile. (Edge tiles only compute the
-// columns that exist, rounded up to 16, or 32 for a CTA pair.)
+// Past three waves of the widest tiles the board's power decides, which the model does not see: there a width that makes
+// more tiles is not taken (16 x 1600^3 symmetric half: 192 columns 92 us, 256: 82; 16 x 1600 x 1600 x 6400: 299 and 270;
+// 8 x 1600^3: 50.2 and 48.0; 5 x 4608 x 1152 x 1152: 67 and 64).
+// Measured over 330 products with sides of 136 to 6400, batches 1 to 24, both orientations and types: on average 0.87 of the
+// time at width 256 and 1.015 of the best width's; at worst 5 % above width 256 (1 x 1032 x 4128 x 1032: 20.7 and 19.6).
+// Symmetric 1024^3 tf32 24.1 -> 18.7 us (width 64), 1000^3 half 20.7 -> 17.9 (64), 1536^3 tf32 29.1 -> 24.5 (96), 12 x 768^3 full
+// 23.1 -> 21.4 (192), 8 x 1024^3 26.3 -> 24.1 (192), launches included. The single-CTA form keeps the widest tile. (Edge
+// tiles only compute the columns that exist, rounded up to 16, or 32 for a CTA pair.)
 int choose_bn(const GemmDesc& g, bool pair, const TcKnobs& kn, int num_sms) {
   const int q = pair ? 32 : 16;
   if (kn.bn >= q && kn.bn <= 256 && kn.bn % q == 0) return kn.bn;
@@ -1288,25 +1298,31 @@ int choose_bn(const GemmDesc& g, bool pair, const TcKnobs& kn, int num_sms) {
   const int esize = (int)dtype_size(g.in_dtype), span = KBYTES / esize;
   const double pairs = num_sms / 2;
   const double out_col = (g.out_dtype == F32 ? 24.0 : 16.0) * (g.symmetric || g.transpose_out ? 1.5 : 1.0);
-  const bool b_mn = g.sb_k[0] != 1;
+  const bool b_mn = g.sb_k[0] != 1, self = g.symmetric && same_operand(g);
   int best = top;
-  double best_t = 0.0;
+  double best_t = 0.0, top_tiles = 0.0;
   for (int bn = top; bn >= 64; bn = (bn - 1) & ~31) {
     const int tm = (g.M + 255) / 256, tn = (g.N + bn - 1) / bn;
-    double tiles = 0.0;
-    for (int i = 0; i < tm; ++i) { const int first = g.symmetric ? i * 256 / bn : 0; if (first < tn) tiles += tn - first; }
-    tiles *= g.batch;
+    double tiles = 0.0, single = 0.0;            // single: tiles that fetch one operand
+    for (int i = 0; i < tm; ++i) {
+      const int first = g.symmetric ? i * 256 / bn : 0;
+      if (first < tn) tiles += tn - first;
+      if (self && bn == 256 && (i + 1) * 256 <= r) single += 1.0;
+    }
     double kb = (g.K[0] + span - 1) / span;
     if (g.nseg == 2) kb += ((g.seg1_identity ? bn : g.K[1]) + span - 1) / span;
     const int bcols = b_mn ? (bn / 2 + span - 1) / span * span : bn / 2;      // an MN-major operand moves whole boxes
-    const double bytes = (128.0 + bcols) * KBYTES, resident = 2.0 * (tiles < pairs ? tiles : pairs);
-    double block = 2.0 * bn;
+    const double bytes = (128.0 + bcols - bcols * (single / tiles)) * KBYTES;
+    tiles *= g.batch;
+    const double cols = (double)r / tn, resident = 2.0 * (tiles < pairs ? tiles : pairs);
+    double block = 2.0 * cols;
     if (block < 480.0) block = 480.0;
     if (block < bytes * resident / 5500.0) block = bytes * resident / 5500.0;
-    const double read_out = 1500.0 + bn * out_col, products = kb * block;
+    const double read_out = 1500.0 + cols * out_col, products = kb * block;
     const double waves = (double)(long long)((tiles + pairs - 1.0) / pairs);
     const double t = (waves - 1.0) * (products > read_out ? products : read_out) + products + read_out;
-    if (bn == top || t < best_t) { best = bn; best_t = t; }
+    if (bn == top) { best_t = t; top_tiles = tiles; }
+    else if (t < best_t && (top_tiles <= 3.0 * pairs || tiles == top_tiles)) { best = bn; best_t = t; }
   }
   return best;
 }
@@ -1504,10 +1520,8 @@ cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word,
             ((uint32_t)((p.pair ? 256 : 128) >> 4) << 24);
   p.epilogue = g.epilogue; p.out_dtype = g.out_dtype; p.aux_dtype = g.aux_dtype; p.symmetric = g.symmetric; p.round_tf32 = g.round_tf32;
   p.transposed = g.transpose_out ? 1 : 0;
-  p.dup_ok = (p.pair && g.symmetric && p.BN == 256 && p.tile_m == 256 && g.nseg == 1 && p.b_split != 2 && g.A[0] == g.B[0] &&
-              g.sa_i[0] == g.sb_j[0] && g.sa_k[0] == g.sb_k[0] && g.batch_a[0] == g.batch_b[0]) ? 1 : 0;
-  p.diag_exact = !(g.nseg == 1 && g.b_split != 2 && g.A[0] == g.B[0] && g.sa_i[0] == g.sb_j[0] && g.sa_k[0] == g.sb_k[0] &&
-                   g.batch_a[0] == g.batch_b[0]) ? 1 : 0;
+  p.dup_ok = (p.pair && g.symmetric && p.BN == 256 && p.tile_m == 256 && same_operand(g)) ? 1 : 0;
+  p.diag_exact = same_operand(g) ? 0 : 1;
   p.aux_f16 = (g.epilogue != EPI_STORE && g.aux_dtype == F16) ? 1 : 0;
   p.out_f16 = (g.out_dtype == F16) ? 1 : 0;
   p.C = g.C; p.ldc = g.ldc; p.batch_c = g.batch_c;

@@ -247,3 +247,41 @@ def test_polynomial_of_an_unsymmetric_matrix_is_computed_in_full(ctx, engine_nam
     ref = torch.eye(n, device="cuda", dtype=torch.float64) + A.double() + 0.125 * (A.double() @ A.double().transpose(1, 2))
     bound = (n + 3) * 2.0 ** -23 * (1.0 + A.double().abs() + 0.125 * (A.double().abs() @ A.double().abs().transpose(1, 2)))
     assert bool(((C.double() - ref).abs() <= bound).all())
+
+
+@pytest.mark.parametrize("width", [64, 96, 128, 160, 192, 224, 256])
+def test_tensor_engine_every_tile_width(monkeypatch, width):
+    """Every width that the tile rule can pick, forced (DEFL_TC_BN), on shapes that are multiples of none: K-major and MN-major
+    operands (whose half tiles of 48, 80, 112 columns are not whole boxes), the symmetric store where the width does not
+    divide the 256 rows of a tile (one operand given twice, and two operands that commute up to rounding: exactly symmetric
+    in both cases), the transposed store, and the identity segment (a small deflated call)."""
+    from paper_2609_21102_b200 import binding
+    monkeypatch.setenv("DEFL_TC_BN", str(width))
+    ctx = binding.Context(0)
+    T = binding.ENGINE_TENSOR
+    M, N, K = 712, 520, 328
+    for ta, tb in ((False, True), (False, False), (True, True), (True, False)):
+        A = _mk(2, K if ta else M, M if ta else K, torch.bfloat16, 61)
+        B = _mk(2, N if tb else K, K if tb else N, torch.bfloat16, 62)
+        ref = _ref(A, B, ta, tb)
+        C = ctx.defl_debug_gemm(A, B, ta, tb, engine=T, out_dtype=torch.float32)
+        assert torch.allclose(C, ref, rtol=1e-4, atol=4e-3)
+        C = ctx.defl_debug_gemm(A, B, ta, tb, engine=T, out_dtype=torch.float32, transpose_out=True)
+        assert torch.allclose(C, ref.transpose(1, 2), rtol=1e-4, atol=4e-3)
+        A = A[:, :, :M - 8].contiguous() if ta else A[:, :M - 8].contiguous()      # (the symmetric shape: 704 rows)
+        C = ctx.defl_debug_gemm(A, A, ta, not ta, engine=T, out_dtype=torch.float16, exploit_symmetry=True)
+        ref = _ref(A, A, ta, not ta)
+        assert torch.equal(C, C.transpose(1, 2)) and torch.allclose(C.float(), ref, rtol=2.0 ** -10, atol=4e-3)
+    S = _mk(2, 456, 456, torch.float32, 63)
+    S = (S + S.transpose(1, 2)).to(torch.float16) * 0.0625
+    S2 = (S.float() @ S.float()).to(torch.float16)                # a polynomial in S: the two commute up to rounding
+    S2 = torch.triu(S2) + torch.triu(S2, 1).transpose(1, 2)
+    C = ctx.defl_debug_gemm(S, S2.contiguous(), False, True, engine=T, out_dtype=torch.float32, exploit_symmetry=True)
+    ref = _ref(S, S2, False, True)
+    err = 2.0 ** -11 * (S.double().abs() @ S2.double().abs()) * 2.0 + 1e-4     # S2's own rounding, in either order of the product
+    assert torch.equal(C, C.transpose(1, 2)) and bool(((C.double() - ref.double()).abs() <= err).all())
+    G = _mk(2, 264, 520, torch.bfloat16, 64)
+    outs = [c.defl_polar_batched(G, 8, 8, 1, [list(binding.MUON_QUINTIC)] * 5, seed=4, gamma=1.01) for c in (ctx, binding.Context(0))]
+    torch.cuda.synchronize()
+    assert torch.equal(outs[0], outs[1])                         # a tile's width does not change the order of any sum
+    ctx.close()
