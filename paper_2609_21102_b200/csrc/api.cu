@@ -61,7 +61,8 @@ bool use_tensor_engine(const GemmDesc& g, int engine) {
 
 // A product of a matrix with its own transpose (X X^T, A A for the symmetric A, the polynomial a I + b A + c A A with the
 // exactly symmetric A itself as `aux`) computes (i, j) and (j, i) from the same terms in the same order on either engine:
-// the upper tiles and their mirror image are the full product for half the work, whatever exploit_symmetry says. On the
+// the upper tiles and their mirror image are the full product, whatever exploit_symmetry says, and are computed instead
+// where that is faster (the mirror store costs more than the plain one, so not where one wave of tiles does it all). On the
 // tensor engine to the bit; the FMA engine counts the tiles when it picks a tile form, and another form adds its K groups
 // in another order. (A_{t+1} = B_t^2 A_t of a paired step is a product of two matrices: without exploit_symmetry it is
 // symmetric up to rounding only, and its polynomial is computed in full.)
@@ -76,8 +77,8 @@ static bool self_product(const GemmDesc& g) {
 // Run one product on the engine the options ask for. Returns a DEFL_* code.
 int run_gemm(defl_ctx* c, const GemmDesc& desc, int engine, const char* what) {
   GemmDesc g = desc;
-  if (self_product(g)) g.symmetric = 1;
   const bool tc = use_tensor_engine(g, engine);
+  if (!g.symmetric && self_product(g) && (tc ? gemm_tc_symmetric_pays(g, c->num_sms, &c->tc_knobs) : gemm_simt_symmetric_pays(g))) g.symmetric = 1;
   if ((engine == DEFL_ENGINE_TENSOR || g.transpose_out) && !tc) {
     snprintf(c->err, sizeof(c->err), "%s: shape/type not supported by the tensor engine", what);
     return DEFL_ERR_UNSUPPORTED;

@@ -87,6 +87,9 @@ struct TmCache {
 // Engines (each returns cudaGetLastError() of its launch; they never synchronise).
 cudaError_t gemm_simt_launch(const GemmDesc& g, cudaStream_t st, long long* launches);
 int gemm_simt_partials_per_batch(const GemmDesc& g);
+// whether computing only the upper tiles of a product that is symmetric anyway is faster than computing it in full
+bool gemm_simt_symmetric_pays(const GemmDesc& g);
+bool gemm_tc_symmetric_pays(const GemmDesc& g, int num_sms, const TcKnobs* knobs);
 // Tensor-core engine: returns cudaErrorNotSupported when the descriptor cannot be expressed
 // as TMA-tiled tcgen05 products (alignment, type), without launching anything.
 cudaError_t gemm_tc_launch(const GemmDesc& g, cudaStream_t st, int* status_word, int num_sms, long long* launches,

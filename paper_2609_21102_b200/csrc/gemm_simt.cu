@@ -399,16 +399,18 @@ bool rank_update_form(const GemmDesc& g) {
 // the smaller of two estimates per SM, fitted to B200 timings: a 64 x 64 tile takes 1 us per K block of 32 and CTA on the
 // SM, a 32 x 32 tile 0.8 us per K block of 64 (4 x (512 x 384 x 384): 31 us with 32 x 32 tiles; 4 x (128 x 128 x 256): 6.2).
 enum SimtForm { FORM_64x64, FORM_32x32, FORM_64x16 };
+double simt_estimate(const GemmDesc& g, bool symmetric, int t) {
+  const int depth = g.K[0] + (g.nseg == 2 ? g.K[1] : 0);
+  const long long tm = (g.M + t - 1) / t, tn = (g.N + t - 1) / t;
+  const double per_sm = (double)(((symmetric ? tm * (tm + 1) / 2 : tm * tn) * g.batch + 147) / 148);
+  return t == 32 ? 0.8 * per_sm * ((depth + 63) / 64) : per_sm * ((depth + 31) / 32);
+}
 SimtForm simt_form(const GemmDesc& g) {
   if (g.M > 32 * 65535) return FORM_64x64;            // (the grid's y extent)
   if (g.N <= 16) return FORM_64x16;
   if (g.N <= 32) return FORM_32x32;
-  const int depth = g.K[0] + (g.nseg == 2 ? g.K[1] : 0);
-  auto per_sm = [&](int t) {
-    const long long tm = (g.M + t - 1) / t, tn = (g.N + t - 1) / t;
-    return (double)(((g.symmetric ? tm * (tm + 1) / 2 : tm * tn) * g.batch + 147) / 148);
-  };
-  return 0.8 * per_sm(32) * ((depth + 63) / 64) < 1.0 * per_sm(64) * ((depth + 31) / 32) ? FORM_32x32 : FORM_64x64;
+  const bool sym = g.symmetric != 0;
+  return simt_estimate(g, sym, 32) < simt_estimate(g, sym, 64) ? FORM_32x32 : FORM_64x64;
 }
 
 template <typename TIn, typename TB>
@@ -421,6 +423,19 @@ void launch_form(const GemmDesc& g, SimtForm f, cudaStream_t st) {
 }
 
 }  // namespace
+
+// The mirror stores (two of one value each instead of one of four) cost 5 to 30 % of a small product, so the upper tiles have
+// to be clearly fewer: estimated at under 0.72 of all tiles, or at 0.76 with at most two thirds of the tiles to compute, or
+// few enough for the smaller tile form. Upper tiles against full, fp32, in graphs: 148 x 64^3 + 30 %, 64 x 128^3 + 31 %,
+// 128 x 104^3 + 31 % (full); 64 x 256^3 - 11 %, 64 x 512^3 - 36 %, 128 x 192 x 192 x 768 - 19 %, 24 x 128 x 128 x 512 - 39 % (upper).
+bool gemm_simt_symmetric_pays(const GemmDesc& g) {
+  if (g.M <= 32 || g.M > 32 * 65535) return false;
+  const double f32 = simt_estimate(g, false, 32), f64 = simt_estimate(g, false, 64);
+  const double s32 = simt_estimate(g, true, 32), s64 = simt_estimate(g, true, 64);
+  const double ratio = fmin(s32, s64) / fmin(f32, f64);
+  const long long t = s32 < s64 ? (g.M + 31) / 32 : (g.M + 63) / 64;
+  return ratio < 0.72 || (ratio <= 0.76 && 3 * (t * (t + 1) / 2) <= 2 * t * t) || (s32 < s64 && !(f32 < f64));
+}
 
 int gemm_simt_partials_per_batch(const GemmDesc& g) {
   const SimtForm f = simt_form(g);

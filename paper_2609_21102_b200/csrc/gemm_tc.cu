@@ -1288,7 +1288,8 @@ bool same_operand(const GemmDesc& g) {
 // Symmetric 1024^3 tf32 24.1 -> 18.7 us (width 64), 1000^3 half 20.7 -> 17.9 (64), 1536^3 tf32 29.1 -> 24.5 (96), 12 x 768^3 full
 // 23.1 -> 21.4 (192), 8 x 1024^3 26.3 -> 24.1 (192), launches included. The single-CTA form keeps the widest tile. (Edge
 // tiles only compute the columns that exist, rounded up to 16, or 32 for a CTA pair.)
-int choose_bn(const GemmDesc& g, bool pair, const TcKnobs& kn, int num_sms) {
+// `cycles`, if given, receives the modelled time (0 where the width is not chosen by the model).
+int choose_bn(const GemmDesc& g, bool pair, const TcKnobs& kn, int num_sms, double* cycles = nullptr) {
   const int q = pair ? 32 : 16;
   if (kn.bn >= q && kn.bn <= 256 && kn.bn % q == 0) return kn.bn;
   const int r = (g.N + q - 1) & ~(q - 1);
@@ -1324,6 +1325,7 @@ int choose_bn(const GemmDesc& g, bool pair, const TcKnobs& kn, int num_sms) {
     if (bn == top) { best_t = t; top_tiles = tiles; }
     else if (t < best_t && (top_tiles <= 3.0 * pairs || tiles == top_tiles)) { best = bn; best_t = t; }
   }
+  if (cycles) *cycles = best_t;
   return best;
 }
 
@@ -1371,6 +1373,21 @@ bool cached_map(TmCache* cache, CUtensorMap* tm, const void* base, int esize, bo
 }
 
 }  // namespace
+
+// Both ways by the model above. Of one tile row nothing is skipped; and within one wave of the widest tiles the model's
+// lead has to be large (half, upper tiles against full, in graphs: 128 x 136^3 + 19 %, 128 x 256^3 + 16 %, 4 x 1024^3 + 7 % where it
+// promises - 11 %; 24 x 264^3 - 11 %, 24 x 320 x 320 x 1280 - 23 %, 64 x 1024^3 - 24 %).
+bool gemm_tc_symmetric_pays(const GemmDesc& g, int num_sms, const TcKnobs* knobs) {
+  const TcKnobs& kn = knobs ? *knobs : kDefaultKnobs;
+  if (g.M <= 256 || !choose_pair(g.M, g.N, kn)) return false;
+  GemmDesc u = g;
+  u.symmetric = 1;
+  double full = 0.0, upper = 0.0;
+  choose_bn(g, true, kn, num_sms, &full);
+  choose_bn(u, true, kn, num_sms, &upper);
+  const long long t = (g.M + 255) / 256;
+  return upper < (t * t * g.batch > num_sms / 2 ? 0.95 : 0.84) * full;
+}
 
 bool gemm_tc_supported(const GemmDesc& g) {
   if (g.batch <= 0 || g.M <= 0 || g.N <= 0) return false;
