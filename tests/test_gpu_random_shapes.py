@@ -111,8 +111,8 @@ def test_random_configurations_add_restore(ctx, seed):
 @pytest.mark.parametrize("form", ["plain", "padded", "gated", "add", "odd_base", "muon"])
 def test_rows_of_no_whole_packets_agree_with_the_fp32_engine(ctx, m, n, form):
     """bf16 shapes whose rows are not whole 16-byte packets run on padded copies and the tensor engine; the fp32 engine takes
-    the same call as it is. Both store the same 16-bit iterates from products that differ in the last bits, so single
-    roundings differ: each result is within the library's 3e-2 of the exact one (half of that here: spectrum with a gap),
+    the same call as it is. The range finder runs on the FMA engine with fp32 panels in both, the head enters X0 as a
+    three-term 16-bit split in the first; the stored 16-bit iterates differ in single roundings: each result is within the library's 3e-2 of the exact one (half of that here: spectrum with a gap),
     their distance within twice that."""
     from paper_2609_21102_b200 import binding
     rng = np.random.default_rng(m * 1000 + n)

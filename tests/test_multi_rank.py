@@ -4,9 +4,9 @@ import json
 import os
 import subprocess
 import sys
+import textwrap
 
 import pytest
-import textwrap
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
