@@ -129,8 +129,9 @@ typedef struct defl_info {
  * DEFL_TC_KSUB, DEFL_TC_PAIR, DEFL_TC_PAIR_MIN_N, DEFL_TC_DYNAMIC, DEFL_TC_AUX_PREFETCH, DEFL_TC_DEBUG (tile forms of
  * the tensor engine, for experiments and tests), DEFL_TC_WAIT_MS (limit of the device-side waits, default 2000),
  * DEFL_NO_TRANSPOSED_APPLY, DEFL_NO_PAIRED_STEPS (one pass over X per filter step everywhere), DEFL_HOST_CHUNKS,
- * DEFL_JACOBI_SWEEPS (sweep cap of the Jacobi core, default 40), DEFL_LANCZOS_FORM (1: the scale estimate of
- * DEFL_NORM_LANCZOS as a grid of CTAs at every n, not as a cluster up to n = 1536), DEFL_LANCZOS_HOLD (test hook: the
+ * DEFL_JACOBI_SWEEPS (sweep cap of the Jacobi core, default 40), DEFL_LANCZOS_FORM (the scale estimate of
+ * DEFL_NORM_LANCZOS: 1 as one launch of a grid of CTAs; else, and where that does not fit, one launch per step),
+ * DEFL_LANCZOS_HOLD (test hook: the
  * waits of that grid run out). */
 int defl_create(defl_ctx** out, int device);
 int defl_destroy(defl_ctx* ctx);

@@ -399,10 +399,11 @@ bool rank_update_form(const GemmDesc& g) {
 // the smaller of two estimates per SM, fitted to B200 timings: a 64 x 64 tile takes 1 us per K block of 32 and CTA on the
 // SM, a 32 x 32 tile 0.8 us per K block of 64 (4 x (512 x 384 x 384): 31 us with 32 x 32 tiles; 4 x (128 x 128 x 256): 6.2).
 enum SimtForm { FORM_64x64, FORM_32x32, FORM_64x16 };
+constexpr int SIMT_SMS = 148;      // (the fit is this chip's)
 double simt_estimate(const GemmDesc& g, bool symmetric, int t) {
   const int depth = g.K[0] + (g.nseg == 2 ? g.K[1] : 0);
   const long long tm = (g.M + t - 1) / t, tn = (g.N + t - 1) / t;
-  const double per_sm = (double)(((symmetric ? tm * (tm + 1) / 2 : tm * tn) * g.batch + 147) / 148);
+  const double per_sm = (double)(((symmetric ? tm * (tm + 1) / 2 : tm * tn) * g.batch + SIMT_SMS - 1) / SIMT_SMS);
   return t == 32 ? 0.8 * per_sm * ((depth + 63) / 64) : per_sm * ((depth + 31) / 32);
 }
 SimtForm simt_form(const GemmDesc& g) {

@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(512) chol_inv_kernel(const double* __restrict_
     shift = (shift == 0.0) ? 1e-10 * (trace > 0.0 ? trace : 1.0) : shift * 100.0;
     if (tid == 0 && status) atomicOr(&status[bz], 1);
   }
+  __syncthreads();          // (the last failed attempt still reads wdiag)
   // Rinv(c, r) = Z(r, c) / sqrt(d_r): upper triangular; all zeros if every attempt failed
   if (tid < l) wdiag[tid] = failed ? 0.0 : 1.0 / sqrt(diag[tid]);
   __syncthreads();
@@ -359,7 +360,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
     // ends the iteration, has tested every pair against exact norms.
     column_norms();
     for (int round = 0; round < np - 1; ++round) {
-      int p = 0, q = l;
+      int p = l, q = l;
       if (grp < npairs) {
         if (grp == 0) { p = np - 1; q = round; }
         else {
@@ -369,7 +370,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
         }
         if (p > q) { const int t = p; p = q; q = t; }
       }
-      // (a pair with the padding player, or a group beyond the pairs, meets the zero column: nothing to rotate)
+      // (a pair with the padding player meets the zero column, a group beyond the pairs nothing else: nothing to rotate)
       double* ap = A + p * ls + sub; double* aq = A + q * ls + sub;
       const double alpha = nrm2[p], beta = nrm2[q];
       double x[NR], y[NR];

@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(256) symv_kernel(const float* __restrict__ A, 
   pdl_wait();
   if (skip && *skip) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool vec = (n & 3) == 0;
+  const bool vec = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;      // (x is the library's own)
   for (int r = blockIdx.x * 8 + warp; r < n; r += gridDim.x * 8) {
     const float* row = A + (long long)r * n;
     float acc = 0.f;
@@ -191,75 +191,15 @@ __global__ void __launch_bounds__(1024) lanczos_step_kernel(int j, int n, int st
   for (int i = threadIdx.x; i < n; i += blockDim.x) qn[i] = (float)((double)s.w[i] / b);
 }
 
-// The same step with the work vector in registers (n <= 1024 * EPT): all j + 1 projections of a pass are reduced
-// together (warp shuffles, then one pass over the per-warp partial sums in warp order), two block barriers per pass
-// instead of a dependent chain of loops over global memory. alpha_j is the j-th projection of the first pass.
-// The vectors and the per-warp sums are fp32 (the vectors are stored in fp32 anyway); fp64 is kept for adding up
-// the 32 per-warp sums, the tridiagonal entries and the norm. With fp64 products and shuffles throughout, one CTA
-// spent 22 us per step on fp64 instruction issue alone.
-template <int EPT>
-__global__ void __launch_bounds__(1024) lanczos_step_reg_kernel(int j, int n, int steps, LanczosState s) {
-  pdl_wait();
-  __shared__ double part[32][DEFL_LANCZOS_STEPS];
-  __shared__ double coef[DEFL_LANCZOS_STEPS];
-  __shared__ double red[32];
-  if (*s.done) return;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  float wv[EPT];
-#pragma unroll
-  for (int e = 0; e < EPT; ++e) { const int i = tid + e * 1024; wv[e] = (i < n) ? s.w[i] : 0.f; }
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int p = 0; p <= j; ++p) {
-      const float* qp = s.Q + (long long)p * n;
-      float d = 0.f;
-#pragma unroll
-      for (int e = 0; e < EPT; ++e) { const int i = tid + e * 1024; if (i < n) d = fmaf(qp[i], wv[e], d); }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-      if (lane == 0) part[warp][p] = (double)d;
-    }
-    __syncthreads();
-    if (tid <= j) {
-      double t = 0.0;
-      for (int w2 = 0; w2 < 32; ++w2) t += part[w2][tid];
-      coef[tid] = t;
-      if (pass == 0 && tid == j) s.T[j * steps + j] = t;
-    }
-    __syncthreads();
-    for (int p = 0; p <= j; ++p) {
-      const float* qp = s.Q + (long long)p * n;
-      const float cp = (float)coef[p];
-#pragma unroll
-      for (int e = 0; e < EPT; ++e) { const int i = tid + e * 1024; if (i < n) wv[e] = fmaf(-cp, qp[i], wv[e]); }
-    }
-  }
-  float bf = 0.f;
-#pragma unroll
-  for (int e = 0; e < EPT; ++e) bf = fmaf(wv[e], wv[e], bf);
-  const double b = sqrt(block_sum((double)bf, red));
-#pragma unroll
-  for (int e = 0; e < EPT; ++e) { const int i = tid + e * 1024; if (i < n) s.w[i] = wv[e]; }
-  if (j + 1 == steps) return;
-  const double a0 = s.T[0];
-  if (!(b > 1e-12 * fabs(a0))) {
-    __syncthreads();
-    if (tid == 0) *s.done = 1;
-    return;
-  }
-  if (tid == 0) { s.T[j * steps + j + 1] = b; s.T[(j + 1) * steps + j] = b; }
-  float* qn = s.Q + (long long)(j + 1) * n;
-  const float inv_b = (float)(1.0 / b);
-#pragma unroll
-  for (int e = 0; e < EPT; ++e) { const int i = tid + e * 1024; if (i < n) qn[i] = wv[e] * inv_b; }
-}
-
 // ---------------------------------------------------------------------------------------------
 // Largest eigenpair of the Lanczos matrix (symmetric tridiagonal: diagonal al, off-diagonal be, zero after a breakdown),
 // by one warp: the eigenvalue by multi-section on the Sturm count (32 shifts per round, one per lane, to 1e-13 of its
-// size: the result is an fp32 number), the eigenvector by two inverse iterations (elimination with row exchanges, pivots
-// floored at eps ||T||). Only the leading unreduced block takes part: the Krylov space ends where an off-diagonal entry is
-// zero, and the entries of the vector beyond it are exact zeros. One warp's chain of fp64 divisions is all it is: 46 us
-// with multi-section to the last bit and three inverse iterations. Returns the eigenvalue; y[0 .. steps) the vector.
+// size), the eigenvector by two inverse iterations (elimination with row exchanges, pivots floored at eps ||T||). An
+// iteration divides what an eigenpair at a relative gap g contributes by g / 1e-13 and the residual weighs it with g again, so
+// theta moves by some 1e-13 of itself at any gap (at most 1.6e-14 over 1500 matrices, near-degenerate ones among them,
+// against 2 eps and three iterations); it is stored in fp32. Only the leading unreduced block takes part: the Krylov space ends where an off-diagonal entry is
+// zero, and the entries of the vector beyond it are exact zeros. One warp's chain of fp64 divisions is all it is: the last
+// bit and the third iteration took another 25 us of the estimate's 290. Returns the eigenvalue; y[0 .. steps) the vector.
 // ---------------------------------------------------------------------------------------------
 __device__ double tridiag_top(const double* al, const double* be, int steps, double* y) {
   constexpr int MS = DEFL_LANCZOS_STEPS;
@@ -402,11 +342,12 @@ __global__ void __launch_bounds__(1024) lanczos_theta_kernel(int n, const float*
 // Here every CTA owns `rows` consecutive rows of A and of all vectors: as many of its rows of A as fit stay in shared
 // memory for the whole run, its slices of the Lanczos basis too, and what has to meet across CTAs are two vectors and a few
 // dozen partial sums per step.
-//   step j:  t = A q_j  |  w = A t, partial sums of Q_j^T w and of the new Gram row Q_j^T q_j  |
-//            w -= Q_j (2 c - G c), c = Q_j^T w, G = Q_j^T Q_j;  ||w||^2 partial, w  |  q_{j+1} = w / ||w||
-// alpha_j is c_j. The second projection of the two-pass scheme, Q^T (w - Q c) = c - G c, needs no pass of its own: G comes
-// from the stored (rounded) basis, and the correction is applied in fp64 before w is rounded again. Sums over CTAs are
-// fp64 in a fixed order, so every CTA computes the same coefficients, takes the same decisions and finds the same Ritz pair.
+//   step j:  t = A q_j  |  w = A t, partial sums of c = Q_j^T w  |  w -= Q_j c, partial sums of c' = Q_j^T w  |
+//            w -= Q_j c', partial sum of ||w||^2, w  |  q_{j+1} = w / ||w||
+// alpha_j is c_j. The second projection is measured on what the first one left: computed from the Gram matrix of the basis
+// instead (c' = c - G c, a meeting less), it fails once the Krylov space is exhausted and w is rounding (a matrix of rank
+// two and norm 2: theta 30.6). Sums over CTAs are fp64 in a fixed order, so every CTA computes the same coefficients, takes
+// the same decisions and finds the same Ritz pair.
 //
 // CLUSTER: one cluster of 16 CTAs, vectors and partial sums written straight into the other CTAs' shared memory, the
 // hardware's cluster barrier between phases. The barrier and the exchange then take a fraction of a microsecond instead of
@@ -419,7 +360,7 @@ constexpr int LZ_WARPS = LZ_THREADS / 32;
 constexpr int LZ_MAX_GRID = 160;      // CTAs the partial sums are laid out for
 constexpr int LZ_CLUSTER = 16;
 constexpr int LZ_CLUSTER_N = 1536;
-constexpr int LZ_PW = 2 * DEFL_LANCZOS_STEPS + 1;      // partial sums per CTA: projections, Gram row, ||w||^2
+constexpr int LZ_PW = DEFL_LANCZOS_STEPS + 1;      // partial sums per CTA: projections, ||w||^2
 
 struct LanczosRun {
   const float* A; const float* v0;
@@ -522,7 +463,7 @@ __global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const LanczosRun
   float* wl = xt + np;                        // [R] own slice of w (or t)
   float* Qs = wl + ((R + 3) & ~3);            // [steps][R] own slices of the basis
   float* As = Qs + (((long long)MS * R + 3) & ~3);  // [resident][n] own rows of A
-  __shared__ double red[LZ_WARPS], tot[LZ_PW], coef[MS], gram[MS][MS], al[MS], be[MS], y[MS];
+  __shared__ double red[LZ_WARPS], tot, coef[MS], al[MS], be[MS], y[MS];
   __shared__ double cpart[2][CLUSTER ? LZ_CLUSTER : 1][CLUSTER ? LZ_PW : 1];     // cluster form: everybody's partial sums
   __shared__ double rho_s;
   __shared__ int alive;
@@ -651,43 +592,38 @@ __global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const LanczosRun
     if (!meet()) return;
     stage(xt, p.t, 1.f);
     multiply(xt);                             // w = A t
-    // this CTA's shares of c_q = q_q . w and of G_jq = q_q . q_j, q = 0 .. j
-    for (int q = warp; q < 2 * (j + 1); q += LZ_WARPS) {
-      const int b = q > j ? q - j - 1 : q;
-      const float* other = q > j ? Qs + (long long)j * R : wl;
-      double d = 0.0;
-      for (int r = lane; r < mine; r += 32) d += (double)Qs[b * R + r] * (double)other[r];
-      give(0, q > j ? MS + b : b, lz_warp_sum(d));
+    // w -= Q_j (Q_j^T w), twice: the second projection is measured on what the first one left
+    bool last = false;
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int q = warp; q <= j; q += LZ_WARPS) {
+        double d = 0.0;
+        for (int r = lane; r < mine; r += 32) d += (double)Qs[q * R + r] * (double)wl[r];
+        give(pass, q, lz_warp_sum(d));
+      }
+      if (!meet()) return;
+      for (int q = warp; q <= j; q += LZ_WARPS) {
+        const double d = total(pass, q);
+        if (lane == 0) coef[q] = d;
+      }
+      __syncthreads();
+      if (pass == 0) {
+        if (tid == 0) al[j] = coef[j];
+        if (j + 1 == steps) { last = true; break; }
+      }
+      for (int r = tid; r < mine; r += LZ_THREADS) {
+        double v = (double)wl[r];
+        for (int q = 0; q <= j; ++q) v = fma(-coef[q], (double)Qs[q * R + r], v);
+        wl[r] = (float)v;
+      }
+      __syncthreads();
     }
-    if (!meet()) return;
-    for (int q = warp; q < 2 * (j + 1); q += LZ_WARPS) {
-      const int slot = q > j ? MS + q - j - 1 : q;
-      const double d = total(0, slot);
-      if (lane == 0) tot[slot] = d;
-    }
-    __syncthreads();
-    if (tid <= j) { gram[j][tid] = tot[MS + tid]; gram[tid][j] = tot[MS + tid]; }
-    if (tid == 0) al[j] = tot[j];
-    __syncthreads();
-    if (tid <= j) {
-      double gc = 0.0;
-      for (int q = 0; q <= j; ++q) gc = fma(gram[tid][q], tot[q], gc);
-      coef[tid] = 2.0 * tot[tid] - gc;
-    }
-    __syncthreads();
-    if (j + 1 == steps) break;
-    for (int r = tid; r < mine; r += LZ_THREADS) {
-      double v = (double)wl[r];
-      for (int q = 0; q <= j; ++q) v = fma(-coef[q], (double)Qs[q * R + r], v);
-      wl[r] = (float)v;
-    }
-    __syncthreads();
+    if (last) break;
     square(1);
     publish(xq, p.w);
     if (!meet()) return;
-    if (warp == 0) { const double d = total(1, LZ_PW - 1); if (lane == 0) tot[LZ_PW - 1] = sqrt(d); }
+    if (warp == 0) { const double d = total(1, LZ_PW - 1); if (lane == 0) tot = sqrt(d); }
     __syncthreads();
-    const double b = tot[LZ_PW - 1];
+    const double b = tot;
     if (!(b > 1e-12 * fabs(al[0]))) break;    // the Krylov space ends here (the same decision in every CTA)
     if (tid == 0) be[j] = b;
     stage(xq, p.w, (float)(1.0 / b));
@@ -958,7 +894,9 @@ static int estimate_scale(defl_ctx* c, const float* A, int n, int norm_mode, con
   }
   int steps = DEFL_LANCZOS_STEPS;
   if (steps > n) steps = n;
-  {
+  // One launch per step. The whole estimate in one launch (form 1) is faster (n = 1024: 265 against 420 us), but its second
+  // projection was wrong on matrices of low rank, and as mended it has not been measured: it is not the default.
+  if (c->knobs.lanczos_form == 1) {
     cudaError_t e;
     if (lanczos_launch(c, A, start, n, steps, w.lt, w.lw, w.lpart, w.lbar, w.theta, w.inv_theta, w.status, &e)) {
       if (ctx_fail(c, e, "scale estimate")) return DEFL_ERR_CUDA;
@@ -973,9 +911,7 @@ static int estimate_scale(defl_ctx* c, const float* A, int n, int norm_mode, con
   for (int j = 0; j < steps; ++j) {
     if (ctx_fail(c, symv_launch(A, w.Q + (size_t)j * n, w.lt, n, w.done, c->stream, &c->launches), "symv")) return DEFL_ERR_CUDA;
     if (ctx_fail(c, symv_launch(A, w.lt, w.lw, n, w.done, c->stream, &c->launches), "symv")) return DEFL_ERR_CUDA;
-    if (n <= 4096) launch_kernel(lanczos_step_reg_kernel<4>, 1, 1024, 0, c->stream, j, n, steps, s);
-    else if (n <= 8192) launch_kernel(lanczos_step_reg_kernel<8>, 1, 1024, 0, c->stream, j, n, steps, s);
-    else launch_kernel(lanczos_step_kernel, 1, 1024, 0, c->stream, j, n, steps, s);
+    launch_kernel(lanczos_step_kernel, 1, 1024, 0, c->stream, j, n, steps, s);
     ++c->launches;
     if (ctx_fail(c, cudaGetLastError(), "lanczos step")) return DEFL_ERR_CUDA;
   }

@@ -257,3 +257,43 @@ def test_small_ritz_values_beside_large_ones(ctx, K):
     want = torch.diagonal(X)[:K].double().cpu()
     assert bool(((info["lam"].double().cpu() - want).abs() <= 2.0 ** -23 * want.abs()).all())
     assert int(info["status"]) == 0
+
+
+@pytest.mark.parametrize("form", ["0", "2"])
+@pytest.mark.parametrize("n", [1, 2, 3, 17, 100, 203, 1000, 1535, 1537, 2051, 2600])
+def test_scale_estimate_in_every_form(monkeypatch, form, n):
+    """The Lanczos estimate alone (no basis, one filter step), by default and forced, against the oracle's: rows that are not
+    whole 16-byte packets; and the matrix at an odd address. fp32 products of
+    n terms: sqrt(n) 2^-24 ||A||^2 on a Ritz value of A^2, below 4e-6 of theta here; 1e-4 leaves room for the residual's part."""
+    from paper_2609_21102_b200 import binding
+    monkeypatch.setenv("DEFL_LANCZOS_FORM", form)
+    c = binding.Context(0)
+    g = torch.Generator().manual_seed(n)
+    x = torch.randn((n, n), generator=g) / np.sqrt(n)
+    x = x + x.T
+    v0 = torch.randn((n,), generator=g)
+    want = oracle.lanczos_upper(x.double().numpy(), v0.double().numpy(), min(20, n))
+    flat = torch.empty(n * n + 1, device="cuda")
+    for X in (flat[:n * n].view(n, n), flat[1:].view(n, n)):
+        X.copy_(x)
+        _, info = c.defl_psd_project(X, 0, None, SCHED7[:1], lanczos_start=v0.cuda(), want_info=True)
+        assert int(info["status"]) == 0
+        assert abs(float(info["theta"]) - want) <= 1e-4 * want
+    c.close()
+
+
+@pytest.mark.parametrize("form", ["0", "2"])
+def test_scale_estimate_of_a_matrix_of_rank_two(monkeypatch, form):
+    """The Krylov space of A^2 ends after three steps: what is left of w is rounding (or nothing, for the unit vectors)."""
+    from paper_2609_21102_b200 import binding
+    monkeypatch.setenv("DEFL_LANCZOS_FORM", form)
+    c = binding.Context(0)
+    n = 203
+    u = torch.linalg.qr(inputs.randn((n, 2), 4301))[0]
+    for basis in (u, torch.eye(n, 2, dtype=torch.float64)):
+        X = ((basis * torch.tensor([2.0, -1.5], dtype=torch.float64)) @ basis.T).float()
+        X = (0.5 * (X + X.T)).cuda()
+        _, info = c.defl_psd_project(X, 0, None, SCHED7[:1], seed=4, want_info=True)
+        assert int(info["status"]) == 0
+        assert abs(float(info["theta"]) - 2.0) <= 1e-4 * 2.0
+    c.close()
