@@ -130,9 +130,8 @@ typedef struct defl_info {
  * the tensor engine, for experiments and tests), DEFL_TC_WAIT_MS (limit of the device-side waits, default 2000),
  * DEFL_NO_TRANSPOSED_APPLY, DEFL_NO_PAIRED_STEPS (one pass over X per filter step everywhere), DEFL_HOST_CHUNKS,
  * DEFL_JACOBI_SWEEPS (sweep cap of the Jacobi core, default 40), DEFL_LANCZOS_FORM (the scale estimate of
- * DEFL_NORM_LANCZOS: 1 as one launch of a grid of CTAs; else, and where that does not fit, one launch per step),
- * DEFL_LANCZOS_HOLD (test hook: the
- * waits of that grid run out). */
+ * DEFL_NORM_LANCZOS: 2 one launch per step, the form for n above 8192; else one launch for all of it),
+ * DEFL_LANCZOS_HOLD (test hook: the waits of that launch run out). */
 int defl_create(defl_ctx** out, int device);
 int defl_destroy(defl_ctx* ctx);
 int defl_set_stream(defl_ctx* ctx, void* cuda_stream); /* cudaStream_t; NULL = default stream */

@@ -158,7 +158,9 @@ __global__ void __launch_bounds__(1024) lanczos_step_kernel(int j, int n, int st
   a = block_sum(a, red);
   if (threadIdx.x == 0) s.T[j * steps + j] = a;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int pass = 0; pass < 2; ++pass) {
+  // w -= Q_j (Q_j^T w), twice; again where less than 1e-5 of w is left (see lanczos_kernel)
+  double b = 0.0, before = 0.0;
+  for (int pass = 0; pass < 4; ++pass) {
     // c = Q_j^T w, one warp per basis vector, then w -= Q_j c
     for (int p = warp; p <= j; p += nw) {
       const float* qp = s.Q + (long long)p * n;
@@ -169,16 +171,23 @@ __global__ void __launch_bounds__(1024) lanczos_step_kernel(int j, int n, int st
       if (lane == 0) coef[p] = d;
     }
     __syncthreads();
+    if (pass == 0) {
+      for (int p = 0; p <= j; ++p) before = fma(coef[p], coef[p], before);
+      before = sqrt(before);
+    }
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       double wi = (double)s.w[i];
       for (int p = 0; p <= j; ++p) wi -= coef[p] * (double)s.Q[(long long)p * n + i];
       s.w[i] = (float)wi;
     }
     __syncthreads();
+    if (pass == 0) continue;
+    b = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) b += (double)s.w[i] * (double)s.w[i];
+    b = sqrt(block_sum(b, red));
+    if (!(b < 1e-5 * before)) break;
+    before = b;
   }
-  double b = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) b += (double)s.w[i] * (double)s.w[i];
-  b = sqrt(block_sum(b, red));
   if (j + 1 == steps) return;
   const double a0 = s.T[0];
   if (!(b > 1e-12 * fabs(a0))) {
@@ -193,110 +202,135 @@ __global__ void __launch_bounds__(1024) lanczos_step_kernel(int j, int n, int st
 
 // ---------------------------------------------------------------------------------------------
 // Largest eigenpair of the Lanczos matrix (symmetric tridiagonal: diagonal al, off-diagonal be, zero after a breakdown),
-// by one warp: the eigenvalue by multi-section on the Sturm count (32 shifts per round, one per lane, to 1e-13 of its
-// size), the eigenvector by two inverse iterations (elimination with row exchanges, pivots floored at eps ||T||). An
-// iteration divides what an eigenpair at a relative gap g contributes by g / 1e-13 and the residual weighs it with g again, so
-// theta moves by some 1e-13 of itself at any gap (at most 1.6e-14 over 1500 matrices, near-degenerate ones among them,
-// against 2 eps and three iterations); it is stored in fp32. Only the leading unreduced block takes part: the Krylov space ends where an off-diagonal entry is
-// zero, and the entries of the vector beyond it are exact zeros. One warp's chain of fp64 divisions is all it is: the last
-// bit and the third iteration took another 25 us of the estimate's 290. Returns the eigenvalue; y[0 .. steps) the vector.
+// by one CTA of any number of warps. The eigenvalue by multi-section on the Sturm count, one shift per thread, to 1e-13 of its
+// size (five rounds with 512 threads): the sign changes of the leading minors of T - x by their three-term
+// recurrence on the matrix scaled to norm one, itself rescaled by powers of two every four rows, so that its chain has no
+// division. The eigenvector from the twisted factorisation of T - lambda: the pivots from the top and from the bottom by two
+// lanes at once, and the recurrences away from the row where they meet with the smallest remainder. theta moves by less than
+// 2e-11 of itself against LAPACK's pair (600 Lanczos matrices, near-degenerate, clustered and of rank two among them); it is
+// stored in fp32. Only the leading unreduced block takes part: the Krylov space ends where an off-diagonal entry is zero,
+// and the entries of the vector beyond it are exact zeros. A chain of dependent fp64 operations is all it is. Returns the
+// eigenvalue; y[0 .. steps) the vector, for every thread of the CTA (all of them call it).
 // ---------------------------------------------------------------------------------------------
-__device__ double tridiag_top(const double* al, const double* be, int steps, double* y) {
-  constexpr int MS = DEFL_LANCZOS_STEPS;
-  const int lane = threadIdx.x & 31;
-  if (lane < steps) y[lane] = 0.0;
-  __syncwarp();
-  int m = 1;
-  while (m < steps && be[m - 1] != 0.0) ++m;                 // size of the leading unreduced block
-  // Gershgorin interval and the scale of the matrix
-  double lo = al[0], hi = al[0], tn = 0.0;
-  for (int i = 0; i < m; ++i) {
-    const double r = (i > 0 ? fabs(be[i - 1]) : 0.0) + (i + 1 < m ? fabs(be[i]) : 0.0);
-    lo = fmin(lo, al[i] - r); hi = fmax(hi, al[i] + r);
-    tn = fmax(tn, fabs(al[i]) + r);
-  }
+struct TridiagScratch {
+  double a[DEFL_LANCZOS_STEPS], e[DEFL_LANCZOS_STEPS], e2[DEFL_LANCZOS_STEPS];      // the scaled matrix
+  double piv[2][DEFL_LANCZOS_STEPS], ratio[2][DEFL_LANCZOS_STEPS];      // from the top, from the bottom
+  double lo, hi, unscale;
+  int m;
+};
+
+__device__ double tridiag_top(const double* al, const double* be, int steps, double* y, TridiagScratch& s) {
+  constexpr unsigned FULL = 0xffffffffu;
   const double eps = 2.220446049250313e-16;
-  const double pivmin = fmax(tn * eps * eps, 1e-300);
-  double a = lo - eps * tn - pivmin, b = hi + eps * tn + pivmin;       // count(a) < m = count(b)
-  for (int round = 0; round < 16; ++round) {
-    const double x = a + (b - a) * ((double)(lane + 1) / 33.0);
-    // number of eigenvalues of the block below x: negative terms of the Sturm recurrence
-    int cnt = 0;
-    double q = 1.0;
-    for (int i = 0; i < m; ++i) {
-      q = al[i] - x - (i > 0 ? be[i - 1] * be[i - 1] / q : 0.0);
-      if (fabs(q) < pivmin) q = -pivmin;
-      cnt += q < 0.0;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  if (tid < 32) {
+    // size of the leading unreduced block; a bracket of the largest eigenvalue: the largest diagonal entry and row sum
+    const bool in = tid < steps;
+    const double d = in ? al[tid] : 0.0, right = (tid + 1 < steps) ? be[tid] : 0.0, left = (in && tid > 0) ? be[tid - 1] : 0.0;
+    const unsigned ends = __ballot_sync(FULL, !(right != 0.0));
+    const int m = __ffs((int)ends);                          // (lane steps - 1 has none to its right)
+    const double r = fabs(left) + (tid + 1 < m ? fabs(right) : 0.0);
+    double lo = tid < m ? d : al[0], tn = tid < m ? fabs(d) + r : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fmax(lo, __shfl_xor_sync(FULL, lo, o));
+      tn = fmax(tn, __shfl_xor_sync(FULL, tn, o));
     }
-    const unsigned full = __ballot_sync(0xffffffffu, cnt >= m);         // shifts above every eigenvalue
-    const int first = full ? __ffs(full) - 1 : 32;
-    const double nb = (first < 32) ? __shfl_sync(0xffffffffu, x, first) : b;
-    const double na = (first > 0) ? __shfl_sync(0xffffffffu, x, first - 1) : a;
+    double scale = 1.0, unscale = 1.0;                       // powers of two around 1 / tn and tn
+    if (tn > 1e-290 && tn < 1e290) {
+      const int ex = (int)((__double_as_longlong(tn) >> 52) & 0x7ff);
+      scale = __longlong_as_double((long long)(2046 - ex) << 52);
+      unscale = __longlong_as_double((long long)ex << 52);
+    }
+    if (tid < m) {
+      const double e = tid + 1 < m ? right * scale : 0.0;
+      s.a[tid] = d * scale; s.e[tid] = e; s.e2[tid] = e * e;
+    }
+    if (tid == 0) { s.m = m; s.lo = lo * scale; s.hi = tn * scale; s.unscale = unscale; }
+  }
+  __syncthreads();
+  const int m = s.m;
+  double a = s.lo - 4.0 * eps - 1e-300, b = s.hi + 4.0 * eps + 1e-300;       // count(a) < m = count(b)
+  const double part = 1.0 / (double)(nt + 1);
+  for (int round = 0; round < 16; ++round) {
+    const double w = (b - a) * part, x = fma(w, (double)(tid + 1), a);
+    // number of eigenvalues of the block below x: sign changes of the minors
+    double pm = 1.0, pc = s.a[0] - x;
+    int sign = __double2hiint(pc) >> 31, cnt = -sign;
+    for (int i = 1; i < m; ++i) {
+      const double pn = fma(s.a[i] - x, pc, -s.e2[i - 1] * pm);
+      pm = pc; pc = pn;
+      const int now = __double2hiint(pc) >> 31;
+      cnt += (now ^ sign) & 1;
+      sign = now;
+      if ((i & 3) == 0) {
+        const double big = fmax(fabs(pm), fabs(pc));
+        if (big < 1e-100) { pm *= 0x1p400; pc *= 0x1p400; }
+      }
+    }
+    const int below = __syncthreads_count(cnt < m);                     // shifts that do not lie above every eigenvalue
+    const double na = below > 0 ? fma(w, (double)below, a) : a, nb = below < nt ? fma(w, (double)(below + 1), a) : b;
     a = na; b = nb;
-    if (b - a <= 1e-13 * fmax(fabs(a), fabs(b)) + 2.0 * pivmin) break;
+    if (!(b - a > 1e-13 * fabs(b))) break;
   }
   const double lam = 0.5 * (a + b);
-  if (lane == 0) {
-    if (m == 1) y[0] = 1.0;
-    else {
-      // inverse iteration from the vector of ones (the off-diagonal entries of a Lanczos matrix are positive, so the
-      // wanted vector has entries of one sign and is not orthogonal to it)
-      double d[MS], du[MS], du2[MS], dl[MS], z[MS];
-      const double floor_p = eps * tn;
-      for (int i = 0; i < m; ++i) z[i] = 1.0;
-      for (int iter = 0; iter < 2; ++iter) {
-        for (int i = 0; i < m; ++i) { d[i] = al[i] - lam; du[i] = (i + 1 < m) ? be[i] : 0.0; dl[i] = du[i]; du2[i] = 0.0; }
-        for (int i = 0; i + 1 < m; ++i) {
-          if (fabs(d[i]) >= fabs(dl[i])) {
-            if (fabs(d[i]) < floor_p) d[i] = (d[i] < 0.0) ? -floor_p : floor_p;
-            const double f = dl[i] / d[i];
-            d[i + 1] -= f * du[i];
-            z[i + 1] -= f * z[i];
-          } else {
-            // rows i and i + 1 change places
-            const double f = d[i] / dl[i];
-            d[i] = dl[i];
-            const double t = d[i + 1];
-            d[i + 1] = du[i] - f * t;
-            du[i] = t;
-            if (i + 2 < m) { du2[i] = du[i + 1]; du[i + 1] = -f * du2[i]; }
-            const double zt = z[i];
-            z[i] = z[i + 1];
-            z[i + 1] = zt - f * z[i + 1];
-          }
-        }
-        if (fabs(d[m - 1]) < floor_p) d[m - 1] = (d[m - 1] < 0.0) ? -floor_p : floor_p;
-        z[m - 1] /= d[m - 1];
-        z[m - 2] = (z[m - 2] - du[m - 2] * z[m - 1]) / d[m - 2];
-        for (int i = m - 3; i >= 0; --i) z[i] = (z[i] - du[i] * z[i + 1] - du2[i] * z[i + 2]) / d[i];
-        double big = 0.0;
-        for (int i = 0; i < m; ++i) big = fmax(big, fabs(z[i]));
-        double nn = 0.0;
-        for (int i = 0; i < m; ++i) { z[i] = (big > 0.0) ? z[i] / big : ((i == 0) ? 1.0 : 0.0); nn += z[i] * z[i]; }
-        const double inv = rsqrt(nn);
-        for (int i = 0; i < m; ++i) z[i] *= inv;
+  if (tid < 32) {
+    if (tid < 2) {
+      // lane 0 from the top, lane 1 from the bottom: piv_i, and ratio_i = (off-diagonal towards the next row) / piv_i
+      double carry = 0.0;
+      for (int k = 0; k < m; ++k) {
+        const int i = tid ? m - 1 - k : k;
+        double d = s.a[i] - lam - carry;
+        s.piv[tid][i] = d;
+        if (fabs(d) < eps) d = (d < 0.0) ? -eps : eps;
+        const double e = (k + 1 < m) ? s.e[tid ? i - 1 : i] : 0.0, q = e * (1.0 / d);
+        s.ratio[tid][i] = q;
+        carry = e * q;
       }
-      for (int i = 0; i < m; ++i) y[i] = z[i];
     }
+    __syncwarp();
+    // the row of the smallest remainder, and products of the ratios away from it
+    double g = tid < m ? fabs(s.piv[0][tid] + s.piv[1][tid] - (s.a[tid] - lam)) : 1e300;
+    int at = tid;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double go = __shfl_xor_sync(FULL, g, o);
+      const int ao = __shfl_xor_sync(FULL, at, o);
+      if (go < g || (go == g && ao < at)) { g = go; at = ao; }
+    }
+    at = min(at, m - 1);
+    double up = (tid < at) ? -s.ratio[0][tid] : 1.0, down = (tid > at && tid < m) ? -s.ratio[1][tid] : 1.0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double u = __shfl_down_sync(FULL, up, o), v = __shfl_up_sync(FULL, down, o);
+      if (tid + o < 32) up *= u;
+      if (tid >= o) down *= v;
+    }
+    const double z = tid < m ? up * down : 0.0;
+    double nn = z * z;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(FULL, nn, o);
+    if (tid < steps) y[tid] = z / sqrt(nn);
   }
-  __syncwarp();
-  return lam;
+  __syncthreads();
+  return lam * s.unscale;
 }
 
 // the same from the dense matrix [steps, steps] in device memory: rho[0] and column 0 of E (fp32, [steps, steps] row-major)
-__global__ void __launch_bounds__(32) tridiag_top_kernel(const double* __restrict__ T, int steps, float* __restrict__ rho,
-                                                         float* __restrict__ E) {
+__global__ void __launch_bounds__(512) tridiag_top_kernel(const double* __restrict__ T, int steps, float* __restrict__ rho,
+                                                          float* __restrict__ E) {
   pdl_wait();
   __shared__ double al[DEFL_LANCZOS_STEPS], be[DEFL_LANCZOS_STEPS], y[DEFL_LANCZOS_STEPS];
-  const int lane = threadIdx.x;
-  if (lane < steps) {
-    al[lane] = T[lane * steps + lane];
-    be[lane] = (lane + 1 < steps) ? T[lane * steps + lane + 1] : 0.0;
+  __shared__ TridiagScratch tri;
+  const int i = threadIdx.x;
+  if (i < steps) {
+    al[i] = T[i * steps + i];
+    be[i] = (i + 1 < steps) ? T[i * steps + i + 1] : 0.0;
   }
-  __syncwarp();
-  const double lam = tridiag_top(al, be, steps, y);
-  if (lane == 0) rho[0] = (float)lam;
-  if (lane < steps) E[lane * steps] = (float)y[lane];
+  __syncthreads();
+  const double lam = tridiag_top(al, be, steps, y, tri);
+  if (i == 0) rho[0] = (float)lam;
+  if (i < steps) E[i * steps] = (float)y[i];
 }
 
 // v = sum_p E[p][0] q_p (the Ritz vector of the largest Ritz value); E is [steps, steps] row-major fp32; rows of Q that
@@ -338,399 +372,477 @@ __global__ void __launch_bounds__(1024) lanczos_theta_kernel(int n, const float*
 
 // ---------------------------------------------------------------------------------------------
 // The whole scale estimate in one launch. As 63 dependent launches (two matrix-vector products and one single-CTA
-// reorthogonalisation per step) it was bound by launches and by one SM's memory path: 440 us at n = 1000, 640 at n = 4096.
-// Here every CTA owns `rows` consecutive rows of A and of all vectors: as many of its rows of A as fit stay in shared
-// memory for the whole run, its slices of the Lanczos basis too, and what has to meet across CTAs are two vectors and a few
-// dozen partial sums per step.
-//   step j:  t = A q_j  |  w = A t, partial sums of c = Q_j^T w  |  w -= Q_j c, partial sums of c' = Q_j^T w  |
+// reorthogonalisation per step) it is bound by launches and by one SM's memory path: 325 us at n = 1024, about 700 at 4096.
+// Here every CTA owns `rows` consecutive rows of A and of all vectors, and every thread up to 4 P columns: as many of the CTA's
+// rows of A as fit stay in shared memory for the whole run, its slices of the Lanczos basis Q and of A Q too, and what has to
+// meet across CTAs are two vectors and a few dozen partial sums per step:
+//   step j:  t = A q_j, partial sums of c = (A Q_j)^T t  |  w = A t - Q_j c, partial sums of c' = Q_j^T w  |
 //            w -= Q_j c', partial sum of ||w||^2, w  |  q_{j+1} = w / ||w||
-// alpha_j is c_j. The second projection is measured on what the first one left: computed from the Gram matrix of the basis
-// instead (c' = c - G c, a meeting less), it fails once the Krylov space is exhausted and w is rounding (a matrix of rank
-// two and norm 2: theta 30.6). Sums over CTAs are fp64 in a fixed order, so every CTA computes the same coefficients, takes
+// c = Q_j^T A t is taken from the slices of A Q_j that the earlier steps left, before t itself has met; alpha_j is c_j. The
+// second projection is measured on what the first one left, and where less than 1e-5 of w remains a third
+// one (and a fourth) is measured on what the second left: the basis is orthonormal to fp32 only, and once the Krylov space is
+// exhausted and w is rounding, two projections leave as much of the basis in w as there is rounding. Of 300 matrices of rank
+// one to seven, two projections alone gave 47 a wrong scale (up to 24 times too large); with the rule the worst is 2e-7 off.
+// Sums over CTAs are fp64 in a fixed order, so every CTA computes the same coefficients, takes
 // the same decisions and finds the same Ritz pair.
 //
-// CLUSTER: one cluster of 16 CTAs, vectors and partial sums written straight into the other CTAs' shared memory, the
-// hardware's cluster barrier between phases. The barrier and the exchange then take a fraction of a microsecond instead of
-// about four through L2 and a counter, which is what bounds small n; 16 SMs can only read 16 times 64 bytes per cycle
-// of what does not fit in their shared memory, which bounds large n. Up to n = LZ_CLUSTER_N the cluster, above it the
-// cooperative grid (n = 1000: 361 us with the grid; n = 4096: 655).
+// A meeting is the exchange itself: every 32-bit word travels in one 64-bit store together with the number of the meeting,
+// and a reader polls the words that it needs until they carry that number. No counter and no fence: one store and one load
+// through L2, 900 cycles from SM to SM on an idle chip. Two things made that ten times longer. What the polls of all CTAs read
+// at once must stay small against L2's bandwidth, or the stores queue behind them: a word of a vector is read by the one
+// thread that owns its column, and above LZ_DIRECT CTAs partial sums are added up by one CTA for all. And a line that many
+// poll must be written by one CTA, in one instruction: every CTA's message has lines of its own and leaves from one warp. A
+// word is overwritten only by the same meeting of the next step, which its owner reaches after it has seen everybody arrive
+// at a later meeting of this step, that is, after everybody has read it. Numbers start at one on zeroed words. What bounds the
+// estimate is the latency of the meetings and of two matrix-vector products per step; above n = 2700 or so also the rows of A
+// that do not fit and come through L2 in every product.
 // ---------------------------------------------------------------------------------------------
 constexpr int LZ_THREADS = 512;
 constexpr int LZ_WARPS = LZ_THREADS / 32;
-constexpr int LZ_MAX_GRID = 160;      // CTAs the partial sums are laid out for
-constexpr int LZ_CLUSTER = 16;
-constexpr int LZ_CLUSTER_N = 1536;
-constexpr int LZ_PW = DEFL_LANCZOS_STEPS + 1;      // partial sums per CTA: projections, ||w||^2
+constexpr int LZ_HALVES = LZ_THREADS / 16;         // groups of 16 lanes: one per basis vector, or per row
+constexpr int LZ_MAX_GRID = 160;                   // CTAs the messages are laid out for
+constexpr int LZ_ROWS = 8;                         // rows per CTA at least, and rows of a pass over the columns
+constexpr int LZ_DIRECT = 64;                      // CTAs up to which everybody reads everybody's partial sums
+constexpr int LZ_QUADS = 4;                        // quads of columns per thread at most: n <= 8192
+constexpr int LZ_PB = 24;                          // partial sums of a message: DEFL_LANCZOS_STEPS, to whole lines of 128 bytes
+constexpr int LZ_LINE = 16;                        // words of a line
+static_assert(LZ_HALVES > LZ_PB && LZ_PB >= DEFL_LANCZOS_STEPS && LZ_PB * 2 % LZ_LINE == 0, "one half-warp per partial sum, and one more");
+static_assert(LZ_WARPS == 16, "a half-warp adds up the warps' sums of a row");
 
 struct LanczosRun {
   const float* A; const float* v0;
-  int n, steps, rows, resident;      // rows per CTA, how many of them stay in shared memory
-  int aligned;                       // rows of A may be read 16 bytes at a time
-  float* t; float* w;                // [n]                       (grid form)
-  double* part;                      // [2][grid][LZ_PW]          (grid form)
-  unsigned int* bar;                 // barrier counter, zero at launch (grid form)
-  int* wait_status;                  // bit 8 when a barrier runs out of time
+  int n, steps, rows, resident;      // rows per CTA (a multiple of four), how many stay in shared memory
+  int aligned;                       // quads of A may be read 16 bytes at a time
+  int block;                         // words of a CTA's message in vec: its rows, its share of ||w||^2 (two words), to whole lines
+  unsigned long long* vec[2];        // [grid][block] t and w
+  unsigned long long* part;          // [2][grid][LZ_PB][2] partial sums of the projections
+  unsigned long long* sum;           // [2][LZ_PB][LZ_LINE] their sums (grids above LZ_DIRECT CTAs)
+  int* wait_status;                  // bit 8 when a meeting runs out of time
   unsigned long long wait_ns;
-  unsigned int hold;                 // test hook (grid form): arrivals that a meeting waits for and that never come
+  unsigned int hold;                 // test hook: the first meeting waits for a number that never comes
   float* theta; float* inv_theta; int* status;
 };
 
-// y_i = A[row_i] . x for up to NR rows at once by the calling warp (x in shared memory, read once for all); every lane
-// gets the sums
-template <int NR>
-__device__ __forceinline__ void row_dots(const float* const* row, const float* x, int n, bool vec, int lane, float* out) {
-  float acc[NR];
-  if (vec) {
-    const float4* x4 = reinterpret_cast<const float4*>(x);
-    float a[NR][4];
+// words that carry a value and the number of its meeting
+__device__ __forceinline__ unsigned long long lz_pack(uint32_t v, uint32_t tag) { return ((unsigned long long)tag << 32) | v; }
+__device__ __forceinline__ void lz_store(unsigned long long* p, unsigned long long w) {
+  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+__device__ __forceinline__ void lz_store2(unsigned long long* p, double d, uint32_t tag) {
+  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};"
+               ::"l"(p), "l"(lz_pack((uint32_t)__double2loint(d), tag)), "l"(lz_pack((uint32_t)__double2hiint(d), tag)) : "memory");
+}
+__device__ __forceinline__ void lz_load2(const unsigned long long* p, unsigned long long& a, unsigned long long& b) {
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
+__device__ __forceinline__ bool lz_tagged(unsigned long long w, uint32_t tag) { return (uint32_t)(w >> 32) == tag; }
+__device__ __forceinline__ double lz_double(unsigned long long a, unsigned long long b) { return __hiloint2double((int)(uint32_t)b, (int)(uint32_t)a); }
+__device__ __forceinline__ double half_sum(double v) {      // over the 16 lanes of a half-warp
 #pragma unroll
-    for (int q = 0; q < NR; ++q)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) a[q][j] = 0.f;
-    const int n4 = n / 4;
-    constexpr int U = NR >= 4 ? 2 : 4;          // 16-byte loads of every row in flight per lane
-    int i = lane;
-    for (; i + 32 * (U - 1) < n4; i += 32 * U) {
-      float4 r[NR][U];
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int q = 0; q < NR; ++q) r[q][u] = reinterpret_cast<const float4*>(row[q])[i + 32 * u];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const float4 v = x4[i + 32 * u];
-#pragma unroll
-        for (int q = 0; q < NR; ++q) {
-          a[q][0] = fmaf(r[q][u].x, v.x, a[q][0]); a[q][1] = fmaf(r[q][u].y, v.y, a[q][1]);
-          a[q][2] = fmaf(r[q][u].z, v.z, a[q][2]); a[q][3] = fmaf(r[q][u].w, v.w, a[q][3]);
-        }
-      }
-    }
-    for (; i < n4; i += 32) {
-      const float4 v = x4[i];
-#pragma unroll
-      for (int q = 0; q < NR; ++q) {
-        const float4 r = reinterpret_cast<const float4*>(row[q])[i];
-        a[q][0] = fmaf(r.x, v.x, a[q][0]); a[q][1] = fmaf(r.y, v.y, a[q][1]);
-        a[q][2] = fmaf(r.z, v.z, a[q][2]); a[q][3] = fmaf(r.w, v.w, a[q][3]);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < NR; ++q) acc[q] = (a[q][0] + a[q][1]) + (a[q][2] + a[q][3]);
-  } else {
-#pragma unroll
-    for (int q = 0; q < NR; ++q) acc[q] = 0.f;
-#pragma unroll 4
-    for (int i = lane; i < n; i += 32) {
-      const float v = x[i];
-#pragma unroll
-      for (int q = 0; q < NR; ++q) acc[q] = fmaf(row[q][i], v, acc[q]);
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < NR; ++q) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
-    out[q] = acc[q];
-  }
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
-// shared memory of CTA `rank` of the cluster at the place of `p` in this one's
-template <typename T>
-__device__ __forceinline__ uint32_t peer_smem(const T* p, int rank) {
-  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void peer_store(uint32_t a, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
-__device__ __forceinline__ void peer_store(uint32_t a, double v) { asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory"); }
-__device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+// limit of one wait, looked at every 256 polls
+struct LzLimit {
+  unsigned int polls = 0;
+  unsigned long long t0 = 0;
+  __device__ __noinline__ bool late(const LanczosRun& p) {
+    unsigned long long now;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
+    if (t0 == 0) { t0 = now; return false; }
+    if (now - t0 <= p.wait_ns) return false;
+    atomicOr(p.wait_status, DEFL_ST_DEVICE_WAIT);
+    return true;
+  }
+  __device__ __forceinline__ bool over(const LanczosRun& p) { return (++polls & 255u) == 0 && late(p); }
+};
+// a double under `tag`, polled by the calling thread
+__device__ __forceinline__ double lz_wait_double(const unsigned long long* w, uint32_t tag, const LanczosRun& p, bool& ok) {
+  unsigned long long a, b;
+  LzLimit limit;
+  while (true) {
+    lz_load2(w, a, b);
+    if (lz_tagged(a, tag) && lz_tagged(b, tag)) break;
+    if (limit.over(p)) { ok = false; break; }
+  }
+  return lz_double(a, b);
 }
 
-template <bool CLUSTER>
-__global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const LanczosRun p) {
-  pdl_wait();
+template <int P>      // quads of columns per thread
+__global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const __grid_constant__ LanczosRun p) {
   extern __shared__ __align__(16) float lz[];
   constexpr int MS = DEFL_LANCZOS_STEPS;
-  const int n = p.n, steps = p.steps, R = p.rows, G = gridDim.x, blk = blockIdx.x;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n = p.n, ns = (n + 3) & ~3, steps = p.steps, R = p.rows, Rc = (R + LZ_ROWS - 1) / LZ_ROWS * LZ_ROWS, G = gridDim.x, blk = blockIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, half = tid >> 4, hl = tid & 15;
   const int first = blk * R, mine = max(0, min(R, n - first));      // this CTA's rows
-  const int np = (n + 3) & ~3;
-  float* xq = lz;                             // [n] the vector being multiplied: q_j (or v), then t
-  float* xt = CLUSTER ? xq + np : xq;         // (the cluster form's CTAs write into each other's: two buffers)
-  float* wl = xt + np;                        // [R] own slice of w (or t)
-  float* Qs = wl + ((R + 3) & ~3);            // [steps][R] own slices of the basis
-  float* As = Qs + (((long long)MS * R + 3) & ~3);  // [resident][n] own rows of A
-  __shared__ double red[LZ_WARPS], tot, coef[MS], al[MS], be[MS], y[MS];
-  __shared__ double cpart[2][CLUSTER ? LZ_CLUSTER : 1][CLUSTER ? LZ_PW : 1];     // cluster form: everybody's partial sums
-  __shared__ double rho_s;
-  __shared__ int alive;
-  unsigned int epoch = 0;
-  const bool vec = (n & 3) == 0 && p.aligned;
+  float* As = lz;                             // [resident][ns] own rows of A
+  float* wl = As + (long long)p.resident * ns;      // [R] own slice of w (or t)
+  float* Qs = wl + R;                         // [steps][R] own slices of the basis
+  float* Ts = Qs + MS * R;                    // [steps][R] own slices of A Q
+  float* red = Ts + MS * R;                   // [warps][Rc] sums over a warp's columns
+  __shared__ double start[LZ_WARPS], before2, pd[LZ_PB], coef[2][LZ_PB], al[MS], be[MS], y[MS];
+  __shared__ double stash[LZ_PB][LZ_DIRECT + 1], share[LZ_MAX_GRID];
+  __shared__ TridiagScratch tri;
+  float x[P][4];                              // the vector being multiplied: columns 4 i .. 4 i + 3 for i = tid + 512 m
+  int at[P];                                  // where those columns stand in a vector's messages
 
-  {
-    const float* src = p.A + (long long)first * n;
-    const int count = min(p.resident, mine) * n;
-    if (vec) {
+  for (int r = warp; r < min(p.resident, mine); r += LZ_WARPS) {
+    const float* src = p.A + (long long)(first + r) * n;
+    float* dst = As + (long long)r * ns;
+    if (p.aligned) {
 #pragma unroll 8
-      for (int e = tid; e < count / 4; e += LZ_THREADS) reinterpret_cast<float4*>(As)[e] = __ldg(reinterpret_cast<const float4*>(src) + e);
+      for (int i = lane; i < n / 4; i += 32) reinterpret_cast<float4*>(dst)[i] = __ldg(reinterpret_cast<const float4*>(src) + i);
     } else {
 #pragma unroll 8
-      for (int e = tid; e < count; e += LZ_THREADS) As[e] = __ldg(src + e);
+      for (int i = lane; i < ns; i += 32) dst[i] = i < n ? __ldg(src + i) : 0.f;
     }
   }
   if (tid < MS) { al[tid] = 0.0; be[tid] = 0.0; }
-  if (tid == 0) alive = 1;
   // (a wait that runs out returns from the middle: the scale is then zero, not what an earlier call left there)
   if (blk == 0 && tid == 0) { p.theta[0] = 0.f; p.inv_theta[0] = 0.f; }
-  __syncthreads();
 
-  // All CTAs meet. Grid form: a counter with a time limit, false (everywhere in the CTA) when it ran out.
-  auto meet = [&]() -> bool {
-    if (CLUSTER) { cluster_barrier(); return true; }
-    __syncthreads();
-    ++epoch;
-    if (tid == 0) {
-      __threadfence();
-      atomicAdd(p.bar, 1u);
-      const unsigned int want = epoch * (unsigned int)G + p.hold;
-      unsigned long long t0 = 0;
-      for (unsigned int polls = 0;; ++polls) {
-        unsigned int v;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p.bar) : "memory");
-        if (v >= want) break;
-        if ((polls & 1023u) == 1023u) {
-          unsigned long long now;
-          asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
-          if (t0 == 0) t0 = now;
-          else if (now - t0 > p.wait_ns) { alive = 0; atomicOr(p.wait_status, DEFL_ST_DEVICE_WAIT); break; }
+  // own columns of the vector that all CTAs have published under `tag`; false when the wait ran out (for the calling thread)
+  auto gather = [&](int which, uint32_t tag) -> bool {
+    unsigned long long a[P][4];
+    LzLimit limit;
+    bool ok = true;
+    while (true) {
+      bool got = true;
+#pragma unroll
+      for (int m = 0; m < P; ++m) {
+        const int c = 4 * (tid + m * LZ_THREADS);
+        if (c < n) { lz_load2(p.vec[which] + at[m], a[m][0], a[m][1]); lz_load2(p.vec[which] + at[m] + 2, a[m][2], a[m][3]); }
+      }
+#pragma unroll
+      for (int m = 0; m < P; ++m) {
+        const int c = 4 * (tid + m * LZ_THREADS);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) if (c + u < n) got &= lz_tagged(a[m][u], tag);
+      }
+      if (got) break;
+      if (limit.over(p)) { ok = false; break; }
+    }
+#pragma unroll
+    for (int m = 0; m < P; ++m) {
+      const int c = 4 * (tid + m * LZ_THREADS);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[m][u] = (c + u < n) ? __uint_as_float((uint32_t)a[m][u]) : 0.f;
+    }
+    return ok;
+  };
+  // the own slice in wl to everybody, by one warp
+  auto publish = [&](int which, uint32_t tag) {
+    for (int r = lane; r < mine; r += 32) lz_store(p.vec[which] + (size_t)blk * p.block + r, lz_pack(__float_as_uint(wl[r]), tag));
+  };
+  // the partial sums pd[0 .. j] to whoever adds them up, by one warp; afterwards coef[set] = their sums over the CTAs, in a
+  // fixed order. Up to LZ_DIRECT CTAs everybody adds up everybody's; above it CTA q adds up those of sum q for all.
+  auto give = [&](int set, int j, uint32_t tag) {
+    if (lane <= j) lz_store2(p.part + ((size_t)(set * G + blk) * LZ_PB + lane) * 2, pd[lane], tag);
+  };
+  auto total = [&](int set, int j, uint32_t tag, bool ok) -> bool {
+    if (G <= LZ_DIRECT) {
+      constexpr int U = LZ_DIRECT * LZ_PB / LZ_THREADS;
+      unsigned long long a[U], b[U];
+      LzLimit limit;
+      while (true) {
+        bool got = true;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int e = tid + u * LZ_THREADS;
+          if (e < G * LZ_PB && e % LZ_PB <= j) lz_load2(p.part + ((size_t)set * G * LZ_PB + e) * 2, a[u], b[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int e = tid + u * LZ_THREADS;
+          if (e < G * LZ_PB && e % LZ_PB <= j) got &= lz_tagged(a[u], tag) && lz_tagged(b[u], tag);
+        }
+        if (got) break;
+        if (limit.over(p)) { ok = false; break; }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int e = tid + u * LZ_THREADS;
+        if (e < G * LZ_PB && e % LZ_PB <= j) stash[e % LZ_PB][e / LZ_PB] = lz_double(a[u], b[u]);
+      }
+      if (!__syncthreads_and(ok)) return false;
+      if (half < LZ_PB) {
+        double d = 0.0;
+        if (half <= j) {
+#pragma unroll
+          for (int u = 0; u < LZ_DIRECT / 16; ++u) if (hl + 16 * u < G) d += stash[half][hl + 16 * u];
+        }
+        d = half_sum(d);
+        if (hl == 0) coef[set][half] = d;
+      }
+      __syncthreads();
+      return true;
+    }
+    if (blk <= j) {                           // (uniform in the block; G > LZ_DIRECT >= LZ_PB CTAs)
+      if (tid < G) share[tid] = lz_wait_double(p.part + ((size_t)(set * G + tid) * LZ_PB + blk) * 2, tag, p, ok);
+      if (!__syncthreads_and(ok)) return false;
+      if (warp == 0) {
+        double d = 0.0;
+        for (int g = lane; g < G; g += 32) d += share[g];
+        d = lz_warp_sum(d);
+        if (lane == 0) lz_store2(p.sum + (size_t)(set * LZ_PB + blk) * LZ_LINE, d, tag);
+      }
+    }
+    if (tid <= j) coef[set][tid] = lz_wait_double(p.sum + (size_t)(set * LZ_PB + tid) * LZ_LINE, tag, p, ok);
+    return __syncthreads_and(ok);
+  };
+  // red[warp][r] = sum over the warp's columns of A[row r] x, for all own rows, eight rows at a time
+  auto multiply = [&]() {
+    for (int r0 = 0; r0 < mine; r0 += LZ_ROWS) {
+      float acc[LZ_ROWS];
+#pragma unroll
+      for (int q = 0; q < LZ_ROWS; ++q) acc[q] = 0.f;
+#pragma unroll
+      for (int m = 0; m < P; ++m) {
+        const int i = tid + m * LZ_THREADS;
+        if (4 * i >= n) continue;
+        float4 v[LZ_ROWS];
+        if (r0 + LZ_ROWS <= p.resident || p.resident >= mine) {
+#pragma unroll
+          for (int q = 0; q < LZ_ROWS; ++q) v[q] = reinterpret_cast<const float4*>(As + (long long)min(r0 + q, mine - 1) * ns)[i];
+        } else if (p.aligned && r0 >= p.resident) {
+#pragma unroll
+          for (int q = 0; q < LZ_ROWS; ++q) v[q] = __ldg(reinterpret_cast<const float4*>(p.A + (long long)(first + min(r0 + q, mine - 1)) * n) + i);
+        } else {                              // both kinds of rows, or rows at any address
+#pragma unroll
+          for (int q = 0; q < LZ_ROWS; ++q) {
+            const int r = min(r0 + q, mine - 1);
+            const float* row = (r < p.resident ? As + (long long)r * ns : p.A + (long long)(first + r) * n) + 4 * i;
+            if (p.aligned) v[q] = *reinterpret_cast<const float4*>(row);
+            else {
+              v[q].x = row[0]; v[q].y = 4 * i + 1 < n ? row[1] : 0.f;
+              v[q].z = 4 * i + 2 < n ? row[2] : 0.f; v[q].w = 4 * i + 3 < n ? row[3] : 0.f;
+            }
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < LZ_ROWS; ++q) {
+          acc[q] = fmaf(v[q].x, x[m][0], acc[q]); acc[q] = fmaf(v[q].y, x[m][1], acc[q]);
+          acc[q] = fmaf(v[q].z, x[m][2], acc[q]); acc[q] = fmaf(v[q].w, x[m][3], acc[q]);
         }
       }
-      __threadfence();
-    }
-    __syncthreads();
-    return alive != 0;
-  };
-  // own slice of a vector to everybody: into their x buffer, or to global memory
-  auto publish = [&](float* x, float* v) {
-    if (CLUSTER) {
-      for (int e = tid; e < mine * G; e += LZ_THREADS) {
-        const int g = e / mine, r = e - g * mine;
-        peer_store(peer_smem(x + first + r, g), wl[r]);
-      }
-    } else {
-      for (int r = tid; r < mine; r += LZ_THREADS) v[first + r] = wl[r];
-    }
-  };
-  // x <- the vector that all CTAs have published (grid form: through L2, the L1 may hold the previous one), times `scale`
-  auto stage = [&](float* x, const float* v, float scale) {
-    if (!CLUSTER || scale != 1.f) {
-      for (int i = tid; i < n; i += LZ_THREADS) x[i] = (CLUSTER ? x[i] : __ldcg(v + i)) * scale;
-      __syncthreads();
-    }
-  };
-  // (A x)[r] for the own rows, in wl
-  auto multiply = [&](const float* x) {
-    for (int r = warp; r < mine; r += 4 * LZ_WARPS) {
-      const float* row[4];
+      // eight sums over 32 lanes: every exchange halves the sums a lane carries, then the lanes of each
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int rr = r + q * LZ_WARPS;
-        row[q] = (rr < p.resident) ? As + (long long)rr * n : p.A + (long long)(first + (rr < mine ? rr : r)) * n;
-      }
-      float o[4];
-      if (r + LZ_WARPS >= mine) row_dots<1>(row, x, n, vec, lane, o);
-      else if (r + 2 * LZ_WARPS >= mine) row_dots<2>(row, x, n, vec, lane, o);
-      else row_dots<4>(row, x, n, vec, lane, o);
-      if (lane == 0) {
+      for (int h = 4; h > 0; h >>= 1) {
+        const bool up = (lane & (4 * h)) != 0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) if (r + q * LZ_WARPS < mine) wl[r + q * LZ_WARPS] = o[q];
+        for (int q = 0; q < h; ++q) {
+          const float keep = up ? acc[q + h] : acc[q], send = up ? acc[q] : acc[q + h];
+          acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * h);
+        }
       }
+      acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
+      acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+      if ((lane & 3) == 0) red[warp * Rc + r0 + (lane >> 2)] = acc[0];
     }
     __syncthreads();
   };
-  // one partial sum of this CTA (the same in every lane of the warp) to where everybody adds them up
-  auto give = [&](int set, int q, double d) {
-    if (CLUSTER) { if (lane < G) peer_store(peer_smem(&cpart[set][blk][q], lane), d); }
-    else if (lane == 0) p.part[((long long)set * G + blk) * LZ_PW + q] = d;
+  // for every own row, by a half-warp: f(row, sum over the warps (with_red) - Q_j coef (c, where given))
+  auto rows = [&](bool with_red, const double* c, int j, auto f) {
+    for (int r0 = 0; r0 < mine; r0 += LZ_HALVES) {
+      const int r = min(r0 + half, mine - 1);
+      double v = with_red ? (double)red[hl * Rc + r] : 0.0;
+      if (c) for (int q = hl; q <= j; q += 16) v = fma(-c[q], (double)Qs[q * R + r], v);
+      v = half_sum(v);
+      if (hl == 0 && r0 + half < mine) f(r, v);
+    }
+    __syncthreads();
   };
-  auto total = [&](int set, int q) -> double {     // sum over the CTAs by one warp, fixed order
+  // pd[q] = S_q . v over the own rows, q <= j
+  auto dots = [&](const float* S, const float* v, int j) {
+    const int q = min(half, j);
     double d = 0.0;
-    if (CLUSTER) { if (lane < G) d = cpart[set][lane][q]; }
-    else for (int g = lane; g < G; g += 32) d += __ldcg(p.part + ((long long)set * G + g) * LZ_PW + q);
-    return lz_warp_sum(d);
-  };
-  auto square = [&](int set) {          // this CTA's share of ||w||^2
-    if (warp == 0) {
-      double d = 0.0;
-      for (int r = lane; r < mine; r += 32) d += (double)wl[r] * (double)wl[r];
-      give(set, LZ_PW - 1, lz_warp_sum(d));
+    if (half == LZ_HALVES - 1) {              // (and ||w||^2 before its projections: all but the last few digits lie in Q_j)
+      for (int i = hl; i <= j; i += 16) d = fma(coef[0][i], coef[0][i], d);
+    } else {
+      for (int r = hl; r < mine; r += 16) d = fma((double)S[q * R + r], (double)v[r], d);
     }
+    d = half_sum(d);
+    if (half <= j && hl == 0) pd[half] = d;
+    if (half == LZ_HALVES - 1 && hl == 0) before2 = d;
+    __syncthreads();
   };
 
   // q_0
   double a = 0.0;
-  for (int i = tid; i < n; i += LZ_THREADS) { const float v = __ldg(p.v0 + i); xq[i] = v; a += (double)v * (double)v; }
+#pragma unroll
+  for (int m = 0; m < P; ++m) {
+    const int c = 4 * (tid + m * LZ_THREADS);
+    at[m] = c / R * p.block + c % R;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      x[m][u] = (c + u < n) ? __ldg(p.v0 + c + u) : 0.f;
+      a = fma((double)x[m][u], (double)x[m][u], a);
+    }
+  }
   a = lz_warp_sum(a);
-  if (lane == 0) red[warp] = a;
+  if (lane == 0) start[warp] = a;
   __syncthreads();
   double nv = 0.0;
-  for (int i = 0; i < LZ_WARPS; ++i) nv += red[i];
+  for (int i = 0; i < LZ_WARPS; ++i) nv += start[i];
   nv = sqrt(nv);
   const bool started = nv > 0.0;
-  for (int i = tid; i < n; i += LZ_THREADS) xq[i] = started ? (float)((double)xq[i] / nv) : 0.f;
-  __syncthreads();
-  for (int r = tid; r < mine; r += LZ_THREADS) Qs[r] = xq[first + r];
-  __syncthreads();
-  if (CLUSTER) cluster_barrier();             // nobody writes into a CTA that has not started
+  const double inv = started ? 1.0 / nv : 0.0;
+#pragma unroll
+  for (int m = 0; m < P; ++m)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[m][u] = (float)((double)x[m][u] * inv);
+  for (int r = tid; r < mine; r += LZ_THREADS) Qs[r] = (float)((double)__ldg(p.v0 + first + r) * inv);
 
+  int other = 1;
   for (int j = 0; started && j < steps; ++j) {
-    multiply(xq);                             // t = A q_j
-    publish(xt, p.t);
-    if (!meet()) return;
-    stage(xt, p.t, 1.f);
-    multiply(xt);                             // w = A t
-    // w -= Q_j (Q_j^T w), twice: the second projection is measured on what the first one left
-    bool last = false;
-    for (int pass = 0; pass < 2; ++pass) {
-      for (int q = warp; q <= j; q += LZ_WARPS) {
-        double d = 0.0;
-        for (int r = lane; r < mine; r += 32) d += (double)Qs[q * R + r] * (double)wl[r];
-        give(pass, q, lz_warp_sum(d));
+    const uint32_t tag = 4u * (uint32_t)j + 1u;
+    multiply();                               // t = A q_j
+    float* tj = Ts + j * R;
+    rows(true, nullptr, 0, [&](int r, double v) { wl[r] = tj[r] = (float)v; });
+    if (warp == LZ_WARPS - 1) publish(0, tag);
+    dots(Ts, tj, j);
+    if (warp == 0) give(0, j, tag);
+    const bool ok = gather(0, tag + (j == 0 ? p.hold : 0u));
+    multiply();                               // A t
+    if (!total(0, j, tag, ok)) return;
+    if (tid == 0) al[j] = coef[0][j];
+    if (j + 1 == steps) break;
+    rows(true, coef[0], j, [&](int r, double v) { wl[r] = (float)v; });
+    double b = 0.0, limit2 = 0.0;
+    for (uint32_t again = 0;; ++again) {
+      dots(Qs, wl, j);
+      if (warp == 0) give(1, j, tag + again);
+      if (!total(1, j, tag + again, true)) return;
+      rows(false, coef[1], j, [&](int r, double v) { wl[r] = (float)((double)wl[r] + v); });
+      if (warp == 0) {
+        publish(1, tag + again);
+        double d = 0.0;                       // this CTA's share of ||w||^2
+        for (int r = lane; r < mine; r += 32) d = fma((double)wl[r], (double)wl[r], d);
+        d = lz_warp_sum(d);
+        if (lane == 0) lz_store2(p.vec[1] + (size_t)blk * p.block + R, d, tag + again);
       }
-      if (!meet()) return;
-      for (int q = warp; q <= j; q += LZ_WARPS) {
-        const double d = total(pass, q);
-        if (lane == 0) coef[q] = d;
-      }
-      __syncthreads();
-      if (pass == 0) {
-        if (tid == 0) al[j] = coef[j];
-        if (j + 1 == steps) { last = true; break; }
-      }
-      for (int r = tid; r < mine; r += LZ_THREADS) {
-        double v = (double)wl[r];
-        for (int q = 0; q <= j; ++q) v = fma(-coef[q], (double)Qs[q * R + r], v);
-        wl[r] = (float)v;
-      }
-      __syncthreads();
+      bool got = gather(1, tag + again);
+      if (tid < G) share[tid] = lz_wait_double(p.vec[1] + (size_t)tid * p.block + R, tag + again, p, got);
+      if (!__syncthreads_and(got)) return;
+      double b2 = 0.0;
+      for (int g = lane; g < G; g += 32) b2 += share[g];
+      b2 = lz_warp_sum(b2);                   // (the same in every warp)
+      b = sqrt(b2);
+      if (again == 0) limit2 = 1e-10 * before2;
+      if (again == 2 || !(b2 < limit2)) break;
+      limit2 = 1e-10 * b2;
     }
-    if (last) break;
-    square(1);
-    publish(xq, p.w);
-    if (!meet()) return;
-    if (warp == 0) { const double d = total(1, LZ_PW - 1); if (lane == 0) tot = sqrt(d); }
-    __syncthreads();
-    const double b = tot;
-    if (!(b > 1e-12 * fabs(al[0]))) break;    // the Krylov space ends here (the same decision in every CTA)
+    if (!(b > 1e-12 * fabs(al[0]))) { other = 0; break; }      // the Krylov space ends here (the same decision in every CTA)
     if (tid == 0) be[j] = b;
-    stage(xq, p.w, (float)(1.0 / b));
-    for (int r = tid; r < mine; r += LZ_THREADS) Qs[(j + 1) * R + r] = xq[first + r];
-    __syncthreads();
+    const float ib = (float)(1.0 / b);
+#pragma unroll
+    for (int m = 0; m < P; ++m)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[m][u] *= ib;
+    for (int r = tid; r < mine; r += LZ_THREADS) Qs[(j + 1) * R + r] = wl[r] * ib;
   }
   __syncthreads();
 
   // largest Ritz pair (rho, v), theta = sqrt(max(rho, 0) + ||A A v - rho v||)
-  if (warp == 0) {
-    const double lam = tridiag_top(al, be, steps, y);
-    if (lane == 0) rho_s = (double)(float)lam;
-  }
-  __syncthreads();
+  const double rho = (double)(float)tridiag_top(al, be, steps, y, tri);
+  const uint32_t end = 4u * (uint32_t)steps + 1u;
+  // (others may still be reading the words of the meeting that the loop was left after: t's, or w's after a breakdown. The
+  // other vector's words are free.)
+  float* vs = Ts;                             // own slice of v
   for (int r = tid; r < mine; r += LZ_THREADS) {
     double v = 0.0;
     for (int q = 0; q < steps; ++q) if (y[q] != 0.0) v += (double)(float)y[q] * (double)Qs[q * R + r];
-    wl[r] = (float)v;
-    Qs[r] = (float)v;                         // (row 0 is this thread's own to overwrite now)
+    vs[r] = wl[r] = (float)v;
   }
-  if (CLUSTER) cluster_barrier(); else __syncthreads();     // (the last x_q may still be read by a slower CTA)
-  publish(xq, p.w);
-  if (!meet()) return;
-  stage(xq, p.w, 1.f);
-  multiply(xq);
-  publish(xt, p.t);
-  if (!meet()) return;
-  stage(xt, p.t, 1.f);
-  multiply(xt);
-  const double rho = rho_s;
-  for (int r = tid; r < mine; r += LZ_THREADS) wl[r] = (float)((double)wl[r] - rho * (double)Qs[r]);
   __syncthreads();
-  square(0);
-  if (!meet()) return;                        // (the last access to another CTA's shared memory lies before this)
-  if (blk == 0 && warp == 0) {
-    const double d = sqrt(total(0, LZ_PW - 1));
+  if (warp == 0) publish(other, end);
+  if (!__syncthreads_and(gather(other, end))) return;
+  multiply();
+  rows(true, nullptr, 0, [&](int r, double v) { wl[r] = (float)v; });
+  if (warp == 0) publish(other ^ 1, end);
+  if (!__syncthreads_and(gather(other ^ 1, end))) return;
+  multiply();
+  rows(true, nullptr, 0, [&](int r, double v) { wl[r] = (float)(v - rho * (double)vs[r]); });
+  if (warp == 0) {
+    double d = 0.0;
+    for (int r = lane; r < mine; r += 32) d = fma((double)wl[r], (double)wl[r], d);
+    d = lz_warp_sum(d);
+    if (lane == 0) lz_store2(p.part + (size_t)blk * LZ_PB * 2, d, end);       // (everybody is past the projections)
+  }
+  if (blk == 0) {
+    bool ok = true;
+    if (tid < G) share[tid] = lz_wait_double(p.part + (size_t)tid * LZ_PB * 2, end, p, ok);
+    if (!__syncthreads_and(ok) || warp != 0) return;
+    double d = 0.0;
+    for (int g = lane; g < G; g += 32) d += share[g];
+    d = sqrt(lz_warp_sum(d));
     if (lane == 0) {
       const double th = sqrt((rho > 0.0 ? rho : 0.0) + d);
-      const bool ok = th > 0.0 && isfinite(th);
+      const bool good = th > 0.0 && isfinite(th);
       p.theta[0] = (float)th;
-      p.inv_theta[0] = ok ? (float)(1.0 / th) : 0.f;
-      if (!ok && p.status) atomicOr(p.status, 4);
+      p.inv_theta[0] = good ? (float)(1.0 / th) : 0.f;
+      if (!good && p.status) atomicOr(p.status, 4);
     }
   }
 }
 
-constexpr size_t LZ_SMEM = 210 * 1024;        // dynamic shared memory at most (static shared memory comes on top)
+constexpr size_t LZ_SMEM = 205 * 1024;        // dynamic shared memory at most (static shared memory comes on top)
 
 cudaError_t psd_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(lanczos_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LZ_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(lanczos_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(lanczos_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LZ_SMEM);
-  return e;
+  const void* forms[] = {(const void*)lanczos_kernel<1>, (const void*)lanczos_kernel<2>, (const void*)lanczos_kernel<LZ_QUADS>};
+  for (const void* f : forms) {
+    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LZ_SMEM);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
-// Launches it, or returns false (nothing launched) where a CTA cannot hold its vectors or the device cannot hold the grid.
-static bool lanczos_launch(defl_ctx* c, const float* A, const float* start, int n, int steps, float* t, float* w, double* part,
-                           unsigned int* bar, float* theta, float* inv_theta, int* status, cudaError_t* err) {
+// words of the exchange: two vectors (what a grid of CTAs adds to n values: three rows to a multiple of four, the share of
+// the norm, and the rest of a line each), the sums, and two sets of partial sums
+static size_t lanczos_words(int n) {
+  return 2 * ((size_t)n + (size_t)LZ_MAX_GRID * (2 * LZ_LINE + 4)) + (size_t)2 * LZ_PB * LZ_LINE + (size_t)2 * LZ_MAX_GRID * LZ_PB * 2;
+}
+
+// Launches it, or returns false (nothing launched) where a thread cannot hold its columns or the device cannot hold the grid.
+static bool lanczos_launch(defl_ctx* c, const float* A, const float* start, int n, int steps, unsigned long long* words,
+                           float* theta, float* inv_theta, int* status, cudaError_t* err) {
   *err = cudaSuccess;
+  if (n > 4 * LZ_THREADS * LZ_QUADS) return false;
   LanczosRun p;
   memset(&p, 0, sizeof(p));
-  p.A = A; p.v0 = start; p.n = n; p.steps = steps; p.t = t; p.w = w; p.part = part; p.bar = bar;
-  p.aligned = (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+  p.A = A; p.v0 = start; p.n = n; p.steps = steps;
+  p.aligned = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
   p.wait_status = c->wait_status;
   p.wait_ns = (unsigned long long)(c->tc_knobs.wait_ms > 0 ? c->tc_knobs.wait_ms : 2000) * 1000000ull;
-  p.hold = (unsigned int)c->knobs.lanczos_hold;
+  p.hold = (unsigned int)c->knobs.lanczos_hold << 20;
   p.theta = theta; p.inv_theta = inv_theta; p.status = status;
-  // rows per CTA, resident rows and shared memory of a form; 0 = does not fit
-  auto layout = [&](int grid, int vectors) -> size_t {
-    p.rows = (n + grid - 1) / grid;
-    const size_t fixed = sizeof(float) * ((size_t)vectors * ((n + 3) & ~3) + (size_t)((p.rows + 3) & ~3) +
-                                          (size_t)((DEFL_LANCZOS_STEPS * p.rows + 3) & ~3));
-    if (fixed > LZ_SMEM) return 0;
-    const size_t fit = (LZ_SMEM - fixed) / ((size_t)n * sizeof(float));
+  const int widest = c->num_sms < LZ_MAX_GRID ? c->num_sms : LZ_MAX_GRID;
+  int grid = (n + LZ_ROWS - 1) / LZ_ROWS;
+  if (grid > LZ_DIRECT) grid = LZ_DIRECT;
+  size_t fixed;
+  while (true) {
+    if (grid > widest) grid = widest;
+    p.rows = ((n + grid - 1) / grid + 3) & ~3;
+    fixed = sizeof(float) * ((size_t)(1 + 2 * DEFL_LANCZOS_STEPS) * p.rows + (size_t)LZ_WARPS * ((p.rows + LZ_ROWS - 1) / LZ_ROWS * LZ_ROWS));
+    const size_t fit = fixed > LZ_SMEM ? 0 : (LZ_SMEM - fixed) / (((size_t)(n + 3) & ~(size_t)3) * sizeof(float));
     p.resident = fit < (size_t)p.rows ? (int)fit : p.rows;
-    return fixed + (size_t)p.resident * n * sizeof(float);
-  };
-  if (n <= LZ_CLUSTER_N && c->knobs.lanczos_form == 0) {
-    const size_t smem = layout(LZ_CLUSTER, 2);
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cudaLaunchAttribute attr[2];
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = LZ_CLUSTER; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(LZ_CLUSTER, 1, 1); cfg.blockDim = dim3(LZ_THREADS, 1, 1); cfg.dynamicSmemBytes = smem; cfg.stream = c->stream;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    int clusters = 0;
-    if (smem > 0 && cudaOccupancyMaxActiveClusters(&clusters, lanczos_kernel<true>, &cfg) == cudaSuccess && clusters > 0) {
-      cfg.numAttrs = 2;
-      *err = cudaLaunchKernelEx(&cfg, lanczos_kernel<true>, p);
-      ++c->launches;
-      return true;
-    }
-    cudaGetLastError();
+    // (all SMs where fewer of them cannot hold the matrix)
+    if (p.resident == p.rows || grid == widest) break;
+    grid = widest;
   }
-  // one CTA per SM at most, at least a row per warp
-  int grid = (n + LZ_WARPS - 1) / LZ_WARPS;
-  if (grid > c->num_sms) grid = c->num_sms;
-  if (grid > LZ_MAX_GRID) grid = LZ_MAX_GRID;
-  const size_t smem = layout(grid, 1);
-  if (smem == 0) return false;
+  if (fixed > LZ_SMEM) return false;
   grid = (n + p.rows - 1) / p.rows;
-  if ((*err = cudaMemsetAsync(bar, 0, sizeof(unsigned int), c->stream)) != cudaSuccess) return true;
+  p.block = (p.rows + 2 + LZ_LINE - 1) / LZ_LINE * LZ_LINE;
+  p.vec[0] = words; p.vec[1] = words + (size_t)grid * p.block;
+  p.sum = p.vec[1] + (size_t)grid * p.block; p.part = p.sum + 2 * LZ_PB * LZ_LINE;
+  const size_t smem = fixed + (size_t)p.resident * ((n + 3) & ~3) * sizeof(float);
+  if ((*err = cudaMemsetAsync(words, 0, lanczos_words(n) * sizeof(unsigned long long), c->stream)) != cudaSuccess) return true;
   void* args[] = {&p};
-  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)lanczos_kernel<false>, dim3(grid), dim3(LZ_THREADS), args, smem, c->stream);
+  const int quads = (n + 4 * LZ_THREADS - 1) / (4 * LZ_THREADS);
+  const void* form = quads <= 1 ? (const void*)lanczos_kernel<1> : quads <= 2 ? (const void*)lanczos_kernel<2> : (const void*)lanczos_kernel<LZ_QUADS>;
+  // (cooperative: all CTAs are resident at once or the launch is refused)
+  const cudaError_t e = cudaLaunchCooperativeKernel(form, dim3(grid), dim3(LZ_THREADS), args, smem, c->stream);
   if (e == cudaErrorCooperativeLaunchTooLarge) { cudaGetLastError(); return false; }
   ++c->launches;
   *err = e;
@@ -837,7 +949,7 @@ struct PsdWs {
   float* Rinv; float* E; float* Es; float* lam; float* coef;   // [K,K] x3, [K], [K]
   float* Q; double* T; float* lw; float* lt; float* lv; float* lE; float* lrho;   // Lanczos state
   int* done; double* beta_prev;
-  double* lpart; unsigned int* lbar;   // partial sums and barrier counter of the one-launch estimate
+  unsigned long long* lwords;   // what the CTAs of the one-launch estimate exchange
   double* npart; float* theta; float* inv_theta; float* dummy; float* rscale;
   int* status;
   int* keff;        // [1] size of the deflated set (gate)
@@ -872,7 +984,7 @@ static PsdWs carve_psd(void* base, int n, int K) {
   w.lw = cv.take<float>(n); w.lt = cv.take<float>(n); w.lv = cv.take<float>(n);
   w.lE = cv.take<float>(S * S); w.lrho = cv.take<float>(S);
   w.done = cv.take<int>(1); w.beta_prev = cv.take<double>(1);
-  w.lpart = cv.take<double>((size_t)2 * LZ_MAX_GRID * LZ_PW); w.lbar = cv.take<unsigned int>(1);
+  w.lwords = cv.take<unsigned long long>(lanczos_words(n));
   w.npart = cv.take<double>(1184);
   w.theta = cv.take<float>(1); w.inv_theta = cv.take<float>(1); w.dummy = cv.take<float>(S * S); w.rscale = cv.take<float>(1);
   w.status = cv.take<int>(1);
@@ -894,15 +1006,14 @@ static int estimate_scale(defl_ctx* c, const float* A, int n, int norm_mode, con
   }
   int steps = DEFL_LANCZOS_STEPS;
   if (steps > n) steps = n;
-  // One launch per step. The whole estimate in one launch (form 1) is faster (n = 1024: 265 against 420 us), but its second
-  // projection was wrong on matrices of low rank, and as mended it has not been measured: it is not the default.
-  if (c->knobs.lanczos_form == 1) {
+  if (c->knobs.lanczos_form != 2) {
     cudaError_t e;
-    if (lanczos_launch(c, A, start, n, steps, w.lt, w.lw, w.lpart, w.lbar, w.theta, w.inv_theta, w.status, &e)) {
+    if (lanczos_launch(c, A, start, n, steps, w.lwords, w.theta, w.inv_theta, w.status, &e)) {
       if (ctx_fail(c, e, "scale estimate")) return DEFL_ERR_CUDA;
       return DEFL_OK;
     }
   }
+  // one launch per step: n above 8192
   LanczosState s;
   s.Q = w.Q; s.T = w.T; s.w = w.lw; s.t = w.lt; s.done = w.done; s.beta_prev = w.beta_prev;
   launch_kernel(lanczos_init_kernel, 1, 1024, 0, c->stream, start, n, steps, s);
@@ -916,7 +1027,7 @@ static int estimate_scale(defl_ctx* c, const float* A, int n, int norm_mode, con
     if (ctx_fail(c, cudaGetLastError(), "lanczos step")) return DEFL_ERR_CUDA;
   }
   // largest Ritz pair of the (zero-padded) tridiagonal matrix
-  launch_kernel(tridiag_top_kernel, 1, 32, 0, c->stream, w.T, steps, w.lrho, w.lE);
+  launch_kernel(tridiag_top_kernel, 1, 512, 0, c->stream, w.T, steps, w.lrho, w.lE);
   ++c->launches;
   if (ctx_fail(c, cudaGetLastError(), "ritz")) return DEFL_ERR_CUDA;
   launch_kernel(lanczos_ritz_kernel, (n + 255) / 256, 256, 0, c->stream, n, steps, w.Q, w.lE, w.lv);
