@@ -267,18 +267,6 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
@@ -306,6 +294,15 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr, uint32_t lbo_
 __device__ __forceinline__ uint64_t smem_desc_hi(uint32_t lbo_bytes, uint32_t sbo_bytes) {
   return make_smem_desc(0, lbo_bytes, sbo_bytes);
 }
+
+// the values are in registers here, whatever the compiler would have preferred
+__device__ __forceinline__ void touch1(float v) { asm volatile("" ::"f"(v)); }
+__device__ __forceinline__ void touch1(int v) { asm volatile("" ::"r"(v)); }
+__device__ __forceinline__ void touch1(uint32_t v) { asm volatile("" ::"r"(v)); }
+__device__ __forceinline__ void touch1(long long v) { asm volatile("" ::"l"(v)); }
+__device__ __forceinline__ void touch1(const void* v) { asm volatile("" ::"l"(v)); }
+template <typename... T>
+__device__ __forceinline__ void touch(T... v) { (touch1(v), ...); }
 
 // ----------------------------------------------------------------------------- the kernel
 // Tile geometry. tile_m = 128: one 128-row accumulator per tile, two accumulator buffers (the epilogue
@@ -510,36 +507,24 @@ __device__ __forceinline__ void aux_fetch_async(const TcParams& p, int lane, int
   cp_async_commit();
 }
 
-// Transposed store of one 32 x 32 block of 16-bit results (EPI_STORE): C[(gj0 + c) * ldc + gi_warp0 + r] = alpha acc[r][c].
-// Each lane packs its row into 16 words of two columns, trades words with its neighbour lane so that a word holds
-// two ROWS of one column, and writes it into the staging buffer laid out as the transposed block (32 columns x 64
-// bytes, conflict-free); the block then leaves in 64-byte rows, 16 bytes per lane. A third of the instructions of
-// gathering the transposed block element by element out of a row-major staging buffer. (Writing the block with one
-// 2-byte store per lane and column instead, 64 contiguous bytes per warp instruction and no staging, takes the same
-// 1.48 ms for the 48 x 1600 x 6400 apply product under the board's power cap: the epilogue is not what bounds it.)
-template <bool F16O>
-__device__ __forceinline__ void store_block_transposed16(const TcParams& p, const uint32_t* r, uint8_t* stg, int lane,
-                                                         int gi_warp0, int gj0, int bz, float alpha) {
-  uint32_t* T = reinterpret_cast<uint32_t*>(stg);          // [32 columns][16 words]
-  const bool odd = (lane & 1) != 0;
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const uint32_t w = pack16x2(alpha * __uint_as_float(r[2 * j]), alpha * __uint_as_float(r[2 * j + 1]), F16O);
-    const uint32_t y = __shfl_xor_sync(0xffffffffu, w, 1);
-    // even lane: column 2j, rows (mine, neighbour's); odd lane: column 2j + 1, rows (neighbour's, mine)
-    const uint32_t word = odd ? __byte_perm(y, w, 0x7632) : __byte_perm(w, y, 0x5410);
-    T[(2 * j + (odd ? 1 : 0)) * 16 + (lane >> 1)] = word;
-  }
-  __syncwarp();
-  uint8_t* mbase = reinterpret_cast<uint8_t*>(p.C) + ((size_t)bz * p.batch_c + (size_t)gj0 * p.ldc + gi_warp0) * 2;
+// Transposed store of a staged 32 x 32 block of 16-bit results: C[(gj0 + c) * ldc + gi_warp0 + r] = block[r][c], the mirror
+// image of a symmetric output or a transposed one. Four transposing matrix loads (8 x 8 values each quarter): the row that a
+// lane points at is chosen so that its four result words are the eight consecutive rows 8 (lane & 3) .. + 7 of one column, i.e. 16
+// bytes of the output as they are stored, 64 bytes per output row and instruction; the key of the staging buffer keeps the eight
+// rows of a quarter on different banks. (Gathering the 32 values of a lane with 2-byte loads took 32 loads and 24 merges.)
+__device__ __forceinline__ void store_staged_transposed16(const TcParams& p, const uint8_t* stg, int lane, int gi_warp0, int gj0, int bz) {
+  const int i = lane >> 3, rho = lane & 7, row = 8 * (rho >> 1) + 2 * i + (rho & 1);
+  const uint32_t base = smem_u32(stg) + (uint32_t)row * 64u, key = (uint32_t)(((row >> 1) ^ (row >> 3)) & 3);
   uint4 q[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const uint4*>(stg + ((lane >> 2) + 8 * i) * 64 + (lane & 3) * 16);
-  uint8_t* mp = mbase + (size_t)(lane >> 2) * p.ldc * 2 + (lane & 3) * 16;
+  for (uint32_t j = 0; j < 4; ++j)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(q[j].x), "=r"(q[j].y), "=r"(q[j].z), "=r"(q[j].w) : "r"(base + ((j ^ key) << 4)) : "memory");
+  uint8_t* mp = reinterpret_cast<uint8_t*>(p.C) +
+                ((size_t)bz * p.batch_c + (size_t)(gj0 + (lane >> 2)) * p.ldc + gi_warp0 + 8 * (lane & 3)) * 2;
   const size_t mstep = (size_t)8 * p.ldc * 2;
 #pragma unroll
-  for (int i = 0; i < 4; ++i, mp += mstep) *reinterpret_cast<uint4*>(mp) = q[i];
-  __syncwarp();
+  for (int j = 0; j < 4; ++j, mp += mstep) *reinterpret_cast<uint4*>(mp) = q[j];
 }
 
 // The calling lane's row of one staged 32 x 32 block, 16 bytes at a time and in place: `aux` values in, results out
@@ -610,13 +595,6 @@ __device__ __forceinline__ void epilogue_block_fast(const TcParams& p, uint32_t 
     __syncwarp();
   }
   tmem_ld_wait();
-  if (EPI == EPI_STORE && ES == 2) {
-    if (p.transposed) {            // (warp-uniform)
-      if (p.out_f16) store_block_transposed16<true>(p, r, stg, lane, gi_warp0, gj0, bz, alpha);
-      else store_block_transposed16<false>(p, r, stg, lane, gi_warp0, gj0, bz, alpha);
-      return;
-    }
-  }
   const int gi = gi_warp0 + lane;
   // the formats of the two-byte types and the position of the diagonal are the same for the whole warp: one
   // branch per block selects a row loop without per-element tests
@@ -656,55 +634,86 @@ __device__ __forceinline__ void epilogue_block_fast(const TcParams& p, uint32_t 
   }
   // (a transposed output is written the way a symmetric one is mirrored)
   if (p.transposed || (p.symmetric && gj0 > gi_warp0)) {
-    // mirror image of a block above the diagonal (the caller guarantees 32 complete rows): transposed row c of the
-    // block is 32 values = pp pieces of 16 bytes; pp consecutive lanes write one such row, each lane gathering its
-    // epp values from one column of the staged block
-    uint8_t* mbase = reinterpret_cast<uint8_t*>(p.C) + ((size_t)bz * p.batch_c + (size_t)gj0 * p.ldc + gi_warp0) * ES;
-    uint4 qm[pp];
+    // mirror image of a block above the diagonal (the caller guarantees 32 complete rows)
+    if (ES == 2) {
+      store_staged_transposed16(p, stg, lane, gi_warp0, gj0, bz);
+    } else {
+      // transposed row c of the block is 32 values = pp pieces of 16 bytes; pp consecutive lanes write one such row, each lane
+      // gathering its epp values from one column of the staged block
+      uint8_t* mbase = reinterpret_cast<uint8_t*>(p.C) + ((size_t)bz * p.batch_c + (size_t)gj0 * p.ldc + gi_warp0) * ES;
+      uint4 qm[pp];
 #pragma unroll
-    for (int i = 0; i < pp; ++i) {
-      const int c = rpi * i + prow;                 // column of the block = row of the mirror image
-      const int cp = c / epp, ce = (c % epp) * ES;  // its piece and byte offset within a staged row
-      uint4& q = qm[i];
-      if (ES == 2) {
-        uint16_t h[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          h[e] = *reinterpret_cast<const uint16_t*>(stg + stage_off(piece * epp + e, cp, rowb, pp) + ce);
-        q = make_uint4((uint32_t)h[0] | ((uint32_t)h[1] << 16), (uint32_t)h[2] | ((uint32_t)h[3] << 16),
-                       (uint32_t)h[4] | ((uint32_t)h[5] << 16), (uint32_t)h[6] | ((uint32_t)h[7] << 16));
-      } else {
+      for (int i = 0; i < pp; ++i) {
+        const int c = rpi * i + prow;                 // column of the block = row of the mirror image
+        const int cp = c / epp, ce = (c % epp) * ES;  // its piece and byte offset within a staged row
         uint32_t w[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e)
           w[e] = *reinterpret_cast<const uint32_t*>(stg + stage_off(piece * epp + e, cp, rowb, pp) + ce);
-        q = make_uint4(w[0], w[1], w[2], w[3]);
+        qm[i] = make_uint4(w[0], w[1], w[2], w[3]);
       }
-    }
-    uint8_t* mp = mbase + (size_t)prow * p.ldc * ES + piece * 16;
-    const size_t mstep = (size_t)rpi * p.ldc * ES;
+      uint8_t* mp = mbase + (size_t)prow * p.ldc * ES + piece * 16;
+      const size_t mstep = (size_t)rpi * p.ldc * ES;
 #pragma unroll
-    for (int i = 0; i < pp; ++i, mp += mstep) *reinterpret_cast<uint4*>(mp) = qm[i];
+      for (int i = 0; i < pp; ++i, mp += mstep) *reinterpret_cast<uint4*>(mp) = qm[i];
+    }
   }
   __syncwarp();
 }
 
+// Which of a warp's 32-column blocks take the coalesced path: the complete ones of aligned rows in matching types, from
+// `first` on below `lim`; `diag` is the block on the diagonal that does not (-1: none).
+// A symmetric output may be the product of two DIFFERENT symmetric matrices (the apply step of the symmetric
+// filter, the Horner steps of a polynomial in the Gram matrix), whose computed (i, j) and (j, i) differ in the last
+// bits. Off the diagonal the mirror store makes the pair equal; the 32 x 32 block ON the diagonal must do the same
+// element by element, or an iterate picks up an antisymmetric part that the symmetric filter doubles at every step:
+// it takes the general path.
+// (A product of a matrix with itself, X X^T or A A, computes (i, j) and (j, i) from the same terms in the same
+// order: its diagonal blocks are symmetric to the bit and stay on the coalesced path.)
+struct FastBlocks { int first, lim, diag; bool on; };
+template <int EPI>
+__device__ __forceinline__ FastBlocks fast_blocks(const TcParams& p, int gi_warp0, int col0, int n_eff, int wsel) {
+  FastBlocks f;
+  const bool a2 = (p.aux_dtype != F32), o2 = (p.out_dtype != F32);
+  // the coalesced path wants `aux` and the output in the same type (true of every product the library makes)
+  // (symmetric output: the mirror stores of the coalesced path assume 32 complete rows)
+  f.on = p.vec_ok != 0 && (EPI == EPI_STORE || EPI == EPI_RESID_NORM || a2 == o2) &&
+         (!p.symmetric || (gi_warp0 + 32 <= p.M && EPI != EPI_RESID_NORM)) && (!p.transposed || gi_warp0 + 32 <= p.M);
+  f.lim = min(p.N - col0, n_eff);
+  f.diag = -1;
+  if ((EPI == EPI_STORE || EPI == EPI_POLY) && p.symmetric && p.diag_exact && gi_warp0 >= col0 && gi_warp0 - col0 < f.lim &&
+      (((gi_warp0 - col0) >> 5) & 1) == wsel)
+    f.diag = gi_warp0 - col0;
+  f.first = wsel * 32;
+  if (!f.on) return f;
+  // symmetric output: nothing to do for blocks entirely left of the warp's rows (they are written as mirror images)
+  if (p.symmetric) while (f.first + 32 <= f.lim && col0 + f.first + 31 < gi_warp0) f.first += 64;
+  // (the block on the diagonal that is left to the general path is the first block of this walk)
+  if (f.first == f.diag) f.first += 64;
+  return f;
+}
+
+// fetches the first block of `aux` that the tile's epilogue will want; returns it (-1: none)
+template <int EPI>
+__device__ __forceinline__ int epilogue_ahead(const TcParams& p, int gi_warp0, int col0, int n_eff, int bz, int wsel, uint8_t* stg, int lane) {
+  const FastBlocks f = fast_blocks<EPI>(p, gi_warp0, col0, n_eff, wsel);
+  if (!f.on || f.first + 32 > f.lim) return -1;
+  if (p.aux_dtype != F32) aux_fetch_async<2>(p, lane, gi_warp0, col0 + f.first, bz, stg);
+  else aux_fetch_async<4>(p, lane, gi_warp0, col0 + f.first, bz, stg);
+  return f.first;
+}
+
 // the warp's complete 32-column blocks c0, c0 + 64, ... below `lim`; returns the first block not done. Two-byte
 // types: the 4 KB staging buffer holds two blocks, and the fetch of block i+1 is issued before block i is
-// processed. Four-byte types: one block at a time.
+// processed. Four-byte types: one block at a time. (`ahead`: the block that has been asked for before.)
 template <int EPI, int ES>
 __device__ __forceinline__ int epilogue_fast_blocks(const TcParams& p, uint32_t taddr, uint8_t* stg, int lane, int gi_warp0,
                                                     int col0, int c0, int lim, int bz, float alpha, float aux_scale,
-                                                    float& sq, int skip_c) {
+                                                    float& sq, int ahead) {
   constexpr bool AHEAD = (ES == 2) && (EPI != EPI_STORE);
   int half = 0;
-  // symmetric output: nothing to do for blocks entirely left of the warp's rows (they are written as mirror images)
-  if (p.symmetric) while (c0 + 32 <= lim && col0 + c0 + 31 < gi_warp0) c0 += 64;
-  // (the block on the diagonal of a plain symmetric store is left to the caller: see epilogue_half; it is the first
-  // block of this walk when it belongs to this warp)
-  if (c0 == skip_c) c0 += 64;
   __syncwarp();
-  if (AHEAD && c0 + 32 <= lim) aux_fetch_async<ES>(p, lane, gi_warp0, col0 + c0, bz, stg);
+  if (AHEAD && c0 + 32 <= lim && ahead != c0) aux_fetch_async<ES>(p, lane, gi_warp0, col0 + c0, bz, stg);
 #pragma unroll 1
   for (; c0 + 32 <= lim; c0 += 64) {
     uint8_t* cur = stg + (AHEAD ? half * (STAGING_BYTES / 2) : 0);
@@ -717,7 +726,7 @@ __device__ __forceinline__ int epilogue_fast_blocks(const TcParams& p, uint32_t 
       }
       half ^= 1;
     } else {
-      if (EPI != EPI_STORE) aux_fetch_async<ES>(p, lane, gi_warp0, col0 + c0, bz, cur);
+      if (EPI != EPI_STORE && ahead != c0) aux_fetch_async<ES>(p, lane, gi_warp0, col0 + c0, bz, cur);
       epilogue_block_fast<EPI, ES, 0>(p, taddr + (uint32_t)c0, cur, lane, gi_warp0, col0 + c0, bz, alpha, aux_scale, sq);
     }
   }
@@ -751,40 +760,22 @@ __device__ __forceinline__ void epilogue_block_general(const TcParams& p, uint32
 template <int EPI>
 __device__ __forceinline__ void epilogue_half(const TcParams& p, uint32_t taddr, int gi, int gi_warp0, int col0, int n_eff,
                                               int bz, int wsel, float alpha, float aux_scale, float& sq, uint8_t* stg,
-                                              int lane) {
+                                              int lane, int ahead) {
   const bool row_ok = gi < p.M;
   const bool aux_bf16 = (p.aux_dtype != F32);       // a 16-bit aux type
   const size_t cbatch = (size_t)bz * p.batch_c;
   const size_t crow = cbatch + (size_t)gi * p.ldc;
   const size_t xrow = (size_t)bz * p.batch_aux + (size_t)gi * p.ld_aux;
   const bool vec_ok = p.vec_ok != 0;
-  const bool a2 = (p.aux_dtype != F32), o2 = (p.out_dtype != F32);
-  // the coalesced path wants `aux` and the output in the same type (true of every product the library makes)
-  // (symmetric output: the mirror stores of the coalesced path assume 32 complete rows)
-  const bool fast_ok = vec_ok && (EPI == EPI_STORE || EPI == EPI_RESID_NORM || a2 == o2) &&
-                       (!p.symmetric || (gi_warp0 + 32 <= p.M && EPI != EPI_RESID_NORM)) &&
-                       (!p.transposed || gi_warp0 + 32 <= p.M);
-  int c0 = wsel * 32;
-  if (fast_ok) {
+  const FastBlocks f = fast_blocks<EPI>(p, gi_warp0, col0, n_eff, wsel);
+  int c0 = f.first;
+  if (f.on) {
     // the complete 32-column blocks come first; whatever is left (a ragged edge) takes the general path below
-    int lim = p.N - col0;
-    if (lim > n_eff) lim = n_eff;
-    // A symmetric output may be the product of two DIFFERENT symmetric matrices (the apply step of the symmetric
-    // filter, the Horner steps of a polynomial in the Gram matrix), whose computed (i, j) and (j, i) differ in the last
-    // bits. Off the diagonal the mirror store makes the pair equal; the 32 x 32 block ON the diagonal must do the same
-    // element by element, or an iterate picks up an antisymmetric part that the symmetric filter doubles at every step:
-    // it takes the general path.
-    // (A product of a matrix with itself, X X^T or A A, computes (i, j) and (j, i) from the same terms in the same
-    // order: its diagonal blocks are symmetric to the bit and stay on the coalesced path.)
-    int c_diag = -1;
-    if ((EPI == EPI_STORE || EPI == EPI_POLY) && p.symmetric && p.diag_exact && gi_warp0 >= col0 && gi_warp0 - col0 < lim &&
-        (((gi_warp0 - col0) >> 5) & 1) == wsel)
-      c_diag = gi_warp0 - col0;
-    const bool two = (EPI == EPI_STORE) ? o2 : a2;
-    if (two) c0 = epilogue_fast_blocks<EPI, 2>(p, taddr, stg, lane, gi_warp0, col0, c0, lim, bz, alpha, aux_scale, sq, c_diag);
-    else c0 = epilogue_fast_blocks<EPI, 4>(p, taddr, stg, lane, gi_warp0, col0, c0, lim, bz, alpha, aux_scale, sq, c_diag);
-    if (c_diag >= 0)
-      epilogue_block_general<EPI>(p, taddr, c_diag, gi, gi_warp0, col0, n_eff, row_ok, vec_ok, aux_bf16, crow, cbatch, xrow,
+    const bool two = (EPI == EPI_STORE ? p.out_dtype : p.aux_dtype) != F32;
+    if (two) c0 = epilogue_fast_blocks<EPI, 2>(p, taddr, stg, lane, gi_warp0, col0, c0, f.lim, bz, alpha, aux_scale, sq, ahead);
+    else c0 = epilogue_fast_blocks<EPI, 4>(p, taddr, stg, lane, gi_warp0, col0, c0, f.lim, bz, alpha, aux_scale, sq, ahead);
+    if (f.diag >= 0)
+      epilogue_block_general<EPI>(p, taddr, f.diag, gi, gi_warp0, col0, n_eff, row_ok, vec_ok, aux_bf16, crow, cbatch, xrow,
                                   alpha, aux_scale, sq);
   }
   for (; c0 < n_eff; c0 += 64)
@@ -866,8 +857,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_tc_kernel(const __grid_co
   if (PAIR) cluster_sync_all();      // the peer's barriers are initialised before anything signals them
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
-  // (barriers, tensor memory and the descriptor fetch above overlap the end of the previous kernel)
-  pdl_wait();
+  // Barriers, tensor memory and the descriptor fetch above overlap the end of the previous kernel, and so does what each
+  // role works out before its first access to global memory, where it waits for that kernel (pdl_wait): a new launch finds its
+  // parameters and code in no cache near the SM, and with the wait here the first copies left 3500-5000 cycles after it.
   pdl_launch();
 
   if (warp == 0) {
@@ -915,6 +907,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_tc_kernel(const __grid_co
       // per pair that tells it to stop; whoever draws the last one puts the counter back to zero
       const long long last_ticket = (total_tiles > npairs ? total_tiles - npairs : 0) + npairs - 1;
       unsigned int ticket = 0;
+      if (dynamic || aux_prefetch) pdl_wait();
       for (int it = 0;; ++it) {
         long long tile;
         if (!dynamic) {
@@ -972,6 +965,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_tc_kernel(const __grid_co
         const int b_loc0 = PAIR ? (int)rank * (t.n_eff >> 1) : 0;                // a pair: this CTA's half of the columns
         const int b_mn0 = t.tn * BN + b_loc0;
         bool live = true;
+        if (it == 0) {
+          touch(a_mn0, b_mn0, my_dst_off, my_tm0, my_tm1, full0_sig, kblocks0, kblocks1, kreal0, kreal1, tx_bytes, tx_sub_bytes);
+          pdl_wait();
+        }
         for (int seg = 0; seg < nseg && live; ++seg) {
           const int nkb = seg ? kblocks1 : kblocks0;
           int left = seg ? kreal1 : kreal0;                   // K blocks of the segment not yet requested
@@ -1117,6 +1114,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_tc_kernel(const __grid_co
     uint32_t acc = 0, acc_phase = 0;
     const int h_first = PAIR ? (int)rank : 0;
     const int h_last = PAIR ? (int)rank : ((p.tile_m == 256) ? 1 : 0);
+    const bool one_half = PAIR || p.tile_m != 256;
+    touch(p.C, p.ldc, p.batch_c, p.aux, p.ld_aux, p.batch_aux, p.alpha, p.pa, p.pb, p.pc, p.N, p.vec_ok, p.out_dtype, p.alpha_dev);
+    pdl_wait();
     for (int it = 0;; ++it) {
       long long tile;
       if (!dynamic) {
@@ -1131,6 +1131,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_tc_kernel(const __grid_co
       const TileInfo t = tile_info(p, tile);
       if (t.skip) continue;
       const int tn = t.tn, tm = t.tm, bz = t.bz;
+      // the first block of `aux` is on its way while the products are still running
+      int ahead = -1;
+      if (one_half && (t.halves & (1 << h_first))) {
+        const int gi0 = tm * p.tile_m + h_first * 128 + q * 32;
+        switch (p.epilogue) {
+          case EPI_POLY: ahead = epilogue_ahead<EPI_POLY>(p, gi0, tn * p.BN, t.n_eff, bz, wsel, stg, lane); break;
+          case EPI_AUX_PLUS: ahead = epilogue_ahead<EPI_AUX_PLUS>(p, gi0, tn * p.BN, t.n_eff, bz, wsel, stg, lane); break;
+          case EPI_RESID_NORM: ahead = epilogue_ahead<EPI_RESID_NORM>(p, gi0, tn * p.BN, t.n_eff, bz, wsel, stg, lane); break;
+          default: break;
+        }
+      }
       const bool ok = mbar_wait(smem_u32(&acc_full_bar[acc]), acc_phase, &abort_flag, p.status, p.wait_ns);
       if (!ok) break;
       tc_fence_after();
@@ -1144,10 +1155,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_tc_kernel(const __grid_co
           const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + tcol;
           const int gi0 = tm * p.tile_m + h * 128 + q * 32, gi = gi0 + lane;
           switch (p.epilogue) {
-            case EPI_STORE: epilogue_half<EPI_STORE>(p, taddr, gi, gi0, tn * p.BN, t.n_eff, bz, wsel, alpha, aux_scale, sq, stg, lane); break;
-            case EPI_POLY: epilogue_half<EPI_POLY>(p, taddr, gi, gi0, tn * p.BN, t.n_eff, bz, wsel, alpha, aux_scale, sq, stg, lane); break;
-            case EPI_AUX_PLUS: epilogue_half<EPI_AUX_PLUS>(p, taddr, gi, gi0, tn * p.BN, t.n_eff, bz, wsel, alpha, aux_scale, sq, stg, lane); break;
-            default: epilogue_half<EPI_RESID_NORM>(p, taddr, gi, gi0, tn * p.BN, t.n_eff, bz, wsel, alpha, aux_scale, sq, stg, lane); break;
+            case EPI_STORE: epilogue_half<EPI_STORE>(p, taddr, gi, gi0, tn * p.BN, t.n_eff, bz, wsel, alpha, aux_scale, sq, stg, lane, ahead); break;
+            case EPI_POLY: epilogue_half<EPI_POLY>(p, taddr, gi, gi0, tn * p.BN, t.n_eff, bz, wsel, alpha, aux_scale, sq, stg, lane, ahead); break;
+            case EPI_AUX_PLUS: epilogue_half<EPI_AUX_PLUS>(p, taddr, gi, gi0, tn * p.BN, t.n_eff, bz, wsel, alpha, aux_scale, sq, stg, lane, ahead); break;
+            default: epilogue_half<EPI_RESID_NORM>(p, taddr, gi, gi0, tn * p.BN, t.n_eff, bz, wsel, alpha, aux_scale, sq, stg, lane, ahead); break;
           }
         }
         if (p.epilogue == EPI_RESID_NORM) {
