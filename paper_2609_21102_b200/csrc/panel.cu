@@ -253,8 +253,12 @@ cudaError_t panel_apply_launch(const float* In, long long in_bs, int ld_in, cons
 // v^T C v with the unshifted matrix (a copy in shared memory): as shifted norms less the shift, 1e-16 ||C||_F is all that
 // would be left of a small one beside a large one. One product of C with V for it: 1 us of 50 at l = 16.
 // What bounds it is the chain of dependent operations of a round (l - 1 rounds a sweep, one barrier each, half a dozen
-// sweeps), not its arithmetic: the block has only the warps that own pairs, and the rotation angle, which merely steers
-// the iteration, comes from approximate fp32 functions.
+// sweeps), not its arithmetic. Only the warps that own pairs take part in the rounds (all of the block loads the partial
+// sums and writes the results). Four lanes per pair: a step of a shuffled fp64 sum takes 38 cycles, so two steps and a
+// longer local sum beat three. The rotation merely steers the iteration, so its cosine and sine come from two fp32 reciprocal
+// square roots (cos 2t = |d| / sqrt(d^2 + g^2), d the difference of the squared norms and g twice the inner product, both over
+// the power of two above their sum) and are scaled in fp64 to c^2 + s^2 = 1; tests and angle are worked out side by side,
+// without branches. A sweep whose largest cosine was below 1e-7 is the last one: convergence is quadratic there.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -262,78 +266,87 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// eight lanes of a warp add up their values (the lanes sub = 0..7 of one column pair)
-__device__ __forceinline__ double group8_sum(double v) {
+// four lanes of a warp add up their values (the lanes sub = 0..3 of one column pair)
+__device__ __forceinline__ double group4_sum(double v) {
   v += __shfl_xor_sync(0xffffffffu, v, 1);
   v += __shfl_xor_sync(0xffffffffu, v, 2);
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
   return v;
 }
 
-// fp32 reciprocal and square root of the hardware's approximation unit (about 1e-7, no special-case handling)
-__device__ __forceinline__ float rcp_approx(float x) { float r; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
-__device__ __forceinline__ float sqrt_approx(float x) { float r; asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
+// fp32 reciprocal square root of the hardware's approximation unit (about 1e-7, no special-case handling)
 __device__ __forceinline__ float rsqrt_approx(float x) { float r; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
 
-constexpr int JAC_THREADS = 256;        // at most 32 column pairs x 8 lanes
+constexpr int JAC_THREADS = 256;
+// doubles between columns: at least four per lane row, four more than a multiple of sixteen, so that the eight pairs of a warp,
+// neighbouring columns mostly, start in different banks
+__host__ __device__ constexpr int jac_stride(int nr) { return (4 * nr - 4 + 15) / 16 * 16 + 4; }
 
-template <int NR>      // rows per lane, ceil(l / 8)
+template <int NR>      // rows per lane, ceil(l / 4) rounded up to even
 __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* __restrict__ partial, int nchunk, int l,
                                                                  int signed_input, float* __restrict__ s_out,
                                                                  float* __restrict__ E, float* __restrict__ Es,
                                                                  int* __restrict__ status, int max_sweeps) {
-  pdl_wait();
   extern __shared__ double sm[];
-  // column-major: A[c * ls + r], rows l .. 8 NR - 1 and column l (the padding player's) all zero, so that no access of a
-  // round needs a test; the stride is odd (the four pairs of a warp start in different banks)
-  constexpr int ls = 8 * NR + 1;
+  // column-major: A[c * ls + r], rows l .. 4 NR - 1 and column l (the padding player's) all zero, so that no access of a
+  // round needs a test
+  constexpr int ls = jac_stride(NR);
   double* A = sm;
   double* C = sm + (l + 1) * ls;      // signed input: the matrix before the shift, stored like A
   __shared__ double lam[MAX_L];       // column norms (eigenvalues of the scaled, shifted matrix), then the eigenvalues
   __shared__ double len[MAX_L];
   __shared__ double nrm2[MAX_L + 1];  // squared column norms of A, carried along by the rotations
   __shared__ int order[MAX_L];
-  __shared__ int rotated;
-  const int bz = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nt = blockDim.x;
+  __shared__ int large[2];            // per parity of the sweep: a rotation with a cosine above 1e-7 was made
+  const int bz = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const double* pb = partial + (long long)bz * nchunk * l * l;
-  for (int e = tid; e < (l + 1) * ls; e += nt) A[e] = 0.0;
+  for (int e = tid; e < (l + 1) * ls; e += JAC_THREADS) A[e] = 0.0;
+  if (tid < 2) large[tid] = 0;
+  if (tid == 0) nrm2[l] = 0.0;
   __syncthreads();
-  for (int e = tid; e < l * l; e += nt) {
-    double t = 0.0;
-#pragma unroll 8
-    for (int ch = 0; ch < nchunk; ++ch) t += pb[(long long)ch * l * l + e];
-    A[(e % l) * ls + e / l] = t;
+  pdl_wait();
+  for (int e0 = tid; e0 < l * l; e0 += 4 * JAC_THREADS) {      // four entries of a thread side by side
+    double t[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+    for (int ch = 0; ch < nchunk; ++ch)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = e0 + u * JAC_THREADS;
+        t[u] += (e < l * l) ? pb[(long long)ch * l * l + e] : 0.0;
+      }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = e0 + u * JAC_THREADS;
+      if (e < l * l) A[(e % l) * ls + e / l] = t[u];
+    }
   }
   __syncthreads();
   // symmetrise (one thread per pair of entries)
-  for (int e = tid; e < l * l; e += nt) {
+  for (int e = tid; e < l * l; e += JAC_THREADS) {
     const int i = e / l, j = e % l;
     if (i < j) { const double a = 0.5 * (A[i * ls + j] + A[j * ls + i]); A[i * ls + j] = a; A[j * ls + i] = a; }
   }
   __syncthreads();
   const int np = (l + 1) & ~1;        // players, padded to even
   const int npairs = np / 2;
-  // Eight lanes per column pair, four pairs per warp: the dot product of a pair takes three shuffle steps.
-  const int grp = tid >> 3, sub = tid & 7;
+  const int grp = tid >> 2, sub = tid & 3;
   // Squared norms of the columns (Frobenius norm for the shift, and for the scale: the matrix is multiplied by the power
-  // of two that brings its norm near one, exactly, so that squared norms and dot products of columns down to 1e-18 of it
-  // are ordinary fp32 numbers for the angle).
-  auto column_norms = [&]() {
-    for (int j0 = 0; j0 < l; j0 += nt >> 3) {      // (the same trip count for every lane: shuffles inside)
+  // of two that brings its norm near one, exactly), by `nt` threads in whole warps
+  auto column_norms = [&](int nt) {
+    for (int j0 = 0; j0 < l; j0 += nt >> 2) {      // (the same trip count for every lane: shuffles inside)
       const int j = j0 + grp;
-      double acc = 0.0;
+      double a0 = 0.0, a1 = 0.0;
 #pragma unroll
-      for (int i = 0; i < NR; ++i) { const double v = A[min(j, l) * ls + sub + 8 * i]; acc = fma(v, v, acc); }
-      acc = group8_sum(acc);
+      for (int i = 0; i < NR; i += 2) {
+        const double v0 = A[min(j, l) * ls + sub + 4 * i], v1 = A[min(j, l) * ls + sub + 4 * i + 4];
+        a0 = fma(v0, v0, a0); a1 = fma(v1, v1, a1);
+      }
+      const double acc = group4_sum(a0 + a1);
       if (sub == 0 && j < l) nrm2[j] = acc;
     }
-    __syncthreads();
   };
-  if (tid == 0) nrm2[l] = 0.0;
-  column_norms();
-  double fro2 = 0.0;
-  for (int j = 0; j < l; ++j) fro2 += nrm2[j];
-  const double fro = sqrt(fro2);
+  column_norms(JAC_THREADS);
+  __syncthreads();
+  const double fro = sqrt(warp_sum((lane < l ? nrm2[lane] : 0.0) + (lane + 32 < l ? nrm2[lane + 32] : 0.0)));      // (the same in every warp)
   double scale = 1.0, unscale = 1.0;
   if (fro > 1e-290 && fro < 1e290) {
     const int ex = (int)((__double_as_longlong(fro) >> 52) & 0x7ff);             // fro in [2^(ex-1023), 2^(ex-1022))
@@ -341,84 +354,83 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
     unscale = __longlong_as_double((long long)ex << 52);
   }
   const double shift = signed_input ? 2.0 * fro * scale : 0.0;
-  __syncthreads();
-  for (int e = tid; e < l * l; e += nt) {
+  for (int e = tid; e < l * l; e += JAC_THREADS) {
     const int c = e / l, r = e % l;
     const double v = A[c * ls + r] * scale;
     A[c * ls + r] = v + ((r == c) ? shift : 0.0);
     if (signed_input) C[c * ls + r] = v;
   }
   if (signed_input)
-    for (int e = tid; e < l * (ls - l); e += nt) C[(e / (ls - l)) * ls + l + e % (ls - l)] = 0.0;
+    for (int e = tid; e < l * (ls - l); e += JAC_THREADS) C[(e / (ls - l)) * ls + l + e % (ls - l)] = 0.0;
   __syncthreads();
-  int sweep = 0;
-  for (; sweep < max_sweeps; ++sweep) {
-    if (tid == 0) rotated = 0;
-    // Squared column norms, exact at the start of every sweep. Within the sweep a rotation by tan t moves
-    // t gamma from one column's squared norm to the other's (alpha' = alpha - t gamma, beta' = beta + t gamma), so
-    // a round computes one dot product per pair instead of three; the sweep that finds nothing to rotate, which
-    // ends the iteration, has tested every pair against exact norms.
-    column_norms();
-    for (int round = 0; round < np - 1; ++round) {
-      int p = l, q = l;
-      if (grp < npairs) {
-        if (grp == 0) { p = np - 1; q = round; }
-        else {
-          // (round + grp) and (round - grp) modulo np - 1: both lie within one period of the range
-          p = round + grp; if (p >= np - 1) p -= np - 1;
-          q = round - grp; if (q < 0) q += np - 1;
+  const int nt = (npairs * 4 + 31) & ~31;          // threads of the rounds
+  if (tid < nt) {
+    auto sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory"); };
+    int sweep = 0;
+    for (; sweep < max_sweeps; ++sweep) {
+      // Squared column norms, exact at the start of every sweep. Within the sweep a rotation moves
+      // s (2 c gamma - s d) from one column's squared norm to the other's, so a round computes one dot product per pair
+      // instead of three.
+      column_norms(nt);
+      sync();
+      if (tid == 0) large[(sweep + 1) & 1] = 0;      // (everybody has looked at the sweep before)
+      bool big = false;
+      // round-robin: group g > 0 has round + g and round - g modulo np - 1, group 0 the round and the player np - 1; worked out
+      // a round ahead. (A pair with the padding player meets the zero column, a group beyond the pairs nothing else: nothing
+      // to rotate.)
+      int one = grp == 0 ? np - 1 : grp, two = grp == 0 ? 0 : np - 1 - grp;
+      if (grp >= npairs) one = two = l;
+      for (int round = 0; round < np - 1; ++round) {
+        const int p = min(one, two), q = max(one, two);
+        if (grp < npairs) {
+          if (grp > 0 && ++one == np - 1) one = 0;
+          if (++two == np - 1) two = 0;
         }
-        if (p > q) { const int t = p; p = q; q = t; }
-      }
-      // (a pair with the padding player meets the zero column, a group beyond the pairs nothing else: nothing to rotate)
-      double* ap = A + p * ls + sub; double* aq = A + q * ls + sub;
-      const double alpha = nrm2[p], beta = nrm2[q];
-      double x[NR], y[NR];
-      double pg0 = 0.0, pg1 = 0.0;
+        double* ap = A + p * ls + sub; double* aq = A + q * ls + sub;
+        double x[NR], y[NR];
 #pragma unroll
-      for (int i = 0; i < NR; ++i) { x[i] = ap[8 * i]; y[i] = aq[8 * i]; }
+        for (int i = 0; i < NR; ++i) { x[i] = ap[4 * i]; y[i] = aq[4 * i]; }
+        const double alpha = nrm2[p], beta = nrm2[q], d = beta - alpha, ab = alpha * beta;
+        // 1 / (the power of two above alpha + beta), for the fp32 angle
+        const double f = __hiloint2double(0x7fd00000 - (__double2hiint(alpha + beta) & 0x7ff00000), 0);
+        const float df = (float)(d * f), adf = fabsf(df);
+        double g0 = 0.0, g1 = 0.0;
 #pragma unroll
-      for (int i = 0; i < NR; ++i) {
-        if (i & 1) pg1 = fma(x[i], y[i], pg1); else pg0 = fma(x[i], y[i], pg0);
-      }
-      const double gamma = group8_sum(pg0 + pg1);
-      // rotate when |gamma| > 1e-11 sqrt(alpha beta) (compared in squares): the eigenvalues are then good to about
-      // 1e-22 and the vectors to 1e-11 over the relative gap, far beyond the fp32 outputs
-      if (gamma != 0.0 && gamma * gamma > 1e-22 * (alpha * beta)) {
-        if (sub == 0) rotated = 1;
-        // The rotation angle only steers the iteration (any exact rotation keeps the invariants intact), so tan is
-        // computed in fp32 with approximate functions; cos comes from an fp32 reciprocal square root refined by two
-        // Newton steps in fp64, which makes c^2 + s^2 = 1 hold to fp64 rounding. A rotation then leaves 1e-7 of the
-        // inner product instead of none, and the pair's next visit removes that. The chain of dependent fp64
-        // operations, which is the latency of a round, shrinks to a third. What fp32 cannot hold takes the fp64 formula.
-        const double d = beta - alpha, g2 = 2.0 * gamma;
-        const float df = (float)d, gf = (float)g2;
-        double t;
-        if (fabsf(gf) > 1e-30f && fabsf(df) < 1e30f) {
-          const float zf = df * rcp_approx(gf), az = fabsf(zf);
-          // t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)): the root of t^2 + 2 zeta t - 1 = 0 of smaller magnitude
-          t = (double)copysignf((az > 1e15f) ? 0.5f * rcp_approx(az) : rcp_approx(az + sqrt_approx(fmaf(zf, zf, 1.0f))), zf);
-        } else {
-          const double zeta = d / g2;
-          t = ((zeta >= 0.0) ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+        for (int i = 0; i < NR; i += 2) { g0 = fma(x[i], y[i], g0); g1 = fma(x[i + 1], y[i + 1], g1); }
+        const double gamma = group4_sum(g0 + g1), g2 = 2.0 * gamma;
+        // rotate when |gamma| > 1e-11 sqrt(alpha beta) (compared in squares): the eigenvalues are then good to about
+        // 1e-22 and the vectors to 1e-11 over the relative gap, far beyond the fp32 outputs
+        const double gg = gamma * gamma;
+        const bool turn = gamma != 0.0 && gg > 1e-22 * ab;
+        const float gf = (float)(g2 * f);
+        const float h = rsqrt_approx(fmaf(gf, gf, df * df));
+        const float xx = fmaf(0.5f * adf, h, 0.5f), ir = rsqrt_approx(xx);
+        double c = (double)(xx * ir), sn = (double)(0.5f * copysignf(gf, __int_as_float(__float_as_int(gf) ^ __float_as_int(df))) * h * ir);
+        if (turn && !(fabsf(gf) > 1e-18f)) {       // what fp32 cannot hold takes the fp64 formula
+          const double zeta = d / g2, t = ((zeta >= 0.0) ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+          c = 1.0 / sqrt(1.0 + t * t); sn = c * t;
         }
-        const double w = fma(t, t, 1.0), h = 0.5 * w;                // w in [1, 2]
-        double c = (double)rsqrt_approx((float)w);
-        c = c * fma(-h * c, c, 1.5);
-        c = c * fma(-h * c, c, 1.5);
-        const double sn = c * t, tg = t * gamma;
-        if (sub == 0) { nrm2[p] = alpha - tg; nrm2[q] = beta + tg; }
+        // c^2 + s^2 = 1 to fp64 rounding: 1 / sqrt(1 - e) = 1 + e/2 + 3/8 e^2 for e of 1e-6
+        const double e = 1.0 - fma(c, c, sn * sn), k = fma(fma(0.375, e, 0.5), e, 1.0);
+        c *= k; sn *= k;
+        if (turn) {
 #pragma unroll
-        for (int i = 0; i < NR; ++i) { ap[8 * i] = c * x[i] - sn * y[i]; aq[8 * i] = sn * x[i] + c * y[i]; }
+          for (int i = 0; i < NR; ++i) { ap[4 * i] = c * x[i] - sn * y[i]; aq[4 * i] = sn * x[i] + c * y[i]; }
+          const double moved = sn * fma(2.0 * c, gamma, -sn * d);
+          if (sub == 0) { nrm2[p] = alpha - moved; nrm2[q] = beta + moved; }
+          big |= gg > 1e-14 * ab;
+        }
+        sync();
       }
-      __syncthreads();
+      if (big && sub == 0) large[sweep & 1] = 1;
+      sync();
+      if (!large[sweep & 1]) break;
     }
-    if (!rotated) break;
-    __syncthreads();
+    if (tid == 0 && sweep >= max_sweeps && status) atomicOr(&status[bz], 2);
   }
-  if (tid == 0 && sweep >= max_sweeps && status) atomicOr(&status[bz], 2);
+  __syncthreads();
   // eigenvalues
-  for (int j = warp; j < l; j += nt >> 5) {
+  for (int j = warp; j < l; j += JAC_THREADS / 32) {
     const double* aj = A + j * ls;
     const double a0 = (lane < l) ? aj[lane] : 0.0, a1 = (lane + 32 < l) ? aj[lane + 32] : 0.0;
     const double nrm = sqrt(warp_sum(a0 * a0 + a1 * a1));
@@ -426,8 +438,8 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
   }
   __syncthreads();
   if (signed_input) {
-    // lambda_j = a_j^T C a_j / ||a_j||^2, eight lanes per column
-    for (int j0 = 0; j0 < l; j0 += nt >> 3) {      // (the same trip count for every lane: shuffles inside)
+    // lambda_j = a_j^T C a_j / ||a_j||^2, four lanes per column
+    for (int j0 = 0; j0 < l; j0 += JAC_THREADS / 4) {      // (the same trip count for every lane: shuffles inside)
       const int j = min(j0 + grp, l);
       const double* aj = A + j * ls;
       double t[NR];
@@ -436,12 +448,12 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
       for (int c = 0; c < l; ++c) {
         const double a = aj[c];
 #pragma unroll
-        for (int i = 0; i < NR; ++i) t[i] = fma(C[c * ls + sub + 8 * i], a, t[i]);
+        for (int i = 0; i < NR; ++i) t[i] = fma(C[c * ls + sub + 4 * i], a, t[i]);
       }
       double acc = 0.0;
 #pragma unroll
-      for (int i = 0; i < NR; ++i) acc = fma(t[i], aj[sub + 8 * i], acc);
-      acc = group8_sum(acc);
+      for (int i = 0; i < NR; ++i) acc = fma(t[i], aj[sub + 4 * i], acc);
+      acc = group4_sum(acc);
       // (a zero matrix has zero columns and no shift)
       if (sub == 0 && j < l) lam[j] = (len[j] <= 1e-150) ? 0.0 : acc / (len[j] * len[j]) * unscale;
     }
@@ -461,7 +473,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
     order[rank] = tid;
   }
   __syncthreads();
-  for (int e = tid; e < l * l; e += nt) {
+  for (int e = tid; e < l * l; e += JAC_THREADS) {
     const int r = e / l, cc = e % l;
     const int src = order[cc];
     // v_j = a_j / ||a_j||; a column that vanished (rank-deficient input) takes its unit vector, which only ever meets a
@@ -475,15 +487,25 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
   }
 }
 
+static const void* jacobi_form(int nr) {
+  switch (nr) {
+    case 2: return (const void*)jacobi_eig_kernel<2>;
+    case 4: return (const void*)jacobi_eig_kernel<4>;
+    case 6: return (const void*)jacobi_eig_kernel<6>;
+    case 8: return (const void*)jacobi_eig_kernel<8>;
+    case 10: return (const void*)jacobi_eig_kernel<10>;
+    case 12: return (const void*)jacobi_eig_kernel<12>;
+    case 14: return (const void*)jacobi_eig_kernel<14>;
+    default: return (const void*)jacobi_eig_kernel<16>;
+  }
+}
+
 cudaError_t jacobi_eig_launch(const double* partial, int nchunk, int batch, int l, int signed_input, float* s_out,
                               float* E, float* Es, int* status, cudaStream_t st, long long* launches, int max_sweeps) {
-  const int threads = (((l + 1) / 2) * 8 + 31) & ~31;        // eight lanes per pair, whole warps
-  const int nr = (l + 7) / 8;
-  const size_t smem = (size_t)(l + 1 + (signed_input ? l : 0)) * (8 * nr + 1) * sizeof(double);
-  auto kern = nr <= 1 ? jacobi_eig_kernel<1> : nr == 2 ? jacobi_eig_kernel<2> : nr == 3 ? jacobi_eig_kernel<3>
-            : nr == 4 ? jacobi_eig_kernel<4> : nr == 5 ? jacobi_eig_kernel<5> : nr == 6 ? jacobi_eig_kernel<6>
-            : nr == 7 ? jacobi_eig_kernel<7> : jacobi_eig_kernel<8>;
-  launch_kernel(kern, batch, threads, smem, st, partial, nchunk, l, signed_input, s_out, E, Es, status, max_sweeps > 0 ? max_sweeps : 40);
+  const int nr = (l + 7) / 8 * 2;
+  const size_t smem = (size_t)(l + 1 + (signed_input ? l : 0)) * jac_stride(nr) * sizeof(double);
+  typedef void (*Form)(const double*, int, int, int, float*, float*, float*, int*, int);
+  launch_kernel((Form)jacobi_form(nr), batch, JAC_THREADS, smem, st, partial, nchunk, l, signed_input, s_out, E, Es, status, max_sweeps > 0 ? max_sweeps : 40);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -1253,10 +1275,11 @@ __global__ void __launch_bounds__(256, 2) panel_fused_kernel(const float* In, lo
 }
 
 cudaError_t panel_prepare() {
-  // (the Jacobi core with a signed input of more than 48 columns; up to there it stays within the default limit)
-  constexpr int jac = (int)((2 * MAX_L + 1) * (MAX_L + 1) * sizeof(double));
-  cudaError_t e = cudaFuncSetAttribute(jacobi_eig_kernel<7>, cudaFuncAttributeMaxDynamicSharedMemorySize, jac);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(jacobi_eig_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, jac);
+  cudaError_t e = cudaSuccess;
+  for (int nr = 2; nr <= 16 && e == cudaSuccess; nr += 2) {      // (signed input, the widest core of the form)
+    const int l = 4 * nr < MAX_L ? 4 * nr : MAX_L;
+    e = cudaFuncSetAttribute(jacobi_form(nr), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)((2 * l + 1) * jac_stride(nr) * sizeof(double)));
+  }
   if (e == cudaSuccess) e = cudaFuncSetAttribute(panel_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM);
   return e;
 }
