@@ -1041,7 +1041,7 @@ namespace defl {
 
 constexpr int FUSED_TILE = 128;
 constexpr int FUSED_TS = MAX_L + 4;
-constexpr size_t FUSED_SMEM = (size_t)(FUSED_TILE + MAX_L) * FUSED_TS * sizeof(float);
+constexpr size_t FUSED_SMEM = (size_t)(2 * FUSED_TILE + MAX_L) * FUSED_TS * sizeof(float);      // two tiles, the matrix
 
 // Rows are split over CTAs in whole 128-row tiles. The split is chosen so that all CTAs of the launch are resident
 // at once (two per SM with this kernel's registers): a fixed 512-row split gave 624 CTAs for 592 places on
@@ -1062,26 +1062,48 @@ int fused_num_chunks(int rows, int batch) {
   return (tiles + t - 1) / t;
 }
 
+// acc = tile * ms for rows ty + 32 i and columns 4 tx .. + 3 (NC = 8: 32 + 4 tx .. + 3 too). Rows of ms beyond l and columns
+// beyond the ones wanted were zeroed when it was staged, so blocks of four are safe.
+template <int NC>
+__device__ __forceinline__ void panel_product(float (*tile)[FUSED_TS], float (*ms)[FUSED_TS], int l, int ty, int tx, float (&acc)[4][NC]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < NC; ++j) acc[i][j] = 0.f;
+  for (int q = 0; q < l; q += 4) {
+    float4 a4[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a4[i] = *reinterpret_cast<const float4*>(&tile[ty + 32 * i][q]);
+#pragma unroll
+    for (int qq = 0; qq < 4; ++qq) {
+      float b[NC];
+#pragma unroll
+      for (int h = 0; h < NC / 4; ++h) {
+        const float4 b4 = *reinterpret_cast<const float4*>(&ms[q + qq][32 * h + tx * 4]);
+        b[4 * h] = b4.x; b[4 * h + 1] = b4.y; b[4 * h + 2] = b4.z; b[4 * h + 3] = b4.w;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float av = (qq == 0) ? a4[i].x : (qq == 1) ? a4[i].y : (qq == 2) ? a4[i].z : a4[i].w;
+#pragma unroll
+        for (int j = 0; j < NC; ++j) acc[i][j] = fmaf(av, b[j], acc[i][j]);
+      }
+    }
+  }
+}
+
 __global__ void __launch_bounds__(256, 2) panel_fused_kernel(const float* In, long long in_bs, int ld_in, int rows, int l,
                                                           const float* __restrict__ Mtx, int ldm, int kout,
                                                           float* Out, long long out_bs, int ld_out,
                                                           __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
                                                           int lp, double* __restrict__ partial, int nchunk) {
-  pdl_wait();
   extern __shared__ __align__(16) float fsm[];
   // row stride 68 floats: rows stay 16-byte aligned, so register blocks are fetched with 128-bit loads
-  float (*tile)[FUSED_TS] = reinterpret_cast<float (*)[FUSED_TS]>(fsm);                          // [128][68]
-  float (*ms)[FUSED_TS] = reinterpret_cast<float (*)[FUSED_TS]>(fsm + FUSED_TILE * FUSED_TS);    // [64][68]
+  float (*tile)[FUSED_TS] = reinterpret_cast<float (*)[FUSED_TS]>(fsm);                              // [128][68], the first of two
+  float (*ms)[FUSED_TS] = reinterpret_cast<float (*)[FUSED_TS]>(fsm + 2 * FUSED_TILE * FUSED_TS);    // [64][68]
   const int chunk = blockIdx.x, bz = blockIdx.y, tid = threadIdx.x;
   const float* Ib = In + (long long)bz * in_bs;
   const int wout = Mtx ? kout : l;      // width of Out
-  if (Mtx) {
-    const float* Mb = Mtx + (long long)bz * l * ldm;
-    for (int e = tid; e < MAX_L * MAX_L; e += 256) {
-      const int r = e / MAX_L, cc = e % MAX_L;
-      ms[r][cc] = (r < l && cc < kout) ? Mb[r * ldm + cc] : 0.f;
-    }
-  }
   // product: thread (ty, tx) computes rows ty, ty + 32, ty + 64, ty + 96 and columns 4 tx .. 4 tx + 3, 32 + 4 tx .. + 3.
   // A warp's four ty values are then four consecutive tile rows (68 floats apart: different banks) and its eight
   // tx values read 128 contiguous bytes of the staged matrix: one shared-memory wavefront per 16-byte load. (With
@@ -1110,56 +1132,58 @@ __global__ void __launch_bounds__(256, 2) panel_fused_kernel(const float* In, lo
   const int tiles = (rows + FUSED_TILE - 1) / FUSED_TILE;
   const int chunk_rows = ((tiles + nchunk - 1) / nchunk) * FUSED_TILE;
   const int r_begin = chunk * chunk_rows, r_end = min(rows, r_begin + chunk_rows);
-  for (int r0 = r_begin; r0 < r_end; r0 += FUSED_TILE) {
-    __syncthreads();
-    if ((ld_in & 3) == 0 && (l & 3) == 0 && ((reinterpret_cast<uintptr_t>(Ib) & 15) == 0)) {
-      // 16 threads per row (one float4 each, up to 64 columns), 16 rows per pass: no index division, and all
-      // eight loads of a thread are issued before the first use
-      const int c4 = tid & 15, rr0 = tid >> 4;
-      const bool col_ok = c4 * 4 < l;
-      float4 buf[FUSED_TILE / 16];
+  // Rows of whole 16-byte packets are copied asynchronously, the next tile into the other half of the memory while this one is
+  // worked on: with load, product and store taking turns a pass over 48 x 6400 x 48 took 94 us, three times its bytes' time.
+  // 16 threads per row (one packet each, up to 64 columns), rows past the end filled with zeros.
+  const bool vec = (ld_in & 3) == 0 && (l & 3) == 0 && ((reinterpret_cast<uintptr_t>(Ib) & 15) == 0);
+  const int c4 = tid & 15, rr0 = tid >> 4;
+  auto fetch = [&](int r0, float (*t)[FUSED_TS]) {
+    if (c4 * 4 < l) {
 #pragma unroll
       for (int it = 0; it < FUSED_TILE / 16; ++it) {
         const int rr = rr0 + it * 16;
-        buf[it] = (col_ok && r0 + rr < r_end) ? *reinterpret_cast<const float4*>(Ib + (long long)(r0 + rr) * ld_in + c4 * 4)
-                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+        const bool ok = r0 + rr < r_end;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                     ::"r"((uint32_t)__cvta_generic_to_shared(&t[rr][c4 * 4])), "l"(Ib + (long long)(ok ? r0 + rr : 0) * ld_in + c4 * 4), "r"(ok ? 16 : 0) : "memory");
       }
-      if (col_ok) {
-#pragma unroll
-        for (int it = 0; it < FUSED_TILE / 16; ++it) *reinterpret_cast<float4*>(&tile[rr0 + it * 16][c4 * 4]) = buf[it];
-      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  pdl_wait();
+  if (vec) fetch(r_begin, tile);
+  if (Mtx) {
+    const float* Mb = Mtx + (long long)bz * l * ldm;
+#pragma unroll 8
+    for (int e = tid; e < MAX_L * MAX_L; e += 256) {
+      const int r = e / MAX_L, cc = e % MAX_L;
+      ms[r][cc] = (r < l && cc < kout) ? Mb[r * ldm + cc] : 0.f;
+    }
+  }
+  for (int r0 = r_begin; r0 < r_end; r0 += FUSED_TILE) {
+    if (vec) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();            // (the tile is there, and everybody is through with the one before)
+      if (r0 + FUSED_TILE < r_end) fetch(r0 + FUSED_TILE, tile == reinterpret_cast<float (*)[FUSED_TS]>(fsm) ? tile + FUSED_TILE : tile - FUSED_TILE);
     } else {
+      __syncthreads();
       const int lr = (l + 3) & ~3;      // columns l..lr-1 are zeroed: the product walks the row in blocks of four
       for (int e = tid; e < FUSED_TILE * lr; e += 256) {
         const int rr = e / lr, c = e % lr;
         tile[rr][c] = (c < l && r0 + rr < r_end) ? Ib[(long long)(r0 + rr) * ld_in + c] : 0.f;
       }
+      __syncthreads();
     }
-    __syncthreads();
-    if (Mtx) {
+    if (Mtx && kout <= 32) {
+      // (half the columns: the same walk without the second half of a thread's)
+      float acc[4][4];
+      panel_product<4>(tile, ms, l, ty, tx, acc);
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(&tile[ty + 32 * i][tx * 4]) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+      __syncthreads();
+    } else if (Mtx) {
       float acc[4][8];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-      // Mtx rows beyond l and columns beyond kout were zeroed when it was staged, so blocks of four are safe
-      for (int q = 0; q < l; q += 4) {
-        float4 a4[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a4[i] = *reinterpret_cast<const float4*>(&tile[ty + 32 * i][q]);
-#pragma unroll
-        for (int qq = 0; qq < 4; ++qq) {
-          const float4 b0 = *reinterpret_cast<const float4*>(&ms[q + qq][tx * 4]);
-          const float4 b1 = *reinterpret_cast<const float4*>(&ms[q + qq][32 + tx * 4]);
-          const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float av = (qq == 0) ? a4[i].x : (qq == 1) ? a4[i].y : (qq == 2) ? a4[i].z : a4[i].w;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(av, b[j], acc[i][j]);
-          }
-        }
-      }
+      panel_product<8>(tile, ms, l, ty, tx, acc);
       __syncthreads();
       // (columns wout.. of the tile receive zeros: the staged matrix has zero columns there)
 #pragma unroll
@@ -1172,7 +1196,6 @@ __global__ void __launch_bounds__(256, 2) panel_fused_kernel(const float* In, lo
     if (Out) {
       float* Ob = Out + (long long)bz * out_bs;
       if ((wout & 3) == 0 && (ld_out & 3) == 0 && ((reinterpret_cast<uintptr_t>(Ob) & 15) == 0)) {
-        const int c4 = tid & 15, rr0 = tid >> 4;
         if (c4 * 4 < wout) {
 #pragma unroll
           for (int it = 0; it < FUSED_TILE / 16; ++it) {
@@ -1192,7 +1215,6 @@ __global__ void __launch_bounds__(256, 2) panel_fused_kernel(const float* In, lo
       if ((lp & 3) == 0 && lp <= 64 && ((reinterpret_cast<uintptr_t>(hi) | reinterpret_cast<uintptr_t>(lo)) & 7) == 0) {
         // four values per thread: 8-byte stores of the hi and lo halves (tile columns wout..lp-1 may hold
         // leftovers of the input, so they are masked here)
-        const int c4 = tid & 15, rr0 = tid >> 4;
         if (c4 * 4 < lp) {
 #pragma unroll
           for (int it = 0; it < FUSED_TILE / 16; ++it) {
@@ -1243,6 +1265,7 @@ __global__ void __launch_bounds__(256, 2) panel_fused_kernel(const float* In, lo
           for (int j = 0; j < 8; ++j) g8[i][j] = fmaf(a[i], b[j], g8[i][j]);
       }
     }
+    if (vec) tile = tile == reinterpret_cast<float (*)[FUSED_TS]>(fsm) ? tile + FUSED_TILE : tile - FUSED_TILE;
   }
   if (partial) {
     // Sum over the groups in fp64 (group order fixed: the result does not depend on timing). Every thread leaves its block
