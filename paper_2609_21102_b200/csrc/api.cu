@@ -222,9 +222,10 @@ int orthonormalise(defl_ctx* c, float* P, int b, int rows, int l, double* gram, 
 }
 
 // Algorithm 3 on the batch: on return w.Lp = Q U_G (left vectors of A, all l), w.Sp... see below.
-// Outputs: w.sv[b,l], w.Uk[b,ml,k_keep] and w.Vk[b,ms,k_keep] (leading k_keep triplets of A = G or G^T).
+// Outputs: w.sv[b,l], w.Uk[b,ml,k_keep] and w.Vk[b,ms,k_keep] (leading k_keep triplets of A = G or G^T), and w.keff[b], how many
+// of them the gate (Algorithm 1, lines 1-2) deflates.
 int run_brsvd(defl_ctx* c, const void* G, int ldg, int b, int m, int n, int dtype, int l, int J, int k_keep,
-              const float* sketch, const PolarWs& w, int engine) {
+              const float* sketch, const PolarWs& w, int engine, float tau = 0.f) {
   const bool tall = m >= n;
   const int ms = tall ? n : m, ml = tall ? m : n;
   // element (i,j) of A (ml x ms): tall G[i*ldg+j]; wide G[j*ldg+i]
@@ -287,16 +288,13 @@ int run_brsvd(defl_ctx* c, const void* G, int ldg, int b, int m, int n, int dtyp
                                      w.gram, c->stream, &c->launches), "gram core"))
     return DEFL_ERR_CUDA;
   if (ctx_fail(c, jacobi_eig_launch(w.gram, fused_num_chunks(ms, b), b, l, 0, w.sv, w.E, w.Es, w.status, c->stream,
-                                    &c->launches, c->knobs.jacobi_sweeps), "jacobi"))
+                                    &c->launches, c->knobs.jacobi_sweeps, w.keff, k_keep, tau), "jacobi"))
     return DEFL_ERR_CUDA;
   if (k_keep > 0) {
     // U = Q E (long side), V = (Q^T A)^T E diag(1/s) (short side); keep the leading k_keep columns
-    if (ctx_fail(c, panel_fused_launch(w.Lp, (long long)ml * l, l, b, ml, l, w.E, l, k_keep, w.Uk, (long long)ml * k_keep,
-                                       k_keep, nullptr, nullptr, 0, nullptr, c->stream, &c->launches), "U = Q E"))
-      return DEFL_ERR_CUDA;
-    if (ctx_fail(c, panel_fused_launch(w.Sp, (long long)ms * l, l, b, ms, l, w.Es, l, k_keep, w.Vk, (long long)ms * k_keep,
-                                       k_keep, nullptr, nullptr, 0, nullptr, c->stream, &c->launches), "V = B^T E / s"))
-      return DEFL_ERR_CUDA;
+    const PanelPass u = panel_pass(w.Lp, (long long)ml * l, l, b, ml, l, w.E, l, k_keep, w.Uk, (long long)ml * k_keep, k_keep, nullptr, nullptr, 0, nullptr);
+    const PanelPass v = panel_pass(w.Sp, (long long)ms * l, l, b, ms, l, w.Es, l, k_keep, w.Vk, (long long)ms * k_keep, k_keep, nullptr, nullptr, 0, nullptr);
+    if (ctx_fail(c, panel_pair_launch(u, v, b, c->stream, &c->launches), "U = Q E, V = B^T E / s")) return DEFL_ERR_CUDA;
   }
   return DEFL_OK;
 }
@@ -659,9 +657,8 @@ static int polar_core(defl_ctx* c, const void* G, void* out, int b, int m, int n
   ctx_profile_begin(c);
   c->err[0] = 0;
   ctx_stage_mark(c);
-  if (ctx_fail(c, fill_int_launch(w.status, b, 0, c->stream, &c->launches), "status")) return DEFL_ERR_CUDA;
-  // the engine's wait word reports this call only (the tile counter next to it stays as the kernels leave it: zero)
-  if (ctx_fail(c, cudaMemsetAsync(c->wait_status, 0, sizeof(int), c->stream), "status word")) return DEFL_ERR_CUDA;
+  // (the engine's wait word reports this call only; the tile counter next to it stays as the kernels leave it: zero)
+  if (ctx_fail(c, begin_call_launch(w.status, b, c->wait_status, c->stream, &c->launches), "status")) return DEFL_ERR_CUDA;
 
   // Row strides: ldx of the iterates, lds of the short-side matrices, ldg of G (or of its padded copy)
   const bool padded = engine == DEFL_ENGINE_AUTO && L > 0 && padded_shape(m, n, dtype);
@@ -680,7 +677,7 @@ static int polar_core(defl_ctx* c, const void* G, void* out, int b, int m, int n
     // (A padded call keeps its panels in fp32 on the FMA engine, as without the padding. The tensor form of these products
     // splits a panel into bf16 hi + lo, 2^-17 of it, and what that leaves of the head in the residual grows with
     // ||head|| / ||R||: 4e-2 .. 2e-1 of the result at 300 and 600, against 8e-3 with fp32 panels.)
-    if ((rc = run_brsvd(c, G, ldg, b, m, n, dtype, l, power_iters, k, sk, w, padded ? (int)DEFL_ENGINE_SIMT : engine))) return rc;
+    if ((rc = run_brsvd(c, G, ldg, b, m, n, dtype, l, power_iters, k, sk, w, padded ? (int)DEFL_ENGINE_SIMT : engine, tau))) return rc;
   }
   ctx_stage_mark(c);
 
@@ -699,9 +696,8 @@ static int polar_core(defl_ctx* c, const void* G, void* out, int b, int m, int n
     // R = G - P diag(s) W^T as a rank-k product on the product engine with G read in the epilogue.
     // bf16 storage: the fp32 factors are split into bf16 hi + lo and the three significant cross terms are
     // laid side by side along K, [hi|hi|lo] x [hi|lo|hi]^T, one tensor-core product of depth 3k.
-    // gate (Algorithm 1, lines 1-2): per matrix, how many of the k triplets are deflated; the columns beyond
-    // that count are zeroed in the scaled right factor, which removes them from every product below
-    if (ctx_fail(c, gate_launch(w.sv, l, b, k, k, tau, w.keff, c->stream, &c->launches), "gate")) return DEFL_ERR_CUDA;
+    // gate: of the k triplets of a matrix, the columns beyond its count w.keff are zeroed in the scaled right factor, which
+    // removes them from every product below
     GemmDesc g = gemm_desc_zero();
     g.batch = b; g.M = m; g.N = n;
     g.aux = G; g.ld_aux = ldg; g.batch_aux = (long long)m * ldg; g.aux_dtype = dtype;

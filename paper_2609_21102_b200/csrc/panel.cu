@@ -92,16 +92,21 @@ cudaError_t gram_partial_launch(const float* Y, long long batch_stride, int batc
 // Symmetric elimination of [W | I] in one l x l array: step j subtracts f_i = W_ij / d_j times row j from every row i > j,
 // the columns right of j holding what is left of W, those up to j the unit lower factor's inverse Z as it grows (column j
 // becomes -f_i). Then L^-1 = diag(d)^(-1/2) Z and R^-1 is its transpose, so factor and inverse take one sweep of l steps
-// with one barrier each, and the only chain per step is barrier, pivot, reciprocal, one multiply-add. Every thread keeps NR
-// consecutive rows of one column in registers; shared memory carries only the pivot row and column (double buffered). The
+// with one barrier each, and the only chain per step is barrier, pivot row, reciprocal, one multiply-add.
+// Every thread keeps NR consecutive rows of one column in registers; shared memory carries only the pivot row, which is the
+// pivot column too (double buffered): with the column published by one lane per group a step took 690 cycles at l = 48, 220 of
+// them for that. Of 16 warps (NR >= 5) only the thread that holds the pivot works out its reciprocal, which takes four warps
+// of a scheduler 220 cycles (l = 48: 29 -> 23 us); of eight or four warps every thread does, off the path of the stores
+// (l = 24: 8.0 -> 7.2 us, 10.6 the other way). The
 // steps run in blocks of NR, so that the pivot's place among a thread's rows is known to the compiler and who takes part
 // is a comparison of warp-uniform numbers: with rows eight apart the selection took more instructions than the update.
 // ---------------------------------------------------------------------------------------------
 template <int NR>      // rows per thread, ceil(l / 8)
 __global__ void __launch_bounds__(512) chol_inv_kernel(const double* __restrict__ partial, int nchunk, int l, int cw_log2,
                                                        float* __restrict__ Rinv, int* __restrict__ status) {
+  constexpr bool OWNER = NR >= 5;
   pdl_wait();
-  __shared__ double prow[2][MAX_L], pcol[2][MAX_L], diag[MAX_L], wdiag[MAX_L];
+  __shared__ double prow[2][MAX_L], pinv[2], diag[MAX_L], wdiag[MAX_L];
   const int bz = blockIdx.x, tid = threadIdx.x;
   const int c = tid & ((1 << cw_log2) - 1), g = tid >> cw_log2;       // column, group of rows g NR .. g NR + NR - 1
   const double* pb = partial + (long long)bz * nchunk * l * l;
@@ -122,15 +127,11 @@ __global__ void __launch_bounds__(512) chol_inv_kernel(const double* __restrict_
   bool failed = false;
   for (int attempt = 0; attempt < 6; ++attempt) {
     __syncthreads();
-    // row j = a NR + u and column j of the array as it stands; below the pivot the column's place is cleared for Z
+    // row j = a NR + u of the array as it stands, and (OWNER) the pivot's reciprocal, by the thread that holds the pivot
     auto publish = [&](int a, int u, int j) {
-      if (g == a) prow[j & 1][c] = m[u];
-      if (c == j) {
-#pragma unroll
-        for (int v = 0; v < NR; ++v) {
-          pcol[j & 1][g * NR + v] = m[v];
-          if (g > a || (g == a && v > u)) m[v] = 0.0;
-        }
+      if (g == a) {
+        prow[j & 1][c] = m[u];
+        if (OWNER && c == j) pinv[j & 1] = 1.0 / m[u];
       }
     };
 #pragma unroll
@@ -147,18 +148,19 @@ __global__ void __launch_bounds__(512) chol_inv_kernel(const double* __restrict_
           const double d = prow[buf][j], pr = prow[buf][c];       // every thread reads the pivot itself: a bad one is seen by all alike
           double f[NR];
 #pragma unroll
-          for (int v = 0; v < NR; ++v) f[v] = pcol[buf][g * NR + v];      // (rows past l: zeros)
+          for (int v = 0; v < NR; ++v) f[v] = prow[buf][g * NR + v];      // W_ij = W_ji (rows past l: zeros)
           if (!(d > 0.0) || !isfinite(d)) failed = true;
           else {
-            const double inv = 1.0 / d;
             if (tid == 0) diag[j] = d;
-            const double s = (c == j) ? inv : inv * pr;
+            const double inv = OWNER ? pinv[buf] : 1.0 / d;
+            // (below the pivot, column j's place becomes Z's)
+            const double sc = (c == j) ? inv : inv * pr;
             if (g > a) {
 #pragma unroll
-              for (int v = 0; v < NR; ++v) m[v] = fma(-f[v], s, m[v]);
+              for (int v = 0; v < NR; ++v) m[v] = fma(-f[v], sc, (c == j) ? 0.0 : m[v]);
             } else if (g == a) {
 #pragma unroll
-              for (int v = u + 1; v < NR; ++v) m[v] = fma(-f[v], s, m[v]);
+              for (int v = u + 1; v < NR; ++v) m[v] = fma(-f[v], sc, (c == j) ? 0.0 : m[v]);
             }
             if (j + 1 < l) publish(u + 1 < NR ? a : a + 1, u + 1 < NR ? u + 1 : 0, j + 1);   // (into the other buffer)
           }
@@ -276,6 +278,20 @@ __device__ __forceinline__ double group4_sum(double v) {
 // fp32 reciprocal square root of the hardware's approximation unit (about 1e-7, no special-case handling)
 __device__ __forceinline__ float rsqrt_approx(float x) { float r; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
 
+// The deflation gate of Algorithms 1 and 2 on the estimated magnitudes s[0..] (descending in magnitude):
+//   tau <= 0: window (deflate exactly the requested number);
+//   tau > 0 : if |s_window| < tau |s_1| then #{i < kmax : |s_i| > tau |s_1|}, else 0.
+__device__ __forceinline__ int gate_count(const float* s, int window, int kmax, float tau) {
+  int k = window;
+  if (tau > 0.f && window > 0) {
+    const float s1 = fabsf(s[0]);
+    k = 0;
+    if (fabsf(s[window - 1]) < tau * s1)
+      for (int i = 0; i < kmax; ++i) if (fabsf(s[i]) > tau * s1) k = i + 1;
+  }
+  return k;
+}
+
 constexpr int JAC_THREADS = 256;
 // doubles between columns: at least four per lane row, four more than a multiple of sixteen, so that the eight pairs of a warp,
 // neighbouring columns mostly, start in different banks
@@ -285,7 +301,8 @@ template <int NR>      // rows per lane, ceil(l / 4) rounded up to even
 __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* __restrict__ partial, int nchunk, int l,
                                                                  int signed_input, float* __restrict__ s_out,
                                                                  float* __restrict__ E, float* __restrict__ Es,
-                                                                 int* __restrict__ status, int max_sweeps) {
+                                                                 int* __restrict__ status, int max_sweeps, int* __restrict__ keff,
+                                                                 int window, float tau) {
   extern __shared__ double sm[];
   // column-major: A[c * ls + r], rows l .. 4 NR - 1 and column l (the padding player's) all zero, so that no access of a
   // round needs a test
@@ -296,6 +313,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
   __shared__ double len[MAX_L];
   __shared__ double nrm2[MAX_L + 1];  // squared column norms of A, carried along by the rotations
   __shared__ int order[MAX_L];
+  __shared__ float sorted[MAX_L];
   __shared__ int large[2];            // per parity of the sweep: a rotation with a cosine above 1e-7 was made
   const int bz = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const double* pb = partial + (long long)bz * nchunk * l * l;
@@ -483,7 +501,12 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
     const double sv = signed_input ? lm : sqrt(lm > 0.0 ? lm : 0.0);
     if (E) E[(long long)bz * l * l + e] = (float)v;
     if (Es) Es[(long long)bz * l * l + e] = (fabs(sv) > 1e-300) ? (float)(v / sv) : 0.f;
+    if (r == 0) sorted[cc] = (float)sv;
     if (r == 0 && s_out) s_out[(long long)bz * l + cc] = (float)sv;
+  }
+  if (keff) {      // the gate on the leading `window` values (a launch of its own took 1.5 us)
+    __syncthreads();
+    if (tid == 0) keff[bz] = gate_count(sorted, window, window, tau);
   }
 }
 
@@ -501,11 +524,13 @@ static const void* jacobi_form(int nr) {
 }
 
 cudaError_t jacobi_eig_launch(const double* partial, int nchunk, int batch, int l, int signed_input, float* s_out,
-                              float* E, float* Es, int* status, cudaStream_t st, long long* launches, int max_sweeps) {
+                              float* E, float* Es, int* status, cudaStream_t st, long long* launches, int max_sweeps, int* keff,
+                              int window, float tau) {
   const int nr = (l + 7) / 8 * 2;
   const size_t smem = (size_t)(l + 1 + (signed_input ? l : 0)) * jac_stride(nr) * sizeof(double);
-  typedef void (*Form)(const double*, int, int, int, float*, float*, float*, int*, int);
-  launch_kernel((Form)jacobi_form(nr), batch, JAC_THREADS, smem, st, partial, nchunk, l, signed_input, s_out, E, Es, status, max_sweeps > 0 ? max_sweeps : 40);
+  typedef void (*Form)(const double*, int, int, int, float*, float*, float*, int*, int, int*, int, float);
+  launch_kernel((Form)jacobi_form(nr), batch, JAC_THREADS, smem, st, partial, nchunk, l, signed_input, s_out, E, Es, status, max_sweeps > 0 ? max_sweeps : 40, keff,
+                window, tau);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -796,6 +821,18 @@ __global__ void fill_int_kernel(int* p, int n, int v) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) p[i] = v;
 }
+// a call starts: its matrices' status words and the engine's wait word are zero
+__global__ void begin_call_kernel(int* status, int n, int* word) {
+  pdl_wait();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) status[i] = 0;
+  if (i == 0) *word = 0;
+}
+cudaError_t begin_call_launch(int* status, int n, int* word, cudaStream_t st, long long* launches) {
+  launch_kernel(begin_call_kernel, (n + 255) / 256, 256, 0, st, status, n, word);
+  if (launches) ++*launches;
+  return cudaGetLastError();
+}
 cudaError_t fill_int_launch(int* p, int n, int v, cudaStream_t st, long long* launches) {
   if (n <= 0) return cudaSuccess;
   launch_kernel(fill_int_kernel, (n + 255) / 256, 256, 0, st, p, n, v);
@@ -1002,23 +1039,11 @@ cudaError_t zero_residual_entry_launch(const int* status, const float* P, const 
   return cudaGetLastError();
 }
 
-// The deflation gate of Algorithms 1 and 2 on the estimated magnitudes s[b, 0..] (descending in magnitude):
-//   tau <= 0: keff = window (deflate exactly the requested number);
-//   tau > 0 : if |s_window| < tau |s_1| then keff = #{i < kmax : |s_i| > tau |s_1|}, else keff = 0.
 __global__ void gate_kernel(const float* __restrict__ s, int ld_s, int batch, int window, int kmax, float tau,
                             int* __restrict__ keff) {
   pdl_wait();
   const int bz = blockIdx.x * blockDim.x + threadIdx.x;
-  if (bz >= batch) return;
-  const float* sb = s + (long long)bz * ld_s;
-  int k = window;
-  if (tau > 0.f && window > 0) {
-    const float s1 = fabsf(sb[0]);
-    k = 0;
-    if (fabsf(sb[window - 1]) < tau * s1)
-      for (int i = 0; i < kmax; ++i) if (fabsf(sb[i]) > tau * s1) k = i + 1;
-  }
-  keff[bz] = k;
+  if (bz < batch) keff[bz] = gate_count(s + (long long)bz * ld_s, window, kmax, tau);
 }
 
 cudaError_t gate_launch(const float* s, int ld_s, int batch, int window, int kmax, float tau, int* keff, cudaStream_t st,
@@ -1092,11 +1117,14 @@ __device__ __forceinline__ void panel_product(float (*tile)[FUSED_TS], float (*m
   }
 }
 
-__global__ void __launch_bounds__(256, 2) panel_fused_kernel(const float* In, long long in_bs, int ld_in, int rows, int l,
-                                                          const float* __restrict__ Mtx, int ldm, int kout,
-                                                          float* Out, long long out_bs, int ld_out,
-                                                          __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
-                                                          int lp, double* __restrict__ partial, int nchunk) {
+// (two passes over panels of one batch may share a launch: blockIdx.z)
+__global__ void __launch_bounds__(256, 2) panel_fused_kernel(const PanelPass first, const PanelPass second) {
+  const PanelPass p = blockIdx.z ? second : first;
+  if ((int)blockIdx.x >= p.nchunk) return;
+  const float* const In = p.In; const float* const Mtx = p.Mtx; float* const Out = p.Out;
+  __nv_bfloat16* const hi = p.hi; __nv_bfloat16* const lo = p.lo; double* const partial = p.partial;
+  const long long in_bs = p.in_bs, out_bs = p.out_bs;
+  const int ld_in = p.ld_in, rows = p.rows, l = p.l, ldm = p.ldm, kout = p.kout, ld_out = p.ld_out, lp = p.lp, nchunk = p.nchunk;
   extern __shared__ __align__(16) float fsm[];
   // row stride 68 floats: rows stay 16-byte aligned, so register blocks are fetched with 128-bit loads
   float (*tile)[FUSED_TS] = reinterpret_cast<float (*)[FUSED_TS]>(fsm);                              // [128][68], the first of two
@@ -1307,12 +1335,26 @@ cudaError_t panel_prepare() {
   return e;
 }
 
+PanelPass panel_pass(const float* In, long long in_bs, int ld_in, int batch, int rows, int l, const float* Mtx, int ldm, int kout,
+                     float* Out, long long out_bs, int ld_out, __nv_bfloat16* hi, __nv_bfloat16* lo, int lp, double* partial) {
+  PanelPass p;
+  p.In = In; p.in_bs = in_bs; p.ld_in = ld_in; p.rows = rows; p.l = l; p.Mtx = Mtx; p.ldm = ldm; p.kout = kout;
+  p.Out = Out; p.out_bs = out_bs; p.ld_out = ld_out; p.hi = hi; p.lo = lo; p.lp = lp; p.partial = partial;
+  p.nchunk = fused_num_chunks(rows, batch);
+  return p;
+}
+
 cudaError_t panel_fused_launch(const float* In, long long in_bs, int ld_in, int batch, int rows, int l, const float* Mtx,
                                int ldm, int kout, float* Out, long long out_bs, int ld_out, __nv_bfloat16* hi,
                                __nv_bfloat16* lo, int lp, double* partial, cudaStream_t st, long long* launches) {
-  const int nchunk = fused_num_chunks(rows, batch);
-  launch_kernel(panel_fused_kernel, dim3(nchunk, batch), 256, FUSED_SMEM, st, In, in_bs, ld_in, rows, l, Mtx, ldm, kout, Out, out_bs, ld_out,
-                                                            hi, lo, lp, partial, nchunk);
+  const PanelPass p = panel_pass(In, in_bs, ld_in, batch, rows, l, Mtx, ldm, kout, Out, out_bs, ld_out, hi, lo, lp, partial);
+  launch_kernel(panel_fused_kernel, dim3(p.nchunk, batch), 256, FUSED_SMEM, st, p, p);
+  if (launches) ++*launches;
+  return cudaGetLastError();
+}
+
+cudaError_t panel_pair_launch(const PanelPass& a, const PanelPass& b, int batch, cudaStream_t st, long long* launches) {
+  launch_kernel(panel_fused_kernel, dim3(a.nchunk > b.nchunk ? a.nchunk : b.nchunk, batch, 2), 256, FUSED_SMEM, st, a, b);
   if (launches) ++*launches;
   return cudaGetLastError();
 }

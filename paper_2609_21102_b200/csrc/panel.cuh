@@ -16,7 +16,8 @@ cudaError_t panel_apply_launch(const float* In, long long in_bs, int ld_in, cons
                                int rows, int l, int kout, float* Out, long long out_bs, int ld_out, cudaStream_t st,
                                long long* launches);
 cudaError_t jacobi_eig_launch(const double* partial, int nchunk, int batch, int l, int signed_input, float* s_out,
-                              float* E, float* Es, int* status, cudaStream_t st, long long* launches, int max_sweeps = 0);
+                              float* E, float* Es, int* status, cudaStream_t st, long long* launches, int max_sweeps = 0,
+                              int* keff = nullptr, int window = 0, float tau = 0.f);
 cudaError_t frob_partial_launch(const void* X, int dtype, int batch, long long count, int nblk, double* partial,
                                 cudaStream_t st, long long* launches);
 constexpr int FROB_VEC_BLOCKS = 148;    // CTAs (and partial sums) per matrix of the vectorised Frobenius pass
@@ -37,6 +38,7 @@ cudaError_t scale_launch(const void* In, int in_dt, void* Out, int out_dt, int b
 cudaError_t fill_gaussian_launch(void* dst, long long count, int dtype, unsigned long long seed, long long per_stream,
                                  unsigned long long seed_stride, cudaStream_t st, long long* launches);
 cudaError_t fill_int_launch(int* p, int n, int v, cudaStream_t st, long long* launches);
+cudaError_t begin_call_launch(int* status, int n, int* word, cudaStream_t st, long long* launches);
 
 }  // namespace defl
 
@@ -64,6 +66,17 @@ int fused_max_chunks(int rows);
 cudaError_t panel_fused_launch(const float* In, long long in_bs, int ld_in, int batch, int rows, int l, const float* Mtx,
                                int ldm, int kout, float* Out, long long out_bs, int ld_out, __nv_bfloat16* hi,
                                __nv_bfloat16* lo, int lp, double* partial, cudaStream_t st, long long* launches);
+// The same passes as arguments: two of them over the panels of one batch in one launch.
+struct PanelPass {
+  const float* In; long long in_bs; int ld_in, rows, l;
+  const float* Mtx; int ldm, kout;
+  float* Out; long long out_bs; int ld_out;
+  __nv_bfloat16* hi; __nv_bfloat16* lo; int lp;
+  double* partial; int nchunk;
+};
+PanelPass panel_pass(const float* In, long long in_bs, int ld_in, int batch, int rows, int l, const float* Mtx, int ldm, int kout,
+                     float* Out, long long out_bs, int ld_out, __nv_bfloat16* hi, __nv_bfloat16* lo, int lp, double* partial);
+cudaError_t panel_pair_launch(const PanelPass& a, const PanelPass& b, int batch, cudaStream_t st, long long* launches);
 // Muon momentum: Mom <- mu Mom + Grad (stored type `dtype`); look (may be null) <- Grad + mu Mom_stored
 cudaError_t momentum_launch(void* Mom, const void* Grad, void* look, int dtype, long long count, float mu, cudaStream_t st,
                             long long* launches);

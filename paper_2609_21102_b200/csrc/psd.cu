@@ -1224,8 +1224,7 @@ static int psd_core(defl_ctx* c, const void* Xv, void* Pv, int n, int k, float* 
   ctx_profile_begin(c);
   c->err[0] = 0;
   ctx_stage_mark(c);
-  if (ctx_fail(c, fill_int_launch(w.status, 1, 0, c->stream, &c->launches), "status")) return DEFL_ERR_CUDA;
-  if (ctx_fail(c, cudaMemsetAsync(c->wait_status, 0, sizeof(int), c->stream), "status word")) return DEFL_ERR_CUDA;
+  if (ctx_fail(c, begin_call_launch(w.status, 1, c->wait_status, c->stream, &c->launches), "status")) return DEFL_ERR_CUDA;
 
   // ---- stage 0: block step and Rayleigh-Ritz (lines 1-2) -------------------------------------------
   if (K > 0) {
