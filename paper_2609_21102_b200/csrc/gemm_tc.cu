@@ -582,7 +582,11 @@ __device__ __forceinline__ float transform_row(const TcParams& p, const uint32_t
 // `aux` and of the output (the same type). Each lane turns its row of the staged block into results 16 bytes at
 // a time, in place; the block then leaves with coalesced 16-byte stores. `pending` = number of cp.async groups
 // that may still be in flight after this block's own (0 or 1).
-template <int EPI, int ES, int PENDING>
+// FIX: the block on the diagonal of a symmetric output of two different operands: what was computed right of the diagonal
+// replaces what was computed left of it (lane r takes the elements (c, r), c < r, of the staged block: one row of it per load).
+// Element by element, every value stored at both places, that block alone took as long as the other three of its tile (n = 256
+// to 1000: 10 us the product instead of 5.5).
+template <int EPI, int ES, int PENDING, bool FIX = false>
 __device__ __forceinline__ void epilogue_block_fast(const TcParams& p, uint32_t taddr, uint8_t* stg, int lane, int gi_warp0,
                                                     int gj0, int bz, float alpha, float aux_scale, float& sq) {
   constexpr int rowb = 32 * ES, pp = rowb >> 4, rpi = 32 / pp, epp = 16 / ES;   // epp = elements per 16-byte piece
@@ -618,6 +622,31 @@ __device__ __forceinline__ void epilogue_block_fast(const TcParams& p, uint32_t 
     return;
   }
   __syncwarp();
+  if (FIX) {
+    uint32_t above[32];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      const uint8_t* e = stg + stage_off(c, lane / epp, rowb, pp) + (lane % epp) * ES;
+      above[c] = (ES == 2) ? (uint32_t)*reinterpret_cast<const uint16_t*>(e) : *reinterpret_cast<const uint32_t*>(e);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int pc = 0; pc < pp; ++pc) {
+      uint4* slot = reinterpret_cast<uint4*>(stg + stage_off(lane, pc, rowb, pp));
+      uint4 q4 = *slot;
+      uint32_t* w = reinterpret_cast<uint32_t*>(&q4);
+#pragma unroll
+      for (int j = 0; j < epp; ++j) {
+        const int c = pc * epp + j;
+        if (c < lane) {
+          if (ES == 4) w[j & 3] = above[c];
+          else w[(j >> 1) & 3] = (j & 1) ? __byte_perm(w[(j >> 1) & 3], above[c], 0x5410) : __byte_perm(w[(j >> 1) & 3], above[c], 0x3254);
+        }
+      }
+      *slot = q4;
+    }
+    __syncwarp();
+  }
   if (!p.transposed) {
     uint8_t* cbase = reinterpret_cast<uint8_t*>(p.C) + ((size_t)bz * p.batch_c + (size_t)gi_warp0 * p.ldc + gj0) * ES;
     // (all reads of the staged block before the first store: the compiler cannot tell that they do not alias, and one by
@@ -662,12 +691,12 @@ __device__ __forceinline__ void epilogue_block_fast(const TcParams& p, uint32_t 
 }
 
 // Which of a warp's 32-column blocks take the coalesced path: the complete ones of aligned rows in matching types, from
-// `first` on below `lim`; `diag` is the block on the diagonal that does not (-1: none).
+// `first` on below `lim`; `diag` is the block on the diagonal that is left out of the walk (-1: none).
 // A symmetric output may be the product of two DIFFERENT symmetric matrices (the apply step of the symmetric
 // filter, the Horner steps of a polynomial in the Gram matrix), whose computed (i, j) and (j, i) differ in the last
 // bits. Off the diagonal the mirror store makes the pair equal; the 32 x 32 block ON the diagonal must do the same
-// element by element, or an iterate picks up an antisymmetric part that the symmetric filter doubles at every step:
-// it takes the general path.
+// within itself, or an iterate picks up an antisymmetric part that the symmetric filter doubles at every step:
+// it is taken by itself, after the others.
 // (A product of a matrix with itself, X X^T or A A, computes (i, j) and (j, i) from the same terms in the same
 // order: its diagonal blocks are symmetric to the bit and stay on the coalesced path.)
 struct FastBlocks { int first, lim, diag; bool on; };
@@ -688,7 +717,7 @@ __device__ __forceinline__ FastBlocks fast_blocks(const TcParams& p, int gi_warp
   if (!f.on) return f;
   // symmetric output: nothing to do for blocks entirely left of the warp's rows (they are written as mirror images)
   if (p.symmetric) while (f.first + 32 <= f.lim && col0 + f.first + 31 < gi_warp0) f.first += 64;
-  // (the block on the diagonal that is left to the general path is the first block of this walk)
+  // (the block on the diagonal, where it is left out, is the first block of this walk)
   if (f.first == f.diag) f.first += 64;
   return f;
 }
@@ -774,9 +803,20 @@ __device__ __forceinline__ void epilogue_half(const TcParams& p, uint32_t taddr,
     const bool two = (EPI == EPI_STORE ? p.out_dtype : p.aux_dtype) != F32;
     if (two) c0 = epilogue_fast_blocks<EPI, 2>(p, taddr, stg, lane, gi_warp0, col0, c0, f.lim, bz, alpha, aux_scale, sq, ahead);
     else c0 = epilogue_fast_blocks<EPI, 4>(p, taddr, stg, lane, gi_warp0, col0, c0, f.lim, bz, alpha, aux_scale, sq, ahead);
-    if (f.diag >= 0)
-      epilogue_block_general<EPI>(p, taddr, f.diag, gi, gi_warp0, col0, n_eff, row_ok, vec_ok, aux_bf16, crow, cbatch, xrow,
-                                  alpha, aux_scale, sq);
+    if (f.diag >= 0) {
+      const uint32_t td = taddr + (uint32_t)f.diag;
+      const int gd = col0 + f.diag;
+      if ((EPI != EPI_STORE && EPI != EPI_POLY) || f.diag + 32 > f.lim || (f.diag & 31)) {
+        epilogue_block_general<EPI>(p, taddr, f.diag, gi, gi_warp0, col0, n_eff, row_ok, vec_ok, aux_bf16, crow, cbatch, xrow,
+                                    alpha, aux_scale, sq);
+      } else if (two) {
+        if (EPI == EPI_POLY) aux_fetch_async<2>(p, lane, gi_warp0, gd, bz, stg);
+        epilogue_block_fast<EPI == EPI_POLY ? EPI_POLY : EPI_STORE, 2, 0, true>(p, td, stg, lane, gi_warp0, gd, bz, alpha, aux_scale, sq);
+      } else {
+        if (EPI == EPI_POLY) aux_fetch_async<4>(p, lane, gi_warp0, gd, bz, stg);
+        epilogue_block_fast<EPI == EPI_POLY ? EPI_POLY : EPI_STORE, 4, 0, true>(p, td, stg, lane, gi_warp0, gd, bz, alpha, aux_scale, sq);
+      }
+    }
   }
   for (; c0 < n_eff; c0 += 64)
     epilogue_block_general<EPI>(p, taddr, c0, gi, gi_warp0, col0, n_eff, row_ok, vec_ok, aux_bf16, crow, cbatch, xrow, alpha,
