@@ -1048,8 +1048,10 @@ int defl_polar_batched_host(defl_ctx* c, const void* G_host, void* out_host, int
   if (ensure_staging(c, bytes)) return DEFL_ERR_CUDA;
   // The batch is independent matrices: it goes through in chunks, the copy of chunk i+1 to the device and of
   // chunk i-1 back to the host running (on streams of their own) while chunk i is computed. Few chunks: the small
-  // kernels of the range finder take about the same time for 12 matrices as for 48.
-  int chunks = b >= 24 ? 3 : (b >= 8 ? 2 : 1);
+  // kernels of the range finder take about the same time for 12 matrices as for 48, 300 us or more, so a second chunk pays only
+  // where it hides more than that of the copies: from 20 MB on (24 x 256 x 512, 6 MB: one chunk 627 us, two 825, three 1083;
+  // 24 x 768 x 768, 28 MB: 1670, 1462, 1556).
+  int chunks = (b < 8 || bytes < ((size_t)20 << 20)) ? 1 : (b >= 24 && bytes >= ((size_t)256 << 20)) ? 3 : 2;
   if (c->knobs.host_chunks >= 1) chunks = c->knobs.host_chunks;
   if (chunks > DEFL_HOST_MAX_CHUNKS) chunks = DEFL_HOST_MAX_CHUNKS;
   if (chunks > b) chunks = b;
