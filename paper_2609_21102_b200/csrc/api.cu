@@ -1051,7 +1051,7 @@ int defl_polar_batched_host(defl_ctx* c, const void* G_host, void* out_host, int
   // kernels of the range finder take about the same time for 12 matrices as for 48, 300 us or more, so a second chunk pays only
   // where it hides more than that of the copies: from 20 MB on (24 x 256 x 512, 6 MB: one chunk 627 us, two 825, three 1083;
   // 24 x 768 x 768, 28 MB: 1670, 1462, 1556).
-  int chunks = (b < 8 || bytes < ((size_t)20 << 20)) ? 1 : (b >= 24 && bytes >= ((size_t)256 << 20)) ? 3 : 2;
+  int chunks = (b < 8 || bytes < ((size_t)20 << 20)) ? 1 : (b >= 24 && bytes >= ((size_t)128 << 20)) ? 3 : 2;
   if (c->knobs.host_chunks >= 1) chunks = c->knobs.host_chunks;
   if (chunks > DEFL_HOST_MAX_CHUNKS) chunks = DEFL_HOST_MAX_CHUNKS;
   if (chunks > b) chunks = b;

@@ -319,3 +319,31 @@ def test_scale_estimate_of_matrices_of_low_rank(monkeypatch, form):
         assert int(info["status"]) == 0
         assert abs(float(info["theta"]) - want) <= 1e-5 * want, (n, r)
     c.close()
+
+
+@pytest.mark.parametrize("n", [136, 1100])
+def test_projection_replayed_from_a_graph(n):
+    """A captured call (its scale estimate is a cooperative launch and clears its own words) gives the eager result every time."""
+    from paper_2609_21102_b200 import binding
+    c = binding.Context(0)
+    g = torch.Generator().manual_seed(n)
+    x = torch.randn((n, n), generator=g) / np.sqrt(n)
+    X = (x + x.T).cuda()
+    v0, P = torch.randn((n,), generator=g).cuda(), torch.empty_like(X)
+    want, info = c.defl_psd_project(X, 0, None, SCHED7[:2], lanczos_start=v0, want_info=True)
+    theta = float(info["theta"])
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        c.defl_psd_project(X, 0, None, SCHED7[:2], lanczos_start=v0, out=P)
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            c.defl_psd_project(X, 0, None, SCHED7[:2], lanczos_start=v0, out=P)
+        for _ in range(3):
+            P.zero_()
+            graph.replay()
+            s.synchronize()
+            assert torch.equal(P, want)
+    assert theta > 0
+    del graph
+    c.close()
