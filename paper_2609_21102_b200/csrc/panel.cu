@@ -260,7 +260,12 @@ cudaError_t panel_apply_launch(const float* In, long long in_bs, int ld_in, cons
 // longer local sum beat three. The rotation merely steers the iteration, so its cosine and sine come from two fp32 reciprocal
 // square roots (cos 2t = |d| / sqrt(d^2 + g^2), d the difference of the squared norms and g twice the inner product, both over
 // the power of two above their sum) and are scaled in fp64 to c^2 + s^2 = 1; tests and angle are worked out side by side,
-// without branches. A sweep whose largest cosine was below 1e-7 is the last one: convergence is quadratic there.
+// without branches. A sweep is the last one when every rotation it made met a cosine below 1e-7 and turned by less than 1e-6: a
+// rotation by s of columns whose cosines with a third are c leaves that third at most s c, 1e-13 at a time and 6e-12 over the 63
+// rotations a column of the widest core takes part in, below the 1e-11 of the rule that ends only where nothing turns (and takes
+// 0.2 sweeps of 10 more). The cosine alone is not enough: values closer than 1e-7 of the shifted norms (the small ones beside
+// large ones of a signed core) turn by an angle of order one at any cosine, and mix couplings of that size back in
+// (values of 1e6 beside a bulk in [-1, 1], l = 24, restated in fp64: small values off by 2.5e-2 of themselves, 5e-7 with the rule).
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -314,7 +319,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
   __shared__ double nrm2[MAX_L + 1];  // squared column norms of A, carried along by the rotations
   __shared__ int order[MAX_L];
   __shared__ float sorted[MAX_L];
-  __shared__ int large[2];            // per parity of the sweep: a rotation with a cosine above 1e-7 was made
+  __shared__ int large[2];            // per parity of the sweep: a rotation with a cosine above 1e-7 or by more than 1e-6 was made
   const int bz = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const double* pb = partial + (long long)bz * nchunk * l * l;
   for (int e = tid; e < (l + 1) * ls; e += JAC_THREADS) A[e] = 0.0;
@@ -436,7 +441,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_eig_kernel(const double* _
           for (int i = 0; i < NR; ++i) { ap[4 * i] = c * x[i] - sn * y[i]; aq[4 * i] = sn * x[i] + c * y[i]; }
           const double moved = sn * fma(2.0 * c, gamma, -sn * d);
           if (sub == 0) { nrm2[p] = alpha - moved; nrm2[q] = beta + moved; }
-          big |= gg > 1e-14 * ab;
+          big |= gg > 1e-14 * ab || fabs(sn) > 1e-6;
         }
         sync();
       }

@@ -259,6 +259,32 @@ def test_small_ritz_values_beside_large_ones(ctx, K):
     assert int(info["status"]) == 0
 
 
+@pytest.mark.parametrize("K", [17, 24, 48, 64])
+def test_small_ritz_values_beside_large_ones_of_a_mixed_core(ctx, K):
+    """A symmetric block B beside a multiple of the identity and the basis of the first unit vectors: the Rayleigh quotient is B to
+    the bit. B has a third of its eigenvalues at +-1e5 and the rest in +-[0.1, 1], in a basis 1e-2 off the unit vectors, so its
+    small values are reached only through rotations among columns whose norms agree to 1e-6. Each value is within the rounding
+    to fp32, 2^-24, and what couplings below 1e-11 leave of it: 4.3e-8 at most over these draws restated in fp64."""
+    from paper_2609_21102_b200 import binding
+    g = torch.Generator().manual_seed(K)
+    n, big = K + 4 - K % 4, K // 3
+    for _ in range(6):
+        sign = 1.0 - 2.0 * torch.randint(0, 2, (K,), generator=g).double()
+        lam = sign * (0.1 + 0.9 * torch.rand(K, generator=g, dtype=torch.float64))
+        lam[:big] = sign[:big] * 1e5 * (0.5 + 0.5 * torch.rand(big, generator=g, dtype=torch.float64))
+        q = torch.linalg.qr(torch.eye(K, dtype=torch.float64) + 1e-2 * torch.randn((K, K), generator=g, dtype=torch.float64))[0]
+        B = ((q * lam) @ q.T).float()
+        B = torch.triu(B) + torch.triu(B, 1).T
+        X = 0.5 * torch.eye(n)
+        X[:K, :K] = B
+        _, info = ctx.defl_psd_project(X.cuda(), 4, torch.eye(n, K).cuda(), SCHED7[:1], gamma=1.1, seed=1, want_info=True)
+        want = torch.linalg.eigvalsh(B.double())
+        got = info["lam"].double().cpu().sort().values
+        # (the panel that becomes the next basis, Z V = B, has a condition number of 1e6, past its fp32 Gram sums: a shifted factor)
+        assert (int(info["status"]) & ~binding.ST_CHOL_SHIFT) == 0
+        assert float(((got - want).abs() / want.abs()).max()) <= 2.0 ** -24 + 1e-7
+
+
 @pytest.mark.parametrize("form", ["0", "2"])
 @pytest.mark.parametrize("n", [1, 2, 3, 17, 100, 203, 1000, 1535, 1537, 2051, 2600])
 def test_scale_estimate_in_every_form(monkeypatch, form, n):
