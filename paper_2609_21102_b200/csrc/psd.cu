@@ -107,7 +107,10 @@ static cudaError_t symv_launch(const float* A, const float* x, float* y, int n, 
 // ---------------------------------------------------------------------------------------------
 // Lanczos on R^2 with full reorthogonalisation (Appendix E.1, "Normalization scale"). One CTA does the vector work of a step:
 //   alpha_j = q_j . w;  w -= Q_j (Q_j^T w) twice;  beta_j = ||w||;  q_{j+1} = w / beta_j
-// State in device memory: Q[steps, n], T[steps, steps] (dense tridiagonal, fp64), done flag.
+// w is scaled by the power of two that brings alpha_0 to [1, 2): it has the size of ||R||^2, and once the Krylov space is
+// exhausted 1e-12 of it, which fp32 holds with few bits or not at all from ||R|| = 1e-12 on (theta of matrices of low rank was up to
+// 30 times too large at 1e-13). Exact, so nothing moves at ordinary norms.
+// State in device memory: Q[steps, n], T[steps, steps] (dense tridiagonal, fp64, scaled), the scale, done flag.
 // ---------------------------------------------------------------------------------------------
 struct LanczosState {
   float* Q;        // [steps, n]
@@ -115,8 +118,14 @@ struct LanczosState {
   float* w;        // [n] work vector (R R q_j)
   float* t;        // [n] work vector (R q_j)
   int* done;       // set when the recurrence broke down (beta ~ 0); later steps become no-ops
-  double* beta_prev;
+  double* scale;   // of w and T
 };
+
+// the power of two that brings a positive a to [1, 2)
+__device__ __forceinline__ double lz_unit(double a) {
+  if (!(a > 1e-290 && a < 1e290)) return 1.0;
+  return __longlong_as_double((2046ll - ((__double_as_longlong(a) >> 52) & 0x7ff)) << 52);
+}
 
 __device__ __forceinline__ double lz_warp_sum(double v) {
 #pragma unroll
@@ -144,7 +153,7 @@ __global__ void __launch_bounds__(1024) lanczos_init_kernel(const float* __restr
   const double nv = sqrt(block_sum(a, red));
   for (int i = threadIdx.x; i < n; i += blockDim.x) s.Q[i] = (nv > 0.0) ? (float)((double)v0[i] / nv) : 0.f;
   for (int i = threadIdx.x; i < steps * steps; i += blockDim.x) s.T[i] = 0.0;
-  if (threadIdx.x == 0) { *s.done = (nv > 0.0) ? 0 : 1; *s.beta_prev = 0.0; }
+  if (threadIdx.x == 0) { *s.done = (nv > 0.0) ? 0 : 1; *s.scale = 1.0; }
 }
 
 __global__ void __launch_bounds__(1024) lanczos_step_kernel(int j, int n, int steps, LanczosState s) {
@@ -156,7 +165,14 @@ __global__ void __launch_bounds__(1024) lanczos_step_kernel(int j, int n, int st
   double a = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) a += (double)q[i] * (double)s.w[i];
   a = block_sum(a, red);
-  if (threadIdx.x == 0) s.T[j * steps + j] = a;
+  const double unit = j == 0 ? lz_unit(a) : *s.scale;
+  a *= unit;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) s.w[i] = (float)((double)s.w[i] * unit);
+  if (threadIdx.x == 0) {
+    s.T[j * steps + j] = a;
+    if (j == 0) *s.scale = unit;
+  }
+  __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   // w -= Q_j (Q_j^T w), twice; again where less than 1e-5 of w is left (see lanczos_kernel)
   double b = 0.0, before = 0.0;
@@ -348,21 +364,21 @@ __global__ void lanczos_ritz_kernel(int n, int steps, const float* __restrict__ 
   v[i] = (float)a;
 }
 
-// theta = sqrt(max(rho, 0) + ||w - rho v||), inv_theta = 1/theta (0 + status bit when theta is not a positive number)
-__global__ void __launch_bounds__(1024) lanczos_theta_kernel(int n, const float* __restrict__ rho_p,
+// theta = sqrt((max(rho, 0) + ||scale w - rho v||) / scale), inv_theta = 1/theta (0 + status bit when theta is not a positive number)
+__global__ void __launch_bounds__(1024) lanczos_theta_kernel(int n, const float* __restrict__ rho_p, const double* __restrict__ scale,
                                                              const float* __restrict__ v, const float* __restrict__ w,
                                                              float* theta, float* inv_theta, int* status) {
   pdl_wait();
   __shared__ double red[32];
-  const double rho = (double)rho_p[0];
+  const double rho = (double)rho_p[0], unit = *scale;
   double a = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double d = (double)w[i] - rho * (double)v[i];
+    const double d = (double)w[i] * unit - rho * (double)v[i];
     a += d * d;
   }
   a = sqrt(block_sum(a, red));
   if (threadIdx.x == 0) {
-    const double th = sqrt((rho > 0.0 ? rho : 0.0) + a);
+    const double th = sqrt(((rho > 0.0 ? rho : 0.0) + a) / unit);
     const bool ok = th > 0.0 && isfinite(th);
     theta[0] = (float)th;
     inv_theta[0] = ok ? (float)(1.0 / th) : 0.f;
@@ -378,7 +394,7 @@ __global__ void __launch_bounds__(1024) lanczos_theta_kernel(int n, const float*
 // meet across CTAs are two vectors and a few dozen partial sums per step:
 //   step j:  t = A q_j, partial sums of c = (A Q_j)^T t  |  w = A t - Q_j c, partial sums of c' = Q_j^T w  |
 //            w -= Q_j c', partial sum of ||w||^2, w  |  q_{j+1} = w / ||w||
-// c = Q_j^T A t is taken from the slices of A Q_j that the earlier steps left, before t itself has met; alpha_j is c_j. The
+// w, and so the Lanczos matrix, is scaled by a power of two as in the step form. c = Q_j^T A t is taken from the slices of A Q_j that the earlier steps left, before t itself has met; alpha_j is c_j. The
 // second projection is measured on what the first one left, and where less than 1e-5 of w remains a third
 // one (and a fourth) is measured on what the second left: the basis is orthonormal to fp32 only, and once the Krylov space is
 // exhausted and w is rounding, two projections leave as much of the basis in w as there is rounding. Of 300 matrices of rank
@@ -695,6 +711,7 @@ __global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const __grid_con
   for (int r = tid; r < mine; r += LZ_THREADS) Qs[r] = (float)((double)__ldg(p.v0 + first + r) * inv);
 
   int other = 1;
+  double unit = 1.0;                          // scale of w and of the Lanczos matrix (the same in every CTA)
   for (int j = 0; started && j < steps; ++j) {
     const uint32_t tag = 4u * (uint32_t)j + 1u;
     multiply();                               // t = A q_j
@@ -706,9 +723,10 @@ __global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const __grid_con
     const bool ok = gather(0, tag + (j == 0 ? p.hold : 0u));
     multiply();                               // A t
     if (!total(0, j, tag, ok)) return;
-    if (tid == 0) al[j] = coef[0][j];
+    if (j == 0) unit = lz_unit(coef[0][0]);
+    if (tid == 0) al[j] = coef[0][j] * unit;
     if (j + 1 == steps) break;
-    rows(true, coef[0], j, [&](int r, double v) { wl[r] = (float)v; });
+    rows(true, coef[0], j, [&](int r, double v) { wl[r] = (float)(v * unit); });
     double b = 0.0, limit2 = 0.0;
     for (uint32_t again = 0;; ++again) {
       dots(Qs, wl, j);
@@ -729,22 +747,24 @@ __global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const __grid_con
       for (int g = lane; g < G; g += 32) b2 += share[g];
       b2 = lz_warp_sum(b2);                   // (the same in every warp)
       b = sqrt(b2);
-      if (again == 0) limit2 = 1e-10 * before2;
+      if (again == 0) limit2 = 1e-10 * before2 * unit * unit;
       if (again == 2 || !(b2 < limit2)) break;
       limit2 = 1e-10 * b2;
     }
     if (!(b > 1e-12 * fabs(al[0]))) { other = 0; break; }      // the Krylov space ends here (the same decision in every CTA)
     if (tid == 0) be[j] = b;
-    const float ib = (float)(1.0 / b);
+    // one rounding per value: 1 / b in two fp32 terms (b lies in 1e-12 .. n here; 16 lanes a cycle convert to fp64)
+    const double ib = 1.0 / b;
+    const float ih = (float)ib, il = (float)(ib - (double)ih);
 #pragma unroll
     for (int m = 0; m < P; ++m)
 #pragma unroll
-      for (int u = 0; u < 4; ++u) x[m][u] *= ib;
-    for (int r = tid; r < mine; r += LZ_THREADS) Qs[(j + 1) * R + r] = wl[r] * ib;
+      for (int u = 0; u < 4; ++u) x[m][u] = fmaf(x[m][u], ih, x[m][u] * il);
+    for (int r = tid; r < mine; r += LZ_THREADS) Qs[(j + 1) * R + r] = fmaf(wl[r], ih, wl[r] * il);
   }
   __syncthreads();
 
-  // largest Ritz pair (rho, v), theta = sqrt(max(rho, 0) + ||A A v - rho v||)
+  // largest Ritz pair (rho, v), theta = sqrt((max(rho, 0) + ||unit A A v - rho v||) / unit)
   const double rho = (double)(float)tridiag_top(al, be, steps, y, tri);
   const uint32_t end = 4u * (uint32_t)steps + 1u;
   // (others may still be reading the words of the meeting that the loop was left after: t's, or w's after a breakdown. The
@@ -763,7 +783,7 @@ __global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const __grid_con
   if (warp == 0) publish(other ^ 1, end);
   if (!__syncthreads_and(gather(other ^ 1, end))) return;
   multiply();
-  rows(true, nullptr, 0, [&](int r, double v) { wl[r] = (float)(v - rho * (double)vs[r]); });
+  rows(true, nullptr, 0, [&](int r, double v) { wl[r] = (float)(v * unit - rho * (double)vs[r]); });
   if (warp == 0) {
     double d = 0.0;
     for (int r = lane; r < mine; r += 32) d = fma((double)wl[r], (double)wl[r], d);
@@ -778,7 +798,7 @@ __global__ void __launch_bounds__(LZ_THREADS, 1) lanczos_kernel(const __grid_con
     for (int g = lane; g < G; g += 32) d += share[g];
     d = sqrt(lz_warp_sum(d));
     if (lane == 0) {
-      const double th = sqrt((rho > 0.0 ? rho : 0.0) + d);
+      const double th = sqrt(((rho > 0.0 ? rho : 0.0) + d) / unit);
       const bool good = th > 0.0 && isfinite(th);
       p.theta[0] = (float)th;
       p.inv_theta[0] = good ? (float)(1.0 / th) : 0.f;
@@ -948,7 +968,7 @@ struct PsdWs {
   double* gram;     // [nchunk, K, K]
   float* Rinv; float* E; float* Es; float* lam; float* coef;   // [K,K] x3, [K], [K]
   float* Q; double* T; float* lw; float* lt; float* lv; float* lE; float* lrho;   // Lanczos state
-  int* done; double* beta_prev;
+  int* done; double* lscale;
   unsigned long long* lwords;   // what the CTAs of the one-launch estimate exchange
   double* npart; float* theta; float* inv_theta; float* dummy; float* rscale;
   int* status;
@@ -983,7 +1003,7 @@ static PsdWs carve_psd(void* base, int n, int K) {
   w.Q = cv.take<float>((size_t)S * n); w.T = cv.take<double>(S * S);
   w.lw = cv.take<float>(n); w.lt = cv.take<float>(n); w.lv = cv.take<float>(n);
   w.lE = cv.take<float>(S * S); w.lrho = cv.take<float>(S);
-  w.done = cv.take<int>(1); w.beta_prev = cv.take<double>(1);
+  w.done = cv.take<int>(1); w.lscale = cv.take<double>(1);
   w.lwords = cv.take<unsigned long long>(lanczos_words(n));
   w.npart = cv.take<double>(1184);
   w.theta = cv.take<float>(1); w.inv_theta = cv.take<float>(1); w.dummy = cv.take<float>(S * S); w.rscale = cv.take<float>(1);
@@ -1015,7 +1035,7 @@ static int estimate_scale(defl_ctx* c, const float* A, int n, int norm_mode, con
   }
   // one launch per step: n above 8192
   LanczosState s;
-  s.Q = w.Q; s.T = w.T; s.w = w.lw; s.t = w.lt; s.done = w.done; s.beta_prev = w.beta_prev;
+  s.Q = w.Q; s.T = w.T; s.w = w.lw; s.t = w.lt; s.done = w.done; s.scale = w.lscale;
   launch_kernel(lanczos_init_kernel, 1, 1024, 0, c->stream, start, n, steps, s);
   ++c->launches;
   if (ctx_fail(c, cudaGetLastError(), "lanczos init")) return DEFL_ERR_CUDA;
@@ -1035,7 +1055,7 @@ static int estimate_scale(defl_ctx* c, const float* A, int n, int norm_mode, con
   if (ctx_fail(c, cudaGetLastError(), "ritz vector")) return DEFL_ERR_CUDA;
   if (ctx_fail(c, symv_launch(A, w.lv, w.lt, n, nullptr, c->stream, &c->launches), "symv")) return DEFL_ERR_CUDA;
   if (ctx_fail(c, symv_launch(A, w.lt, w.lw, n, nullptr, c->stream, &c->launches), "symv")) return DEFL_ERR_CUDA;
-  launch_kernel(lanczos_theta_kernel, 1, 1024, 0, c->stream, n, w.lrho, w.lv, w.lw, w.theta, w.inv_theta, w.status);
+  launch_kernel(lanczos_theta_kernel, 1, 1024, 0, c->stream, n, w.lrho, w.lscale, w.lv, w.lw, w.theta, w.inv_theta, w.status);
   ++c->launches;
   if (ctx_fail(c, cudaGetLastError(), "theta")) return DEFL_ERR_CUDA;
   return DEFL_OK;

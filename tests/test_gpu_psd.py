@@ -347,6 +347,28 @@ def test_scale_estimate_of_matrices_of_low_rank(monkeypatch, form):
     c.close()
 
 
+@pytest.mark.parametrize("form", ["0", "2"])
+@pytest.mark.parametrize("scale", [1e-12, 1e-14, 1e-16])
+def test_scale_estimate_of_tiny_matrices_of_low_rank(monkeypatch, form, scale):
+    """What is left of w once the Krylov space is exhausted is 1e-12 of the norm's square and less, below the fp32 numbers here: theta is
+    the norm within 1e-5 of it all the same, as at ordinary size."""
+    from paper_2609_21102_b200 import binding
+    monkeypatch.setenv("DEFL_LANCZOS_FORM", form)
+    c = binding.Context(0)
+    g = torch.Generator().manual_seed(77)
+    for n, r in [(20, 1), (57, 2), (128, 3), (203, 2), (240, 7), (299, 5)] * 4:
+        u = torch.linalg.qr(torch.randn((n, r), generator=g, dtype=torch.float64))[0]
+        lam = scale * 10.0 ** (torch.rand(r, generator=g, dtype=torch.float64) * 2.0 - 1.0)
+        lam[::2] *= -1.0
+        X = ((u * lam) @ u.T).float()
+        X = 0.5 * (X + X.T)
+        _, info = c.defl_psd_project(X.cuda(), 0, None, SCHED7[:1], lanczos_start=torch.randn((n,), generator=g).cuda(), want_info=True)
+        want = float(lam.abs().max())
+        assert int(info["status"]) == 0
+        assert abs(float(info["theta"]) - want) <= 1e-5 * want, (n, r)
+    c.close()
+
+
 @pytest.mark.parametrize("n", [136, 1100])
 def test_projection_replayed_from_a_graph(n):
     """A captured call (its scale estimate is a cooperative launch and clears its own words) gives the eager result every time."""
