@@ -898,7 +898,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_tc_kernel(const __grid_co
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
   // Barriers, tensor memory and the descriptor fetch above overlap the end of the previous kernel, and so does what each
-  // role works out before its first access to global memory, where it waits for that kernel (pdl_wait): a new launch finds its
+  // role works out before its first access to global memory or its first bounded wait, where it waits for that kernel (pdl_wait): a new launch finds its
   // parameters and code in no cache near the SM, and with the wait here the first copies left 3500-5000 cycles after it.
   pdl_launch();
 
@@ -947,7 +947,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_tc_kernel(const __grid_co
       // per pair that tells it to stop; whoever draws the last one puts the counter back to zero
       const long long last_ticket = (total_tiles > npairs ? total_tiles - npairs : 0) + npairs - 1;
       unsigned int ticket = 0;
-      if (dynamic || aux_prefetch) pdl_wait();
+      bool waited = dynamic || aux_prefetch;
+      if (waited) pdl_wait();
       for (int it = 0;; ++it) {
         long long tile;
         if (!dynamic) {
@@ -1005,9 +1006,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_tc_kernel(const __grid_co
         const int b_loc0 = PAIR ? (int)rank * (t.n_eff >> 1) : 0;                // a pair: this CTA's half of the columns
         const int b_mn0 = t.tn * BN + b_loc0;
         bool live = true;
-        if (it == 0) {
+        if (!waited) {
           touch(a_mn0, b_mn0, my_dst_off, my_tm0, my_tm1, full0_sig, kblocks0, kblocks1, kreal0, kreal1, tx_bytes, tx_sub_bytes);
           pdl_wait();
+          waited = true;
         }
         for (int seg = 0; seg < nseg && live; ++seg) {
           const int nkb = seg ? kblocks1 : kblocks0;
@@ -1077,9 +1079,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_tc_kernel(const __grid_co
       };
       const int prep = total_kblocks >= 2 ? total_kblocks - 2 : 0;
       int it = 0;
+      // (this thread touches no global memory, but the limit of its waits must not run while earlier kernels do)
+      if (dynamic) pdl_wait();
       long long nxt = next_tile(it);
       TileInfo tnx;
       if (nxt >= 0) tnx = tile_info(p, nxt);
+      if (!dynamic) pdl_wait();
       while (nxt >= 0) {
         const TileInfo t = tnx;
         ++it;

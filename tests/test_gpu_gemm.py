@@ -215,6 +215,32 @@ def test_bounded_wait_runs_out_and_is_reported(monkeypatch):
     ctx.close()
 
 
+def test_wait_limit_does_not_count_earlier_products(monkeypatch):
+    """Products of one tile and a very deep K leave most of the chip free, so the next ones are resident while the first runs.
+    The limit of their waits starts when their own work may: eight in a row, each shorter than the limit of 1.6 times
+    one of them, finish without an event, and their results are the first one's."""
+    from paper_2609_21102_b200 import binding
+    K = 1 << 19
+    A, B = _mk(1, 256, K, torch.bfloat16, 43), _mk(1, 256, K, torch.bfloat16, 44)
+    free = binding.Context(0)
+    product = lambda c: c.defl_debug_gemm(A, B, False, True, engine=binding.ENGINE_TENSOR, out_dtype=torch.float32)
+    want = product(free)
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    start.record()
+    for _ in range(8):
+        product(free)
+    end.record()
+    torch.cuda.synchronize()
+    one = start.elapsed_time(end) / 8
+    free.close()
+    monkeypatch.setenv("DEFL_TC_WAIT_MS", str(int(1.6 * one) + 1))
+    c = binding.Context(0)
+    outs = [product(c) for _ in range(8)]
+    assert c.defl_device_wait_status() == 0
+    assert all(torch.equal(o, want) for o in outs)
+    c.close()
+
+
 @pytest.mark.parametrize("engine_name", ["simt", "tensor"])
 @pytest.mark.parametrize("n,K", [(24, 24), (72, 200), (256, 64), (264, 264), (328, 1000), (640, 640)])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.float16])
