@@ -308,6 +308,31 @@ def test_scale_estimate_in_every_form(monkeypatch, form, n):
     c.close()
 
 
+@pytest.mark.parametrize("n", [4100, 6147, 8192, 8196])
+def test_scale_estimate_of_large_matrices(monkeypatch, n):
+    """Up to sixteen columns per thread, some of them past n, and most rows read from global memory (at 4100 and 8192 in groups of
+    which a part is resident; at 6147 at any address); 8196 is past one launch. Against the form of one launch per step: fp32
+    products of n terms on either side, sqrt(n) 2^-24 ||A||^2 on a Ritz value of A^2, half of it on theta. And
+    against the norm of a bulk of radius one (entries of variance 1 / (4 n)) with a direction at -2, which is 2 + 1/8 up to a few 1 / sqrt(n)."""
+    from paper_2609_21102_b200 import binding
+    g = torch.Generator(device="cuda").manual_seed(n)
+    X = torch.randn((n, n), generator=g, device="cuda") / np.sqrt(8.0 * n)
+    X = X + X.T
+    u = torch.nn.functional.normalize(torch.randn((n,), generator=g, device="cuda"), dim=0)
+    X -= 2.0 * u[:, None] * u[None, :]
+    v0 = torch.randn((n,), generator=g, device="cuda")
+    theta = []
+    for form in ("0", "2"):
+        monkeypatch.setenv("DEFL_LANCZOS_FORM", form)
+        c = binding.Context(0)
+        _, info = c.defl_psd_project(X, 0, None, SCHED7[:1], lanczos_start=v0, want_info=True)
+        assert int(info["status"]) == 0
+        theta.append(float(info["theta"]))
+        c.close()
+    assert abs(theta[0] - theta[1]) <= np.sqrt(n) * 2.0 ** -24 * theta[1]
+    assert abs(theta[0] - 2.125) <= 3.0 / np.sqrt(n)
+
+
 @pytest.mark.parametrize("form", ["0", "2"])
 def test_scale_estimate_of_a_matrix_of_rank_two(monkeypatch, form):
     """The Krylov space of A^2 ends after three steps: what is left of w is rounding (or nothing, for the unit vectors)."""
