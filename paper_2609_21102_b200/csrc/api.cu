@@ -1038,6 +1038,27 @@ int defl_muon_step_batched(defl_ctx* c, void* W, int w_dtype, void* Mom, const v
   return polar_core(c, D, c->stage_out, b, m, n, dtype, k, oversample, power_iters, coeff_schedule, L, opts, info, &upd);
 }
 
+// Few chunks: the small kernels of the range finder take about the same time for 12 matrices as for 48, 300 us or more, so another
+// chunk pays only where it hides more than that of the copies; without a range finder that is from a few MB on. fp32 storage takes the
+// third chunk earlier, where its FMA products gain from it as often as they lose (by how their tiles fall into waves: of eleven batches
+// from 20 to 216 MB three chunks were between 13 % faster and 22 % slower than two, equal on average). us with one, two and three
+// chunks, k = 8 unless stated:
+//   bf16       12 MB, 24 x 512 x 512       936   938  1144        15 MB, 16 x 768 x 640     1087  1041  1230
+//              27 MB, 24 x 768 x 768      1682  1480  1570        60 MB, 24 x 1024 x 1280   3423  2536  2650
+//              72 MB, 24 x 1024 x 1536    4097  3059  2936        96 MB, 48 x 1024 x 1024   5452  3969  3583
+//   bf16, k 0   3 MB, 12 x 256 x 512       329   388   489        18 MB, 24 x 512 x 768     1028   837   860
+//              27 MB, 24 x 768 x 768      1520  1148  1114        96 MB, 48 x 1024 x 1024   5075  3618  3167
+//   fp32        3 MB, 24 x 128 x 256       442   614   730        16 MB, 24 x 333 x 517     2358  2407  2553
+//              18 MB, 24 x 384 x 512      2218  2027  2548        24 MB, 24 x 512 x 512     3423  3547  3174
+//              22 MB, 24 x 384 x 640      2614  2381  2894        36 MB, 36 x 512 x 512     4995  4730  5030
+//              48 MB, 24 x 512 x 1024     5852  5670  4917       108 MB, 24 x 768 x 1536   15986 14620 14695
+//   fp32, k 0   6 MB, 12 x 256 x 512       795   639   742        12 MB, 24 x 256 x 512     1165  1310   933
+static int host_chunks(int b, size_t bytes, int dtype, int k) {
+  const bool fp32 = dtype == DEFL_F32;
+  const size_t mb = bytes >> 20, two = k > 0 ? 14 : 4, three = k > 0 ? (fp32 ? 20 : 64) : (fp32 ? 4 : 24);
+  return (b < 8 || mb < two) ? 1 : (b >= 24 && mb >= three) ? 3 : 2;
+}
+
 int defl_polar_batched_host(defl_ctx* c, const void* G_host, void* out_host, int b, int m, int n, int dtype, int k,
                             int oversample, int power_iters, const float* coeff_schedule, int L,
                             const defl_opts* opts) {
@@ -1047,11 +1068,8 @@ int defl_polar_batched_host(defl_ctx* c, const void* G_host, void* out_host, int
   const size_t bytes = (size_t)b * m * n * dtype_size(dtype);
   if (ensure_staging(c, bytes)) return DEFL_ERR_CUDA;
   // The batch is independent matrices: it goes through in chunks, the copy of chunk i+1 to the device and of
-  // chunk i-1 back to the host running (on streams of their own) while chunk i is computed. Few chunks: the small
-  // kernels of the range finder take about the same time for 12 matrices as for 48, 300 us or more, so a second chunk pays only
-  // where it hides more than that of the copies: from 20 MB on (24 x 256 x 512, 6 MB: one chunk 627 us, two 825, three 1083;
-  // 24 x 768 x 768, 28 MB: 1670, 1462, 1556).
-  int chunks = (b < 8 || bytes < ((size_t)20 << 20)) ? 1 : (b >= 24 && bytes >= ((size_t)128 << 20)) ? 3 : 2;
+  // chunk i-1 back to the host running (on streams of their own) while chunk i is computed.
+  int chunks = host_chunks(b, bytes, dtype, k);
   if (c->knobs.host_chunks >= 1) chunks = c->knobs.host_chunks;
   if (chunks > DEFL_HOST_MAX_CHUNKS) chunks = DEFL_HOST_MAX_CHUNKS;
   if (chunks > b) chunks = b;

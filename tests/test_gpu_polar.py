@@ -327,3 +327,26 @@ def test_poly_terms_argument_errors(ctx):
     assert e.value.code == -1
     with pytest.raises(ValueError):
         ctx.defl_polar_batched(G, 0, 0, 0, [[1.0, 0.0, 0.0]] * 2, poly_terms=4)      # three coefficients given, four wanted
+
+
+@pytest.mark.parametrize("b,m,n,dtype,k,chunks", [
+    (7, 1024, 1088, torch.bfloat16, 4, 1), (8, 1024, 800, torch.bfloat16, 4, 1), (8, 1024, 1088, torch.bfloat16, 4, 2),
+    (24, 1024, 1296, torch.bfloat16, 4, 2), (24, 1024, 1376, torch.bfloat16, 4, 3), (23, 1024, 1500, torch.bfloat16, 4, 2),
+    (24, 256, 320, torch.bfloat16, 0, 1), (24, 512, 768, torch.bfloat16, 0, 2), (24, 512, 1040, torch.bfloat16, 0, 3),
+    (24, 256, 512, torch.float32, 4, 1), (24, 256, 704, torch.float32, 4, 2), (24, 256, 896, torch.float32, 4, 3),
+    (24, 128, 256, torch.float32, 0, 1), (8, 256, 640, torch.float32, 0, 2), (24, 128, 384, torch.float32, 0, 3)])
+def test_host_buffers_go_through_in_the_measured_number_of_chunks(ctx, b, m, n, dtype, k, chunks):
+    """Both sides of every threshold: a call launches what its chunks launch as calls of their own."""
+    from paper_2609_21102_b200 import binding
+    sched = [list(binding.MUON_QUINTIC)]
+    G = torch.randn((b, m, n), generator=torch.Generator().manual_seed(b)).to(dtype).pin_memory()
+    per = (b + chunks - 1) // chunks
+    dev = G[:per].cuda()
+    want = 0
+    for b0 in range(0, b, per):
+        before = ctx.defl_launch_count()
+        ctx.defl_polar_batched(dev[:min(per, b - b0)], k, 4 if k else 0, 1, sched, seed=3)
+        want += ctx.defl_launch_count() - before
+    before = ctx.defl_launch_count()
+    ctx.defl_polar_batched_host(G, torch.empty_like(G).pin_memory(), k, 4 if k else 0, 1, sched, seed=3)
+    assert ctx.defl_launch_count() - before == want
