@@ -388,13 +388,15 @@ __global__ void __launch_bounds__(1024) lanczos_theta_kernel(int n, const float*
 
 // ---------------------------------------------------------------------------------------------
 // The whole scale estimate in one launch. As 63 dependent launches (two matrix-vector products and one single-CTA
-// reorthogonalisation per step) it is bound by launches and by one SM's memory path: 325 us at n = 1024, about 700 at 4096.
+// reorthogonalisation per step) it is bound by launches and by one SM's memory path: 303 us at n = 1024, 835 at 4096.
 // Here every CTA owns `rows` consecutive rows of A and of all vectors, and every thread up to 4 P columns: as many of the CTA's
 // rows of A as fit stay in shared memory for the whole run, its slices of the Lanczos basis Q and of A Q too, and what has to
 // meet across CTAs are two vectors and a few dozen partial sums per step:
 //   step j:  t = A q_j, partial sums of c = (A Q_j)^T t  |  w = A t - Q_j c, partial sums of c' = Q_j^T w  |
 //            w -= Q_j c', partial sum of ||w||^2, w  |  q_{j+1} = w / ||w||
-// w, and so the Lanczos matrix, is scaled by a power of two as in the step form. c = Q_j^T A t is taken from the slices of A Q_j that the earlier steps left, before t itself has met; alpha_j is c_j. The
+// w, and so the Lanczos matrix, is scaled by a power of two as in the step form. c = Q_j^T A t is taken from the slices of A Q_j that the earlier steps left, before t itself has met; alpha_j is c_j. (A Q and t
+// are rounded to fp32 there, as w is in the step form: against the same algorithm in fp64 theta is off by at most 9.6e-8 in either
+// form, its own rounding included, over 288 matrices of n = 100 to 2560.) The
 // second projection is measured on what the first one left, and where less than 1e-5 of w remains a third
 // one (and a fourth) is measured on what the second left: the basis is orthonormal to fp32 only, and once the Krylov space is
 // exhausted and w is rounding, two projections leave as much of the basis in w as there is rounding. Of 300 matrices of rank

@@ -122,10 +122,10 @@ def test_half_iterate_overflow_is_reported(ctx):
 
 @pytest.mark.parametrize("root", [0, 2])
 def test_scale_estimate_whose_wait_runs_out_is_reported_and_takes_nothing_from_an_earlier_call(monkeypatch, root):
-    """The grid form of the scale estimate with a meeting that waits for one arrival too many and a limit of 2 ms: the call
+    """The scale estimate in one launch, whose first meeting waits for a number that never comes, with a limit of 2 ms: the call
     returns, says so, and its scale is zero whatever estimate the context made before. The context stays usable."""
     from paper_2609_21102_b200 import binding
-    for k, v in (("DEFL_LANCZOS_FORM", "1"), ("DEFL_LANCZOS_HOLD", "1"), ("DEFL_TC_WAIT_MS", "2")):
+    for k, v in (("DEFL_LANCZOS_FORM", "0"), ("DEFL_LANCZOS_HOLD", "1"), ("DEFL_TC_WAIT_MS", "2")):
         monkeypatch.setenv(k, v)
     c = binding.Context(0)
     n, K = 136, 6

@@ -32,7 +32,7 @@ def _psd(n, K=8):
                                      (lambda: _psd(1000), lambda: _psd(1024)),
                                      (lambda: _psd(2048), lambda: _psd(4096)),
                                      (lambda: _polar(4, 256, 384), lambda: _psd(640))],
-                         ids=["polar_1600", "polar_768_1024", "psd_cluster", "psd_grid", "polar_psd"])
+                         ids=["polar_1600", "polar_768_1024", "psd_sums_by_all", "psd_sums_by_one", "polar_psd"])
 def test_two_contexts_on_two_threads(one, two):
     calls = [one(), two()]
     alone = []
